@@ -404,13 +404,11 @@ k_adj_terminal(const T* __restrict__ x, const T* __restrict__ y, const T* __rest
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_adj_spectral(const cpx<T>* __restrict__ ghat, cpx<T>* __restrict__ abar, cpx<T>* __restrict__ spec, int H,
-               SpecParams sp) {
+               SpecConst<T> sk) {
   const int nh = H / 2 + 1;
   const size_t S = (size_t)H * H * nh;
-  const T two_pi_L = T(6.283185307179586 / sp.L);
-  const T filt = sp.H0 > 0 ? T(-2.0 * 9.869604401089358 / (sp.H0 * sp.H0)) : T(0);
-  const T tau_eps = T(sp.tau / sp.eps), eps_tau = T(sp.eps / sp.tau), k2 = T(sp.k2), tau = T(sp.tau);
-  const T inv_L3 = T(sp.inv_L3);
+  const T two_pi_L = sk.two_pi_L, filt = sk.filt, inv_L3 = sk.inv_L3;
+  const T tau_eps = sk.tau_eps, eps_tau = sk.eps_tau, k2 = sk.k2, tau = sk.tau;
   // 32-bit index arithmetic (S < 2^31 for H <= 256; a 64-bit division costs
   // several times more than the element's own work)
   const unsigned S32 = (unsigned)S, unh = (unsigned)nh, uH = (unsigned)H;
@@ -425,14 +423,14 @@ k_adj_spectral(const cpx<T>* __restrict__ ghat, cpx<T>* __restrict__ abar, cpx<T
     const T q2 = T(qx * qx + qy * qy + qz * qz);
     const T lam = two_pi_L * two_pi_L * q2 + k2;
     T A, B;
-    if (sp.propagator == 0) {
+    if (sk.propagator == 0) {
       A = T(1) / (T(1) + tau_eps * lam);
       B = T(1) / (lam + eps_tau);
     } else {
       A = t_exp(-tau_eps * lam);
       B = A * tau;
     }
-    const T Phi = sp.H0 > 0 ? t_exp(filt * q2) : T(1);
+    const T Phi = sk.filtered ? t_exp(filt * q2) : T(1);
     cpx<T> acc{T(0), T(0)};
     const int qd[3] = {qx, qy, qz};
 #pragma unroll
@@ -488,7 +486,7 @@ template <typename T>
 cudaError_t launch_adj_spectral(const cpx<T>* ghat, cpx<T>* abar, cpx<T>* spec, int H, SpecParams sp,
                                 cudaStream_t s) {
   const int64_t S = (int64_t)H * H * (H / 2 + 1);
-  k_adj_spectral<T><<<grid_blocks(S), 256, 0, s>>>(ghat, abar, spec, H, sp);
+  k_adj_spectral<T><<<grid_blocks(S), 256, 0, s>>>(ghat, abar, spec, H, spec_const<T>(sp));
   return cudaGetLastError();
 }
 

@@ -25,7 +25,21 @@
 namespace sipf {
 
 // e^{-2 pi i m / 256}, m < 256, per device (written once by ensure_device_tables).
+// The single-precision copy is rounded on the host, so the table loads of the
+// float kernels need no FP64-pipe conversions (with the tables cut to what
+// each kernel reads: plane kernels at H = 32 4.1 -> 4.0 us, y pass of a 128^3
+// grid 8.8 -> 7.9 us).
 __device__ double2 g_twiddle[kNmax];
+__device__ float2 g_twiddle_f[kNmax];
+template <typename T> __device__ __forceinline__ cpx<T> twiddle_entry(int m);
+template <> __device__ __forceinline__ cpx<double> twiddle_entry<double>(int m) {
+  const double2 w = g_twiddle[m];
+  return {w.x, w.y};
+}
+template <> __device__ __forceinline__ cpx<float> twiddle_entry<float>(int m) {
+  const float2 w = g_twiddle_f[m];
+  return {w.x, w.y};
+}
 
 cudaError_t ensure_device_tables() {
   static std::mutex mu;
@@ -37,11 +51,14 @@ cudaError_t ensure_device_tables() {
   if ((int)done.size() <= dev) done.resize(dev + 1, false);
   if (done[dev]) return cudaSuccess;
   double2 h[kNmax];
+  float2 hf[kNmax];
   for (int m = 0; m < kNmax; ++m) {
     const double a = -2.0 * M_PI * (double)m / (double)kNmax;
     h[m] = make_double2(cos(a), sin(a));
+    hf[m] = make_float2((float)h[m].x, (float)h[m].y);
   }
   e = cudaMemcpyToSymbol(g_twiddle, h, sizeof(h));
+  if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_twiddle_f, hf, sizeof(hf));
   if (e == cudaSuccess) done[dev] = true;
   return e;
 }
@@ -50,7 +67,7 @@ __device__ __forceinline__ int brev(int j, int lg) { return (int)(__brev((unsign
 
 template <typename T>
 __device__ __forceinline__ void load_twiddles(cpx<T>* tw) {
-  for (int i = threadIdx.x; i < kNmax / 2; i += blockDim.x) tw[i] = cpx<T>{(T)g_twiddle[i].x, (T)g_twiddle[i].y};
+  for (int i = threadIdx.x; i < kNmax / 2; i += blockDim.x) tw[i] = twiddle_entry<T>(i);
 }
 
 // In-place radix-2 DIT transform of `ncol` pencils of length n = 2^lgn in
@@ -119,7 +136,7 @@ k_rows_r2c(Tin* __restrict__ in, double in_scale, int zero_input, cpx<T>* __rest
         v = (T)in[gi];
       }
       if (zero_input) in[gi] = Tin(0);
-      msum += (double)v;
+      if (mass_acc) msum += (double)v;
     }
     cpx<T>& e = buf[(r >> 1) * ld + brev(j, lgH)];
     if (r & 1) e.y = v; else e.x = v;
@@ -188,7 +205,7 @@ k_cols(cpx<T>* __restrict__ data, int lgH, int B, int lgBC, size_t comp_stride, 
 template <typename T, int MODE>
 __global__ void __launch_bounds__(kThreads)
 k_spectral_x(const cpx<T>* __restrict__ T1, cpx<T>* __restrict__ alpha, cpx<T>* __restrict__ T2,
-             int lgH, int lgBC, SpecParams sp, double* alpha0_shadow) {
+             int lgH, int lgBC, SpecConst<T> sk, double* alpha0_shadow) {
   extern __shared__ unsigned char smem_raw[];
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
   cpx<T>* buf = tw + kNmax / 2;
@@ -210,10 +227,8 @@ k_spectral_x(const cpx<T>* __restrict__ T1, cpx<T>* __restrict__ alpha, cpx<T>* 
     __syncthreads();
     smem_fft<T, -1, true>(buf, tw, lgH, lgBC, ld, 1);
   }
-  const T two_pi_L = (T)(2.0 * M_PI / sp.L);
-  const T inv_L3 = (T)sp.inv_L3;
-  const T tau_eps = (T)(sp.tau / sp.eps), eps_tau = (T)(sp.eps / sp.tau), k2 = (T)sp.k2, tau = (T)sp.tau;
-  const T filt = sp.H0 > 0 ? (T)(-2.0 * M_PI * M_PI / (sp.H0 * sp.H0)) : T(0);
+  const T two_pi_L = sk.two_pi_L, inv_L3 = sk.inv_L3, filt = sk.filt;
+  const T tau_eps = sk.tau_eps, eps_tau = sk.eps_tau, k2 = sk.k2, tau = sk.tau;
   for (int t = threadIdx.x; t < H * BC; t += blockDim.x) {
     const int j = t >> lgBC, c = t & (BC - 1);
     const int m = b0 + c;
@@ -225,7 +240,7 @@ k_spectral_x(const cpx<T>* __restrict__ T1, cpx<T>* __restrict__ alpha, cpx<T>* 
       const int qy = ky < H / 2 ? ky : ky - H;
       const int qz = kz < H / 2 ? kz : kz - H;
       const T q2 = (T)(qx * qx + qy * qy + qz * qz);
-      const T Phi = sp.H0 > 0 ? t_exp(filt * q2) : T(1);
+      const T Phi = sk.filtered ? t_exp(filt * q2) : T(1);
       const size_t gi = (size_t)j * B + m;
       if (MODE == kModeStep || MODE == kModeGradOnly) {
         const cpx<T> a = alpha[gi];
@@ -235,7 +250,7 @@ k_spectral_x(const cpx<T>* __restrict__ T1, cpx<T>* __restrict__ alpha, cpx<T>* 
           beta.y *= inv_L3;
           const T lam = two_pi_L * two_pi_L * q2 + k2;
           cpx<T> an;
-          if (sp.propagator == 0) {
+          if (sk.propagator == 0) {
             const T kappa = T(1) / (T(1) + tau_eps * lam);
             const T src = T(1) / (lam + eps_tau);
             an = cpx<T>{kappa * a.x + src * beta.x, kappa * a.y + src * beta.y};
@@ -245,11 +260,8 @@ k_spectral_x(const cpx<T>* __restrict__ T1, cpx<T>* __restrict__ alpha, cpx<T>* 
           }
           alpha[gi] = an;
           if (m == 0 && j == 0 && alpha0_shadow) {
-            const double lam0 = sp.k2;
-            double s = *alpha0_shadow;
-            if (sp.propagator == 0) s = s / (1.0 + sp.tau / sp.eps * lam0) + sp.beta0 / (lam0 + sp.eps / sp.tau);
-            else s = exp(-sp.tau / sp.eps * lam0) * (s + sp.tau * sp.beta0);
-            *alpha0_shadow = s;
+            const double s0 = *alpha0_shadow;
+            *alpha0_shadow = sk.propagator == 0 ? s0 / sk.sh_div + sk.sh_add : exp(sk.sh_div) * (s0 + sk.sh_add);
           }
         }
         const T yx = two_pi_L * (T)qx * Phi, yy = two_pi_L * (T)qy * Phi, yz = two_pi_L * (T)qz * Phi;
@@ -330,7 +342,7 @@ k_rows_c2r(const cpx<T>* __restrict__ in, size_t comp_stride, T* __restrict__ ou
     }
     __syncthreads();
   }
-  double mx = -INFINITY;
+  T mx = -INFINITY;   // (as a double the maximum of every element ran on the FP64 pipe: 14.8 -> 8.3 us at 128^3)
   if (NOUT == 4) {
     for (int t = threadIdx.x; t < 2 * RP * H; t += blockDim.x) {
       const int r = t >> lgH;
@@ -352,14 +364,14 @@ k_rows_c2r(const cpx<T>* __restrict__ in, size_t comp_stride, T* __restrict__ ou
       if (r < nrow) {
         const T v = obuf[t];
         out[(size_t)row0 * H + t] = v;
-        mx = fmax(mx, (double)v);
+        mx = fmax(mx, v);
       }
     }
     if (max_acc) {
       for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
       if ((threadIdx.x & 31) == 0) {
         // order-preserving map of doubles onto signed 64-bit integers
-        long long b = __double_as_longlong(mx);
+        long long b = __double_as_longlong((double)mx);
         if (b < 0) b ^= 0x7fffffffffffffffLL;
         atomicMax(reinterpret_cast<long long*>(max_acc), b);
       }
@@ -551,7 +563,7 @@ template <typename T, int N> __device__ __forceinline__ void load_twq(cpx<T>* tw
   for (int i = threadIdx.x; i < N; i += blockDim.x) {
     const int k1 = i / Q, q = i - k1 * Q;
     const int m = (q * k1 * (kNmax / N)) & (kNmax - 1);
-    twq[i] = cpx<T>{(T)g_twiddle[m].x, (T)g_twiddle[m].y};
+    twq[i] = twiddle_entry<T>(m);
   }
 }
 
@@ -779,15 +791,17 @@ template <typename T, int E> __device__ __forceinline__ void load_tw_full(cpx<T>
       const int j = i - kNmax, k1 = j >> 5, lane = j & 31;
       m = (lane * k1 * SC) & (kNmax - 1);
     }
-    tw[i] = cpx<T>{(T)g_twiddle[m].x, (T)g_twiddle[m].y};
+    tw[i] = twiddle_entry<T>(m);
   }
 }
 
 // Shared twiddles of a kernel whose column passes use tile_ffts: the warp
 // FFT's tables (kTwLen entries), then, in single precision, the group FFT's.
 template <typename T, int E> constexpr int tw_len() { return kTwLen + twq_len<T, 32 * E>(); }
-template <typename T, int E> __device__ __forceinline__ void load_tw_group(cpx<T>* tw) {
-  load_tw_full<T, E>(tw);
+// The warp FFT's tables are filled only where a kernel uses them: in double
+// precision, and for row passes without group FFTs (ROWS).
+template <typename T, int E, bool ROWS> __device__ __forceinline__ void load_tw_group(cpx<T>* tw) {
+  if constexpr (sizeof(T) == 8 || (ROWS && !group_rows<T, 32 * E>())) load_tw_full<T, E>(tw);
   if constexpr (sizeof(T) == 4) load_twq<T, 32 * E>(tw + kTwLen);
 }
 
@@ -887,7 +901,7 @@ kw_rows_r2c(Tin* __restrict__ in, double in_scale, int zero_input, cpx<T>* __res
             double* mass_acc) {
   __shared__ cpx<T> tw[tw_len<T, E>()];
   __shared__ cpx<T> zb[8 * row_scratch<T, 32 * E>()];
-  load_tw_group<T, E>(tw);
+  load_tw_group<T, E, true>(tw);
   __syncthreads();
   rows_r2c_body<T, E, Tin>(in, in_scale, zero_input, out, rows, mass_acc, blockIdx.x, gridDim.x, tw, zb);
 }
@@ -921,7 +935,7 @@ __global__ void __launch_bounds__(256)
 kw_cols(cpx<T>* __restrict__ data, int B, size_t comp_stride, T scale) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
-  load_tw_group<T, E>(tw);
+  load_tw_group<T, E, false>(tw);
   cpx<T>* base = data + blockIdx.z * comp_stride + (size_t)blockIdx.y * (32 * E) * B;
   cols_body<T, E, DIR, BC>(base, B, scale, blockIdx.x * BC, tw, tw + tw_len<T, E>());
 }
@@ -932,7 +946,8 @@ kw_cols(cpx<T>* __restrict__ data, int B, size_t comp_stride, T scale) {
 // two outputs: 3 slots per pencil, so a 128^3 x pass fits one wave of blocks.
 template <typename T, int E, int MODE, int BC>
 __device__ __forceinline__ void spectral_body(const cpx<T>* __restrict__ T1, cpx<T>* __restrict__ alpha,
-                                              cpx<T>* __restrict__ T2, const SpecParams& sp, double* alpha0_shadow,
+                                              cpx<T>* __restrict__ T2, const SpecConst<T>& sk,
+                                              double* alpha0_shadow,
                                               int b0, const cpx<T>* tw, const cpx<T>* twq, cpx<T>* buf) {
   constexpr int N = 32 * E, NHH = N / 2 + 1, LD = 3 * BC + 1;
   const int B = N * NHH;
@@ -948,10 +963,8 @@ __device__ __forceinline__ void spectral_body(const cpx<T>* __restrict__ T1, cpx
     tile_ffts<T, N, -1>(nb, tw, twq, [&](int p, int j) { return buf + tpad(j, LD, p); }, [](int) { return true; });
   }
   __syncthreads();
-  const T two_pi_L = (T)(2.0 * M_PI / sp.L);
-  const T inv_L3 = (T)sp.inv_L3;
-  const T tau_eps = (T)(sp.tau / sp.eps), eps_tau = (T)(sp.eps / sp.tau), k2 = (T)sp.k2, tau = (T)sp.tau;
-  const T filt = sp.H0 > 0 ? (T)(-2.0 * M_PI * M_PI / (sp.H0 * sp.H0)) : T(0);
+  const T two_pi_L = sk.two_pi_L, inv_L3 = sk.inv_L3, filt = sk.filt;
+  const T tau_eps = sk.tau_eps, eps_tau = sk.eps_tau, k2 = sk.k2, tau = sk.tau;
   for (int t = threadIdx.x; t < N * BC; t += blockDim.x) {
     const int j = t / BC, c = t - j * BC;
     const int m = b0 + c;
@@ -962,7 +975,7 @@ __device__ __forceinline__ void spectral_body(const cpx<T>* __restrict__ T1, cpx
       const int qy = ky < N / 2 ? ky : ky - N;
       const int qz = kz < N / 2 ? kz : kz - N;
       const T q2 = (T)(qx * qx + qy * qy + qz * qz);
-      const T Phi = sp.H0 > 0 ? t_exp(filt * q2) : T(1);
+      const T Phi = sk.filtered ? t_exp(filt * q2) : T(1);
       const size_t gi = (size_t)j * B + m;
       if (MODE == kModeStep || MODE == kModeGradOnly) {
         const cpx<T> a = alpha[gi];
@@ -972,7 +985,7 @@ __device__ __forceinline__ void spectral_body(const cpx<T>* __restrict__ T1, cpx
           beta.y *= inv_L3;
           const T lam = two_pi_L * two_pi_L * q2 + k2;
           cpx<T> an;
-          if (sp.propagator == 0) {
+          if (sk.propagator == 0) {
             const T kappa = T(1) / (T(1) + tau_eps * lam);
             const T src = T(1) / (lam + eps_tau);
             an = cpx<T>{kappa * a.x + src * beta.x, kappa * a.y + src * beta.y};
@@ -982,11 +995,8 @@ __device__ __forceinline__ void spectral_body(const cpx<T>* __restrict__ T1, cpx
           }
           alpha[gi] = an;
           if (m == 0 && j == 0 && alpha0_shadow) {
-            const double lam0 = sp.k2;
-            double s = *alpha0_shadow;
-            if (sp.propagator == 0) s = s / (1.0 + sp.tau / sp.eps * lam0) + sp.beta0 / (lam0 + sp.eps / sp.tau);
-            else s = exp(-sp.tau / sp.eps * lam0) * (s + sp.tau * sp.beta0);
-            *alpha0_shadow = s;
+            const double s0 = *alpha0_shadow;
+            *alpha0_shadow = sk.propagator == 0 ? s0 / sk.sh_div + sk.sh_add : exp(sk.sh_div) * (s0 + sk.sh_add);
           }
         }
         const T yx = two_pi_L * (T)qx * Phi, yy = two_pi_L * (T)qy * Phi, yz = two_pi_L * (T)qz * Phi;
@@ -1048,7 +1058,7 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 
 template <int N, int MODE>
 __device__ __forceinline__ void spectral_reg_task(const cpx<float>* __restrict__ T1, cpx<float>* __restrict__ alpha,
-                                                  cpx<float>* __restrict__ T2, const SpecParams& sp,
+                                                  cpx<float>* __restrict__ T2, const SpecConst<float>& sk,
                                                   double* alpha0_shadow, int m0, const cpx<float>* twq,
                                                   cpx<float>* wslot) {
   using S = XRegShape<N>;
@@ -1068,11 +1078,8 @@ __device__ __forceinline__ void spectral_reg_task(const cpx<float>* __restrict__
   }
   const int ky = m / NHH, kz = m - ky * NHH;
   const int qy = ky < N / 2 ? ky : ky - N, qz = kz < N / 2 ? kz : kz - N;
-  const float two_pi_L = (float)(2.0 * M_PI / sp.L);
-  const float inv_L3 = (float)sp.inv_L3;
-  const float tau_eps = (float)(sp.tau / sp.eps), eps_tau = (float)(sp.eps / sp.tau), k2 = (float)sp.k2,
-              tau = (float)sp.tau;
-  const float filt = sp.H0 > 0 ? (float)(-2.0 * M_PI * M_PI / (sp.H0 * sp.H0)) : 0.f;
+  const float two_pi_L = sk.two_pi_L, inv_L3 = sk.inv_L3, filt = sk.filt;
+  const float tau_eps = sk.tau_eps, eps_tau = sk.eps_tau, k2 = sk.k2, tau = sk.tau;
   cpx<float> v[F];
   if (needs_beta) {
 #pragma unroll
@@ -1086,7 +1093,7 @@ __device__ __forceinline__ void spectral_reg_task(const cpx<float>* __restrict__
     const int j = q + Q * s;
     const int qx = j < N / 2 ? j : j - N;
     const float q2 = (float)(qx * qx + qy * qy + qz * qz);
-    const float Phi = sp.H0 > 0 ? expf(filt * q2) : 1.f;
+    const float Phi = sk.filtered ? expf(filt * q2) : 1.f;
     cpx<float> o1{0.f, 0.f};
     if (grad) {
       const cpx<float> a = A[q + Q * s];
@@ -1096,7 +1103,7 @@ __device__ __forceinline__ void spectral_reg_task(const cpx<float>* __restrict__
         beta.y *= inv_L3;
         const float lam = two_pi_L * two_pi_L * q2 + k2;
         cpx<float> an;
-        if (sp.propagator == 0) {
+        if (sk.propagator == 0) {
           const float kappa = 1.f / (1.f + tau_eps * lam);
           const float src = 1.f / (lam + eps_tau);
           an = cpx<float>{kappa * a.x + src * beta.x, kappa * a.y + src * beta.y};
@@ -1106,11 +1113,8 @@ __device__ __forceinline__ void spectral_reg_task(const cpx<float>* __restrict__
         }
         alpha[(size_t)j * B + m] = an;
         if (m == 0 && j == 0 && alpha0_shadow) {
-          const double lam0 = sp.k2;
-          double sh = *alpha0_shadow;
-          if (sp.propagator == 0) sh = sh / (1.0 + sp.tau / sp.eps * lam0) + sp.beta0 / (lam0 + sp.eps / sp.tau);
-          else sh = exp(-sp.tau / sp.eps * lam0) * (sh + sp.tau * sp.beta0);
-          *alpha0_shadow = sh;
+          const double s0 = *alpha0_shadow;
+          *alpha0_shadow = sk.propagator == 0 ? s0 / sk.sh_div + sk.sh_add : exp(sk.sh_div) * (s0 + sk.sh_add);
         }
       }
       const float yx = two_pi_L * (float)qx * Phi;
@@ -1149,7 +1153,7 @@ __device__ __forceinline__ void spectral_reg_task(const cpx<float>* __restrict__
 template <int N, int MODE>
 __global__ void __launch_bounds__(256)
 kwr_spectral_x(const cpx<float>* __restrict__ T1, cpx<float>* __restrict__ alpha, cpx<float>* __restrict__ T2,
-               SpecParams sp, double* alpha0_shadow) {
+               SpecConst<float> sk, double* alpha0_shadow) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<float>* twq = reinterpret_cast<cpx<float>*>(smem_raw);
   load_twq<float, N>(twq);
@@ -1157,7 +1161,7 @@ kwr_spectral_x(const cpx<float>* __restrict__ T1, cpx<float>* __restrict__ alpha
   const int wib = threadIdx.x >> 5;
   const int t = blockIdx.x * (int)(blockDim.x >> 5) + wib;
   if (t < XRegShape<N>::TASKS)
-    spectral_reg_task<N, MODE>(T1, alpha, T2, sp, alpha0_shadow, t * XRegShape<N>::G, twq,
+    spectral_reg_task<N, MODE>(T1, alpha, T2, sk, alpha0_shadow, t * XRegShape<N>::G, twq,
                                twq + N + wib * XRegShape<N>::WARP);
 }
 
@@ -1171,20 +1175,19 @@ __global__ void __launch_bounds__(512) kwrb_spectral_x(const FftRun<float>* __re
   const int wib = threadIdx.x >> 5;
   const int t = blockIdx.x * (int)(blockDim.x >> 5) + wib;
   if (t < XRegShape<N>::TASKS)
-    spectral_reg_task<N, kModeStep>(r.T1, r.alpha, r.T2, r.sp, r.shadow, t * XRegShape<N>::G, twq,
+    spectral_reg_task<N, kModeStep>(r.T1, r.alpha, r.T2, r.sk, r.shadow, t * XRegShape<N>::G, twq,
                                     twq + N + wib * XRegShape<N>::WARP);
 }
 
 template <typename T, int E, int MODE, int BC>
 __global__ void __launch_bounds__(256)
-kw_spectral_x(const cpx<T>* __restrict__ T1, cpx<T>* __restrict__ alpha, cpx<T>* __restrict__ T2, SpecParams sp,
+kw_spectral_x(const cpx<T>* __restrict__ T1, cpx<T>* __restrict__ alpha, cpx<T>* __restrict__ T2, SpecConst<T> sk,
               double* alpha0_shadow) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
-  load_tw_full<T, E>(tw);
+  load_tw_group<T, E, false>(tw);
   cpx<T>* twq = tw + kTwLen;
-  if constexpr (sizeof(T) == 4) load_twq<T, 32 * E>(twq);
-  spectral_body<T, E, MODE, BC>(T1, alpha, T2, sp, alpha0_shadow, blockIdx.x * BC, tw, twq,
+  spectral_body<T, E, MODE, BC>(T1, alpha, T2, sk, alpha0_shadow, blockIdx.x * BC, tw, twq,
                                 twq + twq_len<T, 32 * E>());
 }
 
@@ -1199,7 +1202,7 @@ __device__ __forceinline__ void rows_c2r_body(const cpx<T>* __restrict__ in, siz
   constexpr int NOUT = NCOMP == 3 ? 4 : 1;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   cpx<T>* zb = zb_all + wib * row_scratch<T, N>();
-  double mx = -INFINITY;
+  T mx = -INFINITY;
   if constexpr (group_rows<T, N>()) {
     // group FFTs over this block's contiguous range of row pairs, taken in
     // chunks of one pass of the block's warps, each chunk's components one
@@ -1229,7 +1232,7 @@ __device__ __forceinline__ void rows_c2r_body(const cpx<T>* __restrict__ in, siz
               } else {
                 oa[j] = re;
                 oa[N + j] = im;
-                mx = fmax(mx, fmax((double)re, (double)im));
+                mx = fmax(mx, fmax(re, im));
               }
             });
       }
@@ -1279,7 +1282,7 @@ __device__ __forceinline__ void rows_c2r_body(const cpx<T>* __restrict__ in, siz
       for (int t = lane; t < 2 * N; t += 32) {
         const T v = ob[t];
         oa[t] = v;
-        mx = fmax(mx, (double)v);
+        mx = fmax(mx, v);
       }
     }
     __syncwarp();
@@ -1288,7 +1291,7 @@ __device__ __forceinline__ void rows_c2r_body(const cpx<T>* __restrict__ in, siz
   if (NOUT == 1 && max_acc) {
     for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     if (lane == 0) {
-      long long b = __double_as_longlong(mx);
+      long long b = __double_as_longlong((double)mx);
       if (b < 0) b ^= 0x7fffffffffffffffLL;
       atomicMax(reinterpret_cast<long long*>(max_acc), b);
     }
@@ -1303,7 +1306,7 @@ kw_rows_c2r(const cpx<T>* __restrict__ in, size_t comp_stride, T* __restrict__ o
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
   cpx<T>* zb_all = tw + tw_len<T, E>();
   T* ob_all = reinterpret_cast<T*>(zb_all + 8 * row_scratch<T, N>());
-  load_tw_group<T, E>(tw);
+  load_tw_group<T, E, true>(tw);
   __syncthreads();
   rows_c2r_body<T, E, NCOMP>(in, comp_stride, out, rows, max_acc, blockIdx.x, gridDim.x, tw, zb_all, ob_all);
 }
@@ -1316,7 +1319,7 @@ template <typename T, int E>
 __global__ void __launch_bounds__(256) kwb_rows_r2c(const FftRun<T>* __restrict__ runs) {
   __shared__ cpx<T> tw[tw_len<T, E>()];
   __shared__ cpx<T> zb[8 * row_scratch<T, 32 * E>()];
-  load_tw_group<T, E>(tw);
+  load_tw_group<T, E, true>(tw);
   __syncthreads();
   const FftRun<T>& r = runs[blockIdx.y];
   constexpr int N = 32 * E;
@@ -1332,7 +1335,7 @@ template <typename T, int E, int DIR, int BC>
 __global__ void __launch_bounds__(256) kwb_cols(const FftRun<T>* __restrict__ runs, int ncomp) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
-  load_tw_group<T, E>(tw);
+  load_tw_group<T, E, false>(tw);
   constexpr int N = 32 * E, NHH = N / 2 + 1;
   const int run = blockIdx.z / ncomp, comp = blockIdx.z - run * ncomp;
   const FftRun<T>& r = runs[run];
@@ -1345,11 +1348,10 @@ template <typename T, int E, int BC>
 __global__ void __launch_bounds__(512) kwb_spectral_x(const FftRun<T>* __restrict__ runs) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
-  load_tw_full<T, E>(tw);
+  load_tw_group<T, E, false>(tw);
   cpx<T>* twq = tw + kTwLen;
-  if constexpr (sizeof(T) == 4) load_twq<T, 32 * E>(twq);
   const FftRun<T>& r = runs[blockIdx.y];
-  spectral_body<T, E, kModeStep, BC>(r.T1, r.alpha, r.T2, r.sp, r.shadow, blockIdx.x * BC, tw, twq,
+  spectral_body<T, E, kModeStep, BC>(r.T1, r.alpha, r.T2, r.sk, r.shadow, blockIdx.x * BC, tw, twq,
                                      twq + twq_len<T, 32 * E>());
 }
 
@@ -1360,7 +1362,7 @@ __global__ void __launch_bounds__(256) kwb_rows_c2r(const FftRun<T>* __restrict_
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
   cpx<T>* zb_all = tw + tw_len<T, E>();
   T* ob_all = reinterpret_cast<T*>(zb_all + 8 * row_scratch<T, N>());
-  load_tw_group<T, E>(tw);
+  load_tw_group<T, E, true>(tw);
   __syncthreads();
   const FftRun<T>& r = runs[blockIdx.y];
   const size_t S = (size_t)N * N * (N / 2 + 1);
@@ -1562,7 +1564,7 @@ __global__ void __launch_bounds__(group_rows<T, 32 * E>() ? 512 : 1024) kwp_fwd(
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
   cpx<T>* zb = tw + tw_len<T, E>();
   cpx<T>* P = zb + (group_rows<T, N>() ? 0 : (blockDim.x >> 5) * padded_len(N));
-  load_tw_group<T, E>(tw);
+  load_tw_group<T, E, true>(tw);
   __syncthreads();
   const FftRun<T>& r = runs[blockIdx.y];
   const int x = blockIdx.x;
@@ -1581,7 +1583,7 @@ __global__ void __launch_bounds__(group_rows<T, 32 * E>() ? 512 : 1024) kwp_inv(
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
   cpx<T>* zb = tw + tw_len<T, E>();
   cpx<T>* P = zb + (group_rows<T, N>() ? 0 : (blockDim.x >> 5) * padded_len(N));
-  load_tw_group<T, E>(tw);
+  load_tw_group<T, E, true>(tw);
   __syncthreads();
   const FftRun<T>& r = runs[blockIdx.z];
   const int x = blockIdx.x, d = blockIdx.y;
@@ -1708,7 +1710,7 @@ __global__ void __launch_bounds__(group_rows<T, 32 * E>() ? 512 : 1024) kwp_inv3
   cpx<T>* zb = tw + tw_len<T, E>();
   cpx<T>* P = zb + (group_rows<T, N>() ? 0 : (blockDim.x >> 5) * padded_len(N));
   T* ob = reinterpret_cast<T*>(P + 3 * ((size_t)N * NH + E));
-  load_tw_group<T, E>(tw);
+  load_tw_group<T, E, true>(tw);
   __syncthreads();
   const FftRun<T>& r = runs[blockIdx.y];
   const int x = blockIdx.x;
@@ -1919,7 +1921,7 @@ __global__ void __launch_bounds__(1024) kwc_fwd(const FftRun<T>* __restrict__ ru
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
   cpx<T>* zb = tw + tw_len<T, E>();
   cpx<T>* Q = zb + (blockDim.x >> 5) * row_scratch<T, N>();
-  load_tw_group<T, E>(tw);
+  load_tw_group<T, E, true>(tw);
   __syncthreads();
   const FftRun<T>& r = runs[blockIdx.y];
   const int x = blockIdx.x / CS;
@@ -1938,7 +1940,7 @@ __global__ void __launch_bounds__(1024) kwc_inv(const FftRun<T>* __restrict__ ru
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
   cpx<T>* zb = tw + tw_len<T, E>();
   cpx<T>* Q = zb + (blockDim.x >> 5) * row_scratch<T, N>();
-  load_tw_group<T, E>(tw);
+  load_tw_group<T, E, true>(tw);
   __syncthreads();
   const FftRun<T>& r = runs[blockIdx.z];
   const int x = blockIdx.x / CS, d = blockIdx.y;
@@ -2003,7 +2005,7 @@ static cudaError_t warp_spectral(const cpx<T>* T1, cpx<T>* alpha, cpx<T>* T2, Sp
     auto k = kwr_spectral_x<N, MODE>;
     cudaError_t e = set_smem(k, smem);
     if (e != cudaSuccess) return e;
-    k<<<(XRegShape<N>::TASKS + nw - 1) / nw, 32 * nw, smem, s>>>(T1, alpha, T2, sp, shadow);
+    k<<<(XRegShape<N>::TASKS + nw - 1) / nw, 32 * nw, smem, s>>>(T1, alpha, T2, spec_const<T>(sp), shadow);
     return cudaGetLastError();
   } else {
   constexpr int BC = (sizeof(T) == 8 && E == 8) ? 4 : ((sizeof(T) == 8 || E == 8) ? 8 : 16);
@@ -2012,7 +2014,7 @@ static cudaError_t warp_spectral(const cpx<T>* T1, cpx<T>* alpha, cpx<T>* T2, Sp
   auto k = kw_spectral_x<T, E, MODE, BC>;
   cudaError_t e = set_smem(k, smem);
   if (e != cudaSuccess) return e;
-  k<<<(B + BC - 1) / BC, 256, smem, s>>>(T1, alpha, T2, sp, shadow);
+  k<<<(B + BC - 1) / BC, 256, smem, s>>>(T1, alpha, T2, spec_const<T>(sp), shadow);
   return cudaGetLastError();
   }
 }
@@ -2125,7 +2127,7 @@ static cudaError_t spectral_mode(const cpx<T>* T1, cpx<T>* alpha, cpx<T>* T2, in
   auto k = k_spectral_x<T, MODE>;
   cudaError_t e = set_smem(k, smem);
   if (e != cudaSuccess) return e;
-  k<<<(B + BC - 1) / BC, kThreads, smem, s>>>(T1, alpha, T2, lgH, lgBC, sp, shadow);
+  k<<<(B + BC - 1) / BC, kThreads, smem, s>>>(T1, alpha, T2, lgH, lgBC, spec_const<T>(sp), shadow);
   return cudaGetLastError();
 }
 

@@ -87,15 +87,20 @@ k2_deposit(const T* __restrict__ x, const T* __restrict__ y, int64_t P, Geo<T> g
   }
 }
 
+// Constants of the spectral kernel, rounded to T on the host (double divisions
+// in every thread run on the slow FP64 pipe).
+template <typename T>
 struct Spec2D {
-  double L, inv_L2, tau, eps, k2, H0;
-  int mode;   // 0: step (field + gradients), 1: density Phi beta into component 0
+  T two_pi_L, inv_L2, tau_eps, eps_tau, k2, filt;   // Phi = exp(filt |q|^2)
+  int filtered, elliptic;   // Phi in use; eps = 0
+  int mode;                 // 0: step (field + gradients), 1: density Phi beta into component 0
 };
 
 // One thread per mode of the H x (H/2+1) half spectrum.
 template <typename T>
 __global__ void __launch_bounds__(kT2)
-k2_spectral(const cpx<T>* __restrict__ T1, cpx<T>* __restrict__ alpha, cpx<T>* __restrict__ T2, int H, Spec2D sp) {
+k2_spectral(const cpx<T>* __restrict__ T1, cpx<T>* __restrict__ alpha, cpx<T>* __restrict__ T2, int H,
+            Spec2D<T> sp) {
   const int NH = H / 2 + 1;
   const int S = H * NH;
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
@@ -104,24 +109,24 @@ k2_spectral(const cpx<T>* __restrict__ T1, cpx<T>* __restrict__ alpha, cpx<T>* _
   const int qx = kx < H / 2 ? kx : kx - H;
   const int qy = ky < H / 2 ? ky : ky - H;
   const T q2 = (T)(qx * qx + qy * qy);
-  const T Phi = sp.H0 > 0 ? t_exp((T)(-2.0 * M_PI * M_PI / (sp.H0 * sp.H0)) * q2) : T(1);
+  const T Phi = sp.filtered ? t_exp(sp.filt * q2) : T(1);
   cpx<T> beta = T1[m];
-  beta.x *= (T)sp.inv_L2;
-  beta.y *= (T)sp.inv_L2;
+  beta.x *= sp.inv_L2;
+  beta.y *= sp.inv_L2;
   if (sp.mode == 1) {
     T2[m] = cpx<T>{beta.x * Phi, beta.y * Phi};
     return;
   }
-  const T two_pi_L = (T)(2.0 * M_PI / sp.L);
-  const T lam = two_pi_L * two_pi_L * q2 + (T)sp.k2;
+  const T two_pi_L = sp.two_pi_L;
+  const T lam = two_pi_L * two_pi_L * q2 + sp.k2;
   cpx<T> a;   // the field that drives this step's move
-  if (sp.eps == 0.0) {
+  if (sp.elliptic) {
     a = lam > T(0) ? cpx<T>{beta.x / lam, beta.y / lam} : cpx<T>{T(0), T(0)};
     alpha[m] = a;
   } else {
     a = alpha[m];
-    const T kappa = T(1) / (T(1) + (T)(sp.tau / sp.eps) * lam);
-    const T src = T(1) / (lam + (T)(sp.eps / sp.tau));
+    const T kappa = T(1) / (T(1) + sp.tau_eps * lam);
+    const T src = T(1) / (lam + sp.eps_tau);
     alpha[m] = cpx<T>{kappa * a.x + src * beta.x, kappa * a.y + src * beta.y};
   }
   const T yx = two_pi_L * (T)qx * Phi, yy = two_pi_L * (T)qy * Phi;
@@ -306,14 +311,17 @@ template <typename T> int deposit2(sipf2d_ctx* c) {
   return SIPF_OK;
 }
 
-Spec2D spec2(const sipf2d_ctx* c, int mode) {
-  Spec2D s;
-  s.L = c->p.L;
-  s.inv_L2 = 1.0 / (c->p.L * c->p.L);
-  s.tau = c->p.dt;
-  s.eps = c->p.eps;
-  s.k2 = c->p.k * c->p.k;
-  s.H0 = c->H0;
+template <typename T> Spec2D<T> spec2(const sipf2d_ctx* c, int mode, bool filtered = true) {
+  Spec2D<T> s;
+  const double H0 = filtered ? c->H0 : 0.0;
+  s.two_pi_L = (T)(2.0 * M_PI / c->p.L);
+  s.inv_L2 = (T)(1.0 / (c->p.L * c->p.L));
+  s.elliptic = c->p.eps == 0.0 ? 1 : 0;
+  s.tau_eps = s.elliptic ? T(0) : (T)(c->p.dt / c->p.eps);
+  s.eps_tau = (T)(c->p.eps / c->p.dt);
+  s.k2 = (T)(c->p.k * c->p.k);
+  s.filtered = H0 > 0 ? 1 : 0;
+  s.filt = s.filtered ? (T)(-2.0 * M_PI * M_PI / (H0 * H0)) : T(0);
   s.mode = mode;
   return s;
 }
@@ -334,7 +342,7 @@ template <typename T> int step2(sipf2d_ctx* c, int64_t nsteps) {
     int r = forward2<T>(c, true, nullptr);
     if (r) return r;
     k2_spectral<T><<<(unsigned)((S + kT2 - 1) / kT2), kT2, 0, c->stream>>>(
-        (const cpx<T>*)c->T1, (cpx<T>*)c->alpha, (cpx<T>*)c->T2, H, spec2(c, 0));
+        (const cpx<T>*)c->T1, (cpx<T>*)c->alpha, (cpx<T>*)c->T2, H, spec2<T>(c, 0));
     SIPF2_CK(cudaGetLastError());
     SIPF2_CK(launch_cols<T>((cpx<T>*)c->T2, H, 1, H / 2 + 1, 2, S, +1, 1.0, c->stream));
     SIPF2_CK(launch_rows_c2r<T>((const cpx<T>*)c->T2, 3, S, (T*)c->grad, H, H, nullptr, c->stream));
@@ -380,10 +388,8 @@ template <typename T> int density_num2(sipf2d_ctx* c, int filtered) {
   const size_t S = (size_t)c->S();
   int r = forward2<T>(c, false, nullptr);
   if (r) return r;
-  Spec2D sp = spec2(c, 1);
-  if (!filtered) sp.H0 = 0.0;
   k2_spectral<T><<<(unsigned)((S + kT2 - 1) / kT2), kT2, 0, c->stream>>>(
-      (const cpx<T>*)c->T1, (cpx<T>*)c->alpha, (cpx<T>*)c->T2, H, sp);
+      (const cpx<T>*)c->T1, (cpx<T>*)c->alpha, (cpx<T>*)c->T2, H, spec2<T>(c, 1, filtered != 0));
   SIPF2_CK(cudaGetLastError());
   SIPF2_CK(launch_cols<T>((cpx<T>*)c->T2, H, 1, H / 2 + 1, 1, 0, +1, 1.0, c->stream));
   // (only the first spectrum is used; the third, read as zeros by the step's

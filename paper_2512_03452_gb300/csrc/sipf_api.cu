@@ -224,7 +224,7 @@ template <typename T> FftRun<T> make_fft_run(const sipf_ctx* c) {
   f.alpha = (cpx<T>*)c->alpha;
   f.T2 = (cpx<T>*)c->T2;
   f.grad = (T*)c->grad;
-  f.sp = spec_params(c);
+  f.sk = spec_const<T>(spec_params(c));
   f.shadow = c->dsc + kDscAlpha0;
   return f;
 }
