@@ -9,14 +9,15 @@
 //             each particle then written into the bin of its new tile in the
 //             other buffer (one global reservation per round and tile; the
 //             particles of a merged item reserve one slot each);
-//   chunk lists: work items of up to 4096 particles of one bin, and one
-//             merged item per window of m consecutive bins for the bins
-//             under 256 particles (m = 4 for a single run, 16 in a batch);
-//   k_binned (deposit): the deposit I of the new positions (Algorithm 2), a
+//   chunk lists: work items of up to `chunk` particles of one bin (64 to 4096,
+//             chosen for the number of particles), and one merged item per
+//             window of 8 consecutive bins for its small bins;
+//   k_binned_deposit: the deposit I of the new positions (Algorithm 2), a
 //             block per work item, into a shared-memory integer window over
 //             the tile and the stencil halo (several copies, chosen per lane
 //             so that a warp's atomics fall into distinct banks), then added
-//             to the grid with coalesced reductions.  Particles outside the
+//             to the grid with coalesced reductions; the bins of a merged
+//             item a warp each, in windows of one copy.  Particles outside the
 //             window (the overflow bin) deposit with global reductions.
 // Batched forms take the work items of many runs from one counter.  Also
 // here: the re-binning of particle-order arrays, the read-backs to particle
@@ -149,11 +150,8 @@ __device__ __forceinline__ int find_run(const long long* prefix, int nruns, long
 }
 
 // ---------------------------------------------------------------------------
-// The binned particle kernel.  Template flags:
-//   MOVE:    advance X^{n-1} -> X^n (Algorithm 4, particle loop)
-//   DEPOSIT: deposit the positions into phi
-//   REBIN:   write each particle into the destination bins of its tile
-// A step runs MOVE+REBIN, then DEPOSIT over the new bins: the chemotactic
+// Deposit and re-bin over the tile bins.  A step moves every particle into the
+// bin of its new tile (k_move), then deposits from those bins: the chemotactic
 // drift can carry particles many cells in one step, so the deposit reads the
 // bins of the new positions, where every particle lies in the tile of its bin
 // and the window only needs the stencil halo.
@@ -172,22 +170,29 @@ constexpr int kReplicas = 4;                  // whole-grid window copies (lane 
 // 32 / kTileReps: far fewer bank conflicts than copies stored one after
 // another, whose random slots spread over all 32 banks at random.
 constexpr int kTileReps = 8;
-constexpr int kChunk = 4096;                  // particles per work item
-// Work items with fewer particles deposit with global reductions: clearing
-// and flushing a tile window (11^3 slots x 8 copies) costs more than their
-// 32 reductions per particle.
+// Work items hold at most `chunk` particles of one bin (BinArgs / ChunkListArgs,
+// chosen for the number of particles by particle_chunk below), so that a small
+// run still gives every SM several items.
+constexpr int kChunkMax = 4096, kChunkMin = 64;
+// Pieces of a bin with fewer particles deposit with global reductions:
+// clearing and flushing a tile window (11^3 slots x 8 copies) costs more than
+// their 32 reductions per particle.
 constexpr int kWinMinLen = 64;
-// Sparse bins are taken together: the bins with fewer than kSmall particles
-// (the overflow bin excepted) of each window of m consecutive bins form one
-// work item, marked by bin = -m with the window index in `start` and the
+// Sparse bins are taken together: the bins with fewer than `small` particles
+// (the overflow bin excepted) of each window of kMerge consecutive bins form
+// one work item, marked by bin = -1 with the window index in `start` and the
 // bins' total in `len`.  A sparse region then costs the move one round per
-// window instead of one per bin.  m (a power of two, 2 ... kMergeMax) is set
-// per chunk list: 4 for a single run (longer merged items left the deposit's
-// last blocks idle), 16 for the runs of a batch (many sparse runs).
-constexpr int kMergeMax = 16;
-constexpr int kSmall = 256;
-__device__ __forceinline__ int merge_of(const ChunkDesc& d) { return -d.bin; }
-__device__ __forceinline__ bool bin_is_small(int b, int count, int NT) { return b < NT && count > 0 && count < kSmall; }
+// window instead of one per bin, and the deposit a warp per bin: a block has
+// kMerge warps.  (Windows of 4 and 16 bins: 241 and 267 us per step of a batch
+// of 24 runs against 237; torus of 1e7 453 and 445 against 446.)
+constexpr int kMerge = 8;
+constexpr int kSmallMax = 256;
+// In a merged item's deposit, a warp takes a bin of at least this many
+// particles into a window of its own (below it: global reductions).
+constexpr int kWarpWinMin = 24;
+__device__ __forceinline__ bool bin_is_small(int b, int count, int NT, int small) {
+  return b < NT && count > 0 && count < small;
+}
 
 // Calls fn(slot) for every particle of work item d, the block's threads
 // striding over each run of slots (all threads take the same bins).
@@ -197,12 +202,11 @@ __device__ __forceinline__ void item_slots(const BinArgs<T>& a, const ChunkDesc&
     for (int i = threadIdx.x; i < d.len; i += blockDim.x) fn(d.start + i);
     return;
   }
-  const int m = merge_of(d);
-  for (int k = 0; k < m; ++k) {
-    const int b = (int)d.start * m + k;
+  for (int k = 0; k < kMerge; ++k) {
+    const int b = (int)d.start * kMerge + k;
     if (b > a.NT) break;
     const int c = a.src_count[b];
-    if (!bin_is_small(b, c, a.NT)) continue;
+    if (!bin_is_small(b, c, a.NT, a.small)) continue;
     const long long s0 = a.src_base[b];
     for (int i = threadIdx.x; i < c; i += blockDim.x) fn(s0 + i);
   }
@@ -224,12 +228,19 @@ template <> __device__ __forceinline__ float sum_to_real<float>(long long v) {
 }
 template <> __device__ __forceinline__ double sum_to_real<double>(long long v) { return (double)v; }
 
+// One window node's sum v (units of 2^-K) added to grid node gi.
+template <typename T, bool FIXED>
+__device__ __forceinline__ void add_node(const BinArgs<T>& a, int gi, long long v, T unit) {
+  if (FIXED) atomicAdd(static_cast<unsigned long long*>(a.phi) + gi, (unsigned long long)v);
+  else atomicAdd(static_cast<T*>(a.phi) + gi, sum_to_real<T>(v) * unit);
+}
+
 template <typename T, bool FIXED, bool WHOLE>
 __device__ __forceinline__ void window_flush(const BinArgs<T>& a, typename WinType<T>::type* win, int wslots, int ox,
-                                             int oy, int oz, T wwin) {
+                                             int oy, int oz, int K) {
   using A = typename WinType<T>::type;
   const int H = a.g.H, mask = a.g.mask;
-  const T unit = a.wmass / wwin;   // M0/P * 2^-K
+  const T unit = a.wmass * pow2<T>(-K);   // M0/P * 2^-K
   if constexpr (!WHOLE && sizeof(A) == 4) {
     // Tile window of ints: a warp takes 32 consecutive slots (1 KB) per pass.
     // Lane l reads 16-byte pieces l and 32 + l (halves of slots l/2 and
@@ -260,8 +271,7 @@ __device__ __forceinline__ void window_flush(const BinArgs<T>& a, typename WinTy
       if (sidx < wslots && v != 0) {
         const int c = sidx % kWin, b = (sidx / kWin) % kWin, aa = sidx / (kWin * kWin);
         const int gi = (((ox + aa) & mask) * H + ((oy + b) & mask)) * H + ((oz + c) & mask);
-        if (FIXED) atomicAdd(static_cast<unsigned long long*>(a.phi) + gi, (unsigned long long)(long long)v);
-        else atomicAdd(static_cast<T*>(a.phi) + gi, sum_to_real<T>(v) * unit);
+        add_node<T, FIXED>(a, gi, v, unit);
       }
     }
   } else {
@@ -288,21 +298,66 @@ __device__ __forceinline__ void window_flush(const BinArgs<T>& a, typename WinTy
           const int c = sidx % kWin, b = (sidx / kWin) % kWin, aa = sidx / (kWin * kWin);
           gi = (((ox + aa) & mask) * H + ((oy + b) & mask)) * H + ((oz + c) & mask);
         }
-        if (FIXED) atomicAdd(static_cast<unsigned long long*>(a.phi) + gi, (unsigned long long)(long long)v);
-        else atomicAdd(static_cast<T*>(a.phi) + gi, sum_to_real<T>(v) * unit);
+        add_node<T, FIXED>(a, gi, v, unit);
       }
     }
   }
 }
 
-// One work item of k_binned (deposit and/or re-bin without a move).
-// seg_cnt / seg_base (shared memory, nseg entries; NULL: the item is the
-// contiguous slots start ... start + len - 1): the item's particles are the
-// runs of seg_cnt[k] slots from seg_base[k], one after another.
-template <typename T, bool FIXED, bool MOVE, bool DEPOSIT, bool REBIN, bool WHOLE>
-__device__ __forceinline__ void binned_chunk(const BinArgs<T>& a, const ChunkDesc& cur,
-                                             typename WinType<T>::type* win, const int* seg_cnt = nullptr,
-                                             const long long* seg_base = nullptr, int nseg = 0) {
+// The particle in slot s deposited with global reductions.
+template <typename T, bool FIXED>
+__device__ __forceinline__ void deposit_global(const BinArgs<T>& a, long long s) {
+  int cx, cy, cz;
+  T lx, ly, lz;
+  cell_lambda(__ldcs(a.sx + s), a.g, cx, lx);
+  cell_lambda(__ldcs(a.sy + s), a.g, cy, ly);
+  cell_lambda(__ldcs(a.sz + s), a.g, cz, lz);
+  if (FIXED) {
+    unsigned long long* grid = static_cast<unsigned long long*>(a.phi);
+    stencil_visit_global<T>(a.p2g, cx, cy, cz, lx, ly, lz, pow2<T>(a.fix_k), a.g, [&](int idx, T f) {
+      atomicAdd(grid + idx, (unsigned long long)(long long)WinType<T>::round(f));
+    });
+  } else {
+    T* grid = static_cast<T*>(a.phi);
+    stencil_visit_global<T>(a.p2g, cx, cy, cz, lx, ly, lz, a.wmass, a.g,
+                            [&](int idx, T f) { atomicAdd(grid + idx, f); });
+  }
+}
+
+// Window slot of base node (cx - 1, cy - 1, cz - 1) of a tile window with
+// origin (ox, oy, oz); false if the 4^3 box of the stencil leaves the window.
+__device__ __forceinline__ bool tile_slot(int cx, int cy, int cz, int ox, int oy, int oz, int mask, int& slot) {
+  const int sx = (cx - 1 - ox) & mask, sy = (cy - 1 - oy) & mask, sz = (cz - 1 - oz) & mask;
+  slot = ((sx * kWin) + sy) * kWin + sz;
+  return sx <= kWin - 4 && sy <= kWin - 4 && sz <= kWin - 4;
+}
+
+// Adds a particle's weights (scale wwin = 2^K) to a tile window whose slots
+// are STRIDE words apart, from its base slot's word on.
+template <typename T, int STRIDE>
+__device__ __forceinline__ void deposit_window(int p2g, typename WinType<T>::type* wb, T lx, T ly, T lz, T wwin) {
+  int ix[4], iy[4], iz[4];
+#pragma unroll
+  for (int o = 0; o < 4; ++o) {   // compile-time offsets of the 4^3 box
+    ix[o] = o * (kWin * kWin * STRIDE);
+    iy[o] = o * (kWin * STRIDE);
+    iz[o] = o * STRIDE;
+  }
+  stencil_visit<T>(p2g, ix, iy, iz, lx, ly, lz, wwin, [&](int idx, T f) { win_add(wb + idx, WinType<T>::round(f)); });
+}
+
+__device__ __forceinline__ void tile_origin(int bin, int ntx, int& ox, int& oy, int& oz) {
+  const int tz = bin % ntx, ty = (bin / ntx) % ntx, tx = bin / (ntx * ntx);
+  ox = tx * kTileE - kMargin - 1;
+  oy = ty * kTileE - kMargin - 1;
+  oz = tz * kTileE - kMargin - 1;
+}
+
+// Deposit of one work item of a single bin by the block.  WHOLE: the window is
+// the whole grid (use_win: the launch has one).
+template <typename T, bool FIXED, bool WHOLE>
+__device__ __forceinline__ void deposit_chunk(const BinArgs<T>& a, const ChunkDesc& cur,
+                                              typename WinType<T>::type* win, bool use_win) {
   using A = typename WinType<T>::type;
   const int H = a.g.H, mask = a.g.mask;
   const int wslots = WHOLE ? H * H * H : kWinSlots;
@@ -311,217 +366,211 @@ __device__ __forceinline__ void binned_chunk(const BinArgs<T>& a, const ChunkDes
   A* const my_win = win + (lane & (kReplicas - 1)) * wslots;
   const int bin = cur.bin, len = cur.len;
   const long long start = cur.start;
-  // window origin (node coordinates of slot (0,0,0))
-  bool has_win = DEPOSIT && (WHOLE || (bin < a.NT && len >= kWinMinLen));
-  int ox = 0, oy = 0, oz = 0;
-  if (!WHOLE && bin < a.NT) {
-    const int tz = bin % a.ntx, ty = (bin / a.ntx) % a.ntx, tx = bin / (a.ntx * a.ntx);
-    ox = tx * kTileE - kMargin - 1;
-    oy = ty * kTileE - kMargin - 1;
-    oz = tz * kTileE - kMargin - 1;
-  }
+  const bool has_win = use_win && (WHOLE || (bin < a.NT && len >= kWinMinLen));
+  int ox = 0, oy = 0, oz = 0;   // node coordinates of window slot (0,0,0)
+  if (!WHOLE && bin < a.NT) tile_origin(bin, a.ntx, ox, oy, oz);
   // window scale 2^K: no copy's node sum can reach 2^30 (int32 windows; see
   // win_copy_load) or 2^62 (int64 windows: the whole chunk's sum)
   const int K = FIXED ? a.fix_k
                       : (sizeof(A) == 4 ? 30 - ceil_log2(win_copy_load(WHOLE ? 8 : 7, len, blockDim.x) + 1)
                                         : WinType<T>::bits - ceil_log2(len + 1));
   const T wwin = pow2<T>(K);
-  const int iters = (len + blockDim.x - 1) / blockDim.x;
   // next particle's data is loaded one iteration ahead (streaming loads: the
-  // particle arrays are read once per pass, the grids stay in L2)
-  auto slot_of = [&](int i) -> long long {
-    if (!seg_cnt) return start + i;
-    int k = 0;
-    while (k < nseg - 1 && i >= seg_cnt[k]) i -= seg_cnt[k++];
-    return seg_base[k] + i;
-  };
-  T px = T(0), py = T(0), pz = T(0);
-  uint32_t pid = 0;
-  if ((int)threadIdx.x < len) {
-    const long long s = slot_of(threadIdx.x);
-    px = __ldcs(a.sx + s);
-    py = __ldcs(a.sy + s);
-    pz = __ldcs(a.sz + s);
-    pid = __ldcs(a.sid + s);
-  }
-  for (int it = 0; it < iters; ++it) {
-    const int i = it * blockDim.x + threadIdx.x;
-    const bool valid = i < len;
-    T x = px, y = py, z = pz;
-    const uint32_t id = pid;
-    if (i + (int)blockDim.x < len) {
-      const long long s = slot_of(i + blockDim.x);
+  // particle arrays are read once per pass, the grids stay in L2).  Particles
+  // whose stencil leaves the window are noted in a bit per iteration and
+  // deposited after the loop: their code inside it costs the loop spills.
+  uint32_t missed = has_win ? 0u : 0xFFFFFFFFu;
+  if (has_win) {
+    T px = T(0), py = T(0), pz = T(0);
+    if ((int)threadIdx.x < len) {
+      const long long s = start + threadIdx.x;
       px = __ldcs(a.sx + s);
       py = __ldcs(a.sy + s);
       pz = __ldcs(a.sz + s);
-      pid = __ldcs(a.sid + s);
     }
-    if (MOVE && valid) {
-      T nz[6];
-      normals6(a.seed, (uint64_t)id, a.n, nz);
-      if (a.split == 0) {
-        // Z = X + W^- + chi tau I*(grad c)(X + W^-),  X^n = Z + W^+
-        const T yx = x + a.s_noise * nz[0], yy = y + a.s_noise * nz[1], yz = z + a.s_noise * nz[2];
-        const V3<T> gr = gather_grad(a.grad4, a.g2p, yx, yy, yz, a.g);
-        x = wrap_coord((yx + a.chitau * gr.x) + a.s_noise * nz[3], a.g);
-        y = wrap_coord((yy + a.chitau * gr.y) + a.s_noise * nz[4], a.g);
-        z = wrap_coord((yz + a.chitau * gr.z) + a.s_noise * nz[5], a.g);
-      } else {
-        // X^n = X + chi tau I*(grad c)(X) + W,  W ~ N(0, 2 mu tau I)
-        const V3<T> gr = gather_grad(a.grad4, a.g2p, x, y, z, a.g);
-        x = wrap_coord((x + a.chitau * gr.x) + a.s_noise * nz[0], a.g);
-        y = wrap_coord((y + a.chitau * gr.y) + a.s_noise * nz[1], a.g);
-        z = wrap_coord((z + a.chitau * gr.z) + a.s_noise * nz[2], a.g);
+    uint32_t bit = 1u;   // at most kChunkMax / 256 iterations
+    for (int i0 = 0; i0 < len; i0 += blockDim.x, bit <<= 1) {
+      const int i = i0 + threadIdx.x;
+      const T x = px, y = py, z = pz;
+      if (i + (int)blockDim.x < len) {
+        const long long s = start + i + blockDim.x;
+        px = __ldcs(a.sx + s);
+        py = __ldcs(a.sy + s);
+        pz = __ldcs(a.sz + s);
       }
-      if (!(t_finite(x) && t_finite(y) && t_finite(z))) atomicOr(a.err, 1);
-    }
-    int cx = 0, cy = 0, cz = 0;
-    T lx = T(0), ly = T(0), lz = T(0);
-    cell_lambda(x, a.g, cx, lx);
-    cell_lambda(y, a.g, cy, ly);
-    cell_lambda(z, a.g, cz, lz);
-    // reserve the destination slot first: the atomic's round trip overlaps the deposit
-    int t = 0, rank = 0, leader = 0, b0 = 0;
-    if (REBIN) {
-      t = tile_of(cx & mask, cy & mask, cz & mask, a.tile_shift, a.ntx);
-      const unsigned key = valid ? (unsigned)t : 0xFFFFFFFFu;
-      const unsigned peers = __match_any_sync(0xFFFFFFFFu, key);
-      leader = __ffs(peers) - 1;
-      rank = __popc(peers & ((1u << lane) - 1u));
-      if (valid && lane == leader) b0 = atomicAdd(a.dst_cursor + t, __popc(peers));
-    }
-    bool fits = DEPOSIT && valid && has_win;
-    int sx = 0, sy = 0, sz = 0;
-    if (!WHOLE && fits) {
-      sx = (cx - 1 - ox) & mask;
-      sy = (cy - 1 - oy) & mask;
-      sz = (cz - 1 - oz) & mask;
-      fits = sx <= kWin - 4 && sy <= kWin - 4 && sz <= kWin - 4;
-    }
-    // Copy of the tile window each lane adds into.  A slot's kTileReps copies
-    // cover a fixed group of banks, and the group of every stencil node of a
-    // particle is its base slot's group shifted by the same amount for all
-    // lanes; so lanes whose base slots share a group are ranked and take
-    // distinct copies (conflict-free while at most kTileReps share a group).
-    int cpy = lane & (kTileReps - 1);
-    if (DEPOSIT && !WHOLE) {
-      constexpr int kGroups = 32 * 4 / (kTileReps * (int)sizeof(A));   // bank groups: 4 (int), 2 (long long)
-      const int cls = fits ? ((((sx * kWin) + sy) * kWin + sz) & (kGroups - 1)) : kGroups;
-      const unsigned m0 = __ballot_sync(0xFFFFFFFFu, cls & 1), m1 = __ballot_sync(0xFFFFFFFFu, cls & 2),
-                     m2 = __ballot_sync(0xFFFFFFFFu, cls & 4);
-      const unsigned peers = ((cls & 1) ? m0 : ~m0) & ((cls & 2) ? m1 : ~m1) & ((cls & 4) ? m2 : ~m2);
-      cpy = __popc(peers & ((1u << lane) - 1u)) & (kTileReps - 1);
-    }
-    if (DEPOSIT && valid) {
-      if (fits) {
-        int ix[4], iy[4], iz[4];
-        if (WHOLE) {
+      int cx = 0, cy = 0, cz = 0;
+      T lx = T(0), ly = T(0), lz = T(0);
+      cell_lambda(x, a.g, cx, lx);
+      cell_lambda(y, a.g, cy, ly);
+      cell_lambda(z, a.g, cz, lz);
+      bool fits = i < len;
+      if (WHOLE) {
+        if (fits) {
+          int ix[4], iy[4], iz[4];
           axis_layers_global(cx, mask, H * H, ix);
           axis_layers_global(cy, mask, H, iy);
           axis_layers_global(cz, mask, 1, iz);
           stencil_visit<T>(a.p2g, ix, iy, iz, lx, ly, lz, wwin,
                            [&](int idx, T f) { win_add(my_win + idx, WinType<T>::round(f)); });
-        } else {
-          // base slot plus compile-time offsets of the 4x4x4 box (interleaved copies)
-          A* wb = win + (((sx * kWin) + sy) * kWin + sz) * kTileReps + cpy;
-#pragma unroll
-          for (int o = 0; o < 4; ++o) {
-            ix[o] = o * (kWin * kWin * kTileReps);
-            iy[o] = o * (kWin * kTileReps);
-            iz[o] = o * kTileReps;
-          }
-          stencil_visit<T>(a.p2g, ix, iy, iz, lx, ly, lz, wwin,
-                           [&](int idx, T f) { win_add(wb + idx, WinType<T>::round(f)); });
         }
-      } else if (FIXED) {
-        unsigned long long* grid = static_cast<unsigned long long*>(a.phi);
-        stencil_visit_global<T>(a.p2g, cx, cy, cz, lx, ly, lz, wwin, a.g, [&](int idx, T f) {
-          atomicAdd(grid + idx, (unsigned long long)(long long)WinType<T>::round(f));
-        });
-      } else {
-        T* grid = static_cast<T*>(a.phi);
-        stencil_visit_global<T>(a.p2g, cx, cy, cz, lx, ly, lz, a.wmass, a.g,
-                                [&](int idx, T f) { atomicAdd(grid + idx, f); });
+        continue;
       }
-    }
-    if (REBIN) {
-      b0 = __shfl_sync(0xFFFFFFFFu, b0, leader);
-      if (valid) {
-        long long slot;
-        const int r = b0 + rank;
-        if (r < a.dst_cap[t]) {
-          slot = a.dst_base[t] + r;
-        } else {
-          const int o = atomicAdd(a.dst_cursor + a.NT, 1);
-          slot = o < a.dst_cap[a.NT] ? a.dst_base[a.NT] + o : -1;
-        }
-        if (slot >= 0) {
-          a.dx[slot] = x;
-          a.dy[slot] = y;
-          a.dz[slot] = z;
-          a.did[slot] = id;
-        } else {
-          atomicOr(a.err, 2);   // overflow bin full: the particle is lost
-        }
+      int slot = 0;
+      if (fits && !tile_slot(cx, cy, cz, ox, oy, oz, mask, slot)) {
+        fits = false;
+        missed |= bit;
       }
+      // Copy of the tile window each lane adds into.  A slot's kTileReps copies
+      // cover a fixed group of banks, and the group of every stencil node of a
+      // particle is its base slot's group shifted by the same amount for all
+      // lanes; so lanes whose base slots share a group are ranked and take
+      // distinct copies (conflict-free while at most kTileReps share a group).
+      constexpr int kGroups = 32 * 4 / (kTileReps * (int)sizeof(A));   // bank groups: 4 (int), 2 (long long)
+      const int cls = fits ? (slot & (kGroups - 1)) : kGroups;
+      const unsigned m0 = __ballot_sync(0xFFFFFFFFu, cls & 1), m1 = __ballot_sync(0xFFFFFFFFu, cls & 2),
+                     m2 = __ballot_sync(0xFFFFFFFFu, cls & 4);
+      const unsigned peers = ((cls & 1) ? m0 : ~m0) & ((cls & 2) ? m1 : ~m1) & ((cls & 4) ? m2 : ~m2);
+      const int cpy = __popc(peers & ((1u << lane) - 1u)) & (kTileReps - 1);
+      if (fits) deposit_window<T, kTileReps>(a.p2g, win + slot * kTileReps + cpy, lx, ly, lz, wwin);
     }
   }
-  if (DEPOSIT && has_win) {
+  if (missed)
+    for (int i = threadIdx.x; i < len; i += blockDim.x, missed >>= 1)
+      if (missed & 1u) deposit_global<T, FIXED>(a, start + i);
+  if (has_win) {
     __syncthreads();
-    window_flush<T, FIXED, WHOLE>(a, win, wslots, ox, oy, oz, wwin);
+    window_flush<T, FIXED, WHOLE>(a, win, wslots, ox, oy, oz, K);
   }
 }
 
-// A work item of k_binned: one bin's chunk, or a merged item: its bins under
-// kWinMinLen particles in one pass without a window, then each other small
-// bin with its own window.
-template <typename T, bool FIXED, bool MOVE, bool DEPOSIT, bool REBIN, bool WHOLE>
-__device__ __forceinline__ void binned_item(const BinArgs<T>& a, const ChunkDesc& cur,
-                                            typename WinType<T>::type* win) {
-  if (cur.bin >= 0) {
-    binned_chunk<T, FIXED, MOVE, DEPOSIT, REBIN, WHOLE>(a, cur, win);
-    return;
-  }
-  // the window's bins, looked up together
-  const int m = merge_of(cur);
-  __shared__ int s_cnt[kMergeMax], s_tiny[kMergeMax];
-  __shared__ long long s_base[kMergeMax];
-  if (threadIdx.x < m) {
-    const int b = (int)cur.start * m + threadIdx.x;
-    int c = b <= a.NT ? a.src_count[b] : 0;
-    if (!bin_is_small(b, c, a.NT)) c = 0;
-    s_cnt[threadIdx.x] = c;
-    s_tiny[threadIdx.x] = !WHOLE && c < kWinMinLen ? c : 0;
-    s_base[threadIdx.x] = c ? a.src_base[b] : 0;
-  }
-  __syncthreads();
-  // bins too small for a window: all of them in one pass (global reductions)
-  int tiny = 0;
-  for (int k = 0; k < m; ++k) tiny += s_tiny[k];
-  if (tiny > 0)
-    binned_chunk<T, FIXED, MOVE, DEPOSIT, REBIN, WHOLE>(a, ChunkDesc{0, a.NT, tiny}, win, s_tiny, s_base, m);
-  // the others each with its window
-  for (int k = 0; k < m; ++k) {
-    const int c = s_cnt[k];
-    if (c == 0 || s_tiny[k] != 0) continue;
-    binned_chunk<T, FIXED, MOVE, DEPOSIT, REBIN, WHOLE>(a, ChunkDesc{s_base[k], (int)cur.start * m + k, c}, win);
-    __syncthreads();   // the window's flush (which clears it) ends before the next bin adds into it
-  }
-}
-
-template <typename T, bool FIXED, bool MOVE, bool DEPOSIT, bool REBIN, bool WHOLE>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2)
-k_binned(BinArgs<T> a) {
+// Deposit of a merged item: each warp takes small bins of its own, with a
+// window of one copy in its eighth of the block's window, so the bins of an
+// item run beside one another with no block barrier.  (Taken one after another
+// by the whole block, a bin of some 80 particles cost about 10 us of barriers
+// and dependent loads, and an item was as many of them.)  A bin adds at most once per particle to a
+// node, so K = 31 - ceil(log2(c + 1)) keeps c 2^K below 2^31: 24 for up to 127
+// particles, 23 for up to 255.
+template <typename T, bool FIXED, bool WHOLE>
+__device__ __forceinline__ void deposit_merged(const BinArgs<T>& a, const ChunkDesc& cur,
+                                               typename WinType<T>::type* win) {
   using A = typename WinType<T>::type;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  A* win = reinterpret_cast<A*>(smem_raw);
-  __shared__ ChunkDesc s_desc[2];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = (int)(blockDim.x >> 5);
+  const int H = a.g.H, mask = a.g.mask;
+  A* const ww = win + warp * kWinSlots;
+  for (int k = warp; k < kMerge; k += nwarps) {
+    const int b = (int)cur.start * kMerge + k;
+    const int c = b < a.NT ? a.src_count[b] : 0;
+    if (!bin_is_small(b, c, a.NT, a.small)) continue;
+    const long long s0 = a.src_base[b];
+    const bool has_win = !WHOLE && c >= kWarpWinMin;
+    int ox = 0, oy = 0, oz = 0;
+    if (!WHOLE) tile_origin(b, a.ntx, ox, oy, oz);
+    const int K = FIXED ? a.fix_k : (sizeof(A) == 4 ? 31 : WinType<T>::bits) - ceil_log2(c + 1);
+    const T wwin = pow2<T>(K);
+    uint32_t missed = has_win ? 0u : 0xFFFFFFFFu;   // a bit per iteration (at most kSmallMax / 32)
+    if (has_win) {
+      T px = T(0), py = T(0), pz = T(0);
+      if (lane < c) {
+        px = __ldcs(a.sx + s0 + lane);
+        py = __ldcs(a.sy + s0 + lane);
+        pz = __ldcs(a.sz + s0 + lane);
+      }
+      uint32_t bit = 1u;
+      for (int i = lane; i < c; i += 32, bit <<= 1) {
+        const T x = px, y = py, z = pz;
+        if (i + 32 < c) {
+          px = __ldcs(a.sx + s0 + i + 32);
+          py = __ldcs(a.sy + s0 + i + 32);
+          pz = __ldcs(a.sz + s0 + i + 32);
+        }
+        int cx, cy, cz;
+        T lx, ly, lz;
+        cell_lambda(x, a.g, cx, lx);
+        cell_lambda(y, a.g, cy, ly);
+        cell_lambda(z, a.g, cz, lz);
+        int slot = 0;
+        if (tile_slot(cx, cy, cz, ox, oy, oz, mask, slot)) deposit_window<T, 1>(a.p2g, ww + slot, lx, ly, lz, wwin);
+        else missed |= bit;
+      }
+    }
+    if (missed)
+      for (int i = lane; i < c; i += 32, missed >>= 1)
+        if (missed & 1u) deposit_global<T, FIXED>(a, s0 + i);
+    if (has_win) {
+      __syncwarp();
+      const T unit = a.wmass * pow2<T>(-K);
+#pragma unroll 4
+      for (int s = lane; s < kWinSlots; s += 32) {
+        const A v = ww[s];
+        if (v != 0) {
+          ww[s] = A(0);
+          const int sc = s % kWin, sb = (s / kWin) % kWin, sa = s / (kWin * kWin);
+          add_node<T, FIXED>(a, (((ox + sa) & mask) * H + ((oy + sb) & mask)) * H + ((oz + sc) & mask), v, unit);
+        }
+      }
+      __syncwarp();
+    }
+  }
+}
+
+// One particle of a re-bin pass written into the destination bin of its tile;
+// all lanes of the warp take part (valid: this lane has a particle).
+template <typename T>
+__device__ __forceinline__ void rebin_one(const BinArgs<T>& a, bool valid, T x, T y, T z, uint32_t id) {
+  const int lane = threadIdx.x & 31, mask = a.g.mask;
+  int cx, cy, cz;
+  T l;
+  cell_lambda(x, a.g, cx, l);
+  cell_lambda(y, a.g, cy, l);
+  cell_lambda(z, a.g, cz, l);
+  const int t = tile_of(cx & mask, cy & mask, cz & mask, a.tile_shift, a.ntx);
+  const unsigned peers = __match_any_sync(0xFFFFFFFFu, valid ? (unsigned)t : 0xFFFFFFFFu);
+  const int leader = __ffs(peers) - 1, rank = __popc(peers & ((1u << lane) - 1u));
+  int b0 = 0;
+  if (valid && lane == leader) b0 = atomicAdd(a.dst_cursor + t, __popc(peers));
+  b0 = __shfl_sync(0xFFFFFFFFu, b0, leader);
+  if (!valid) return;
+  const int r = b0 + rank;
+  long long slot;
+  if (r < a.dst_cap[t]) {
+    slot = a.dst_base[t] + r;
+  } else {
+    const int o = atomicAdd(a.dst_cursor + a.NT, 1);
+    slot = o < a.dst_cap[a.NT] ? a.dst_base[a.NT] + o : -1;
+  }
+  if (slot >= 0) {
+    a.dx[slot] = x;
+    a.dy[slot] = y;
+    a.dz[slot] = z;
+    a.did[slot] = id;
+  } else {
+    atomicOr(a.err, 2);   // overflow bin full: the particle is lost
+  }
+}
+
+// `len` particles from slot `start` re-binned by `width` threads (whole warps).
+template <typename T>
+__device__ __forceinline__ void rebin_run(const BinArgs<T>& a, long long start, int len, int t0, int width) {
+  for (int i0 = 0; i0 < len; i0 += width) {
+    const int i = i0 + t0;
+    const bool valid = i < len;
+    T x = T(0), y = T(0), z = T(0);
+    uint32_t id = 0;
+    if (valid) {
+      x = __ldcs(a.sx + start + i);
+      y = __ldcs(a.sy + start + i);
+      z = __ldcs(a.sz + start + i);
+      id = __ldcs(a.sid + start + i);
+    }
+    rebin_one(a, valid, x, y, z, id);
+  }
+}
+
+// Work items are taken from a global counter by persistent blocks; the next
+// one is fetched while the current one is processed.
+template <typename T, typename Fn>
+__device__ __forceinline__ void for_items(const BinArgs<T>& a, ChunkDesc* s_desc, Fn&& fn) {
   const long long nchunks = a.chunk_start[a.NT + 1];
-  const int wslots = WHOLE ? a.g.H * a.g.H * a.g.H : kWinSlots;
-  if (DEPOSIT)
-    for (int i = threadIdx.x; i < (WHOLE ? kReplicas : kTileReps) * wslots; i += blockDim.x) win[i] = A(0);
-  // work items are taken from a global counter; the next one is fetched
-  // while the current one is processed
   if (threadIdx.x == 0) {
     const long long c = (long long)atomicAdd(a.work, 1ULL);
     s_desc[0] = c < nchunks ? a.chunks[c] : ChunkDesc{0, 0, 0};
@@ -535,10 +584,44 @@ k_binned(BinArgs<T> a) {
       const long long c = (long long)atomicAdd(a.work, 1ULL);
       if (c < nchunks) nxt = a.chunks[c];
     }
-    binned_item<T, FIXED, MOVE, DEPOSIT, REBIN, WHOLE>(a, cur, win);
+    fn(cur);
     if (threadIdx.x == 0) s_desc[buf ^ 1] = nxt;
     __syncthreads();
   }
+}
+
+template <typename T, bool FIXED, bool WHOLE>
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2)
+k_binned_deposit(const __grid_constant__ BinArgs<T> a, int use_win) {
+  using A = typename WinType<T>::type;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  A* win = reinterpret_cast<A*>(smem_raw);
+  __shared__ ChunkDesc s_desc[2];
+  if (use_win) {
+    const int n = WHOLE ? kReplicas * a.g.H * a.g.H * a.g.H : kTileReps * kWinSlots;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) win[i] = A(0);
+  }
+  for_items(a, s_desc, [&](const ChunkDesc& cur) {
+    if (cur.bin >= 0) deposit_chunk<T, FIXED, WHOLE>(a, cur, win, use_win != 0);
+    else deposit_merged<T, FIXED, WHOLE>(a, cur, win);
+  });
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256)
+k_binned_rebin(const __grid_constant__ BinArgs<T> a) {
+  __shared__ ChunkDesc s_desc[2];
+  for_items(a, s_desc, [&](const ChunkDesc& cur) {
+    if (cur.bin >= 0) {
+      rebin_run(a, cur.start, cur.len, threadIdx.x, blockDim.x);
+      return;
+    }
+      for (int k = threadIdx.x >> 5; k < kMerge; k += (int)(blockDim.x >> 5)) {   // a warp per small bin
+      const int b = (int)cur.start * kMerge + k;
+      const int c = b < a.NT ? a.src_count[b] : 0;
+      if (bin_is_small(b, c, a.NT, a.small)) rebin_run(a, a.src_base[b], c, threadIdx.x & 31, 32);
+    }
+  });
 }
 
 // Batched deposit over the bins of all runs (tile windows, H >= 32).
@@ -577,7 +660,8 @@ k_deposit_batch(const BinArgs<T>* __restrict__ table, const long long* __restric
         nxt = table[nrun].chunks[c - prefix[nrun]];
       }
     }
-    binned_item<T, FIXED, false, true, false, false>(table[run], cur, win);
+    if (cur.bin >= 0) deposit_chunk<T, FIXED, false>(table[run], cur, win, true);
+    else deposit_merged<T, FIXED, false>(table[run], cur, win);
     if (threadIdx.x == 0) {
       s_desc[buf ^ 1] = nxt;
       s_run[buf ^ 1] = nrun;
@@ -616,8 +700,8 @@ struct MoveSmem {
   int meta[R];        // neighbour slot (0..124) | rank << 7, or -1 - tile for far moves
   int cnt[kNbr], base[kNbr], tile[kNbr], cap[kNbr];
   long long gbase[kNbr];   // first slot of each destination bin
-  long long seg_base[kMergeMax];   // merged items: first slot and particles of each small bin
-  int seg_cnt[kMergeMax];
+  long long seg_base[kMerge];   // merged items: first slot and particles of each small bin
+  int seg_cnt[kMerge];
   __align__(8) uint64_t bar;
   int abort;
 };
@@ -700,15 +784,14 @@ template <typename T> __device__ __forceinline__ void move_write_out(const BinAr
 template <typename T, bool MOVE, int G2P>
 __device__ __forceinline__ void move_merged(const BinArgs<T>& a, const ChunkDesc& cur, uint32_t n, MoveSmem<T>& sm) {
   constexpr int R = MoveRound<T>::n;
-  const int m = merge_of(cur);
-  if (threadIdx.x < m) {
-    const int b = (int)cur.start * m + threadIdx.x;
+  if (threadIdx.x < kMerge) {
+    const int b = (int)cur.start * kMerge + threadIdx.x;
     int c = 0;
     long long base = 0;
     if (b <= a.NT) {
       c = a.src_count[b];
       base = a.src_base[b];
-      if (!bin_is_small(b, c, a.NT)) c = 0;
+      if (!bin_is_small(b, c, a.NT, a.small)) c = 0;
     }
     sm.seg_cnt[threadIdx.x] = c;
     sm.seg_base[threadIdx.x] = base;
@@ -720,7 +803,7 @@ __device__ __forceinline__ void move_merged(const BinArgs<T>& a, const ChunkDesc
     for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
       // the bin holding item particle r0 + i
       int k = 0, o = r0 + i;
-      while (k < m - 1 && o >= sm.seg_cnt[k]) o -= sm.seg_cnt[k++];
+      while (k < kMerge - 1 && o >= sm.seg_cnt[k]) o -= sm.seg_cnt[k++];
       const long long slot = sm.seg_base[k] + o;
       T x = a.sx[slot], y = a.sy[slot], z = a.sz[slot];
       const uint32_t id = a.sid[slot];
@@ -918,15 +1001,27 @@ k_move_batch(const BinArgs<T>* __restrict__ table, const long long* __restrict__
   }
 }
 
-template <typename T> cudaError_t launch_move(const BinArgs<T>& a, cudaStream_t s) {
+static cudaError_t resident_blocks(const void* kern, int threads, size_t smem, int* blocks) {
   int dev = 0, sms = 0, per_sm = 0;
   cudaError_t e;
+  if (smem > 48 * 1024 &&
+      (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+    return e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem)) != cudaSuccess) return e;
+  *blocks = sms * (per_sm < 1 ? 1 : per_sm);
+  return cudaSuccess;
+}
+
+// (No more blocks than there can be work items: a small run's idle blocks only
+// lengthen the launch.)
+template <typename T> cudaError_t launch_move(const BinArgs<T>& a, cudaStream_t s) {
+  int blocks = 0;
   auto k = a.g2p == 4 ? k_move<T, 4> : k_move<T, 2>;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kMoveThreads, 0)) != cudaSuccess) return e;
-  if (per_sm < 1) per_sm = 1;
-  k<<<sms * per_sm, kMoveThreads, 0, s>>>(a);
+  const cudaError_t e = resident_blocks((const void*)k, kMoveThreads, 0, &blocks);
+  if (e != cudaSuccess) return e;
+  k<<<min(blocks, a.max_items), kMoveThreads, 0, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -1001,15 +1096,15 @@ __device__ __forceinline__ void chunk_count_body(const ChunkListArgs& a, int blk
   if (b < nb) {
     const int c = min(a.cursor[b], a.cap[b]);
     a.count[b] = c;
-    small = bin_is_small(b, c, a.NT);
-    ch = small ? 0 : (c + kChunk - 1) / kChunk;
+    small = bin_is_small(b, c, a.NT, a.small);
+    ch = small ? 0 : (c + a.chunk - 1) / a.chunk;
     a.other_cursor[b] = 0;
   }
-  // the first bin of a window (a.merge lanes of a warp) also holds the
+  // the first bin of a window (kMerge lanes of a warp) also holds the
   // window's merged item, if it has small bins
   const unsigned sm = __ballot_sync(0xFFFFFFFFu, small);
-  const int lane = threadIdx.x & 31, mw = a.merge;
-  if ((lane & (mw - 1)) == 0 && ((sm >> lane) & ((1u << mw) - 1u)) != 0u) ch += 1;
+  const int lane = threadIdx.x & 31;
+  if ((lane & (kMerge - 1)) == 0 && ((sm >> lane) & ((1u << kMerge) - 1u)) != 0u) ch += 1;
   long long total;
   const long long ex = block_exclusive_scan_ll(ch, total);
   if (b < nb) a.chunk_start[b] = ex;
@@ -1046,22 +1141,22 @@ __device__ __forceinline__ void chunk_emit_body(const ChunkListArgs& a, int blk,
       if (s_ls[i + step] <= q) i += step;
     const int bin = blk * kCLBlock + i;
     int j = (int)(q - s_ls[i]);
-    if ((bin & (a.merge - 1)) == 0) {
+    if ((bin & (kMerge - 1)) == 0) {
       int tot = 0;
-      for (int k = 0; k < a.merge && bin + k < nb; ++k) {
+      for (int k = 0; k < kMerge && bin + k < nb; ++k) {
         const int cc = a.count[bin + k];
-        if (bin_is_small(bin + k, cc, a.NT)) tot += cc;
+        if (bin_is_small(bin + k, cc, a.NT, a.small)) tot += cc;
       }
       if (tot > 0) {
         if (j == 0) {   // the window's merged item comes first
-          a.chunks[off + q] = ChunkDesc{(long long)(bin / a.merge), -a.merge, tot};
+          a.chunks[off + q] = ChunkDesc{(long long)(bin / kMerge), -1, tot};
           continue;
         }
         j -= 1;
       }
     }
     const int c = a.count[bin];
-    a.chunks[off + q] = ChunkDesc{a.base[bin] + (long long)j * kChunk, bin, min(kChunk, c - j * kChunk)};
+    a.chunks[off + q] = ChunkDesc{a.base[bin] + (long long)j * a.chunk, bin, min(a.chunk, c - j * a.chunk)};
   }
   if (blk == nblk - 1 && threadIdx.x == 0) {
     a.chunk_start[nb] = off + total;
@@ -1327,7 +1422,7 @@ k_gather_slots(const uint32_t* __restrict__ slot_of, const T* __restrict__ bx, c
 // entries lie in the same grid tile; items land in the order their blocks
 // reserve their ranges (cursor: zeroed before the launch).
 template <typename T>
-__global__ void __launch_bounds__(1024)
+__global__ void __launch_bounds__(256)
 k_compact(BinArgs<T> a, unsigned long long* cursor, T* __restrict__ ox, T* __restrict__ oy, T* __restrict__ oz,
           uint32_t* __restrict__ oid) {
   __shared__ long long s_base;
@@ -1350,12 +1445,11 @@ k_compact(BinArgs<T> a, unsigned long long* cursor, T* __restrict__ ox, T* __res
     copy_run(d.start, d.len);
     return;
   }
-  const int m = merge_of(d);
-  for (int k = 0; k < m; ++k) {
-    const int b = (int)d.start * m + k;
+  for (int k = 0; k < kMerge; ++k) {
+    const int b = (int)d.start * kMerge + k;
     if (b > a.NT) break;
     const int n = a.src_count[b];
-    if (bin_is_small(b, n, a.NT)) copy_run(a.src_base[b], n);
+    if (bin_is_small(b, n, a.NT, a.small)) copy_run(a.src_base[b], n);
   }
 }
 
@@ -1601,41 +1695,55 @@ __global__ void __launch_bounds__(256) k_alpha_energy(const cpx<T>* __restrict__
 // ---------------------------------------------------------------------------
 // Launchers.
 // ---------------------------------------------------------------------------
-int binned_window_slots(int H) { return H <= 16 ? kReplicas * H * H * H : kTileReps * kWinSlots; }
-int binned_chunk() { return kChunk; }
 int binned_tile_shift(int H) { return H <= 16 ? 30 : kTileShift; }
 
-template <typename T, bool FIXED, bool MOVE, bool DEPOSIT, bool REBIN>
-static cudaError_t launch_binned_t(const BinArgs<T>& a, cudaStream_t s) {
-  const bool whole = a.g.H <= 16;
-  const size_t smem = DEPOSIT ? (size_t)binned_window_slots(a.g.H) * sizeof(typename WinType<T>::type) : 0;
-  auto kern = whole ? k_binned<T, FIXED, MOVE, DEPOSIT, REBIN, true> : k_binned<T, FIXED, MOVE, DEPOSIT, REBIN, false>;
-  cudaError_t e;
-  if (smem > 48 * 1024) {
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  int dev = 0, sms = 0, per_sm = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem)) != cudaSuccess) return e;
-  if (per_sm < 1) per_sm = 1;
-  kern<<<sms * per_sm, 256, smem, s>>>(a);
+// Work-item length: the longest power of two that leaves the 152 SMs six
+// items each, so that few particles still spread over the chip and the last
+// wave of many is short, but long enough that a tile window's flush stays
+// small next to its particles.  Measured per step (us) by item length:
+//   FP32, P = 1e7, H = 128: 512 612, 2048 455, 4096 453; P = 1e6, H = 64: 512 103,
+//   1024 95, 4096 110; P = 2e5, H = 64: 128 78, 512 63, 2048 63; P = 16384,
+//   H = 32: 64 to 256 46, 1024 54, 4096 65;
+//   FP64 (the FP64 pipe wants every SM busy), P = 1e6, H = 64: 256 1170, 1024
+//   1159, 4096 1273; P = 1e4, H = 16 (whole-grid tile): 32 98, 64 86, 256 124, 4096 866.
+int particle_chunk(int64_t P, int H, bool fp64) {
+  const int least = H <= 16 ? kChunkMin : fp64 ? 128 : P < (1 << 16) ? 256 : 512;
+  int c = kChunkMax;
+  while (c > least && P / c < 152 * 6) c >>= 1;
+  return c;
+}
+// A merged item (up to kMerge bins) is then at most twice an item of one bin.
+int particle_small(int chunk) {
+  const int s = chunk / 4;
+  return s > kSmallMax ? kSmallMax : s < 32 ? 32 : s;
+}
+
+template <typename T, bool FIXED, bool WHOLE>
+static cudaError_t launch_deposit_t(const BinArgs<T>& a, cudaStream_t s) {
+  // whole-grid window: only for items with enough particles to pay for its flush
+  const int nodes = a.g.H * a.g.H * a.g.H;
+  const int use_win = !WHOLE || a.chunk >= nodes / 8;
+  const size_t slots = WHOLE ? (size_t)kReplicas * nodes : (size_t)kTileReps * kWinSlots;
+  const size_t smem = use_win ? slots * sizeof(typename WinType<T>::type) : 0;
+  auto kern = k_binned_deposit<T, FIXED, WHOLE>;
+  int blocks = 0;
+  const cudaError_t e = resident_blocks((const void*)kern, 256, smem, &blocks);
+  if (e != cudaSuccess) return e;
+  kern<<<min(blocks, a.max_items), 256, smem, s>>>(a, use_win);
   return cudaGetLastError();
 }
 
-template <typename T>
-cudaError_t launch_binned(const BinArgs<T>& a, int move, int deposit, int rebin, cudaStream_t s) {
-  if (a.fixed) {
-    if (move && !deposit && rebin) return launch_binned_t<T, true, true, false, true>(a, s);
-    if (!move && deposit && !rebin) return launch_binned_t<T, true, false, true, false>(a, s);
-    if (!move && !deposit && rebin) return launch_binned_t<T, true, false, false, true>(a, s);
-  } else {
-    if (move && !deposit && rebin) return launch_binned_t<T, false, true, false, true>(a, s);
-    if (!move && deposit && !rebin) return launch_binned_t<T, false, false, true, false>(a, s);
-    if (!move && !deposit && rebin) return launch_binned_t<T, false, false, false, true>(a, s);
-  }
-  return cudaErrorInvalidValue;
+template <typename T> cudaError_t launch_binned_deposit(const BinArgs<T>& a, cudaStream_t s) {
+  if (a.g.H <= 16) return a.fixed ? launch_deposit_t<T, true, true>(a, s) : launch_deposit_t<T, false, true>(a, s);
+  return a.fixed ? launch_deposit_t<T, true, false>(a, s) : launch_deposit_t<T, false, false>(a, s);
+}
+
+template <typename T> cudaError_t launch_binned_rebin(const BinArgs<T>& a, cudaStream_t s) {
+  int blocks = 0;
+  const cudaError_t e = resident_blocks((const void*)k_binned_rebin<T>, 256, 0, &blocks);
+  if (e != cudaSuccess) return e;
+  k_binned_rebin<T><<<min(blocks, a.max_items), 256, 0, s>>>(a);
+  return cudaGetLastError();
 }
 
 int chunk_list_blocks(int NT) { return (NT + 1 + kCLBlock - 1) / kCLBlock; }
@@ -1760,7 +1868,7 @@ cudaError_t launch_compact(const BinArgs<T>& a, int64_t max_chunks, unsigned lon
                            uint32_t* id, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(cursor, 0, sizeof(unsigned long long), s);
   if (e != cudaSuccess || max_chunks < 1) return e;
-  k_compact<T><<<(unsigned)max_chunks, 1024, 0, s>>>(a, cursor, x, y, z, id);   // a work item per block
+  k_compact<T><<<(unsigned)max_chunks, 256, 0, s>>>(a, cursor, x, y, z, id);   // a work item per block
   return cudaGetLastError();
 }
 
@@ -1859,7 +1967,8 @@ template <typename T> cudaError_t launch_alpha_energy(const cpx<T>* alpha, int H
 }
 
 #define SIPF_INST(T)                                                                                          \
-  template cudaError_t launch_binned<T>(const BinArgs<T>&, int, int, int, cudaStream_t);                       \
+  template cudaError_t launch_binned_deposit<T>(const BinArgs<T>&, cudaStream_t);                             \
+  template cudaError_t launch_binned_rebin<T>(const BinArgs<T>&, cudaStream_t);                               \
   template cudaError_t launch_move<T>(const BinArgs<T>&, cudaStream_t);                                       \
   template cudaError_t launch_move_batch<T>(const BinArgs<T>*, const long long*, int, unsigned long long*,     \
                                             const uint32_t*, bool, cudaStream_t, int, int);                  \

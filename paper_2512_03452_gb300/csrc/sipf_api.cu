@@ -4,6 +4,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <cstdio>
 #include <mutex>
 #include <string>
@@ -187,11 +188,9 @@ struct sipf_ctx {
   int64_t H3() const { return (int64_t)p.H * p.H * p.H; }
   int64_t S() const { return (int64_t)p.H * p.H * (p.H / 2 + 1); }
   bool fixed() const { return p.deposit_mode == SIPF_DEPOSIT_DETERMINISTIC; }
-  int64_t max_chunks() const { return p.P / binned_chunk() + NT + 2; }
+  int64_t max_chunks() const { return p.P / chunk + NT + 2; }
   int resort() const { return p.resort_every > 0 ? p.resort_every : 16; }
-  // bins per merge window of the chunk lists (small bins of a window form one
-  // work item): 4 for a single run, 16 for the runs of a batch
-  int merge = 4;
+  int chunk = 4096, small = 256;   // work-item length and merge threshold (particle_chunk, particle_small)
 };
 
 enum { kDscMass = 0, kDscAlpha0 = 1, kDscM2 = 2, kDscRing = 3, kDscHF = 4, kDscTot = 5, kDscMax = 6, kDscCount = 8 };
@@ -262,6 +261,9 @@ template <typename T> BinArgs<T> bin_args(sipf_ctx* c, int src_buf, int src_lay,
   a.NT = c->NT;
   a.ntx = c->ntx;
   a.tile_shift = c->shift;
+  a.max_items = (int)std::min<int64_t>(c->max_chunks(), INT32_MAX);
+  a.chunk = c->chunk;
+  a.small = c->small;
   a.phi = c->phi;
   a.grad4 = (const T*)c->grad;
   a.g = make_geo<T>(c->p.L, c->p.H);
@@ -282,7 +284,8 @@ template <typename T> BinArgs<T> bin_args(sipf_ctx* c, int src_buf, int src_lay,
 // Chunk-list arguments: bins of (cursor, cap, base) into the context's chunk
 // arrays; `other` are the cursors to clear for the next pass.
 ChunkListArgs cl_args(sipf_ctx* c, const int* cursor, const int* cap, const long long* base, int* other) {
-  return ChunkListArgs{cursor, cap, base, c->count, c->chunk_start, c->chunks, other, c->NT, c->part, c->merge};
+  return ChunkListArgs{cursor, cap, base, c->count, c->chunk_start, c->chunks, other, c->NT, c->part,
+                       c->chunk, c->small};
 }
 
 // The current bins are final (positions of step n, before their deposit):
@@ -304,7 +307,7 @@ template <typename T> int flush_deposit(sipf_ctx* c) {
   if (!c->dep_pending) return SIPF_OK;
   if (!c->phi_zero)
     SIPF_CK(cudaMemsetAsync(c->phi, 0, (size_t)c->H3() * (c->fixed() ? 8 : sizeof(T)), c->stream));
-  SIPF_CK(launch_binned<T>(bin_args<T>(c, c->cur, c->lc, -1, 0), 0, 1, 0, c->stream));
+  SIPF_CK(launch_binned_deposit<T>(bin_args<T>(c, c->cur, c->lc, -1, 0), c->stream));
   c->launches += 1;
   c->dep_pending = false;
   c->phi_zero = false;
@@ -329,7 +332,7 @@ template <typename T> int rebin_from_staging(sipf_ctx* c) {
                              (T*)c->bx[d][2], c->bid[d], c->lbase[L], c->lcap[L], c->cursor[d], c->err, c->stream,
                              &e)) {
     SIPF_CK(cudaMemsetAsync(c->work, 0, sizeof(unsigned long long), c->stream));
-    e = launch_binned<T>(bin_args<T>(c, -1, 0, d, L), 0, 0, 1, c->stream);
+    e = launch_binned_rebin<T>(bin_args<T>(c, -1, 0, d, L), c->stream);
   }
   SIPF_CK(e);
   SIPF_CK(launch_chunk_list(cl_args(c, c->cursor[d], c->lcap[L], c->lbase[L], c->cursor[1 - d]), c->work, nullptr,
@@ -416,7 +419,7 @@ template <typename T> int step_impl(sipf_ctx* c, int64_t nsteps) {
       const int L = 1 - c->lc, d2 = 1 - c->cur;
       SIPF_CK(launch_layout(c->cursor[c->cur], c->lcap[L], c->lbase[L], c->NT, c->ntx, (int)c->p.P, c->stream));
       SIPF_CK(cudaMemsetAsync(c->work, 0, sizeof(unsigned long long), c->stream));
-      SIPF_CK(launch_binned<T>(bin_args<T>(c, c->cur, c->lc, d2, L), 0, 0, 1, c->stream));
+      SIPF_CK(launch_binned_rebin<T>(bin_args<T>(c, c->cur, c->lc, d2, L), c->stream));
       SIPF_CK(launch_chunk_list(cl_args(c, c->cursor[d2], c->lcap[L], c->lbase[L], c->cursor[c->cur]), c->work, nullptr,
                                 c->stream));
       c->launches += 4;
@@ -827,6 +830,8 @@ int sipf_init(const sipf_params* p, const double* X0, void* stream, sipf_ctx** o
   c->shift = binned_tile_shift(p->H);
   c->ntx = p->H <= 16 ? 1 : p->H >> c->shift;
   c->NT = c->ntx * c->ntx * c->ntx;
+  c->chunk = particle_chunk(p->P, p->H, p->precision == 64);
+  c->small = particle_small(c->chunk);
   const size_t nb = (size_t)c->NT + 1;
   // bins hold at most 1.5 P + 64 NT + 6 P / 4 (capacities with spare room), the overflow bin P
   c->cap_total = (int64_t)(4 * P + 68 * (size_t)c->NT + 1024);
@@ -1562,6 +1567,8 @@ int sipf_batch_init(int32_t nruns, const sipf_params* params, const double* cons
     }
     b->own_stream = true;
   }
+  int64_t total = 0;
+  for (int r = 0; r < nruns; ++r) total += params[r].P;
   for (int r = 0; r < nruns; ++r) {
     sipf_ctx* c = nullptr;
     int v = sipf_init(&params[r], X0[r], b->stream, &c);
@@ -1570,9 +1577,11 @@ int sipf_batch_init(int32_t nruns, const sipf_params* params, const double* cons
       return v;
     }
     b->runs.push_back(c);
-    // many sparse runs: merge windows of 16 bins; the current bins' chunk
-    // list is made again with them (their counts are unchanged)
-    c->merge = 16;
+    // the work items sized for all runs' particles together (never shorter than
+    // the run's own); the current bins' chunk list is made again with them
+    // (their counts are unchanged)
+    c->chunk = std::max(c->chunk, particle_chunk(total, c->p.H, c->p.precision == 64));
+    c->small = particle_small(c->chunk);
     cudaError_t e = launch_chunk_list(cl_args(c, c->cursor[c->cur], c->lcap[c->lc], c->lbase[c->lc],
                                               c->cursor[1 - c->cur]),
                                       c->work, nullptr, c->stream);

@@ -160,7 +160,8 @@ template <typename T>
 cudaError_t launch_adj_spectral(const cpx<T>* ghat, cpx<T>* abar, cpx<T>* spec, int H, SpecParams sp, cudaStream_t s);
 
 // ---- particle launchers (particle_kernels.cu) -----------------------------------
-// One work item of the binned kernel: `len` particles of bin `bin` from slot `start`.
+// One work item of the particle passes: `len` particles of bin `bin` from slot
+// `start`; bin = -1: the small bins of merge window `start` (see particle_kernels.cu).
 struct ChunkDesc {
   long long start;
   int bin, len;
@@ -182,6 +183,8 @@ struct BinArgs {
   int* dst_cursor;               // [NT+1] fill cursors (zeroed before the launch)
   unsigned long long* work;      // chunk counter of the persistent grid (zeroed before the launch)
   int NT, ntx, tile_shift;       // tiles, tiles per axis, log2 tile edge
+  int max_items;                 // bound of the number of work items
+  int chunk, small;              // the chunk list's item length and merge threshold (see ChunkListArgs)
   // physics
   void* phi;                     // deposit target (T, or int64 fixed point)
   const T* grad4;                // H^3 nodes x 4 (gx, gy, gz, 0)
@@ -206,7 +209,7 @@ struct ChunkListArgs {
   int* other_cursor;        // cursors of the other buffer (cleared)
   int NT;
   long long* part;          // chunk totals of the blocks of kCLBlock bins (chunk_list_blocks(NT))
-  int merge;                // bins per merge window of the small bins (power of two, 2 ... 16)
+  int chunk, small;         // most particles of an item of one bin; bins below `small` are merged
 };
 struct LayoutArgs {
   const int* want;
@@ -225,10 +228,13 @@ cudaError_t launch_chunk_list_batch(const ChunkListArgs* t, int nruns, int max_N
 cudaError_t launch_run_prefix(const ChunkListArgs* t, int nruns, long long* prefix, unsigned long long* work,
                               uint32_t* step, int bump, cudaStream_t s);
 cudaError_t launch_layout_batch(const LayoutArgs* t, int nruns, cudaStream_t s);
-int binned_window_slots(int H);
-int binned_chunk();
+// Work-item length for P particles on an H^3 grid, and the bin size below which bins are merged.
+int particle_chunk(int64_t P, int H, bool fp64);
+int particle_small(int chunk);
 int binned_tile_shift(int H);
-template <typename T> cudaError_t launch_binned(const BinArgs<T>& a, int move, int deposit, int rebin, cudaStream_t s);
+// Deposit of the source bins; re-bin of the source bins into the destination bins.
+template <typename T> cudaError_t launch_binned_deposit(const BinArgs<T>& a, cudaStream_t s);
+template <typename T> cudaError_t launch_binned_rebin(const BinArgs<T>& a, cudaStream_t s);
 // The move + re-bin pass of a step (Algorithm 4 particle loop).
 template <typename T> cudaError_t launch_move(const BinArgs<T>& a, cudaStream_t s);
 // From fill cursors: clamped counts, chunk prefix sums and chunk descriptors
