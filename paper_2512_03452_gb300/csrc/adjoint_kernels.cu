@@ -214,6 +214,7 @@ __device__ __forceinline__ A3<T> deposit_adjoint4_quads(const T* __restrict__ qu
 template <typename T>
 __global__ void __launch_bounds__(256) k_adj_quads(const T* __restrict__ phibar, T* __restrict__ quads, int H,
                                                    int64_t H3) {
+  pdl_wait();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < H3; i += (int64_t)gridDim.x * blockDim.x) {
     const int z = (int)(i & (H - 1));
     const int64_t row = i - z;
@@ -318,6 +319,7 @@ template <typename T> __device__ __forceinline__ void block_acc2(T a, T b, doubl
 template <typename T, int G2P, int P2G>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? ((G2P && P2G) ? 4 : 2) : 1)
 k_adj_step(AdjArgs<T> a) {
+  pdl_wait();
   const int g2p = G2P ? G2P : a.g2p, p2g = P2G ? P2G : a.p2g;
   T chi_part = T(0), s_part = T(0);
   const Geo<T> g = a.g;
@@ -374,6 +376,7 @@ k_adj_step(AdjArgs<T> a) {
 // the nodes are cleared for the next step's accumulation.
 template <typename T>
 __global__ void __launch_bounds__(256) k_adj_planes(T* __restrict__ gbar4, T* __restrict__ planes, int64_t H3) {
+  pdl_wait();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < H3; i += (int64_t)gridDim.x * blockDim.x) {
     T* node = gbar4 + (size_t)i * 4;
     planes[i] = node[0];
@@ -391,6 +394,7 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 k_adj_terminal(const T* __restrict__ x, const T* __restrict__ y, const T* __restrict__ z, int64_t P,
                const T* __restrict__ phibar, int p2g, T w_inv_h, Geo<T> g, T* __restrict__ xb4) {
+  pdl_wait();
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += (int64_t)gridDim.x * blockDim.x) {
     const A3<T> dp = deposit_adjoint<T>(phibar, p2g, x[p], y[p], z[p], w_inv_h, g);
     Rec4<T>::store(xb4 + (size_t)p * 4, dp.x, dp.y, dp.z);
@@ -405,6 +409,7 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 k_adj_spectral(const cpx<T>* __restrict__ ghat, cpx<T>* __restrict__ abar, cpx<T>* __restrict__ spec, int H,
                SpecConst<T> sk) {
+  pdl_wait();
   const int nh = H / 2 + 1;
   const size_t S = (size_t)H * H * nh;
   const T two_pi_L = sk.two_pi_L, filt = sk.filt, inv_L3 = sk.inv_L3;
@@ -459,18 +464,18 @@ int grid_blocks(int64_t n) {
 template <typename T> cudaError_t launch_adj_step(const AdjArgs<T>& a, cudaStream_t s) {
   if (a.P <= 0) return cudaSuccess;
   auto k = (a.g2p == 2 && a.p2g == 4) ? k_adj_step<T, 2, 4> : k_adj_step<T, 0, 0>;
-  k<<<grid_blocks(a.P), 256, 0, s>>>(a);
+  launch_k(k, grid_blocks(a.P), 256, 0, s, a);
   return cudaGetLastError();
 }
 
 template <typename T> cudaError_t launch_adj_quads(const T* phibar, T* quads, int H, cudaStream_t s) {
   const int64_t H3 = (int64_t)H * H * H;
-  k_adj_quads<T><<<grid_blocks(H3), 256, 0, s>>>(phibar, quads, H, H3);
+  launch_k(k_adj_quads<T>, grid_blocks(H3), 256, 0, s, phibar, quads, H, H3);
   return cudaGetLastError();
 }
 
 template <typename T> cudaError_t launch_adj_planes(T* gbar4, T* planes, int64_t H3, cudaStream_t s) {
-  k_adj_planes<T><<<grid_blocks(H3), 256, 0, s>>>(gbar4, planes, H3);
+  launch_k(k_adj_planes<T>, grid_blocks(H3), 256, 0, s, gbar4, planes, H3);
   return cudaGetLastError();
 }
 
@@ -478,7 +483,7 @@ template <typename T>
 cudaError_t launch_adj_terminal(const T* x, const T* y, const T* z, int64_t P, const T* phibar, int p2g, T w_inv_h,
                                 Geo<T> g, T* xb4, cudaStream_t s) {
   if (P <= 0) return cudaSuccess;
-  k_adj_terminal<T><<<grid_blocks(P), 256, 0, s>>>(x, y, z, P, phibar, p2g, w_inv_h, g, xb4);
+  launch_k(k_adj_terminal<T>, grid_blocks(P), 256, 0, s, x, y, z, P, phibar, p2g, w_inv_h, g, xb4);
   return cudaGetLastError();
 }
 
@@ -486,7 +491,7 @@ template <typename T>
 cudaError_t launch_adj_spectral(const cpx<T>* ghat, cpx<T>* abar, cpx<T>* spec, int H, SpecParams sp,
                                 cudaStream_t s) {
   const int64_t S = (int64_t)H * H * (H / 2 + 1);
-  k_adj_spectral<T><<<grid_blocks(S), 256, 0, s>>>(ghat, abar, spec, H, spec_const<T>(sp));
+  launch_k(k_adj_spectral<T>, grid_blocks(S), 256, 0, s, ghat, abar, spec, H, spec_const<T>(sp));
   return cudaGetLastError();
 }
 

@@ -116,6 +116,7 @@ template <typename T, typename Tin>
 __global__ void __launch_bounds__(kThreads)
 k_rows_r2c(Tin* __restrict__ in, double in_scale, int zero_input, cpx<T>* __restrict__ out,
            int lgH, int rows, int RP, double* mass_acc) {
+  pdl_wait();
   extern __shared__ unsigned char smem_raw[];
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
   cpx<T>* buf = tw + kNmax / 2;
@@ -166,6 +167,7 @@ k_rows_r2c(Tin* __restrict__ in, double in_scale, int zero_input, cpx<T>* __rest
 template <typename T, int DIR>
 __global__ void __launch_bounds__(kThreads)
 k_cols(cpx<T>* __restrict__ data, int lgH, int B, int lgBC, size_t comp_stride, T scale) {
+  pdl_wait();
   extern __shared__ unsigned char smem_raw[];
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
   cpx<T>* buf = tw + kNmax / 2;
@@ -206,6 +208,7 @@ template <typename T, int MODE>
 __global__ void __launch_bounds__(kThreads)
 k_spectral_x(const cpx<T>* __restrict__ T1, cpx<T>* __restrict__ alpha, cpx<T>* __restrict__ T2,
              int lgH, int lgBC, SpecConst<T> sk, double* alpha0_shadow) {
+  pdl_wait();
   extern __shared__ unsigned char smem_raw[];
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
   cpx<T>* buf = tw + kNmax / 2;
@@ -303,6 +306,7 @@ template <typename T, int NCOMP>
 __global__ void __launch_bounds__(kThreads)
 k_rows_c2r(const cpx<T>* __restrict__ in, size_t comp_stride, T* __restrict__ out, int lgH, int rows,
            int RP, double* max_acc) {
+  pdl_wait();
   extern __shared__ unsigned char smem_raw[];
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
   cpx<T>* buf = tw + kNmax / 2;
@@ -899,6 +903,7 @@ template <typename T, int E, typename Tin>
 __global__ void __launch_bounds__(256)
 kw_rows_r2c(Tin* __restrict__ in, double in_scale, int zero_input, cpx<T>* __restrict__ out, int rows,
             double* mass_acc) {
+  pdl_wait();
   __shared__ cpx<T> tw[tw_len<T, E>()];
   __shared__ cpx<T> zb[8 * row_scratch<T, 32 * E>()];
   load_tw_group<T, E, true>(tw);
@@ -933,6 +938,7 @@ __device__ __forceinline__ void cols_body(cpx<T>* __restrict__ base, int B, T sc
 template <typename T, int E, int DIR, int BC>
 __global__ void __launch_bounds__(256)
 kw_cols(cpx<T>* __restrict__ data, int B, size_t comp_stride, T scale) {
+  pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
   load_tw_group<T, E, false>(tw);
@@ -1154,6 +1160,7 @@ template <int N, int MODE>
 __global__ void __launch_bounds__(256)
 kwr_spectral_x(const cpx<float>* __restrict__ T1, cpx<float>* __restrict__ alpha, cpx<float>* __restrict__ T2,
                SpecConst<float> sk, double* alpha0_shadow) {
+  pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<float>* twq = reinterpret_cast<cpx<float>*>(smem_raw);
   load_twq<float, N>(twq);
@@ -1167,6 +1174,7 @@ kwr_spectral_x(const cpx<float>* __restrict__ T1, cpx<float>* __restrict__ alpha
 
 template <int N>
 __global__ void __launch_bounds__(512) kwrb_spectral_x(const FftRun<float>* __restrict__ runs) {
+  pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<float>* twq = reinterpret_cast<cpx<float>*>(smem_raw);
   load_twq<float, N>(twq);
@@ -1183,6 +1191,7 @@ template <typename T, int E, int MODE, int BC>
 __global__ void __launch_bounds__(256)
 kw_spectral_x(const cpx<T>* __restrict__ T1, cpx<T>* __restrict__ alpha, cpx<T>* __restrict__ T2, SpecConst<T> sk,
               double* alpha0_shadow) {
+  pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
   load_tw_group<T, E, false>(tw);
@@ -1301,6 +1310,7 @@ __device__ __forceinline__ void rows_c2r_body(const cpx<T>* __restrict__ in, siz
 template <typename T, int E, int NCOMP>
 __global__ void __launch_bounds__(256)
 kw_rows_c2r(const cpx<T>* __restrict__ in, size_t comp_stride, T* __restrict__ out, int rows, double* max_acc) {
+  pdl_wait();
   constexpr int N = 32 * E;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
@@ -1559,6 +1569,7 @@ __device__ __forceinline__ void plane_inv_body(const cpx<T>* __restrict__ in, T*
 
 template <typename T, int E>
 __global__ void __launch_bounds__(group_rows<T, 32 * E>() ? 512 : 1024) kwp_fwd(const FftRun<T>* __restrict__ runs) {
+  pdl_wait();
   constexpr int N = 32 * E, NH = N / 2 + 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
@@ -1578,6 +1589,7 @@ __global__ void __launch_bounds__(group_rows<T, 32 * E>() ? 512 : 1024) kwp_fwd(
 
 template <typename T, int E>
 __global__ void __launch_bounds__(group_rows<T, 32 * E>() ? 512 : 1024) kwp_inv(const FftRun<T>* __restrict__ runs) {
+  pdl_wait();
   constexpr int N = 32 * E, NH = N / 2 + 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
@@ -1916,6 +1928,7 @@ __device__ __forceinline__ void cplane_inv_body(const cpx<T>* __restrict__ in, T
 
 template <typename T, int E, int CS>
 __global__ void __launch_bounds__(1024) kwc_fwd(const FftRun<T>* __restrict__ runs) {
+  pdl_wait();
   constexpr int N = 32 * E, NH = N / 2 + 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
@@ -1935,6 +1948,7 @@ __global__ void __launch_bounds__(1024) kwc_fwd(const FftRun<T>* __restrict__ ru
 
 template <typename T, int E, int CS>
 __global__ void __launch_bounds__(1024) kwc_inv(const FftRun<T>* __restrict__ runs) {
+  pdl_wait();
   constexpr int N = 32 * E, NH = N / 2 + 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
@@ -1957,13 +1971,15 @@ static cudaError_t launch_cluster(K kernel, dim3 grid, int threads, size_t smem,
   cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = cs;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // see launch_k
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = grid.x * grid.y * grid.z <= kPdlBlocks ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
@@ -1976,9 +1992,9 @@ template <typename T, int E>
 static cudaError_t warp_rows_r2c(const void* in, int in_kind, double in_scale, bool zero_input, cpx<T>* out, int rows,
                                  double* mass_acc, cudaStream_t s) {
   if (in_kind == 0)
-    kw_rows_r2c<T, E, T><<<warp_blocks(rows), 256, 0, s>>>((T*)in, in_scale, zero_input ? 1 : 0, out, rows, mass_acc);
+    launch_k(kw_rows_r2c<T, E, T>, warp_blocks(rows), 256, 0, s, (T*)in, in_scale, zero_input ? 1 : 0, out, rows, mass_acc);
   else
-    kw_rows_r2c<T, E, unsigned long long><<<warp_blocks(rows), 256, 0, s>>>((unsigned long long*)in, in_scale,
+    launch_k(kw_rows_r2c<T, E, unsigned long long>, warp_blocks(rows), 256, 0, s, (unsigned long long*)in, in_scale,
                                                                            zero_input ? 1 : 0, out, rows, mass_acc);
   return cudaGetLastError();
 }
@@ -1991,7 +2007,7 @@ static cudaError_t warp_cols(cpx<T>* data, int A, int B, int ncomp, size_t comp_
   cudaError_t e = set_smem(k, smem);
   if (e != cudaSuccess) return e;
   dim3 grid((B + BC - 1) / BC, A, ncomp);
-  k<<<grid, 256, smem, s>>>(data, B, comp_stride, (T)scale);
+  launch_k(k, grid, 256, smem, s, data, B, comp_stride, (T)scale);
   return cudaGetLastError();
 }
 
@@ -2005,7 +2021,7 @@ static cudaError_t warp_spectral(const cpx<T>* T1, cpx<T>* alpha, cpx<T>* T2, Sp
     auto k = kwr_spectral_x<N, MODE>;
     cudaError_t e = set_smem(k, smem);
     if (e != cudaSuccess) return e;
-    k<<<(XRegShape<N>::TASKS + nw - 1) / nw, 32 * nw, smem, s>>>(T1, alpha, T2, spec_const<T>(sp), shadow);
+    launch_k(k, (XRegShape<N>::TASKS + nw - 1) / nw, 32 * nw, smem, s, T1, alpha, T2, spec_const<T>(sp), shadow);
     return cudaGetLastError();
   } else {
   constexpr int BC = (sizeof(T) == 8 && E == 8) ? 4 : ((sizeof(T) == 8 || E == 8) ? 8 : 16);
@@ -2014,7 +2030,7 @@ static cudaError_t warp_spectral(const cpx<T>* T1, cpx<T>* alpha, cpx<T>* T2, Sp
   auto k = kw_spectral_x<T, E, MODE, BC>;
   cudaError_t e = set_smem(k, smem);
   if (e != cudaSuccess) return e;
-  k<<<(B + BC - 1) / BC, 256, smem, s>>>(T1, alpha, T2, spec_const<T>(sp), shadow);
+  launch_k(k, (B + BC - 1) / BC, 256, smem, s, T1, alpha, T2, spec_const<T>(sp), shadow);
   return cudaGetLastError();
   }
 }
@@ -2027,7 +2043,7 @@ static cudaError_t warp_rows_c2r(const cpx<T>* in, size_t comp_stride, T* out, i
   auto k = kw_rows_c2r<T, E, NCOMP>;
   cudaError_t e = set_smem(k, smem);
   if (e != cudaSuccess) return e;
-  k<<<warp_blocks(rows), 256, smem, s>>>(in, comp_stride, out, rows, max_acc);
+  launch_k(k, warp_blocks(rows), 256, smem, s, in, comp_stride, out, rows, max_acc);
   return cudaGetLastError();
 }
 
@@ -2067,11 +2083,11 @@ cudaError_t launch_rows_r2c(const void* in, int in_kind, double in_scale, bool z
   if (in_kind == 0) {
     auto k = k_rows_r2c<T, T>;
     if ((e = set_smem(k, smem)) != cudaSuccess) return e;
-    k<<<blocks, kThreads, smem, s>>>((T*)in, in_scale, zero_input ? 1 : 0, out, lgH, rows, RP, mass_acc);
+    launch_k(k, blocks, kThreads, smem, s, (T*)in, in_scale, zero_input ? 1 : 0, out, lgH, rows, RP, mass_acc);
   } else {
     auto k = k_rows_r2c<T, unsigned long long>;
     if ((e = set_smem(k, smem)) != cudaSuccess) return e;
-    k<<<blocks, kThreads, smem, s>>>((unsigned long long*)in, in_scale, zero_input ? 1 : 0, out, lgH, rows,
+    launch_k(k, blocks, kThreads, smem, s, (unsigned long long*)in, in_scale, zero_input ? 1 : 0, out, lgH, rows,
                                      RP, mass_acc);
   }
   return cudaGetLastError();
@@ -2106,11 +2122,11 @@ cudaError_t launch_cols(cpx<T>* data, int H, int A, int B, int ncomp, size_t com
   if (dir < 0) {
     auto k = k_cols<T, -1>;
     if ((e = set_smem(k, smem)) != cudaSuccess) return e;
-    k<<<grid, kThreads, smem, s>>>(data, lgH, B, lgBC, comp_stride, (T)scale);
+    launch_k(k, grid, kThreads, smem, s, data, lgH, B, lgBC, comp_stride, (T)scale);
   } else {
     auto k = k_cols<T, +1>;
     if ((e = set_smem(k, smem)) != cudaSuccess) return e;
-    k<<<grid, kThreads, smem, s>>>(data, lgH, B, lgBC, comp_stride, (T)scale);
+    launch_k(k, grid, kThreads, smem, s, data, lgH, B, lgBC, comp_stride, (T)scale);
   }
   return cudaGetLastError();
 }
@@ -2127,7 +2143,7 @@ static cudaError_t spectral_mode(const cpx<T>* T1, cpx<T>* alpha, cpx<T>* T2, in
   auto k = k_spectral_x<T, MODE>;
   cudaError_t e = set_smem(k, smem);
   if (e != cudaSuccess) return e;
-  k<<<(B + BC - 1) / BC, kThreads, smem, s>>>(T1, alpha, T2, lgH, lgBC, spec_const<T>(sp), shadow);
+  launch_k(k, (B + BC - 1) / BC, kThreads, smem, s, T1, alpha, T2, lgH, lgBC, spec_const<T>(sp), shadow);
   return cudaGetLastError();
 }
 
@@ -2179,11 +2195,11 @@ cudaError_t launch_rows_c2r(const cpx<T>* in, int ncomp, size_t comp_stride, T* 
   if (ncomp == 3) {
     auto k = k_rows_c2r<T, 3>;
     if ((e = set_smem(k, smem)) != cudaSuccess) return e;
-    k<<<blocks, kThreads, smem, s>>>(in, comp_stride, out, lgH, rows, RP, nullptr);
+    launch_k(k, blocks, kThreads, smem, s, in, comp_stride, out, lgH, rows, RP, nullptr);
   } else {
     auto k = k_rows_c2r<T, 1>;
     if ((e = set_smem(k, smem)) != cudaSuccess) return e;
-    k<<<blocks, kThreads, smem, s>>>(in, comp_stride, out, lgH, rows, RP, max_acc);
+    launch_k(k, blocks, kThreads, smem, s, in, comp_stride, out, lgH, rows, RP, max_acc);
   }
   return cudaGetLastError();
 }
@@ -2206,7 +2222,7 @@ static cudaError_t kwb_cols_launch(const FftRun<T>* runs, int nruns, int ncomp, 
   if (smc > kMaxSmem) return cudaErrorInvalidValue;
   cudaError_t e;
   if ((e = set_smem(kwb_cols<T, E, DIR, BC>, smc)) != cudaSuccess) return e;
-  kwb_cols<T, E, DIR, BC><<<dim3((NHH + BC - 1) / BC, N, nruns * ncomp), 256, smc, s>>>(runs, ncomp);
+  launch_plain(kwb_cols<T, E, DIR, BC>, dim3((NHH + BC - 1) / BC, N, nruns * ncomp), 256, smc, s, runs, ncomp);
   return cudaGetLastError();
 }
 
@@ -2227,13 +2243,13 @@ static cudaError_t kwb_spectral_launch(const FftRun<T>* runs, int nruns, int nw,
     const size_t smr = xreg_smem_bytes<N>(nw);
     if (smr > kMaxSmem) return cudaErrorInvalidValue;
     if ((e = set_smem(kwrb_spectral_x<N>, smr)) != cudaSuccess) return e;
-    kwrb_spectral_x<N><<<dim3((XRegShape<N>::TASKS + nw - 1) / nw, nruns), 32 * nw, smr, s>>>(runs);
+    launch_k(kwrb_spectral_x<N>, dim3((XRegShape<N>::TASKS + nw - 1) / nw, nruns), 32 * nw, smr, s, runs);
     return cudaGetLastError();
   } else {
     const size_t sms = spectral_smem<T, E, SBC>();
     if (sms > kMaxSmem) return cudaErrorInvalidValue;
     if ((e = set_smem(kwb_spectral_x<T, E, SBC>, sms)) != cudaSuccess) return e;
-    kwb_spectral_x<T, E, SBC><<<dim3((N * NHH + SBC - 1) / SBC, nruns), 32 * nw, sms, s>>>(runs);
+    launch_plain(kwb_spectral_x<T, E, SBC>, dim3((N * NHH + SBC - 1) / SBC, nruns), 32 * nw, sms, s, runs);
     return cudaGetLastError();
   }
 }
@@ -2295,11 +2311,11 @@ static cudaError_t field_batch_e(const FftRun<T>* runs, int nruns, int stages, c
       nk += 1;
     } else if (planes) {
       if ((e = set_smem(kwp_fwd<T, E>, fsm)) != cudaSuccess) return e;
-      kwp_fwd<T, E><<<dim3(N, nruns), 32 * fnw, fsm, s>>>(runs);
+      launch_k(kwp_fwd<T, E>, dim3(N, nruns), 32 * fnw, fsm, s, runs);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
       nk += 1;
     } else {
-      kwb_rows_r2c<T, E><<<dim3(rblocks, nruns), 256, 0, s>>>(runs);
+      launch_plain(kwb_rows_r2c<T, E>, dim3(rblocks, nruns), 256, 0, s, runs);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
       if ((e = kwb_cols_bc<T, E, -1>(runs, nruns, 1, bc, s)) != cudaSuccess) return e;
       nk += 2;
@@ -2322,20 +2338,20 @@ static cudaError_t field_batch_e(const FftRun<T>* runs, int nruns, int stages, c
   } else if ((stages & kFieldInverse) && inv3) {
     if constexpr (E <= 2) {
       if ((e = set_smem(kwp_inv3<T, E>, i3sm)) != cudaSuccess) return e;
-      kwp_inv3<T, E><<<dim3(N, nruns), 32 * i3nw, i3sm, s>>>(runs);
+      launch_plain(kwp_inv3<T, E>, dim3(N, nruns), 32 * i3nw, i3sm, s, runs);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
       nk += 1;
     }
   } else if ((stages & kFieldInverse) && planes) {
     if ((e = set_smem(kwp_inv<T, E>, ism)) != cudaSuccess) return e;
-    kwp_inv<T, E><<<dim3(N, 3, nruns), 32 * inw, ism, s>>>(runs);
+    launch_k(kwp_inv<T, E>, dim3(N, 3, nruns), 32 * inw, ism, s, runs);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     nk += 1;
   } else if (stages & kFieldInverse) {
     if ((e = kwb_cols_bc<T, E, +1>(runs, nruns, 3, bc, s)) != cudaSuccess) return e;
     const size_t smr = row_c2r_smem<T, E, 4>();
     if ((e = set_smem(kwb_rows_c2r<T, E>, smr)) != cudaSuccess) return e;
-    kwb_rows_c2r<T, E><<<dim3(rblocks, nruns), 256, smr, s>>>(runs);
+    launch_plain(kwb_rows_c2r<T, E>, dim3(rblocks, nruns), 256, smr, s, runs);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     nk += 2;
   }

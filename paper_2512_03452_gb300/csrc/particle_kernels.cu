@@ -601,6 +601,7 @@ k_binned_deposit(const __grid_constant__ BinArgs<T> a, int use_win) {
     const int n = WHOLE ? kReplicas * a.g.H * a.g.H * a.g.H : kTileReps * kWinSlots;
     for (int i = threadIdx.x; i < n; i += blockDim.x) win[i] = A(0);
   }
+  pdl_wait();
   for_items(a, s_desc, [&](const ChunkDesc& cur) {
     if (cur.bin >= 0) deposit_chunk<T, FIXED, WHOLE>(a, cur, win, use_win != 0);
     else deposit_merged<T, FIXED, WHOLE>(a, cur, win);
@@ -610,6 +611,7 @@ k_binned_deposit(const __grid_constant__ BinArgs<T> a, int use_win) {
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_binned_rebin(const __grid_constant__ BinArgs<T> a) {
+  pdl_wait();
   __shared__ ChunkDesc s_desc[2];
   for_items(a, s_desc, [&](const ChunkDesc& cur) {
     if (cur.bin >= 0) {
@@ -634,8 +636,9 @@ k_deposit_batch(const BinArgs<T>* __restrict__ table, const long long* __restric
   A* win = reinterpret_cast<A*>(smem_raw);
   __shared__ ChunkDesc s_desc[2];
   __shared__ int s_run[2];
-  const long long total = prefix[nruns];
   for (int i = threadIdx.x; i < kTileReps * kWinSlots; i += blockDim.x) win[i] = A(0);
+  pdl_wait();
+  const long long total = prefix[nruns];
   if (threadIdx.x == 0) {
     const long long c = (long long)atomicAdd(work, 1ULL);
     if (c < total) {
@@ -931,6 +934,7 @@ __device__ __forceinline__ void move_chunk(const BinArgs<T>& a, const ChunkDesc&
 template <typename T, int G2P>
 __global__ void __launch_bounds__(kMoveThreads, move_min_blocks<T>())
 k_move(BinArgs<T> a) {
+  pdl_wait();
   __shared__ MoveSmem<T> sm;
   const long long nchunks = a.chunk_start[a.NT + 1];
   if (threadIdx.x == 0) {
@@ -962,6 +966,7 @@ template <typename T, bool MOVE, int G2P>
 __global__ void __launch_bounds__(kMoveThreads, move_min_blocks<T>())
 k_move_batch(const BinArgs<T>* __restrict__ table, const long long* __restrict__ prefix, int nruns,
              unsigned long long* work, const uint32_t* step) {
+  pdl_wait();
   __shared__ MoveSmem<T> sm;
   const long long total = prefix[nruns];
   const uint32_t n = *step + 1;
@@ -1021,7 +1026,7 @@ template <typename T> cudaError_t launch_move(const BinArgs<T>& a, cudaStream_t 
   auto k = a.g2p == 4 ? k_move<T, 4> : k_move<T, 2>;
   const cudaError_t e = resident_blocks((const void*)k, kMoveThreads, 0, &blocks);
   if (e != cudaSuccess) return e;
-  k<<<min(blocks, a.max_items), kMoveThreads, 0, s>>>(a);
+  launch_k(k, min(blocks, a.max_items), kMoveThreads, 0, s, a);
   return cudaGetLastError();
 }
 
@@ -1170,21 +1175,27 @@ __device__ __forceinline__ void chunk_emit_body(const ChunkListArgs& a, int blk,
 
 __device__ __forceinline__ int chunk_list_blocks_dev(int NT) { return (NT + 1 + kCLBlock - 1) / kCLBlock; }
 
-__global__ void __launch_bounds__(kCLBlock) k_chunk_count(ChunkListArgs a) { chunk_count_body(a, blockIdx.x); }
+__global__ void __launch_bounds__(kCLBlock) k_chunk_count(ChunkListArgs a) {
+  pdl_wait();
+  chunk_count_body(a, blockIdx.x);
+}
 
 __global__ void __launch_bounds__(kCLBlock)
 k_chunk_emit(ChunkListArgs a, unsigned long long* work, unsigned long long* ovf_total) {
+  pdl_wait();
   chunk_emit_body(a, blockIdx.x, gridDim.x, work, ovf_total);
 }
 
 // Batched: grid (blocks of the largest run, runs).
 __global__ void __launch_bounds__(kCLBlock) k_chunk_count_batch(const ChunkListArgs* __restrict__ t) {
+  pdl_wait();
   const ChunkListArgs a = t[blockIdx.y];
   if ((int)blockIdx.x >= chunk_list_blocks_dev(a.NT)) return;
   chunk_count_body(a, blockIdx.x);
 }
 
 __global__ void __launch_bounds__(kCLBlock) k_chunk_emit_batch(const ChunkListArgs* __restrict__ t) {
+  pdl_wait();
   const ChunkListArgs a = t[blockIdx.y];
   const int nblk = chunk_list_blocks_dev(a.NT);
   if ((int)blockIdx.x >= nblk) return;
@@ -1196,6 +1207,7 @@ __global__ void __launch_bounds__(kCLBlock) k_chunk_emit_batch(const ChunkListAr
 __global__ void __launch_bounds__(1024)
 k_run_prefix(const ChunkListArgs* __restrict__ t, int nruns, long long* __restrict__ prefix, unsigned long long* work,
              uint32_t* step, int bump) {
+  pdl_wait();
   __shared__ long long s_part[1024];
   const int per = (nruns + blockDim.x - 1) / blockDim.x;
   const int r0 = threadIdx.x * per;
@@ -1268,11 +1280,13 @@ __device__ __forceinline__ void layout_body(const int* __restrict__ want, int* _
 __global__ void __launch_bounds__(1024)
 k_layout(const int* __restrict__ want, int* __restrict__ cap, long long* __restrict__ base, int NT, int ntx,
          int ovf_cap) {
+  pdl_wait();
   layout_body(want, cap, base, NT, ntx, ovf_cap);
 }
 
 // One block per run.
 __global__ void __launch_bounds__(1024) k_layout_batch(const LayoutArgs* __restrict__ t) {
+  pdl_wait();
   const LayoutArgs& a = t[blockIdx.x];
   layout_body(a.want, a.cap, a.base, a.NT, a.ntx, a.ovf_cap);
 }
@@ -1284,6 +1298,7 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 k_tile_hist(const T* __restrict__ x, const T* __restrict__ y, const T* __restrict__ z, int64_t P, Geo<T> g,
             int shift, int ntx, int NT, int* __restrict__ hist, int use_smem) {
+  pdl_wait();
   extern __shared__ int s_cnt[];
   const int lane = threadIdx.x & 31;
   if (use_smem) {
@@ -1335,6 +1350,7 @@ k_rebin_plain(const T* __restrict__ x, const T* __restrict__ y, const T* __restr
               T* __restrict__ dx, T* __restrict__ dy, T* __restrict__ dz, uint32_t* __restrict__ did,
               const long long* __restrict__ dst_base, const int* __restrict__ dst_cap, int* __restrict__ dst_cursor,
               int* err, int64_t id0, int wrap) {
+  pdl_wait();
   extern __shared__ int s_cnt[];
   for (int t = threadIdx.x; t < NT; t += blockDim.x) s_cnt[t] = 0;
   __syncthreads();
@@ -1382,6 +1398,7 @@ k_rebin_plain(const T* __restrict__ x, const T* __restrict__ y, const T* __restr
 // device can address) is written whole lines at a time.
 template <typename T>
 __global__ void __launch_bounds__(256) k_slot_map(BinArgs<T> a, uint32_t* __restrict__ slot_of) {
+  pdl_wait();
   const long long c = blockIdx.x;
   if (c >= a.chunk_start[a.NT + 1]) return;
   const ChunkDesc d = a.chunks[c];
@@ -1392,6 +1409,7 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 k_gather_slots(const uint32_t* __restrict__ slot_of, const T* __restrict__ bx, const T* __restrict__ by,
                const T* __restrict__ bz, int64_t P, T* __restrict__ ox, T* __restrict__ oy, T* __restrict__ oz) {
+  pdl_wait();
   // four ids per thread and iteration, their gathers issued together
   constexpr int U = 4;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -1425,6 +1443,7 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 k_compact(BinArgs<T> a, unsigned long long* cursor, T* __restrict__ ox, T* __restrict__ oy, T* __restrict__ oz,
           uint32_t* __restrict__ oid) {
+  pdl_wait();
   __shared__ long long s_base;
   const long long c = blockIdx.x;
   if (c >= a.chunk_start[a.NT + 1]) return;
@@ -1457,6 +1476,7 @@ k_compact(BinArgs<T> a, unsigned long long* cursor, T* __restrict__ ox, T* __res
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_unbin(BinArgs<T> a, T* __restrict__ ox, T* __restrict__ oy, T* __restrict__ oz) {
+  pdl_wait();
   const long long c = blockIdx.x;
   if (c >= a.chunk_start[a.NT + 1]) return;
   const ChunkDesc d = a.chunks[c];
@@ -1487,6 +1507,7 @@ template <> struct Vec4Store<double> {
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_unbin_aos(BinArgs<T> a, T* __restrict__ aos) {
+  pdl_wait();
   const long long c = blockIdx.x;
   if (c >= a.chunk_start[a.NT + 1]) return;
   const ChunkDesc d = a.chunks[c];
@@ -1503,6 +1524,7 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 k_partition_pieces(BinArgs<T> a, PieceBounds pb, int* __restrict__ cursor, T* __restrict__ rx, T* __restrict__ ry,
                    T* __restrict__ rz, uint32_t* __restrict__ rid) {
+  pdl_wait();
   __shared__ int cnt[PieceBounds::kMax], base[PieceBounds::kMax];
   const long long c = blockIdx.x;
   if (c >= a.chunk_start[a.NT + 1]) return;
@@ -1541,6 +1563,7 @@ __global__ void __launch_bounds__(256)
 k_scatter_piece(const T* __restrict__ rx, const T* __restrict__ ry, const T* __restrict__ rz,
                 const uint32_t* __restrict__ rid, int64_t a0, int64_t n, int64_t P, T* __restrict__ ox,
                 T* __restrict__ oy, T* __restrict__ oz) {
+  pdl_wait();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t s = a0 + i;
     const uint32_t id = rid[s];
@@ -1555,6 +1578,7 @@ k_scatter_piece(const T* __restrict__ rx, const T* __restrict__ ry, const T* __r
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_aos4_to_soa(const T* __restrict__ aos, int64_t P, T* __restrict__ ox, T* __restrict__ oy, T* __restrict__ oz) {
+  pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += stride) {
     const T* v = aos + (size_t)p * 4;
@@ -1566,6 +1590,7 @@ k_aos4_to_soa(const T* __restrict__ aos, int64_t P, T* __restrict__ ox, T* __res
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_iota(uint32_t* id, int64_t P) {
+  pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += stride) id[p] = (uint32_t)p;
 }
@@ -1577,6 +1602,7 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 k_deposit(const T* __restrict__ x, const T* __restrict__ y, const T* __restrict__ z, int64_t P, Geo<T> g, T w,
           T* __restrict__ phi, int order) {
+  pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += stride) {
     int cx, cy, cz;
@@ -1592,6 +1618,7 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 k_gather(const T* __restrict__ x, const T* __restrict__ y, const T* __restrict__ z, int64_t P, Geo<T> g,
          const T* __restrict__ f, int ncomp, int order, T* __restrict__ out) {
+  pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const size_t N = (size_t)g.H * g.H * g.H;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += stride) {
@@ -1611,6 +1638,7 @@ k_gather(const T* __restrict__ x, const T* __restrict__ y, const T* __restrict__
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_noise(uint64_t seed, uint32_t step, int64_t first, int64_t P, T* z) {
+  pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += stride) {
     T v[6];
@@ -1629,6 +1657,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_moments(const T* __restrict__ x, const T* __restrict__ y, const T* __restrict__ z, int64_t P, double* acc2) {
+  pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   double s2 = 0.0, sr = 0.0;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += stride) {
@@ -1647,6 +1676,7 @@ k_moments(const T* __restrict__ x, const T* __restrict__ y, const T* __restrict_
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_aos_to_soa(const double* __restrict__ aos, int64_t P, Geo<T> g, T* x, T* y, T* z) {
+  pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += stride) {
     x[p] = wrap_coord((T)aos[3 * p + 0], g);
@@ -1657,6 +1687,7 @@ k_aos_to_soa(const double* __restrict__ aos, int64_t P, Geo<T> g, T* x, T* y, T*
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_wrap_soa(int64_t P, Geo<T> g, T* x, T* y, T* z) {
+  pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += stride) {
     x[p] = wrap_coord(x[p], g);
@@ -1669,6 +1700,7 @@ __global__ void __launch_bounds__(256) k_wrap_soa(int64_t P, Geo<T> g, T* x, T* 
 // (mult = 2 for 0 < kz < H/2 accounts for the Hermitian partner).
 template <typename T>
 __global__ void __launch_bounds__(256) k_alpha_energy(const cpx<T>* __restrict__ alpha, int H, double* acc2) {
+  pdl_wait();
   const int nh = H / 2 + 1;
   const int64_t n = (int64_t)H * H * nh;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -1729,7 +1761,7 @@ static cudaError_t launch_deposit_t(const BinArgs<T>& a, cudaStream_t s) {
   int blocks = 0;
   const cudaError_t e = resident_blocks((const void*)kern, 256, smem, &blocks);
   if (e != cudaSuccess) return e;
-  kern<<<min(blocks, a.max_items), 256, smem, s>>>(a, use_win);
+  launch_k(kern, min(blocks, a.max_items), 256, smem, s, a, use_win);
   return cudaGetLastError();
 }
 
@@ -1742,7 +1774,7 @@ template <typename T> cudaError_t launch_binned_rebin(const BinArgs<T>& a, cudaS
   int blocks = 0;
   const cudaError_t e = resident_blocks((const void*)k_binned_rebin<T>, 256, 0, &blocks);
   if (e != cudaSuccess) return e;
-  k_binned_rebin<T><<<min(blocks, a.max_items), 256, 0, s>>>(a);
+  launch_k(k_binned_rebin<T>, min(blocks, a.max_items), 256, 0, s, a);
   return cudaGetLastError();
 }
 
@@ -1751,10 +1783,10 @@ int chunk_list_blocks(int NT) { return (NT + 1 + kCLBlock - 1) / kCLBlock; }
 cudaError_t launch_chunk_list(const ChunkListArgs& a, unsigned long long* work, unsigned long long* ovf_total,
                               cudaStream_t s) {
   const int nblk = chunk_list_blocks(a.NT);
-  k_chunk_count<<<nblk, kCLBlock, 0, s>>>(a);
+  launch_k(k_chunk_count, nblk, kCLBlock, 0, s, a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_chunk_emit<<<nblk, kCLBlock, 0, s>>>(a, work, ovf_total);
+  launch_k(k_chunk_emit, nblk, kCLBlock, 0, s, a, work, ovf_total);
   return cudaGetLastError();
 }
 
@@ -1771,7 +1803,7 @@ cudaError_t launch_move_batch(const BinArgs<T>* table, const long long* prefix, 
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kMoveThreads, 0)) != cudaSuccess) return e;
   if (blocks_per_sm > 0 && blocks_per_sm < per_sm) per_sm = blocks_per_sm;
   if (per_sm < 1) per_sm = 1;
-  k<<<sms * per_sm, kMoveThreads, 0, s>>>(table, prefix, nruns, work, step);
+  launch_k(k, sms * per_sm, kMoveThreads, 0, s, table, prefix, nruns, work, step);
   return cudaGetLastError();
 }
 
@@ -1789,32 +1821,32 @@ cudaError_t launch_deposit_batch(const BinArgs<T>* table, const long long* prefi
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 256, smem)) != cudaSuccess) return e;
   if (blocks_per_sm > 0 && blocks_per_sm < per_sm) per_sm = blocks_per_sm;
   if (per_sm < 1) per_sm = 1;
-  k<<<sms * per_sm, 256, smem, s>>>(table, prefix, nruns, work);
+  launch_k(k, sms * per_sm, 256, smem, s, table, prefix, nruns, work);
   return cudaGetLastError();
 }
 
 cudaError_t launch_chunk_list_batch(const ChunkListArgs* t, int nruns, int max_NT, cudaStream_t s) {
   const dim3 grid(chunk_list_blocks(max_NT), nruns);
-  k_chunk_count_batch<<<grid, kCLBlock, 0, s>>>(t);
+  launch_k(k_chunk_count_batch, grid, kCLBlock, 0, s, t);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_chunk_emit_batch<<<grid, kCLBlock, 0, s>>>(t);
+  launch_k(k_chunk_emit_batch, grid, kCLBlock, 0, s, t);
   return cudaGetLastError();
 }
 
 cudaError_t launch_run_prefix(const ChunkListArgs* t, int nruns, long long* prefix, unsigned long long* work,
                               uint32_t* step, int bump, cudaStream_t s) {
-  k_run_prefix<<<1, 1024, 0, s>>>(t, nruns, prefix, work, step, bump);
+  launch_k(k_run_prefix, 1, 1024, 0, s, t, nruns, prefix, work, step, bump);
   return cudaGetLastError();
 }
 
 cudaError_t launch_layout_batch(const LayoutArgs* t, int nruns, cudaStream_t s) {
-  k_layout_batch<<<nruns, 1024, 0, s>>>(t);
+  launch_k(k_layout_batch, nruns, 1024, 0, s, t);
   return cudaGetLastError();
 }
 
 cudaError_t launch_layout(const int* want, int* cap, long long* base, int NT, int ntx, int ovf_cap, cudaStream_t s) {
-  k_layout<<<1, 1024, 0, s>>>(want, cap, base, NT, ntx, ovf_cap);
+  launch_k(k_layout, 1, 1024, 0, s, want, cap, base, NT, ntx, ovf_cap);
   return cudaGetLastError();
 }
 
@@ -1829,7 +1861,7 @@ cudaError_t launch_tile_hist(const T* x, const T* y, const T* z, int64_t P, Geo<
                              int* hist, cudaStream_t s) {
   const int use_smem = NT <= kMaxSmemTiles ? 1 : 0;
   const int b = use_smem ? plain_blocks(P) : (grid_for(P, 256) > 152 * 16 ? 152 * 16 : grid_for(P, 256));
-  k_tile_hist<T><<<b, 256, use_smem ? NT * sizeof(int) : 0, s>>>(x, y, z, P, g, shift, ntx, NT, hist, use_smem);
+  launch_k(k_tile_hist<T>, b, 256, use_smem ? NT * sizeof(int) : 0, s, x, y, z, P, g, shift, ntx, NT, hist, use_smem);
   return cudaGetLastError();
 }
 
@@ -1839,7 +1871,7 @@ bool launch_rebin_plain(const T* x, const T* y, const T* z, const uint32_t* id, 
                         const int* dst_cap, int* dst_cursor, int* err, cudaStream_t s, cudaError_t* e, int64_t id0,
                         bool wrap) {
   if (NT > kMaxSmemTiles) return false;
-  k_rebin_plain<T><<<plain_blocks(P), 256, NT * sizeof(int), s>>>(x, y, z, id, P, g, shift, ntx, NT, dx, dy, dz, did,
+  launch_k(k_rebin_plain<T>, plain_blocks(P), 256, NT * sizeof(int), s, x, y, z, id, P, g, shift, ntx, NT, dx, dy, dz, did,
                                                                  dst_base, dst_cap, dst_cursor, err, id0,
                                                                  wrap ? 1 : 0);
   *e = cudaGetLastError();
@@ -1850,7 +1882,7 @@ int rebin_plain_max_tiles() { return kMaxSmemTiles; }
 
 template <typename T>
 cudaError_t launch_unbin_aos(const BinArgs<T>& a, int64_t max_chunks, T* aos, cudaStream_t s) {
-  k_unbin_aos<T><<<(unsigned)max_chunks, 256, 0, s>>>(a, aos);
+  launch_k(k_unbin_aos<T>, (unsigned)max_chunks, 256, 0, s, a, aos);
   return cudaGetLastError();
 }
 
@@ -1859,7 +1891,7 @@ cudaError_t launch_partition_pieces(const BinArgs<T>& a, int64_t max_chunks, con
                                     T* ry, T* rz, uint32_t* rid, cudaStream_t s) {
   if (pb.np < 1 || pb.np > PieceBounds::kMax) return cudaErrorInvalidValue;
   if (max_chunks < 1) return cudaSuccess;
-  k_partition_pieces<T><<<(unsigned)max_chunks, 256, 0, s>>>(a, pb, cursor, rx, ry, rz, rid);
+  launch_k(k_partition_pieces<T>, (unsigned)max_chunks, 256, 0, s, a, pb, cursor, rx, ry, rz, rid);
   return cudaGetLastError();
 }
 
@@ -1868,7 +1900,7 @@ cudaError_t launch_compact(const BinArgs<T>& a, int64_t max_chunks, unsigned lon
                            uint32_t* id, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(cursor, 0, sizeof(unsigned long long), s);
   if (e != cudaSuccess || max_chunks < 1) return e;
-  k_compact<T><<<(unsigned)max_chunks, 256, 0, s>>>(a, cursor, x, y, z, id);   // a work item per block
+  launch_k(k_compact<T>, (unsigned)max_chunks, 256, 0, s, a, cursor, x, y, z, id);   // a work item per block
   return cudaGetLastError();
 }
 
@@ -1876,11 +1908,11 @@ template <typename T>
 cudaError_t launch_read_back_mapped(const BinArgs<T>& a, int64_t max_chunks, uint32_t* slot_of, int64_t P, T* x, T* y,
                                    T* z, cudaStream_t s) {
   if (max_chunks < 1 || P < 1) return cudaSuccess;
-  k_slot_map<T><<<(unsigned)max_chunks, 256, 0, s>>>(a, slot_of);
+  launch_k(k_slot_map<T>, (unsigned)max_chunks, 256, 0, s, a, slot_of);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int64_t b = (P + 255) / 256;
-  k_gather_slots<T><<<(unsigned)(b > 152 * 16 ? 152 * 16 : b), 256, 0, s>>>(slot_of, a.sx, a.sy, a.sz, P, x, y, z);
+  launch_k(k_gather_slots<T>, (unsigned)(b > 152 * 16 ? 152 * 16 : b), 256, 0, s, slot_of, a.sx, a.sy, a.sz, P, x, y, z);
   return cudaGetLastError();
 }
 
@@ -1889,13 +1921,13 @@ cudaError_t launch_scatter_piece(const T* rx, const T* ry, const T* rz, const ui
                                  int64_t P, T* x, T* y, T* z, cudaStream_t s) {
   if (n < 1) return cudaSuccess;
   const int64_t b = (n + 255) / 256;
-  k_scatter_piece<T><<<(unsigned)(b > 152 * 8 ? 152 * 8 : b), 256, 0, s>>>(rx, ry, rz, rid, a0, n, P, x, y, z);
+  launch_k(k_scatter_piece<T>, (unsigned)(b > 152 * 8 ? 152 * 8 : b), 256, 0, s, rx, ry, rz, rid, a0, n, P, x, y, z);
   return cudaGetLastError();
 }
 
 template <typename T> cudaError_t launch_aos4_to_soa(const T* aos, int64_t P, T* x, T* y, T* z, cudaStream_t s) {
   const int64_t b = (P + 255) / 256;
-  k_aos4_to_soa<T><<<(unsigned)(b > 152 * 16 ? 152 * 16 : (b < 1 ? 1 : b)), 256, 0, s>>>(aos, P, x, y, z);
+  launch_k(k_aos4_to_soa<T>, (unsigned)(b > 152 * 16 ? 152 * 16 : (b < 1 ? 1 : b)), 256, 0, s, aos, P, x, y, z);
   return cudaGetLastError();
 }
 
@@ -1903,39 +1935,39 @@ template <typename T>
 cudaError_t launch_unbin(const BinArgs<T>& a, int64_t max_chunks, T* x, T* y, T* z, T* aos_scratch, int64_t P,
                          cudaStream_t s) {
   if (!aos_scratch) {
-    k_unbin<T><<<(unsigned)max_chunks, 256, 0, s>>>(a, x, y, z);
+    launch_k(k_unbin<T>, (unsigned)max_chunks, 256, 0, s, a, x, y, z);
     return cudaGetLastError();
   }
-  k_unbin_aos<T><<<(unsigned)max_chunks, 256, 0, s>>>(a, aos_scratch);
+  launch_k(k_unbin_aos<T>, (unsigned)max_chunks, 256, 0, s, a, aos_scratch);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int64_t b = (P + 255) / 256;
-  k_aos4_to_soa<T><<<(unsigned)(b > 152 * 16 ? 152 * 16 : (b < 1 ? 1 : b)), 256, 0, s>>>(aos_scratch, P, x, y, z);
+  launch_k(k_aos4_to_soa<T>, (unsigned)(b > 152 * 16 ? 152 * 16 : (b < 1 ? 1 : b)), 256, 0, s, aos_scratch, P, x, y, z);
   return cudaGetLastError();
 }
 
 cudaError_t launch_iota(uint32_t* id, int64_t P, cudaStream_t s) {
-  k_iota<int><<<grid_for(P, 256), 256, 0, s>>>(id, P);
+  launch_k(k_iota<int>, grid_for(P, 256), 256, 0, s, id, P);
   return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_deposit(const T* x, const T* y, const T* z, int64_t P, Geo<T> g, T w, T* phi, int order,
                            cudaStream_t s) {
-  k_deposit<T><<<grid_for(P, 256), 256, 0, s>>>(x, y, z, P, g, w, phi, order);
+  launch_k(k_deposit<T>, grid_for(P, 256), 256, 0, s, x, y, z, P, g, w, phi, order);
   return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_gather(const T* x, const T* y, const T* z, int64_t P, Geo<T> g, const T* f, int ncomp, int order,
                           T* out, cudaStream_t s) {
-  k_gather<T><<<grid_for(P, 256), 256, 0, s>>>(x, y, z, P, g, f, ncomp, order, out);
+  launch_k(k_gather<T>, grid_for(P, 256), 256, 0, s, x, y, z, P, g, f, ncomp, order, out);
   return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_noise(uint64_t seed, int64_t step, int64_t first, int64_t P, T* z, cudaStream_t s) {
-  k_noise<T><<<grid_for(P, 256), 256, 0, s>>>(seed, (uint32_t)step, first, P, z);
+  launch_k(k_noise<T>, grid_for(P, 256), 256, 0, s, seed, (uint32_t)step, first, P, z);
   return cudaGetLastError();
 }
 
@@ -1943,18 +1975,18 @@ template <typename T>
 cudaError_t launch_moments(const T* x, const T* y, const T* z, int64_t P, double* acc2, cudaStream_t s) {
   int b = grid_for(P, 256);
   if (b > 152 * 8) b = 152 * 8;
-  k_moments<T><<<b, 256, 0, s>>>(x, y, z, P, acc2);
+  launch_k(k_moments<T>, b, 256, 0, s, x, y, z, P, acc2);
   return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_aos_to_soa(const double* aos, int64_t P, Geo<T> g, T* x, T* y, T* z, cudaStream_t s) {
-  k_aos_to_soa<T><<<grid_for(P, 256), 256, 0, s>>>(aos, P, g, x, y, z);
+  launch_k(k_aos_to_soa<T>, grid_for(P, 256), 256, 0, s, aos, P, g, x, y, z);
   return cudaGetLastError();
 }
 
 template <typename T> cudaError_t launch_wrap_soa(int64_t P, Geo<T> g, T* x, T* y, T* z, cudaStream_t s) {
-  k_wrap_soa<T><<<grid_for(P, 256), 256, 0, s>>>(P, g, x, y, z);
+  launch_k(k_wrap_soa<T>, grid_for(P, 256), 256, 0, s, P, g, x, y, z);
   return cudaGetLastError();
 }
 
@@ -1962,7 +1994,7 @@ template <typename T> cudaError_t launch_alpha_energy(const cpx<T>* alpha, int H
   const int64_t n = (int64_t)H * H * (H / 2 + 1);
   int b = grid_for(n, 256);
   if (b > 152 * 8) b = 152 * 8;
-  k_alpha_energy<T><<<b, 256, 0, s>>>(alpha, H, acc2);
+  launch_k(k_alpha_energy<T>, b, 256, 0, s, alpha, H, acc2);
   return cudaGetLastError();
 }
 

@@ -77,6 +77,7 @@ template <typename T>
 __global__ void __launch_bounds__(kT2)
 k2_deposit(const T* __restrict__ x, const T* __restrict__ y, int64_t P, Geo<T> g, T w, int order,
            T* __restrict__ phi) {
+  pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += stride) {
     int cx, cy;
@@ -101,6 +102,7 @@ template <typename T>
 __global__ void __launch_bounds__(kT2)
 k2_spectral(const cpx<T>* __restrict__ T1, cpx<T>* __restrict__ alpha, cpx<T>* __restrict__ T2, int H,
             Spec2D<T> sp) {
+  pdl_wait();
   const int NH = H / 2 + 1;
   const int S = H * NH;
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
@@ -138,6 +140,7 @@ template <typename T>
 __global__ void __launch_bounds__(kT2)
 k2_move(T* __restrict__ x, T* __restrict__ y, int64_t P, Geo<T> g, const T* __restrict__ grad4, int g2p, int split,
         T s_noise, T chitau, uint64_t seed, uint32_t n, int* err) {
+  pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += stride) {
     T z[4];
@@ -179,6 +182,7 @@ template <typename T>
 __global__ void __launch_bounds__(kT2)
 k2_sums(const T* __restrict__ x, const T* __restrict__ y, int64_t P, const T* __restrict__ phi, int64_t N,
         double* acc) {
+  pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   double m2 = 0.0, mass = 0.0;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += stride)
@@ -196,6 +200,7 @@ k2_sums(const T* __restrict__ x, const T* __restrict__ y, int64_t P, const T* __
 // the columns ky = 0 and ky = H/2 once, the others twice)
 template <typename T>
 __global__ void __launch_bounds__(kT2) k2_energy(const cpx<T>* __restrict__ alpha, int H, double* acc) {
+  pdl_wait();
   const int NH = H / 2 + 1, S = H * NH;
   double hi = 0.0, tot = 0.0;
   for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < S; m += gridDim.x * blockDim.x) {
@@ -217,6 +222,7 @@ __global__ void __launch_bounds__(kT2) k2_energy(const cpx<T>* __restrict__ alph
 template <typename T>
 __global__ void __launch_bounds__(kT2)
 k2_load_aos(const double* __restrict__ X, int64_t P, Geo<T> g, T* __restrict__ x, T* __restrict__ y) {
+  pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += stride) {
     x[p] = wrap_coord((T)X[2 * p], g);
@@ -227,6 +233,7 @@ k2_load_aos(const double* __restrict__ X, int64_t P, Geo<T> g, T* __restrict__ x
 template <typename T>
 __global__ void __launch_bounds__(kT2)
 k2_store_aos(const T* __restrict__ x, const T* __restrict__ y, int64_t P, double* __restrict__ X) {
+  pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += stride) {
     X[2 * p] = (double)x[p];
@@ -305,7 +312,7 @@ template <typename T> Geo<T> geo2(const sipf2d_ctx* c) { return make_geo<T>(c->p
 
 template <typename T> int deposit2(sipf2d_ctx* c) {
   const T w = (T)(c->p.mass / (double)c->p.P);
-  k2_deposit<T><<<grid_for2(c->p.P, kT2), kT2, 0, c->stream>>>((const T*)c->x, (const T*)c->y, c->p.P, geo2<T>(c), w,
+  launch_k(k2_deposit<T>, grid_for2(c->p.P, kT2), kT2, 0, c->stream, (const T*)c->x, (const T*)c->y, c->p.P, geo2<T>(c), w,
                                                                 c->p.p2g_order, (T*)c->phi);
   SIPF2_CK(cudaGetLastError());
   return SIPF_OK;
@@ -341,13 +348,11 @@ template <typename T> int step2(sipf2d_ctx* c, int64_t nsteps) {
   for (int64_t i = 0; i < nsteps; ++i) {
     int r = forward2<T>(c, true, nullptr);
     if (r) return r;
-    k2_spectral<T><<<(unsigned)((S + kT2 - 1) / kT2), kT2, 0, c->stream>>>(
-        (const cpx<T>*)c->T1, (cpx<T>*)c->alpha, (cpx<T>*)c->T2, H, spec2<T>(c, 0));
+    launch_k(k2_spectral<T>, (unsigned)((S + kT2 - 1) / kT2), kT2, 0, c->stream, (const cpx<T>*)c->T1, (cpx<T>*)c->alpha, (cpx<T>*)c->T2, H, spec2<T>(c, 0));
     SIPF2_CK(cudaGetLastError());
     SIPF2_CK(launch_cols<T>((cpx<T>*)c->T2, H, 1, H / 2 + 1, 2, S, +1, 1.0, c->stream));
     SIPF2_CK(launch_rows_c2r<T>((const cpx<T>*)c->T2, 3, S, (T*)c->grad, H, H, nullptr, c->stream));
-    k2_move<T><<<grid_for2(c->p.P, kT2), kT2, 0, c->stream>>>(
-        (T*)c->x, (T*)c->y, c->p.P, geo2<T>(c), (const T*)c->grad, c->p.g2p_order, c->p.splitting, s_noise,
+    launch_k(k2_move<T>, grid_for2(c->p.P, kT2), kT2, 0, c->stream, (T*)c->x, (T*)c->y, c->p.P, geo2<T>(c), (const T*)c->grad, c->p.g2p_order, c->p.splitting, s_noise,
         (T)(c->p.chi * c->p.dt), c->p.seed, (uint32_t)(c->n + 1), c->err);
     SIPF2_CK(cudaGetLastError());
     c->n += 1;
@@ -360,14 +365,14 @@ template <typename T> int step2(sipf2d_ctx* c, int64_t nsteps) {
 template <typename T> int init_positions2(sipf2d_ctx* c, const double* X0) {
   const size_t bytes = (size_t)c->p.P * 2 * sizeof(double);
   SIPF2_CK(cudaMemcpyAsync(c->aos, X0, bytes, cudaMemcpyHostToDevice, c->stream));
-  k2_load_aos<T><<<grid_for2(c->p.P, kT2), kT2, 0, c->stream>>>(c->aos, c->p.P, geo2<T>(c), (T*)c->x, (T*)c->y);
+  launch_k(k2_load_aos<T>, grid_for2(c->p.P, kT2), kT2, 0, c->stream, c->aos, c->p.P, geo2<T>(c), (T*)c->x, (T*)c->y);
   SIPF2_CK(cudaGetLastError());
   SIPF2_CK(cudaMemsetAsync(c->phi, 0, (size_t)c->N() * c->esz, c->stream));
   return deposit2<T>(c);
 }
 
 template <typename T> int positions2(sipf2d_ctx* c, double* out) {
-  k2_store_aos<T><<<grid_for2(c->p.P, kT2), kT2, 0, c->stream>>>((const T*)c->x, (const T*)c->y, c->p.P, c->aos);
+  launch_k(k2_store_aos<T>, grid_for2(c->p.P, kT2), kT2, 0, c->stream, (const T*)c->x, (const T*)c->y, c->p.P, c->aos);
   SIPF2_CK(cudaGetLastError());
   SIPF2_CK(cudaMemcpyAsync(out, c->aos, (size_t)c->p.P * 2 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   SIPF2_CK(cudaStreamSynchronize(c->stream));
@@ -388,8 +393,7 @@ template <typename T> int density_num2(sipf2d_ctx* c, int filtered) {
   const size_t S = (size_t)c->S();
   int r = forward2<T>(c, false, nullptr);
   if (r) return r;
-  k2_spectral<T><<<(unsigned)((S + kT2 - 1) / kT2), kT2, 0, c->stream>>>(
-      (const cpx<T>*)c->T1, (cpx<T>*)c->alpha, (cpx<T>*)c->T2, H, spec2<T>(c, 1, filtered != 0));
+  launch_k(k2_spectral<T>, (unsigned)((S + kT2 - 1) / kT2), kT2, 0, c->stream, (const cpx<T>*)c->T1, (cpx<T>*)c->alpha, (cpx<T>*)c->T2, H, spec2<T>(c, 1, filtered != 0));
   SIPF2_CK(cudaGetLastError());
   SIPF2_CK(launch_cols<T>((cpx<T>*)c->T2, H, 1, H / 2 + 1, 1, 0, +1, 1.0, c->stream));
   // (only the first spectrum is used; the third, read as zeros by the step's
@@ -409,10 +413,9 @@ template <typename T> int diag2(sipf2d_ctx* c, sipf_diag* d) {
     memcpy(&init[4], &b, 8);
   }
   SIPF2_CK(cudaMemcpyAsync(c->acc, init, sizeof(init), cudaMemcpyHostToDevice, c->stream));
-  k2_sums<T><<<grid_for2(c->p.P > c->N() ? c->p.P : c->N(), kT2, 152 * 8), kT2, 0, c->stream>>>(
-      (const T*)c->x, (const T*)c->y, c->p.P, (const T*)c->phi, c->N(), c->acc);
+  launch_k(k2_sums<T>, grid_for2(c->p.P > c->N() ? c->p.P : c->N(), kT2, 152 * 8), kT2, 0, c->stream, (const T*)c->x, (const T*)c->y, c->p.P, (const T*)c->phi, c->N(), c->acc);
   SIPF2_CK(cudaGetLastError());
-  k2_energy<T><<<grid_for2(c->S(), kT2, 152 * 8), kT2, 0, c->stream>>>((const cpx<T>*)c->alpha, c->p.H, c->acc);
+  launch_k(k2_energy<T>, grid_for2(c->S(), kT2, 152 * 8), kT2, 0, c->stream, (const cpx<T>*)c->alpha, c->p.H, c->acc);
   SIPF2_CK(cudaGetLastError());
   int r = density_num2<T>(c, c->H0 > 0 ? 1 : 0);
   if (r) return r;

@@ -9,6 +9,16 @@ namespace sipf {
 
 template <typename T> struct cpx { T x, y; };
 
+// Programmatic dependent launch (see launch_k): in a grid of at most
+// kPdlBlocks blocks, waits until the kernel before this one has completed and
+// its writes are visible.  (Larger grids are launched the ordinary way.)
+// Every block of such a kernel executes it first of all, so a kernel's
+// completion implies that of all kernels before it.
+constexpr unsigned kPdlBlocks = 152 * 8;
+__device__ __forceinline__ void pdl_wait() {
+  if (gridDim.x * gridDim.y * gridDim.z <= kPdlBlocks) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 __device__ __forceinline__ int ilog2_dev(int v) { return 31 - __clz(v); }   // v a power of two
 __device__ __forceinline__ float t_floor(float v) { return floorf(v); }
 __device__ __forceinline__ double t_floor(double v) { return ::floor(v); }

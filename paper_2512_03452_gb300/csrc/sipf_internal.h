@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include <string>
+#include <utility>
 
 #include "sipf_device.cuh"
 
@@ -52,6 +53,43 @@ template <typename T> inline SpecConst<T> spec_const(const SpecParams& sp) {
   c.sh_div = sp.propagator == 0 ? fma(sp.tau / sp.eps, sp.k2, 1.0) : -sp.tau / sp.eps * sp.k2;
   c.sh_add = sp.propagator == 0 ? sp.beta0 / (sp.k2 + sp.eps / sp.tau) : sp.tau * sp.beta0;
   return c;
+}
+
+// Kernel launches.  launch_k: grids of at most kPdlBlocks blocks use programmatic
+// stream serialisation: the kernel is set up and its blocks become resident
+// while the kernel before it drains, and its first statement (pdl_wait,
+// sipf_device.cuh) waits for that kernel.  A small run's step is some ten
+// dependent launches of 2 to 8 us whose gaps were about 1.8 us each: 938 -> 622
+// us for 20 steps of P = 16384, H = 32.  An explicit trigger at the start of
+// the kernels, so that the next kernel's blocks come in as soon as there is
+// room, measured slower (643 us; FP64 P = 1e6 2.52 -> 2.77 ms): the early blocks
+// pile up on the SMs that drain first.
+// launch_plain: kernels only used for grids of many waves.  They do not contain
+// the wait: the instruction alone, executed or not, made such kernels slower
+// (y pass at H = 256, 6912 blocks: 125 -> 201 us; x pass 170 -> 198).
+template <typename... KA, typename... A>
+inline cudaError_t launch_plain(void (*kernel)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+template <typename... KA, typename... A>
+inline cudaError_t launch_k(void (*kernel)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = grid.x * grid.y * grid.z <= kPdlBlocks ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 
 enum SpecMode { kModeStep = 0, kModeDensity = 1, kModeField = 2, kModeGradOnly = 3 };
