@@ -30,7 +30,8 @@ namespace {
 
 constexpr int kT2 = 256;
 
-inline int grid_for2(int64_t n, int threads, int cap = 152 * 16) {
+// (at most eight blocks of 256 per SM: one resident wave)
+inline int grid_for2(int64_t n, int threads, int cap = 152 * 8) {
   int64_t b = (n + threads - 1) / threads;
   if (b > cap) b = cap;
   if (b < 1) b = 1;
@@ -85,6 +86,53 @@ k2_deposit(const T* __restrict__ x, const T* __restrict__ y, int64_t P, Geo<T> g
     cell_lambda(x[p], g, cx, lx);
     cell_lambda(y[p], g, cy, ly);
     stencil2d<T>(order, cx, cy, lx, ly, w, g.H, g.mask, [&](int idx, T f) { atomicAdd(phi + idx, f); });
+  }
+}
+
+// Deposit through a window of the grid in shared memory.  The window holds the
+// `rows` grid rows (all of them for H <= 128, 226 of 256 in single precision)
+// around row 0, where the studies' data is centred; a block adds its share of
+// the particles there with shared atomics and the window's non-zero nodes to
+// the grid once, rows outside with global reductions.  With one global
+// reduction per node and particle the dense disk's some 2000 cells serialised
+// in L2: 218 -> 28 us for P = 2^20, H = 256 (what is left is the shared
+// atomics: no native float add).  The sums stay in T (a block's
+// partial sums, then the blocks').
+constexpr int kT2Win = 1024;                      // threads of a block (one block per SM)
+constexpr size_t kWin2Bytes = 226 * 1024;
+template <typename T> int win2_rows(int H) {
+  const int r = (int)(kWin2Bytes / ((size_t)H * sizeof(T)));
+  return r < H ? r : H;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kT2Win, 1)
+k2_deposit_win(const T* __restrict__ x, const T* __restrict__ y, int64_t P, Geo<T> g, T w, int order, int rows,
+               T* __restrict__ phi) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* win = reinterpret_cast<T*>(smem_raw);
+  const int H = g.H, mask = g.mask, n = rows * H;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) win[i] = T(0);
+  pdl_wait();
+  __syncthreads();
+  const int lo = rows / 2;   // window row r holds grid row (r - lo) mod H
+  const int64_t per = (P + gridDim.x - 1) / gridDim.x;
+  const int64_t p0 = (int64_t)blockIdx.x * per, p1 = p0 + per < P ? p0 + per : P;
+  for (int64_t p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
+    int cx, cy;
+    T lx, ly;
+    cell_lambda(x[p], g, cx, lx);
+    cell_lambda(y[p], g, cy, ly);
+    stencil2d<T>(order, cx, cy, lx, ly, w, H, mask, [&](int idx, T f) {
+      const int s = (idx + lo * H) & (H * H - 1);   // row (idx / H + lo) mod H, same column
+      if (s < n) atomicAdd(win + s, f);
+      else atomicAdd(phi + idx, f);
+    });
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    const T v = win[i];
+    if (v != T(0)) atomicAdd(phi + ((i - lo * H) & (H * H - 1)), v);
   }
 }
 
@@ -312,6 +360,16 @@ template <typename T> Geo<T> geo2(const sipf2d_ctx* c) { return make_geo<T>(c->p
 
 template <typename T> int deposit2(sipf2d_ctx* c) {
   const T w = (T)(c->p.mass / (double)c->p.P);
+  // a window per block pays from some thousand particles on (its clearing and
+  // flush, about 2 us)
+  if (c->p.P >= 8 * kT2Win) {
+    const int rows = win2_rows<T>(c->p.H);
+    const size_t smem = (size_t)rows * c->p.H * sizeof(T);
+    SIPF2_CK(cudaFuncSetAttribute(k2_deposit_win<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    SIPF2_CK(launch_k(k2_deposit_win<T>, grid_for2(c->p.P, kT2Win, 152), kT2Win, smem, c->stream, (const T*)c->x,
+                      (const T*)c->y, c->p.P, geo2<T>(c), w, c->p.p2g_order, rows, (T*)c->phi));
+    return SIPF_OK;
+  }
   launch_k(k2_deposit<T>, grid_for2(c->p.P, kT2), kT2, 0, c->stream, (const T*)c->x, (const T*)c->y, c->p.P, geo2<T>(c), w,
                                                                 c->p.p2g_order, (T*)c->phi);
   SIPF2_CK(cudaGetLastError());
@@ -413,9 +471,9 @@ template <typename T> int diag2(sipf2d_ctx* c, sipf_diag* d) {
     memcpy(&init[4], &b, 8);
   }
   SIPF2_CK(cudaMemcpyAsync(c->acc, init, sizeof(init), cudaMemcpyHostToDevice, c->stream));
-  launch_k(k2_sums<T>, grid_for2(c->p.P > c->N() ? c->p.P : c->N(), kT2, 152 * 8), kT2, 0, c->stream, (const T*)c->x, (const T*)c->y, c->p.P, (const T*)c->phi, c->N(), c->acc);
+  launch_k(k2_sums<T>, grid_for2(c->p.P > c->N() ? c->p.P : c->N(), kT2), kT2, 0, c->stream, (const T*)c->x, (const T*)c->y, c->p.P, (const T*)c->phi, c->N(), c->acc);
   SIPF2_CK(cudaGetLastError());
-  launch_k(k2_energy<T>, grid_for2(c->S(), kT2, 152 * 8), kT2, 0, c->stream, (const cpx<T>*)c->alpha, c->p.H, c->acc);
+  launch_k(k2_energy<T>, grid_for2(c->S(), kT2), kT2, 0, c->stream, (const cpx<T>*)c->alpha, c->p.H, c->acc);
   SIPF2_CK(cudaGetLastError());
   int r = density_num2<T>(c, c->H0 > 0 ? 1 : 0);
   if (r) return r;
