@@ -2056,9 +2056,15 @@ static cudaError_t set_smem(K kernel, size_t bytes) {
   return cudaSuccess;
 }
 
-static int rows_per_pair_block(int H, size_t elem, bool with_out4) {
+// Shapes of the H < 32 kernels: blocks as small as it takes to give every SM
+// one (a 16^3 grid has 256 rows and 144 x pencils; with 8 row pairs or 16
+// pencils a block its FP64 transforms ran on 9 to 16 SMs: a step of P = 1e4
+// 64.5 -> 60.2 us).
+constexpr int kSmallThreads = 64;   // threads of a block that holds a single row pair or pencil pair
+static int rows_per_pair_block(int H, int rows, size_t elem, bool with_out4) {
   // row pairs per block: up to 8, bounded so the shared buffers stay <= ~96 KB
   int rp = 8;
+  while (rp > 1 && rows / (2 * rp) < 152) rp >>= 1;
   auto bytes = [&](int r) {
     size_t b = (size_t)r * (H + 1) * 2 * elem;
     if (with_out4) b += (size_t)2 * r * H * 4 * elem;
@@ -2076,18 +2082,18 @@ cudaError_t launch_rows_r2c(const void* in, int in_kind, double in_scale, bool z
   if (H == 128) return warp_rows_r2c<T, 4>(in, in_kind, in_scale, zero_input, out, rows, mass_acc, s);
   if (H == 256) return warp_rows_r2c<T, 8>(in, in_kind, in_scale, zero_input, out, rows, mass_acc, s);
   const int lgH = ilog2(H);
-  const int RP = rows_per_pair_block(H, sizeof(T), false);
+  const int RP = rows_per_pair_block(H, rows, sizeof(T), false);
   const size_t smem = (kNmax / 2 + (size_t)RP * (H + 1)) * sizeof(cpx<T>);
   const int blocks = (rows + 2 * RP - 1) / (2 * RP);
   cudaError_t e;
   if (in_kind == 0) {
     auto k = k_rows_r2c<T, T>;
     if ((e = set_smem(k, smem)) != cudaSuccess) return e;
-    launch_k(k, blocks, kThreads, smem, s, (T*)in, in_scale, zero_input ? 1 : 0, out, lgH, rows, RP, mass_acc);
+    launch_k(k, blocks, RP > 2 ? kThreads : kSmallThreads, smem, s, (T*)in, in_scale, zero_input ? 1 : 0, out, lgH, rows, RP, mass_acc);
   } else {
     auto k = k_rows_r2c<T, unsigned long long>;
     if ((e = set_smem(k, smem)) != cudaSuccess) return e;
-    launch_k(k, blocks, kThreads, smem, s, (unsigned long long*)in, in_scale, zero_input ? 1 : 0, out, lgH, rows,
+    launch_k(k, blocks, RP > 2 ? kThreads : kSmallThreads, smem, s, (unsigned long long*)in, in_scale, zero_input ? 1 : 0, out, lgH, rows,
                                      RP, mass_acc);
   }
   return cudaGetLastError();
@@ -2115,18 +2121,19 @@ cudaError_t launch_cols(cpx<T>* data, int H, int A, int B, int ncomp, size_t com
   const int lgH = ilog2(H);
   int BC = col_chunk<T>(H, 1);
   if (BC > 16) BC = 16;
-  const int lgBC = ilog2(BC);
+  while (BC > 1 && (B + BC - 1) / BC * A * ncomp < 152) BC >>= 1;
+  const int lgBC = ilog2(BC), nt = BC > 2 ? kThreads : kSmallThreads;
   const size_t smem = (kNmax / 2 + (size_t)H * BC) * sizeof(cpx<T>);
   dim3 grid((B + BC - 1) / BC, A, ncomp);
   cudaError_t e;
   if (dir < 0) {
     auto k = k_cols<T, -1>;
     if ((e = set_smem(k, smem)) != cudaSuccess) return e;
-    launch_k(k, grid, kThreads, smem, s, data, lgH, B, lgBC, comp_stride, (T)scale);
+    launch_k(k, grid, nt, smem, s, data, lgH, B, lgBC, comp_stride, (T)scale);
   } else {
     auto k = k_cols<T, +1>;
     if ((e = set_smem(k, smem)) != cudaSuccess) return e;
-    launch_k(k, grid, kThreads, smem, s, data, lgH, B, lgBC, comp_stride, (T)scale);
+    launch_k(k, grid, nt, smem, s, data, lgH, B, lgBC, comp_stride, (T)scale);
   }
   return cudaGetLastError();
 }
@@ -2135,15 +2142,16 @@ template <typename T, int MODE>
 static cudaError_t spectral_mode(const cpx<T>* T1, cpx<T>* alpha, cpx<T>* T2, int H, SpecParams sp,
                                  double* shadow, cudaStream_t s) {
   const int lgH = ilog2(H);
+  const int B = H * (H / 2 + 1);
   int BC = col_chunk<T>(H, 4);
   if (BC > 16) BC = 16;
-  const int lgBC = ilog2(BC);
-  const int B = H * (H / 2 + 1);
+  while (BC > 1 && (B + BC - 1) / BC < 152) BC >>= 1;
+  const int lgBC = ilog2(BC), nt = BC > 2 ? kThreads : kSmallThreads;
   const size_t smem = (kNmax / 2 + (size_t)H * 4 * BC) * sizeof(cpx<T>);
   auto k = k_spectral_x<T, MODE>;
   cudaError_t e = set_smem(k, smem);
   if (e != cudaSuccess) return e;
-  launch_k(k, (B + BC - 1) / BC, kThreads, smem, s, T1, alpha, T2, lgH, lgBC, spec_const<T>(sp), shadow);
+  launch_k(k, (B + BC - 1) / BC, nt, smem, s, T1, alpha, T2, lgH, lgBC, spec_const<T>(sp), shadow);
   return cudaGetLastError();
 }
 
@@ -2187,7 +2195,7 @@ cudaError_t launch_rows_c2r(const cpx<T>* in, int ncomp, size_t comp_stride, T* 
   if (H == 256) return ncomp == 3 ? warp_rows_c2r<T, 8, 3>(in, comp_stride, out, rows, nullptr, s)
                                   : warp_rows_c2r<T, 8, 1>(in, comp_stride, out, rows, max_acc, s);
   const int lgH = ilog2(H);
-  const int RP = rows_per_pair_block(H, sizeof(T), true);
+  const int RP = rows_per_pair_block(H, rows, sizeof(T), true);
   const int NOUT = ncomp == 3 ? 4 : 1;
   const size_t smem = (kNmax / 2 + (size_t)RP * (H + 1)) * sizeof(cpx<T>) + (size_t)2 * RP * H * NOUT * sizeof(T);
   const int blocks = (rows + 2 * RP - 1) / (2 * RP);
@@ -2195,11 +2203,11 @@ cudaError_t launch_rows_c2r(const cpx<T>* in, int ncomp, size_t comp_stride, T* 
   if (ncomp == 3) {
     auto k = k_rows_c2r<T, 3>;
     if ((e = set_smem(k, smem)) != cudaSuccess) return e;
-    launch_k(k, blocks, kThreads, smem, s, in, comp_stride, out, lgH, rows, RP, nullptr);
+    launch_k(k, blocks, RP > 2 ? kThreads : kSmallThreads, smem, s, in, comp_stride, out, lgH, rows, RP, nullptr);
   } else {
     auto k = k_rows_c2r<T, 1>;
     if ((e = set_smem(k, smem)) != cudaSuccess) return e;
-    launch_k(k, blocks, kThreads, smem, s, in, comp_stride, out, lgH, rows, RP, max_acc);
+    launch_k(k, blocks, RP > 2 ? kThreads : kSmallThreads, smem, s, in, comp_stride, out, lgH, rows, RP, max_acc);
   }
   return cudaGetLastError();
 }
