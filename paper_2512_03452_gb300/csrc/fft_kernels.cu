@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(kThreads)
 k_rows_r2c(Tin* __restrict__ in, double in_scale, int zero_input, cpx<T>* __restrict__ out,
            int lgH, int rows, int RP, double* mass_acc) {
   pdl_wait();
-  extern __shared__ unsigned char smem_raw[];
+  extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
   cpx<T>* buf = tw + kNmax / 2;
   const int H = 1 << lgH, nh = H / 2 + 1, ld = H + 1;
@@ -168,7 +168,7 @@ template <typename T, int DIR>
 __global__ void __launch_bounds__(kThreads)
 k_cols(cpx<T>* __restrict__ data, int lgH, int B, int lgBC, size_t comp_stride, T scale) {
   pdl_wait();
-  extern __shared__ unsigned char smem_raw[];
+  extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
   cpx<T>* buf = tw + kNmax / 2;
   const int H = 1 << lgH, BC = 1 << lgBC;
@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(kThreads)
 k_spectral_x(const cpx<T>* __restrict__ T1, cpx<T>* __restrict__ alpha, cpx<T>* __restrict__ T2,
              int lgH, int lgBC, SpecConst<T> sk, double* alpha0_shadow) {
   pdl_wait();
-  extern __shared__ unsigned char smem_raw[];
+  extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
   cpx<T>* buf = tw + kNmax / 2;
   const int H = 1 << lgH, BC = 1 << lgBC, nh = H / 2 + 1;
@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(kThreads)
 k_rows_c2r(const cpx<T>* __restrict__ in, size_t comp_stride, T* __restrict__ out, int lgH, int rows,
            int RP, double* max_acc) {
   pdl_wait();
-  extern __shared__ unsigned char smem_raw[];
+  extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
   cpx<T>* buf = tw + kNmax / 2;
   const int H = 1 << lgH, nh = H / 2 + 1, ld = H + 1;
@@ -946,16 +946,24 @@ kw_cols(cpx<T>* __restrict__ data, int B, size_t comp_stride, T scale) {
   cols_body<T, E, DIR, BC>(base, B, scale, blockIdx.x * BC, tw, tw + tw_len<T, E>());
 }
 
+// H = 256: the x pass hands on two spectra (see spectral_body's TWO).
+template <int E> constexpr bool two_spectra() { return E == 8; }
+
 // x-axis pass fused with the spectral work (as k_spectral_x), warp FFTs.
 // Shared tile: [N][3 BC + 1]; slot 0 = beta, then the first output (each
 // element's beta is read before its outputs are written), slots 1, 2 the other
 // two outputs: 3 slots per pencil, so a 128^3 x pass fits one wave of blocks.
-template <typename T, int E, int MODE, int BC>
+// TWO (the step at H = 256): q_y and q_z are constant along an x pencil, so only
+// G_x and Phi alpha are transformed back and stored (T2 components 0 and 2);
+// the y pass forms G_y and G_z from the latter (kwb_cols_inv3): 3 instead of 4
+// transforms a pencil, and a third less to write here and to read there (x pass
+// 170 -> 123 us, inverse y pass 125 -> 112).
+template <typename T, int E, int MODE, int BC, bool TWO = false>
 __device__ __forceinline__ void spectral_body(const cpx<T>* __restrict__ T1, cpx<T>* __restrict__ alpha,
                                               cpx<T>* __restrict__ T2, const SpecConst<T>& sk,
                                               double* alpha0_shadow,
                                               int b0, const cpx<T>* tw, const cpx<T>* twq, cpx<T>* buf) {
-  constexpr int N = 32 * E, NHH = N / 2 + 1, LD = 3 * BC + 1;
+  constexpr int N = 32 * E, NHH = N / 2 + 1, LD = (TWO ? 2 : 3) * BC + 1;
   const int B = N * NHH;
   const size_t S = (size_t)N * B;
   const int nb = min(BC, B - b0);
@@ -1007,8 +1015,12 @@ __device__ __forceinline__ void spectral_body(const cpx<T>* __restrict__ T1, cpx
         }
         const T yx = two_pi_L * (T)qx * Phi, yy = two_pi_L * (T)qy * Phi, yz = two_pi_L * (T)qz * Phi;
         if (qx != -N / 2) o1 = cpx<T>{-yx * a.y, yx * a.x};
-        if (qy != -N / 2) o2 = cpx<T>{-yy * a.y, yy * a.x};
-        if (qz != -N / 2) o3 = cpx<T>{-yz * a.y, yz * a.x};
+        if (TWO) {
+          o2 = cpx<T>{Phi * a.x, Phi * a.y};
+        } else {
+          if (qy != -N / 2) o2 = cpx<T>{-yy * a.y, yy * a.x};
+          if (qz != -N / 2) o3 = cpx<T>{-yz * a.y, yz * a.x};
+        }
       } else if (MODE == kModeDensity) {
         const cpx<T> beta = buf[tpad(j, LD, c)];
         o1 = cpx<T>{beta.x * inv_L3 * Phi, beta.y * inv_L3 * Phi};
@@ -1018,10 +1030,10 @@ __device__ __forceinline__ void spectral_body(const cpx<T>* __restrict__ T1, cpx
     }
     buf[tpad(j, LD, c)] = o1;
     buf[tpad(j, LD, BC + c)] = o2;
-    buf[tpad(j, LD, 2 * BC + c)] = o3;
+    if (!TWO) buf[tpad(j, LD, 2 * BC + c)] = o3;
   }
   __syncthreads();
-  constexpr int nout = (MODE == kModeStep || MODE == kModeGradOnly) ? 3 : 1;
+  constexpr int nout = TWO ? 2 : (MODE == kModeStep || MODE == kModeGradOnly) ? 3 : 1;
   tile_ffts<T, N, +1>(nout * BC, tw, twq, [&](int p, int j) { return buf + tpad(j, LD, p); },
                       [&](int p) { return p % BC < nb; });
   __syncthreads();
@@ -1029,7 +1041,7 @@ __device__ __forceinline__ void spectral_body(const cpx<T>* __restrict__ T1, cpx
     const int j = t / BC, c = t - j * BC;
     if (c < nb) {
 #pragma unroll
-      for (int d = 0; d < nout; ++d) T2[d * S + (size_t)j * B + b0 + c] = buf[tpad(j, LD, d * BC + c)];
+      for (int d = 0; d < nout; ++d) T2[(TWO ? 2 * d : d) * S + (size_t)j * B + b0 + c] = buf[tpad(j, LD, d * BC + c)];
     }
   }
 }
@@ -1354,6 +1366,59 @@ __global__ void __launch_bounds__(256) kwb_cols(const FftRun<T>* __restrict__ ru
   cols_body<T, E, DIR, BC>(data + (size_t)blockIdx.y * N * NHH, NHH, T(1), blockIdx.x * BC, tw, tw + tw_len<T, E>());
 }
 
+// Inverse y pass of the two spectra the x pass handed on, G_x (T2 component 0)
+// and Phi alpha (component 2), for one x-plane's tile of BC columns: G_x, then
+// G_y = i y_y Phi alpha (to component 1), then Phi alpha, whose outputs times
+// i y_z (constant along the column) are G_z (back to component 2, read by
+// then).  One block does all three, so Phi alpha's tile is read from DRAM once.
+template <typename T, int E, int BC>
+__global__ void __launch_bounds__(256) kwb_cols_inv3(const FftRun<T>* __restrict__ runs) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
+  load_tw_group<T, E, false>(tw);
+  cpx<T>* buf = tw + tw_len<T, E>();
+  constexpr int N = 32 * E, B = N / 2 + 1, LD = BC + 1;
+  const FftRun<T>& r = runs[blockIdx.z];
+  const size_t S = (size_t)N * N * B;
+  const int b0 = blockIdx.x * BC, nb = min(BC, B - b0);
+  cpx<T>* const gx = r.T2 + (size_t)blockIdx.y * N * B + b0;
+  cpx<T>* const gy = gx + S;
+  cpx<T>* const ga = gy + S;
+  const T two_pi_L = r.sk.two_pi_L;
+#pragma unroll 1
+  for (int d = 0; d < 3; ++d) {
+    const cpx<T>* src = d == 0 ? gx : ga;
+    cpx<T>* dst = d == 0 ? gx : d == 1 ? gy : ga;
+    for (int t = threadIdx.x; t < N * BC; t += blockDim.x) {
+      const int j = t / BC, c = t - j * BC;
+      cpx<T> v = c < nb ? src[(size_t)j * B + c] : cpx<T>{T(0), T(0)};
+      if (d == 1) {
+        const int qy = j < N / 2 ? j : j - N;
+        const T cy = qy != -N / 2 ? two_pi_L * (T)qy : T(0);
+        v = cpx<T>{-cy * v.y, cy * v.x};
+      }
+      buf[tpad(j, LD, c)] = v;
+    }
+    __syncthreads();
+    tile_ffts<T, N, +1>(nb, tw, tw + kTwLen, [&](int p, int j) { return buf + tpad(j, LD, p); },
+                        [](int) { return true; });
+    __syncthreads();
+    for (int t = threadIdx.x; t < N * BC; t += blockDim.x) {
+      const int j = t / BC, c = t - j * BC;
+      if (c < nb) {
+        cpx<T> v = buf[tpad(j, LD, c)];
+        if (d == 2) {
+          const int qz = b0 + c;
+          const T cz = qz != N / 2 ? two_pi_L * (T)qz : T(0);
+          v = cpx<T>{-cz * v.y, cz * v.x};
+        }
+        dst[(size_t)j * B + c] = v;
+      }
+    }
+    __syncthreads();
+  }
+}
+
 template <typename T, int E, int BC>
 __global__ void __launch_bounds__(512) kwb_spectral_x(const FftRun<T>* __restrict__ runs) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1361,8 +1426,8 @@ __global__ void __launch_bounds__(512) kwb_spectral_x(const FftRun<T>* __restric
   load_tw_group<T, E, false>(tw);
   cpx<T>* twq = tw + kTwLen;
   const FftRun<T>& r = runs[blockIdx.y];
-  spectral_body<T, E, kModeStep, BC>(r.T1, r.alpha, r.T2, r.sk, r.shadow, blockIdx.x * BC, tw, twq,
-                                     twq + twq_len<T, 32 * E>());
+  spectral_body<T, E, kModeStep, BC, two_spectra<E>()>(r.T1, r.alpha, r.T2, r.sk, r.shadow, blockIdx.x * BC, tw, twq,
+                                                       twq + twq_len<T, 32 * E>());
 }
 
 template <typename T, int E>
@@ -1377,6 +1442,69 @@ __global__ void __launch_bounds__(256) kwb_rows_c2r(const FftRun<T>* __restrict_
   const FftRun<T>& r = runs[blockIdx.y];
   const size_t S = (size_t)N * N * (N / 2 + 1);
   rows_c2r_body<T, E, 3>(r.T2, S, r.grad, N * N, nullptr, blockIdx.x, gridDim.x, tw, zb_all, ob_all);
+}
+
+// Rows c2r of the three gradient components by group FFTs with whole nodes
+// written: a group keeps its row pair's transforms of all three components in
+// registers (lane q holds the same nodes of each) and stores (gx, gy, gz, 0)
+// vectors.  Written one component at a time, every node's sector was stored
+// in part three times and, never complete, filled from DRAM before it could
+// be evicted: 175 -> 81 us at H = 256.
+template <int N>
+__global__ void __launch_bounds__(128) kwrb_rows_c2r3(const FftRun<float>* __restrict__ runs) {
+  using T = float;
+  constexpr int F = GroupShape<N>::F, Q = GroupShape<N>::Q, G = 32 / Q, R = F / Q, NH = N / 2 + 1;
+  constexpr int KI = (NH + Q - 1) / Q;
+  __shared__ cpx<T> twq[N];
+  __shared__ cpx<T> slots[4 * G * group_ps<N>()];
+  load_twq<T, N>(twq);
+  __syncthreads();
+  const FftRun<T>& r = runs[blockIdx.y];
+  constexpr size_t S = (size_t)N * N * NH;
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const int g = lane / Q, q = lane & (Q - 1);
+  cpx<T>* z = slots + (wib * G + g) * group_ps<N>();
+  const int pr = (blockIdx.x * 4 + wib) * G + g;   // N N / 2 row pairs, a whole number of blocks
+  const cpx<T>* ra = r.T2 + (size_t)(2 * pr) * NH;
+  cpx<T> v[3][F];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    cpx<T> a[KI], b[KI];
+#pragma unroll
+    for (int i = 0; i < KI; ++i) {
+      const int k = q + Q * i;
+      if (k < NH) {
+        a[i] = ra[d * S + k];
+        b[i] = ra[d * S + NH + k];
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < KI; ++i) {
+      const int k = q + Q * i;
+      if (k < NH) {
+        cpx<T> A = a[i], Bv = b[i];
+        if (k == 0 || k == N / 2) {
+          A.y = T(0);
+          Bv.y = T(0);
+        }
+        z[k] = cpx<T>{A.x - Bv.y, A.y + Bv.x};
+        if (k > 0 && k < N / 2) z[N - k] = cpx<T>{A.x + Bv.y, -A.y + Bv.x};   // conj A + i conj B
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int m = 0; m < F; ++m) v[d][m] = z[q + Q * m];
+    group_fft<T, N, +1>(v[d], q, twq, 0xffffffffu, [z](int j) { return z + j; });
+  }
+  float4* oa = reinterpret_cast<float4*>(r.grad) + (size_t)(2 * pr) * N;
+#pragma unroll
+  for (int rr = 0; rr < R; ++rr)
+#pragma unroll
+    for (int k2 = 0; k2 < Q; ++k2) {
+      const int j = q + Q * rr + F * k2, i = rr * Q + k2;
+      oa[j] = make_float4(v[0][i].x, v[1][i].x, v[2][i].x, 0.f);
+      oa[N + j] = make_float4(v[0][i].y, v[1][i].y, v[2][i].y, 0.f);
+    }
 }
 
 // Shared bytes of the row c2r kernels: twiddles, per-warp scratch and, in
@@ -1851,7 +1979,9 @@ __device__ __forceinline__ void cplane_fwd_body(Tin* __restrict__ in, double in_
 
 template <typename T, int E, int CS>
 __device__ __forceinline__ void cplane_inv_body(const cpx<T>* __restrict__ in, T* __restrict__ out, int x, int d,
-                                                const cpx<T>* tw, cpx<T>* Q, cpx<T>* zball) {
+                                                T two_pi_L, const cpx<T>* tw, cpx<T>* Q, cpx<T>* zball) {
+  // H = 256: G_y and G_z from Phi alpha, as in kwb_cols_inv3
+  const bool from_y = two_spectra<E>() && d == 1, from_z = two_spectra<E>() && d == 2;
   namespace cg = cooperative_groups;
   constexpr int N = 32 * E;
   using CSp = ColSplit<N, CS>;
@@ -1863,7 +1993,13 @@ __device__ __forceinline__ void cplane_inv_body(const cpx<T>* __restrict__ in, T
   const int c0 = CSp::first(rank), nc = CSp::count(rank);
   for (int t = threadIdx.x; t < N * nc; t += blockDim.x) {
     const int j = t / nc, c = t - j * nc;
-    Q[tpad(j, LD, c)] = in[(size_t)j * NH + c0 + c];
+    cpx<T> v = in[(size_t)j * NH + c0 + c];
+    if (from_y) {
+      const int qy = j < N / 2 ? j : j - N;
+      const T cy = qy != -N / 2 ? two_pi_L * (T)qy : T(0);
+      v = cpx<T>{-cy * v.y, cy * v.x};
+    }
+    Q[tpad(j, LD, c)] = v;
   }
   __syncthreads();
   // 1. y-axis inverse of this CTA's columns
@@ -1883,6 +2019,11 @@ __device__ __forceinline__ void cplane_inv_body(const cpx<T>* __restrict__ in, T
           const int row = 2 * (rank * PAIRS + pr), o = k / LD, kl = k - o * LD;
           A = peer[o][tpad(row, LD, kl)];
           B = peer[o][tpad(row + 1, LD, kl)];
+          if (from_z) {
+            const T cz = k != N / 2 ? two_pi_L * (T)k : T(0);
+            A = cpx<T>{-cz * A.y, cz * A.x};
+            B = cpx<T>{-cz * B.y, cz * B.x};
+          }
         },
         [&](int, int g) { return zs + g * group_ps<N>(); },
         [&](int pr, int j, T re, T im) {
@@ -1896,6 +2037,11 @@ __device__ __forceinline__ void cplane_inv_body(const cpx<T>* __restrict__ in, T
     for (int k = lane; k < NH; k += 32) {
       const int o = k / LD, kl = k - o * LD;
       cpx<T> A = peer[o][tpad(2 * pr, LD, kl)], Bv = peer[o][tpad(2 * pr + 1, LD, kl)];
+      if (from_z) {
+        const T cz = k != N / 2 ? two_pi_L * (T)k : T(0);
+        A = cpx<T>{-cz * A.y, cz * A.x};
+        Bv = cpx<T>{-cz * Bv.y, cz * Bv.x};
+      }
       if (k == 0 || k == N / 2) {
         A.y = T(0);
         Bv.y = T(0);
@@ -1959,7 +2105,8 @@ __global__ void __launch_bounds__(1024) kwc_inv(const FftRun<T>* __restrict__ ru
   const FftRun<T>& r = runs[blockIdx.z];
   const int x = blockIdx.x / CS, d = blockIdx.y;
   const size_t S = (size_t)N * N * NH;
-  cplane_inv_body<T, E, CS>(r.T2 + d * S + (size_t)x * N * NH, r.grad, x, d, tw, Q, zb);
+  const int comp = two_spectra<E>() && d == 1 ? 2 : d;   // G_y from Phi alpha
+  cplane_inv_body<T, E, CS>(r.T2 + comp * S + (size_t)x * N * NH, r.grad, x, d, r.sk.two_pi_L, tw, Q, zb);
 }
 
 // Launch with a cluster of CS CTAs along x.
@@ -2220,7 +2367,8 @@ static size_t cols_smem() {
 }
 template <typename T, int E, int SBC>
 static size_t spectral_smem() {
-  return (kTwLen + twq_len<T, 32 * E>() + (size_t)32 * E * (3 * SBC + 1) + E) * sizeof(cpx<T>);
+  return (kTwLen + twq_len<T, 32 * E>() + (size_t)32 * E * ((two_spectra<E>() ? 2 : 3) * SBC + 1) + E) *
+         sizeof(cpx<T>);
 }
 
 template <typename T, int E, int DIR, int BC>
@@ -2241,6 +2389,16 @@ static cudaError_t kwb_cols_bc(const FftRun<T>* runs, int nruns, int ncomp, int 
     case 32: return kwb_cols_launch<T, E, DIR, 32>(runs, nruns, ncomp, s);
     default: return kwb_cols_launch<T, E, DIR, 16>(runs, nruns, ncomp, s);
   }
+}
+
+template <typename T, int E, int BC>
+static cudaError_t kwb_cols_inv3_launch(const FftRun<T>* runs, int nruns, cudaStream_t s) {
+  constexpr int N = 32 * E, NHH = N / 2 + 1;
+  const size_t smc = cols_smem<T, E, BC>();
+  if (smc > kMaxSmem) return cudaErrorInvalidValue;
+  const cudaError_t e = set_smem(kwb_cols_inv3<T, E, BC>, smc);
+  if (e != cudaSuccess) return e;
+  return launch_plain(kwb_cols_inv3<T, E, BC>, dim3((NHH + BC - 1) / BC, N, nruns), 256, smc, s, runs);
 }
 
 template <typename T, int E, int SBC>
@@ -2356,11 +2514,24 @@ static cudaError_t field_batch_e(const FftRun<T>* runs, int nruns, int stages, c
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     nk += 1;
   } else if (stages & kFieldInverse) {
-    if ((e = kwb_cols_bc<T, E, +1>(runs, nruns, 3, bc, s)) != cudaSuccess) return e;
-    const size_t smr = row_c2r_smem<T, E, 4>();
-    if ((e = set_smem(kwb_rows_c2r<T, E>, smr)) != cudaSuccess) return e;
-    launch_plain(kwb_rows_c2r<T, E>, dim3(rblocks, nruns), 256, smr, s, runs);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if constexpr (two_spectra<E>()) {
+      switch (bc) {
+        case 8: e = kwb_cols_inv3_launch<T, E, 8>(runs, nruns, s); break;
+        case 32: e = kwb_cols_inv3_launch<T, E, 32>(runs, nruns, s); break;
+        default: e = kwb_cols_inv3_launch<T, E, 16>(runs, nruns, s); break;
+      }
+    } else {
+      e = kwb_cols_bc<T, E, +1>(runs, nruns, 3, bc, s);
+    }
+    if (e != cudaSuccess) return e;
+    if constexpr (group_rows<T, N>()) {
+      e = launch_plain(kwrb_rows_c2r3<N>, dim3(N * N / 2 / (4 * (32 / GroupShape<N>::Q)), nruns), 128, 0, s, runs);
+    } else {
+      const size_t smr = row_c2r_smem<T, E, 4>();
+      if ((e = set_smem(kwb_rows_c2r<T, E>, smr)) != cudaSuccess) return e;
+      e = launch_plain(kwb_rows_c2r<T, E>, dim3(rblocks, nruns), 256, smr, s, runs);
+    }
+    if (e != cudaSuccess) return e;
     nk += 2;
   }
   return cudaSuccess;
