@@ -139,16 +139,6 @@ __device__ __forceinline__ int tile_of(int cx, int cy, int cz, int shift, int nt
   return (((cx >> shift) * ntx) + (cy >> shift)) * ntx + (cz >> shift);
 }
 
-// Find the run of global work item c: largest r with prefix[r] <= c.
-__device__ __forceinline__ int find_run(const long long* prefix, int nruns, long long c) {
-  int lo = 0, hi = nruns - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (prefix[mid] <= c) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
-
 // ---------------------------------------------------------------------------
 // Deposit and re-bin over the tile bins.  A step moves every particle into the
 // bin of its new tile (k_move), then deposits from those bins: the chemotactic
@@ -355,9 +345,9 @@ __device__ __forceinline__ void tile_origin(int bin, int ntx, int& ox, int& oy, 
 
 // Deposit of one work item of a single bin by the block.  WHOLE: the window is
 // the whole grid (use_win: the launch has one).
-template <typename T, bool FIXED, bool WHOLE>
+template <typename T, bool FIXED, bool WHOLE, typename Fetch>
 __device__ __forceinline__ void deposit_chunk(const BinArgs<T>& a, const ChunkDesc& cur,
-                                              typename WinType<T>::type* win, bool use_win) {
+                                              typename WinType<T>::type* win, bool use_win, Fetch& fetch) {
   using A = typename WinType<T>::type;
   const int H = a.g.H, mask = a.g.mask;
   const int wslots = WHOLE ? H * H * H : kWinSlots;
@@ -388,6 +378,7 @@ __device__ __forceinline__ void deposit_chunk(const BinArgs<T>& a, const ChunkDe
       py = __ldcs(a.sy + s);
       pz = __ldcs(a.sz + s);
     }
+    fetch.load();
     uint32_t bit = 1u;   // at most kChunkMax / 256 iterations
     for (int i0 = 0; i0 < len; i0 += blockDim.x, bit <<= 1) {
       const int i = i0 + threadIdx.x;
@@ -434,6 +425,7 @@ __device__ __forceinline__ void deposit_chunk(const BinArgs<T>& a, const ChunkDe
       if (fits) deposit_window<T, kTileReps>(a.p2g, win + slot * kTileReps + cpy, lx, ly, lz, wwin);
     }
   }
+  if (!has_win) fetch.load();
   if (missed)
     for (int i = threadIdx.x; i < len; i += blockDim.x, missed >>= 1)
       if (missed & 1u) deposit_global<T, FIXED>(a, start + i);
@@ -499,13 +491,41 @@ __device__ __forceinline__ void deposit_merged(const BinArgs<T>& a, const ChunkD
     if (has_win) {
       __syncwarp();
       const T unit = a.wmass * pow2<T>(-K);
+      if constexpr (sizeof(A) == 4 && !FIXED) {
+        // float grid: aligned quads of a window row along z (1, 4, 4 and 2 of
+        // its 11 nodes) as 16-byte reductions, 484 a window instead of some
+        // 900 non-zero nodes (see k_deposit_vec)
+        float* const grid = reinterpret_cast<float*>(a.phi);
+        for (int t = lane; t < kWin * kWin * 4; t += 32) {
+          const int row = t >> 2, k0 = 4 * (t & 3) - 3;
+          A* const wr = ww + row * kWin + k0;
+          float v[4];
+          bool any = false;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            A c4 = 0;
+            if (k0 + i >= 0 && k0 + i < kWin) c4 = wr[i];
+            if (c4 != 0) {
+              wr[i] = 0;
+              any = true;
+            }
+            v[i] = sum_to_real<float>(c4) * unit;
+          }
+          if (any) {
+            const int sa = row / kWin, sb = row - sa * kWin;
+            const int gi = (((ox + sa) & mask) * H + ((oy + sb) & mask)) * H + ((oz + k0) & mask);
+            atomicAdd(reinterpret_cast<float4*>(grid + gi), make_float4(v[0], v[1], v[2], v[3]));
+          }
+        }
+      } else {
 #pragma unroll 4
-      for (int s = lane; s < kWinSlots; s += 32) {
-        const A v = ww[s];
-        if (v != 0) {
-          ww[s] = A(0);
-          const int sc = s % kWin, sb = (s / kWin) % kWin, sa = s / (kWin * kWin);
-          add_node<T, FIXED>(a, (((ox + sa) & mask) * H + ((oy + sb) & mask)) * H + ((oz + sc) & mask), v, unit);
+        for (int s = lane; s < kWinSlots; s += 32) {
+          const A v = ww[s];
+          if (v != 0) {
+            ww[s] = A(0);
+            const int sc = s % kWin, sb = (s / kWin) % kWin, sa = s / (kWin * kWin);
+            add_node<T, FIXED>(a, (((ox + sa) & mask) * H + ((oy + sb) & mask)) * H + ((oz + sc) & mask), v, unit);
+          }
         }
       }
       __syncwarp();
@@ -566,26 +586,45 @@ __device__ __forceinline__ void rebin_run(const BinArgs<T>& a, long long start, 
   }
 }
 
-// Work items are taken from a global counter by persistent blocks; the next
-// one is fetched while the current one is processed.
-template <typename T, typename Fn>
-__device__ __forceinline__ void for_items(const BinArgs<T>& a, ChunkDesc* s_desc, Fn&& fn) {
-  const long long nchunks = a.chunk_start[a.NT + 1];
-  if (threadIdx.x == 0) {
-    const long long c = (long long)atomicAdd(a.work, 1ULL);
-    s_desc[0] = c < nchunks ? a.chunks[c] : ChunkDesc{0, 0, 0};
+// Work items are taken from a global counter by persistent blocks.  Thread 0
+// takes the next item's index when the current item starts and loads its
+// description when fn calls mid(), by when the counter's answer has come
+// back, so that neither latency lies between two items.  (Both at the start
+// of an item, with a search over the runs for a batch's items, put some 2 and
+// 4 us in front of every item: batch of 24 runs, move 62 -> MEASURED us and
+// deposit 61 -> MEASURED us a step.)
+__device__ __forceinline__ ChunkDesc desc_of(const ChunkDesc& d) { return d; }
+__device__ __forceinline__ ChunkDesc desc_of(const BatchItem& b) { return b.d; }
+template <typename Item>
+struct ItemFetch {
+  const Item* list;
+  long long n;
+  unsigned long long* work;
+  long long c;
+  Item nxt;
+  __device__ __forceinline__ void take() {
+    if (threadIdx.x == 0) c = (long long)atomicAdd(work, 1ULL);
   }
+  __device__ __forceinline__ void load() {
+    nxt = Item{};
+    if (threadIdx.x == 0 && c < n) nxt = list[c];
+  }
+};
+// s_item: two shared items.  fn(item, fetch) must call fetch.load() once.
+template <typename Item, typename Fn>
+__device__ __forceinline__ void for_items(const Item* list, long long n, unsigned long long* work, Item* s_item,
+                                          Fn&& fn) {
+  ItemFetch<Item> fetch{list, n, work, 0, Item{}};
+  fetch.take();
+  fetch.load();
+  if (threadIdx.x == 0) s_item[0] = fetch.nxt;
   __syncthreads();
   for (int buf = 0;; buf ^= 1) {
-    const ChunkDesc cur = s_desc[buf];
-    if (cur.len == 0) break;
-    ChunkDesc nxt{0, 0, 0};
-    if (threadIdx.x == 0) {
-      const long long c = (long long)atomicAdd(a.work, 1ULL);
-      if (c < nchunks) nxt = a.chunks[c];
-    }
-    fn(cur);
-    if (threadIdx.x == 0) s_desc[buf ^ 1] = nxt;
+    const Item cur = s_item[buf];
+    if (desc_of(cur).len == 0) break;
+    fetch.take();
+    if (!fn(cur, fetch)) break;
+    if (threadIdx.x == 0) s_item[buf ^ 1] = fetch.nxt;
     __syncthreads();
   }
 }
@@ -596,15 +635,20 @@ k_binned_deposit(const __grid_constant__ BinArgs<T> a, int use_win) {
   using A = typename WinType<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   A* win = reinterpret_cast<A*>(smem_raw);
-  __shared__ ChunkDesc s_desc[2];
+  __shared__ ChunkDesc s_item[2];
   if (use_win) {
     const int n = WHOLE ? kReplicas * a.g.H * a.g.H * a.g.H : kTileReps * kWinSlots;
     for (int i = threadIdx.x; i < n; i += blockDim.x) win[i] = A(0);
   }
   pdl_wait();
-  for_items(a, s_desc, [&](const ChunkDesc& cur) {
-    if (cur.bin >= 0) deposit_chunk<T, FIXED, WHOLE>(a, cur, win, use_win != 0);
-    else deposit_merged<T, FIXED, WHOLE>(a, cur, win);
+  for_items(a.chunks, a.chunk_start[a.NT + 1], a.work, s_item, [&](const ChunkDesc& cur, auto& fetch) {
+    if (cur.bin >= 0) {
+      deposit_chunk<T, FIXED, WHOLE>(a, cur, win, use_win != 0, fetch);
+    } else {
+      fetch.load();
+      deposit_merged<T, FIXED, WHOLE>(a, cur, win);
+    }
+    return true;
   });
 }
 
@@ -612,65 +656,44 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 k_binned_rebin(const __grid_constant__ BinArgs<T> a) {
   pdl_wait();
-  __shared__ ChunkDesc s_desc[2];
-  for_items(a, s_desc, [&](const ChunkDesc& cur) {
+  __shared__ ChunkDesc s_item[2];
+  for_items(a.chunks, a.chunk_start[a.NT + 1], a.work, s_item, [&](const ChunkDesc& cur, auto& fetch) {
+    fetch.load();
     if (cur.bin >= 0) {
       rebin_run(a, cur.start, cur.len, threadIdx.x, blockDim.x);
-      return;
+      return true;
     }
       for (int k = threadIdx.x >> 5; k < kMerge; k += (int)(blockDim.x >> 5)) {   // a warp per small bin
       const int b = (int)cur.start * kMerge + k;
       const int c = b < a.NT ? a.src_count[b] : 0;
       if (bin_is_small(b, c, a.NT, a.small)) rebin_run(a, a.src_base[b], c, threadIdx.x & 31, 32);
     }
+    return true;
   });
 }
 
-// Batched deposit over the bins of all runs (tile windows, H >= 32).
+// Batched deposit over the bins of all runs (tile windows, H >= 32): items of
+// all runs from one list.
 template <typename T, bool FIXED>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2)
-k_deposit_batch(const BinArgs<T>* __restrict__ table, const long long* __restrict__ prefix, int nruns,
-                unsigned long long* work) {
+k_deposit_batch(const BinArgs<T>* __restrict__ table, const BatchItem* __restrict__ list,
+                const long long* __restrict__ total, unsigned long long* work) {
   using A = typename WinType<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   A* win = reinterpret_cast<A*>(smem_raw);
-  __shared__ ChunkDesc s_desc[2];
-  __shared__ int s_run[2];
+  __shared__ BatchItem s_item[2];
   for (int i = threadIdx.x; i < kTileReps * kWinSlots; i += blockDim.x) win[i] = A(0);
   pdl_wait();
-  const long long total = prefix[nruns];
-  if (threadIdx.x == 0) {
-    const long long c = (long long)atomicAdd(work, 1ULL);
-    if (c < total) {
-      const int r = find_run(prefix, nruns, c);
-      s_run[0] = r;
-      s_desc[0] = table[r].chunks[c - prefix[r]];
+  for_items(list, *total, work, s_item, [&](const BatchItem& cur, auto& fetch) {
+    const BinArgs<T>& a = table[cur.run];
+    if (cur.d.bin >= 0) {
+      deposit_chunk<T, FIXED, false>(a, cur.d, win, true, fetch);
     } else {
-      s_desc[0] = ChunkDesc{0, 0, 0};
+      fetch.load();
+      deposit_merged<T, FIXED, false>(a, cur.d, win);
     }
-  }
-  __syncthreads();
-  for (int buf = 0;; buf ^= 1) {
-    const ChunkDesc cur = s_desc[buf];
-    if (cur.len == 0) break;
-    const int run = s_run[buf];
-    ChunkDesc nxt{0, 0, 0};
-    int nrun = 0;
-    if (threadIdx.x == 0) {
-      const long long c = (long long)atomicAdd(work, 1ULL);
-      if (c < total) {
-        nrun = find_run(prefix, nruns, c);
-        nxt = table[nrun].chunks[c - prefix[nrun]];
-      }
-    }
-    if (cur.bin >= 0) deposit_chunk<T, FIXED, false>(table[run], cur, win, true);
-    else deposit_merged<T, FIXED, false>(table[run], cur, win);
-    if (threadIdx.x == 0) {
-      s_desc[buf ^ 1] = nxt;
-      s_run[buf ^ 1] = nrun;
-    }
-    __syncthreads();
-  }
+    return true;
+  });
 }
 
 // ---------------------------------------------------------------------------
@@ -694,8 +717,7 @@ template <typename T> constexpr int move_min_blocks() { return sizeof(T) == 4 ? 
 template <typename T>
 struct MoveSmem {
   static constexpr int R = MoveRound<T>::n;
-  ChunkDesc desc[2];
-  int run[2];
+  BatchItem item[2];   // (single runs use the first ChunkDesc-sized part)
   __align__(16) T x[R];
   __align__(16) T y[R];
   __align__(16) T z[R];
@@ -784,8 +806,9 @@ template <typename T> __device__ __forceinline__ void move_write_out(const BinAr
 // source tiles, are read straight from their bins in rounds, moved, staged
 // and written out, each reserving its own destination slot (sparse bins, so
 // the destination cursors see little contention).
-template <typename T, bool MOVE, int G2P>
-__device__ __forceinline__ void move_merged(const BinArgs<T>& a, const ChunkDesc& cur, uint32_t n, MoveSmem<T>& sm) {
+template <typename T, bool MOVE, int G2P, typename Fetch>
+__device__ __forceinline__ void move_merged(const BinArgs<T>& a, const ChunkDesc& cur, uint32_t n, MoveSmem<T>& sm,
+                                            Fetch& fetch) {
   constexpr int R = MoveRound<T>::n;
   if (threadIdx.x < kMerge) {
     const int b = (int)cur.start * kMerge + threadIdx.x;
@@ -800,6 +823,7 @@ __device__ __forceinline__ void move_merged(const BinArgs<T>& a, const ChunkDesc
     sm.seg_base[threadIdx.x] = base;
   }
   __syncthreads();
+  fetch.load();
   for (int r0 = 0; r0 < cur.len; r0 += R) {
     const int cnt = min(R, cur.len - r0);
 #pragma unroll 1
@@ -837,13 +861,14 @@ __device__ __forceinline__ void prefetch_round(const BinArgs<T>& a, long long s0
 
 // One work item of the move + re-bin pass (see above).  n: step index of the
 // move (noise counter).  MOVE = false only re-bins (capacity rebuilds).
-// nxt / na (thread 0; na nullable): the block's next work item and its run's
-// arguments, whose first round is prefetched during this item's last round.
-template <typename T, bool MOVE, int G2P = 0>
+// fetch: the block's next work item, loaded while this one's first round is
+// staged; its first round is prefetched (args_of: its run's arguments) during
+// this item's last round.
+template <typename T, bool MOVE, int G2P, typename Fetch, typename ArgsOf>
 __device__ __forceinline__ void move_chunk(const BinArgs<T>& a, const ChunkDesc& cur, uint32_t n, MoveSmem<T>& sm,
-                                           uint32_t& phase, const ChunkDesc& nxt, const BinArgs<T>* na) {
+                                           uint32_t& phase, Fetch& fetch, ArgsOf&& args_of) {
   if (cur.bin < 0) {
-    move_merged<T, MOVE, G2P>(a, cur, n, sm);
+    move_merged<T, MOVE, G2P>(a, cur, n, sm, fetch);
     return;
   }
   constexpr int R = MoveRound<T>::n;
@@ -873,6 +898,7 @@ __device__ __forceinline__ void move_chunk(const BinArgs<T>& a, const ChunkDesc&
       if (r0 + R < cur.len) prefetch_round(a, s0 + R, min(R, cur.len - r0 - R));
     }
     for (int k = threadIdx.x; k < kNbr; k += blockDim.x) sm.cnt[k] = 0;
+    if (r0 == 0) fetch.load();
     if (!mbar_wait(&sm.bar, phase, 1u << 26)) {
       atomicOr(a.err, 4);   // staging copy did not complete
       sm.abort = 1;
@@ -912,8 +938,10 @@ __device__ __forceinline__ void move_chunk(const BinArgs<T>& a, const ChunkDesc&
     }
     __syncthreads();
     // (the next item's descriptor has arrived by now)
-    if (threadIdx.x == 0 && r0 + R >= cur.len && nxt.len > 0 && nxt.bin >= 0 && na)
-      prefetch_round(*na, nxt.start, min(R, nxt.len));
+    if (threadIdx.x == 0 && r0 + R >= cur.len) {
+      const ChunkDesc nd = desc_of(fetch.nxt);
+      if (nd.len > 0 && nd.bin >= 0) prefetch_round(args_of(fetch.nxt), nd.start, min(R, nd.len));
+    }
     // 2. one reservation per destination tile (with its capacity and first slot)
     for (int k = threadIdx.x; k < kNbr; k += blockDim.x) {
       const int c = sm.cnt[k];
@@ -936,77 +964,44 @@ __global__ void __launch_bounds__(kMoveThreads, move_min_blocks<T>())
 k_move(BinArgs<T> a) {
   pdl_wait();
   __shared__ MoveSmem<T> sm;
-  const long long nchunks = a.chunk_start[a.NT + 1];
   if (threadIdx.x == 0) {
     mbar_init(&sm.bar, 1);
     sm.abort = 0;
-    const long long c = (long long)atomicAdd(a.work, 1ULL);
-    sm.desc[0] = c < nchunks ? a.chunks[c] : ChunkDesc{0, 0, 0};
   }
-  __syncthreads();
   uint32_t phase = 0;
-  for (int buf = 0;; buf ^= 1) {
-    const ChunkDesc cur = sm.desc[buf];
-    if (cur.len == 0 || sm.abort) break;
-    ChunkDesc nxt{0, 0, 0};
-    if (threadIdx.x == 0) {
-      const long long c = (long long)atomicAdd(a.work, 1ULL);
-      if (c < nchunks) nxt = a.chunks[c];
-    }
-    move_chunk<T, true, G2P>(a, cur, a.n, sm, phase, nxt, &a);
-    if (threadIdx.x == 0) sm.desc[buf ^ 1] = nxt;
-    __syncthreads();
-  }
+  for_items(a.chunks, a.chunk_start[a.NT + 1], a.work, reinterpret_cast<ChunkDesc*>(sm.item),
+            [&](const ChunkDesc& cur, auto& fetch) {
+              move_chunk<T, true, G2P>(a, cur, a.n, sm, phase, fetch,
+                                       [&](const ChunkDesc&) -> const BinArgs<T>& { return a; });
+              return sm.abort == 0;
+            });
 }
 
 
-// Batched move (MOVE) or re-bin (!MOVE): work items of all runs from one
-// counter; run r's arguments at table[r]; the step index from device memory.
+// Batched move (MOVE) or re-bin (!MOVE): work items of all runs from one list;
+// run r's arguments at table[r]; the step index from device memory.
 template <typename T, bool MOVE, int G2P>
 __global__ void __launch_bounds__(kMoveThreads, move_min_blocks<T>())
-k_move_batch(const BinArgs<T>* __restrict__ table, const long long* __restrict__ prefix, int nruns,
-             unsigned long long* work, const uint32_t* step) {
+k_move_batch(const BinArgs<T>* __restrict__ table, const BatchItem* __restrict__ list,
+             const long long* __restrict__ total, unsigned long long* work, const uint32_t* step) {
   pdl_wait();
   __shared__ MoveSmem<T> sm;
-  const long long total = prefix[nruns];
   const uint32_t n = *step + 1;
   if (threadIdx.x == 0) {
     mbar_init(&sm.bar, 1);
     sm.abort = 0;
-    const long long c = (long long)atomicAdd(work, 1ULL);
-    if (c < total) {
-      const int r = find_run(prefix, nruns, c);
-      sm.run[0] = r;
-      sm.desc[0] = table[r].chunks[c - prefix[r]];
-    } else {
-      sm.desc[0] = ChunkDesc{0, 0, 0};
-    }
   }
-  __syncthreads();
   uint32_t phase = 0;
-  for (int buf = 0;; buf ^= 1) {
-    const ChunkDesc cur = sm.desc[buf];
-    if (cur.len == 0 || sm.abort) break;
-    const int run = sm.run[buf];
-    ChunkDesc nxt{0, 0, 0};
-    int nrun = 0;
-    if (threadIdx.x == 0) {
-      const long long c = (long long)atomicAdd(work, 1ULL);
-      if (c < total) {
-        nrun = find_run(prefix, nruns, c);
-        nxt = table[nrun].chunks[c - prefix[nrun]];
-      }
-    }
-    move_chunk<T, MOVE, G2P>(table[run], cur, n, sm, phase, nxt, nxt.len > 0 ? table + nrun : nullptr);
-    if (threadIdx.x == 0) {
-      sm.desc[buf ^ 1] = nxt;
-      sm.run[buf ^ 1] = nrun;
-    }
-    __syncthreads();
-  }
+  for_items(list, *total, work, sm.item, [&](const BatchItem& cur, auto& fetch) {
+    move_chunk<T, MOVE, G2P>(table[cur.run], cur.d, n, sm, phase, fetch,
+                             [&](const BatchItem& i) -> const BinArgs<T>& { return table[i.run]; });
+    return sm.abort == 0;
+  });
 }
 
-static cudaError_t resident_blocks(const void* kern, int threads, size_t smem, int* blocks) {
+// Blocks of a persistent grid: as many as are resident at once (at most
+// blocks_per_sm of them on an SM, if given).
+static cudaError_t resident_blocks(const void* kern, int threads, size_t smem, int* blocks, int blocks_per_sm = 0) {
   int dev = 0, sms = 0, per_sm = 0;
   cudaError_t e;
   if (smem > 48 * 1024 &&
@@ -1015,6 +1010,7 @@ static cudaError_t resident_blocks(const void* kern, int threads, size_t smem, i
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem)) != cudaSuccess) return e;
+  if (blocks_per_sm > 0 && blocks_per_sm < per_sm) per_sm = blocks_per_sm;
   *blocks = sms * (per_sm < 1 ? 1 : per_sm);
   return cudaSuccess;
 }
@@ -1116,8 +1112,9 @@ __device__ __forceinline__ void chunk_count_body(const ChunkListArgs& a, int blk
   if (threadIdx.x == 0) a.part[blk] = total;
 }
 
+// (list: a batch's items, where this run's go from its entry on)
 __device__ __forceinline__ void chunk_emit_body(const ChunkListArgs& a, int blk, int nblk, unsigned long long* work,
-                                                unsigned long long* ovf_total) {
+                                                unsigned long long* ovf_total, BatchItem* list = nullptr, int run = 0) {
   __shared__ long long s_off;
   __shared__ long long s_ls[kCLBlock];   // block-local first chunk of each bin
   if (threadIdx.x == 0) {
@@ -1154,14 +1151,18 @@ __device__ __forceinline__ void chunk_emit_body(const ChunkListArgs& a, int blk,
       }
       if (tot > 0) {
         if (j == 0) {   // the window's merged item comes first
-          a.chunks[off + q] = ChunkDesc{(long long)(bin / kMerge), -1, tot};
+          const ChunkDesc d{(long long)(bin / kMerge), -1, tot};
+          a.chunks[off + q] = d;
+          if (list) list[off + q] = BatchItem{d, run, 0};
           continue;
         }
         j -= 1;
       }
     }
     const int c = a.count[bin];
-    a.chunks[off + q] = ChunkDesc{a.base[bin] + (long long)j * a.chunk, bin, min(a.chunk, c - j * a.chunk)};
+    const ChunkDesc d{a.base[bin] + (long long)j * a.chunk, bin, min(a.chunk, c - j * a.chunk)};
+    a.chunks[off + q] = d;
+    if (list) list[off + q] = BatchItem{d, run, 0};
   }
   if (blk == nblk - 1 && threadIdx.x == 0) {
     a.chunk_start[nb] = off + total;
@@ -1194,12 +1195,20 @@ __global__ void __launch_bounds__(kCLBlock) k_chunk_count_batch(const ChunkListA
   chunk_count_body(a, blockIdx.x);
 }
 
-__global__ void __launch_bounds__(kCLBlock) k_chunk_emit_batch(const ChunkListArgs* __restrict__ t) {
+__global__ void __launch_bounds__(kCLBlock)
+k_chunk_emit_batch(const ChunkListArgs* __restrict__ t, const long long* __restrict__ prefix, BatchItem* list) {
   pdl_wait();
   const ChunkListArgs a = t[blockIdx.y];
   const int nblk = chunk_list_blocks_dev(a.NT);
   if ((int)blockIdx.x >= nblk) return;
-  chunk_emit_body(a, blockIdx.x, nblk, nullptr, nullptr);
+  chunk_emit_body(a, blockIdx.x, nblk, nullptr, nullptr, list + prefix[blockIdx.y], blockIdx.y);
+}
+
+// Work items of a run from its blocks' totals (k_chunk_count_batch).
+__device__ __forceinline__ long long run_items(const ChunkListArgs& a) {
+  long long s = 0;
+  for (int i = 0; i < chunk_list_blocks_dev(a.NT); ++i) s += a.part[i];
+  return s;
 }
 
 // Prefix over runs of their work-item counts; clears the work counter and,
@@ -1212,7 +1221,7 @@ k_run_prefix(const ChunkListArgs* __restrict__ t, int nruns, long long* __restri
   const int per = (nruns + blockDim.x - 1) / blockDim.x;
   const int r0 = threadIdx.x * per;
   long long local = 0;
-  for (int r = r0; r < min(r0 + per, nruns); ++r) local += t[r].chunk_start[t[r].NT + 1];
+  for (int r = r0; r < min(r0 + per, nruns); ++r) local += run_items(t[r]);
   s_part[threadIdx.x] = local;
   __syncthreads();
   for (int off = 1; off < (int)blockDim.x; off <<= 1) {
@@ -1224,11 +1233,12 @@ k_run_prefix(const ChunkListArgs* __restrict__ t, int nruns, long long* __restri
   long long run = s_part[threadIdx.x] - local;
   for (int r = r0; r < min(r0 + per, nruns); ++r) {
     prefix[r] = run;
-    run += t[r].chunk_start[t[r].NT + 1];
+    run += run_items(t[r]);
   }
   if (threadIdx.x == blockDim.x - 1) prefix[nruns] = s_part[threadIdx.x];
   if (threadIdx.x == 0) {
-    *work = 0ULL;
+    work[0] = 0ULL;   // deposit / re-bin
+    work[1] = 0ULL;   // move
     if (bump) *step += 1u;
   }
 }
@@ -1863,53 +1873,37 @@ cudaError_t launch_chunk_list(const ChunkListArgs& a, unsigned long long* work, 
 }
 
 template <typename T>
-cudaError_t launch_move_batch(const BinArgs<T>* table, const long long* prefix, int nruns, unsigned long long* work,
-                              const uint32_t* step, bool move, cudaStream_t s, int blocks_per_sm, int g2p) {
-  int dev = 0, sms = 0, per_sm = 0;
-  cudaError_t e;
+cudaError_t launch_move_batch(const BinArgs<T>* table, const BatchItem* list, const long long* total,
+                              unsigned long long* work, const uint32_t* step, bool move, cudaStream_t s,
+                              int blocks_per_sm, int g2p) {
   // the gather order fixed at compile time when every run uses the same one
   auto k = !move ? k_move_batch<T, false, 0>
                  : (g2p == 2 ? k_move_batch<T, true, 2> : g2p == 4 ? k_move_batch<T, true, 4> : k_move_batch<T, true, 0>);
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kMoveThreads, 0)) != cudaSuccess) return e;
-  if (blocks_per_sm > 0 && blocks_per_sm < per_sm) per_sm = blocks_per_sm;
-  if (per_sm < 1) per_sm = 1;
-  launch_k(k, sms * per_sm, kMoveThreads, 0, s, table, prefix, nruns, work, step);
-  return cudaGetLastError();
+  int blocks = 0;
+  const cudaError_t e = resident_blocks((const void*)k, kMoveThreads, 0, &blocks, blocks_per_sm);
+  if (e != cudaSuccess) return e;
+  return launch_k(k, blocks, kMoveThreads, 0, s, table, list, total, work, step);
 }
 
 template <typename T>
-cudaError_t launch_deposit_batch(const BinArgs<T>* table, const long long* prefix, int nruns,
+cudaError_t launch_deposit_batch(const BinArgs<T>* table, const BatchItem* list, const long long* total,
                                  unsigned long long* work, bool fixed, cudaStream_t s, int blocks_per_sm) {
   const size_t smem = (size_t)kTileReps * kWinSlots * sizeof(typename WinType<T>::type);
   auto k = fixed ? k_deposit_batch<T, true> : k_deposit_batch<T, false>;
-  cudaError_t e;
-  if (smem > 48 * 1024 && (e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-    return e;
-  int dev = 0, sms = 0, per_sm = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 256, smem)) != cudaSuccess) return e;
-  if (blocks_per_sm > 0 && blocks_per_sm < per_sm) per_sm = blocks_per_sm;
-  if (per_sm < 1) per_sm = 1;
-  launch_k(k, sms * per_sm, 256, smem, s, table, prefix, nruns, work);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_chunk_list_batch(const ChunkListArgs* t, int nruns, int max_NT, cudaStream_t s) {
-  const dim3 grid(chunk_list_blocks(max_NT), nruns);
-  launch_k(k_chunk_count_batch, grid, kCLBlock, 0, s, t);
-  cudaError_t e = cudaGetLastError();
+  int blocks = 0;
+  const cudaError_t e = resident_blocks((const void*)k, 256, smem, &blocks, blocks_per_sm);
   if (e != cudaSuccess) return e;
-  launch_k(k_chunk_emit_batch, grid, kCLBlock, 0, s, t);
-  return cudaGetLastError();
+  return launch_k(k, blocks, 256, smem, s, table, list, total, work);
 }
 
-cudaError_t launch_run_prefix(const ChunkListArgs* t, int nruns, long long* prefix, unsigned long long* work,
-                              uint32_t* step, int bump, cudaStream_t s) {
-  launch_k(k_run_prefix, 1, 1024, 0, s, t, nruns, prefix, work, step, bump);
-  return cudaGetLastError();
+cudaError_t launch_chunk_list_batch(const ChunkListArgs* t, int nruns, int max_NT, long long* prefix,
+                                    unsigned long long* work, uint32_t* step, int bump, BatchItem* list,
+                                    cudaStream_t s) {
+  const dim3 grid(chunk_list_blocks(max_NT), nruns);
+  cudaError_t e = launch_k(k_chunk_count_batch, grid, kCLBlock, 0, s, t);
+  if (e == cudaSuccess) e = launch_k(k_run_prefix, 1, 1024, 0, s, t, nruns, prefix, work, step, bump);
+  if (e == cudaSuccess) e = launch_k(k_chunk_emit_batch, grid, kCLBlock, 0, s, t, prefix, list);
+  return e;
 }
 
 cudaError_t launch_layout_batch(const LayoutArgs* t, int nruns, cudaStream_t s) {
@@ -2077,10 +2071,10 @@ template <typename T> cudaError_t launch_alpha_energy(const cpx<T>* alpha, int H
   template cudaError_t launch_binned_deposit<T>(const BinArgs<T>&, cudaStream_t);                             \
   template cudaError_t launch_binned_rebin<T>(const BinArgs<T>&, cudaStream_t);                               \
   template cudaError_t launch_move<T>(const BinArgs<T>&, cudaStream_t);                                       \
-  template cudaError_t launch_move_batch<T>(const BinArgs<T>*, const long long*, int, unsigned long long*,     \
-                                            const uint32_t*, bool, cudaStream_t, int, int);                  \
-  template cudaError_t launch_deposit_batch<T>(const BinArgs<T>*, const long long*, int, unsigned long long*,  \
-                                               bool, cudaStream_t, int);                                      \
+  template cudaError_t launch_move_batch<T>(const BinArgs<T>*, const BatchItem*, const long long*,             \
+                                            unsigned long long*, const uint32_t*, bool, cudaStream_t, int, int); \
+  template cudaError_t launch_deposit_batch<T>(const BinArgs<T>*, const BatchItem*, const long long*,          \
+                                               unsigned long long*, bool, cudaStream_t, int);                 \
   template cudaError_t launch_tile_hist<T>(const T*, const T*, const T*, int64_t, Geo<T>, int, int, int, int*, \
                                            cudaStream_t);                                                    \
   template bool launch_rebin_plain<T>(const T*, const T*, const T*, const uint32_t*, int64_t, Geo<T>, int, int, \

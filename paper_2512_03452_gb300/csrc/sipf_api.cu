@@ -1233,7 +1233,8 @@ struct sipf_batch {
   void* dep_tab[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
   ChunkListArgs* cl_tab[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
   LayoutArgs* ly_tab[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
-  long long* prefix = nullptr;
+  long long* prefix = nullptr;      // first item of each run in `list`, then their number
+  BatchItem* list = nullptr;        // all runs' work items
   unsigned long long* work = nullptr;
   uint32_t* step = nullptr;
   int cur = 0, lc = 1, since = 0;
@@ -1271,6 +1272,7 @@ void batch_free(sipf_batch* b) {
       cudaFree(b->ly_tab[i][j]);
     }
   cudaFree(b->prefix);
+  cudaFree(b->list);
   cudaFree(b->work);
   cudaFree(b->step);
   for (cudaEvent_t e : b->ev) cudaEventDestroy(e);
@@ -1338,28 +1340,27 @@ template <typename T> int batch_issue_step(sipf_batch* b) {
     SIPF_CK(mark(2 * g + 1));
   }
   SIPF_CK(mark(2 * G));
-  SIPF_CK(cudaMemsetAsync(b->work, 0, sizeof(unsigned long long), s));
-  SIPF_CK(launch_move_batch<T>((const BinArgs<T>*)b->move_tab[b->cur][b->lc], b->prefix, R, b->work, b->step, true, s,
-                               b->move_bps, b->g2p));
-  SIPF_CK(launch_chunk_list_batch(b->cl_tab[1 - b->cur][b->lc], R, b->max_NT, s));
-  SIPF_CK(launch_run_prefix(b->cl_tab[1 - b->cur][b->lc], R, b->prefix, b->work, b->step, 1, s));
+  SIPF_CK(launch_move_batch<T>((const BinArgs<T>*)b->move_tab[b->cur][b->lc], b->list, b->prefix + R, b->work + 1, b->step, true,
+                               s, b->move_bps, b->g2p));
+  SIPF_CK(launch_chunk_list_batch(b->cl_tab[1 - b->cur][b->lc], R, b->max_NT, b->prefix, b->work, b->step, 1, b->list,
+                                  s));
   SIPF_CK(mark(2 * G + 1));
   b->launches += fk + 4;
   b->field_kernels = fk;
   b->cur = 1 - b->cur;
   if (++b->since >= kBatchResort) {
     SIPF_CK(launch_layout_batch(b->ly_tab[b->cur][1 - b->lc], R, s));
-    SIPF_CK(launch_move_batch<T>((const BinArgs<T>*)b->rebin_tab[b->cur][b->lc], b->prefix, R, b->work, b->step, false,
+    SIPF_CK(launch_move_batch<T>((const BinArgs<T>*)b->rebin_tab[b->cur][b->lc], b->list, b->prefix + R, b->work, b->step, false,
                                  s, b->move_bps));
-    SIPF_CK(launch_chunk_list_batch(b->cl_tab[1 - b->cur][1 - b->lc], R, b->max_NT, s));
-    SIPF_CK(launch_run_prefix(b->cl_tab[1 - b->cur][1 - b->lc], R, b->prefix, b->work, b->step, 0, s));
+    SIPF_CK(launch_chunk_list_batch(b->cl_tab[1 - b->cur][1 - b->lc], R, b->max_NT, b->prefix, b->work, b->step, 0,
+                                    b->list, s));
     b->launches += 5;
     b->cur = 1 - b->cur;
     b->lc = 1 - b->lc;
     b->since = 0;
   }
   SIPF_CK(mark(2 * G + 2));
-  SIPF_CK(launch_deposit_batch<T>((const BinArgs<T>*)b->dep_tab[b->cur][b->lc], b->prefix, R, b->work, b->fixed, s,
+  SIPF_CK(launch_deposit_batch<T>((const BinArgs<T>*)b->dep_tab[b->cur][b->lc], b->list, b->prefix + R, b->work, b->fixed, s,
                                   b->dep_bps));
   SIPF_CK(mark(2 * G + 3));
   b->launches += 1;
@@ -1604,13 +1605,16 @@ int sipf_batch_init(int32_t nruns, const sipf_params* params, const double* cons
   }
   b->field_tune.assign(b->group_H.size(), FieldTune{});
   for (sipf_ctx* c : b->runs) b->max_NT = std::max(b->max_NT, c->NT);
+  int64_t items = 0;
+  for (sipf_ctx* c : b->runs) items += c->max_chunks();
   cudaError_t e = cudaMalloc(&b->prefix, (nruns + 1) * sizeof(long long));
+  if (e == cudaSuccess) e = cudaMalloc(&b->list, (size_t)items * sizeof(BatchItem));
   for (size_t i = 0; i < 2 * b->group_H.size() + 4 && e == cudaSuccess; ++i) {
     cudaEvent_t ev = nullptr;
     e = cudaEventCreate(&ev);
     if (e == cudaSuccess) b->ev.push_back(ev);
   }
-  if (e == cudaSuccess) e = cudaMalloc(&b->work, sizeof(unsigned long long));
+  if (e == cudaSuccess) e = cudaMalloc(&b->work, 2 * sizeof(unsigned long long));   // deposit / re-bin, move
   if (e == cudaSuccess) e = cudaMalloc(&b->step, sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMemsetAsync(b->step, 0, sizeof(uint32_t), b->stream);
   if (e != cudaSuccess) {
@@ -1621,7 +1625,8 @@ int sipf_batch_init(int32_t nruns, const sipf_params* params, const double* cons
   b->lc = b->runs[0]->lc;
   int r = b->precision == 64 ? batch_tables<double>(b) : batch_tables<float>(b);
   if (!r) {
-    cudaError_t e3 = launch_run_prefix(b->cl_tab[b->cur][b->lc], nruns, b->prefix, b->work, b->step, 0, b->stream);
+    cudaError_t e3 = launch_chunk_list_batch(b->cl_tab[b->cur][b->lc], nruns, b->max_NT, b->prefix, b->work, b->step, 0,
+                                             b->list, b->stream);
     if (e3 == cudaSuccess) e3 = cudaStreamSynchronize(b->stream);
     if (e3 != cudaSuccess) r = cuda_fail(e3, "sipf_batch_init prefix");
   }

@@ -205,6 +205,12 @@ struct ChunkDesc {
   int bin, len;
 };
 
+// One work item of a batch: run `run`'s item d.
+struct BatchItem {
+  ChunkDesc d;
+  int run, pad;
+};
+
 // Arguments of the binned particle kernel (see particle_kernels.cu).
 template <typename T>
 struct BinArgs {
@@ -256,15 +262,20 @@ struct LayoutArgs {
   int NT, ntx, ovf_cap;
 };
 template <typename T>
-cudaError_t launch_move_batch(const BinArgs<T>* table, const long long* prefix, int nruns, unsigned long long* work,
-                              const uint32_t* step, bool move, cudaStream_t s, int blocks_per_sm = 0,
+cudaError_t launch_move_batch(const BinArgs<T>* table, const BatchItem* list, const long long* total,
+                              unsigned long long* work, const uint32_t* step, bool move, cudaStream_t s,
+                              int blocks_per_sm = 0,
                               int g2p = 0);   // g2p: 2 or 4 when all runs use that gather order, else 0
 template <typename T>
-cudaError_t launch_deposit_batch(const BinArgs<T>* table, const long long* prefix, int nruns,
+cudaError_t launch_deposit_batch(const BinArgs<T>* table, const BatchItem* list, const long long* total,
                                  unsigned long long* work, bool fixed, cudaStream_t s, int blocks_per_sm = 0);
-cudaError_t launch_chunk_list_batch(const ChunkListArgs* t, int nruns, int max_NT, cudaStream_t s);
-cudaError_t launch_run_prefix(const ChunkListArgs* t, int nruns, long long* prefix, unsigned long long* work,
-                              uint32_t* step, int bump, cudaStream_t s);
+// Chunk lists of every run and the batch's list of all their items (three
+// launches: count, prefix over runs, emit).  prefix[r]: run r's first item,
+// prefix[nruns]: their number; clears the two work counters (deposit and
+// re-bin, move) and, if `bump`, advances the step counter.
+cudaError_t launch_chunk_list_batch(const ChunkListArgs* t, int nruns, int max_NT, long long* prefix,
+                                    unsigned long long* work, uint32_t* step, int bump, BatchItem* list,
+                                    cudaStream_t s);
 cudaError_t launch_layout_batch(const LayoutArgs* t, int nruns, cudaStream_t s);
 // Work-item length for P particles on an H^3 grid, and the bin size below which bins are merged.
 int particle_chunk(int64_t P, int H, bool fp64);
