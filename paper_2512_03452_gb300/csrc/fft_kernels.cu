@@ -1527,6 +1527,14 @@ template <typename T, int E, int NOUT> constexpr size_t row_c2r_smem() {
 // ---------------------------------------------------------------------------
 constexpr int kDefaultPlaneWarps = 8;      // warps per block of the plane kernels
 constexpr int kDefaultSpectralWarps = 8;   // warps per block of the fused x pass
+// The register x pass of few pencils in smaller blocks, so that its warps lie
+// on different SMs (one 64^3 grid is 528 warps, one 32^3 grid 68: 8.1 -> 6.5 and
+// 6.5 -> 4.8 us).
+static int spread_warps(int tasks, int most) {
+  int nw = most;
+  while (nw > 1 && (tasks + nw - 1) / nw < 152) nw >>= 1;
+  return nw;
+}
 
 template <typename T, int E> constexpr size_t plane_smem_bytes(int nw) {
   // plane: H rows of H/2+1 plus one slot per 32 rows; one padded pencil per warp
@@ -2163,7 +2171,7 @@ static cudaError_t warp_spectral(const cpx<T>* T1, cpx<T>* alpha, cpx<T>* T2, Sp
                                  cudaStream_t s) {
   constexpr int N = 32 * E;
   if constexpr (sizeof(T) == 4 && N <= 128) {
-    constexpr int nw = 8;
+    const int nw = spread_warps(XRegShape<N>::TASKS, kDefaultSpectralWarps);
     const size_t smem = xreg_smem_bytes<N>(nw);
     auto k = kwr_spectral_x<N, MODE>;
     cudaError_t e = set_smem(k, smem);
@@ -2406,12 +2414,14 @@ static cudaError_t kwb_spectral_launch(const FftRun<T>* runs, int nruns, int nw,
   constexpr int N = 32 * E, NHH = N / 2 + 1;
   cudaError_t e;
   if constexpr (sizeof(T) == 4 && N <= 128) {
+    if (nw == 0) nw = spread_warps(XRegShape<N>::TASKS * nruns, kDefaultSpectralWarps);
     const size_t smr = xreg_smem_bytes<N>(nw);
     if (smr > kMaxSmem) return cudaErrorInvalidValue;
     if ((e = set_smem(kwrb_spectral_x<N>, smr)) != cudaSuccess) return e;
     launch_k(kwrb_spectral_x<N>, dim3((XRegShape<N>::TASKS + nw - 1) / nw, nruns), 32 * nw, smr, s, runs);
     return cudaGetLastError();
   } else {
+    if (nw == 0) nw = kDefaultSpectralWarps;
     const size_t sms = spectral_smem<T, E, SBC>();
     if (sms > kMaxSmem) return cudaErrorInvalidValue;
     if ((e = set_smem(kwb_spectral_x<T, E, SBC>, sms)) != cudaSuccess) return e;
@@ -2451,7 +2461,7 @@ static cudaError_t field_batch_e(const FftRun<T>* runs, int nruns, int stages, c
   const int fnw = plane_warps(nruns * N, 2, SP ? 16 : 32), inw = SP ? (tune.plane_nw > 0 ? tune.plane_nw : 8)
                                                                      : plane_warps(3 * nruns * N, 4, 16),
             i3nw = plane_warps(nruns * N, 2, SP ? 16 : 32);
-  const int snw = tune.spec_nw > 0 ? tune.spec_nw : kDefaultSpectralWarps;
+  const int snw = tune.spec_nw;   // 0: by the number of pencils
   const size_t fsm = plane_smem_bytes<T, E>(fnw), ism = plane_smem_bytes<T, E>(inw);
   const size_t i3sm = plane3_smem_bytes<T, E>(i3nw);
   // cluster plane kernels (CS = 2 at H <= 128, 4 at H = 256) when asked: at
