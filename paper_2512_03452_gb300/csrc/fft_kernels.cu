@@ -911,17 +911,36 @@ kw_rows_r2c(Tin* __restrict__ in, double in_scale, int zero_input, cpx<T>* __res
   rows_r2c_body<T, E, Tin>(in, in_scale, zero_input, out, rows, mass_acc, blockIdx.x, gridDim.x, tw, zb);
 }
 
+__device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_addr(smem)), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// One thread's elements of a tile, element (j, c) of [N][BC] from src[j * B + c]
+// to shared column `col + c` (c < nb).  ASYNC (single precision, the library's
+// own arrays, 8-byte aligned): all of them in flight at once as asynchronous
+// copies; the caller's wait is included, a block barrier is not.
+template <typename T, int N, int BC, bool ASYNC>
+__device__ __forceinline__ void load_tile(const cpx<T>* __restrict__ src, int B, int nb, cpx<T>* buf, int LD, int col) {
+  for (int t = threadIdx.x; t < N * BC; t += blockDim.x) {
+    const int j = t / BC, c = t - j * BC;
+    if constexpr (ASYNC && sizeof(T) == 4) {
+      if (c < nb) cp_async8(buf + tpad(j, LD, col + c), src + (size_t)j * B + c);
+    } else {
+      buf[tpad(j, LD, col + c)] = c < nb ? src[(size_t)j * B + c] : cpx<T>{T(0), T(0)};
+    }
+  }
+}
+
 // c2c along the middle axis of [A][H][B]: a block stages an H x BC tile
 // (coalesced row segments), warps transform its columns from shared memory.
-template <typename T, int E, int DIR, int BC>
+template <typename T, int E, int DIR, int BC, bool ASYNC = false>
 __device__ __forceinline__ void cols_body(cpx<T>* __restrict__ base, int B, T scale, int b0, const cpx<T>* tw,
                                           cpx<T>* buf) {
   constexpr int N = 32 * E, LD = BC + 1;
   const int nb = min(BC, B - b0);
-  for (int t = threadIdx.x; t < N * BC; t += blockDim.x) {
-    const int j = t / BC, c = t - j * BC;
-    buf[tpad(j, LD, c)] = c < nb ? base[(size_t)j * B + b0 + c] : cpx<T>{T(0), T(0)};
-  }
+  load_tile<T, N, BC, ASYNC>(base + b0, B, nb, buf, LD, 0);
+  if (ASYNC) cp_async_wait_all();
   __syncthreads();
   tile_ffts<T, N, DIR>(nb, tw, tw + kTwLen, [&](int p, int j) { return buf + tpad(j, LD, p); },
                        [](int) { return true; });
@@ -968,11 +987,12 @@ __device__ __forceinline__ void spectral_body(const cpx<T>* __restrict__ T1, cpx
   const size_t S = (size_t)N * B;
   const int nb = min(BC, B - b0);
   constexpr bool needs_beta = (MODE == kModeStep || MODE == kModeDensity);
+  // (alpha's tile comes with beta's, in the second output's slot)
+  constexpr bool alpha_tile = MODE == kModeStep;
   if (needs_beta) {
-    for (int t = threadIdx.x; t < N * BC; t += blockDim.x) {
-      const int j = t / BC, c = t - j * BC;
-      buf[tpad(j, LD, c)] = c < nb ? T1[(size_t)j * B + b0 + c] : cpx<T>{T(0), T(0)};
-    }
+    load_tile<T, N, BC, true>(T1 + b0, B, nb, buf, LD, 0);
+    if (alpha_tile) load_tile<T, N, BC, true>(alpha + b0, B, nb, buf, LD, BC);
+    cp_async_wait_all();
     __syncthreads();
     tile_ffts<T, N, -1>(nb, tw, twq, [&](int p, int j) { return buf + tpad(j, LD, p); }, [](int) { return true; });
   }
@@ -992,7 +1012,7 @@ __device__ __forceinline__ void spectral_body(const cpx<T>* __restrict__ T1, cpx
       const T Phi = sk.filtered ? t_exp(filt * q2) : T(1);
       const size_t gi = (size_t)j * B + m;
       if (MODE == kModeStep || MODE == kModeGradOnly) {
-        const cpx<T> a = alpha[gi];
+        const cpx<T> a = alpha_tile ? buf[tpad(j, LD, BC + c)] : alpha[gi];
         if (MODE == kModeStep) {
           cpx<T> beta = buf[tpad(j, LD, c)];
           beta.x *= inv_L3;
@@ -1068,11 +1088,6 @@ template <int N> struct XRegShape {
 template <int N> constexpr size_t xreg_smem_bytes(int nw) {
   return ((size_t)N + (size_t)nw * XRegShape<N>::WARP) * sizeof(cpx<float>);
 }
-
-__device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_addr(smem)), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 template <int N, int MODE>
 __device__ __forceinline__ void spectral_reg_task(const cpx<float>* __restrict__ T1, cpx<float>* __restrict__ alpha,
@@ -1363,7 +1378,8 @@ __global__ void __launch_bounds__(256) kwb_cols(const FftRun<T>* __restrict__ ru
   const FftRun<T>& r = runs[run];
   const size_t S = (size_t)N * N * NHH;
   cpx<T>* data = DIR < 0 ? r.T1 : r.T2 + comp * S;
-  cols_body<T, E, DIR, BC>(data + (size_t)blockIdx.y * N * NHH, NHH, T(1), blockIdx.x * BC, tw, tw + tw_len<T, E>());
+  cols_body<T, E, DIR, BC, true>(data + (size_t)blockIdx.y * N * NHH, NHH, T(1), blockIdx.x * BC, tw,
+                                 tw + tw_len<T, E>());
 }
 
 // Inverse y pass of the two spectra the x pass handed on, G_x (T2 component 0)
@@ -1372,7 +1388,7 @@ __global__ void __launch_bounds__(256) kwb_cols(const FftRun<T>* __restrict__ ru
 // i y_z (constant along the column) are G_z (back to component 2, read by
 // then).  One block does all three, so Phi alpha's tile is read from DRAM once.
 template <typename T, int E, int BC>
-__global__ void __launch_bounds__(256) kwb_cols_inv3(const FftRun<T>* __restrict__ runs) {
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1) kwb_cols_inv3(const FftRun<T>* __restrict__ runs) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
   load_tw_group<T, E, false>(tw);
@@ -1389,16 +1405,16 @@ __global__ void __launch_bounds__(256) kwb_cols_inv3(const FftRun<T>* __restrict
   for (int d = 0; d < 3; ++d) {
     const cpx<T>* src = d == 0 ? gx : ga;
     cpx<T>* dst = d == 0 ? gx : d == 1 ? gy : ga;
-    for (int t = threadIdx.x; t < N * BC; t += blockDim.x) {
-      const int j = t / BC, c = t - j * BC;
-      cpx<T> v = c < nb ? src[(size_t)j * B + c] : cpx<T>{T(0), T(0)};
-      if (d == 1) {
+    load_tile<T, N, BC, true>(src, B, nb, buf, LD, 0);
+    cp_async_wait_all();
+    if (d == 1)
+      for (int t = threadIdx.x; t < N * BC; t += blockDim.x) {   // the elements this thread loaded
+        const int j = t / BC, c = t - j * BC;
         const int qy = j < N / 2 ? j : j - N;
         const T cy = qy != -N / 2 ? two_pi_L * (T)qy : T(0);
-        v = cpx<T>{-cy * v.y, cy * v.x};
+        const cpx<T> v = buf[tpad(j, LD, c)];
+        buf[tpad(j, LD, c)] = cpx<T>{-cy * v.y, cy * v.x};
       }
-      buf[tpad(j, LD, c)] = v;
-    }
     __syncthreads();
     tile_ffts<T, N, +1>(nb, tw, tw + kTwLen, [&](int p, int j) { return buf + tpad(j, LD, p); },
                         [](int) { return true; });
@@ -1442,6 +1458,64 @@ __global__ void __launch_bounds__(256) kwb_rows_c2r(const FftRun<T>* __restrict_
   const FftRun<T>& r = runs[blockIdx.y];
   const size_t S = (size_t)N * N * (N / 2 + 1);
   rows_c2r_body<T, E, 3>(r.T2, S, r.grad, N * N, nullptr, blockIdx.x, gridDim.x, tw, zb_all, ob_all);
+}
+
+// Rows r2c by group FFTs, one row pair per group of lanes and no loop, so that
+// a warp's 32 row loads are all in flight and the next blocks' loads follow as
+// soon as registers are free (the persistent pass over row pairs left the
+// memory idle between a warp's pairs: 76 -> 71 us at H = 256).
+template <int N, typename Tin>
+__device__ __forceinline__ void rows_r2c_pair(Tin* __restrict__ in, double in_scale, cpx<float>* __restrict__ out, int pr,
+                                              int q, const cpx<float>* twq, cpx<float>* z) {
+  using T = float;
+  constexpr int F = GroupShape<N>::F, Q = GroupShape<N>::Q, R = F / Q, NH = N / 2 + 1;
+  constexpr int KI = (NH + Q - 1) / Q;
+  Tin* ra = in + (size_t)(2 * pr) * N + q;
+  cpx<T> v[F];
+#pragma unroll
+  for (int m = 0; m < F; ++m) {
+    if constexpr (sizeof(Tin) == 8)
+      v[m] = cpx<T>{(T)((double)(long long)ra[Q * m] * in_scale), (T)((double)(long long)ra[N + Q * m] * in_scale)};
+    else
+      v[m] = cpx<T>{(T)ra[Q * m], (T)ra[N + Q * m]};
+  }
+#pragma unroll
+  for (int m = 0; m < F; ++m) {
+    ra[Q * m] = Tin(0);
+    ra[N + Q * m] = Tin(0);
+  }
+  group_fft<T, N, -1>(v, q, twq, 0xffffffffu, [z](int j) { return z + j; });
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+#pragma unroll
+    for (int k2 = 0; k2 < Q; ++k2) z[q + Q * r + F * k2] = v[r * Q + k2];
+  __syncwarp();
+  cpx<T>* oa = out + (size_t)(2 * pr) * NH;
+#pragma unroll
+  for (int i = 0; i < KI; ++i) {
+    const int k = q + Q * i;
+    if (k < NH) {
+      const cpx<T> zk = z[k], zm = cconj(z[(N - k) & (N - 1)]), d = csub(zk, zm);
+      oa[k] = cpx<T>{(zk.x + zm.x) * T(0.5), (zk.y + zm.y) * T(0.5)};
+      oa[NH + k] = cpx<T>{d.y * T(0.5), -d.x * T(0.5)};
+    }
+  }
+}
+template <int N>
+__global__ void __launch_bounds__(128) kwrb_rows_r2c(const FftRun<float>* __restrict__ runs) {
+  constexpr int Q = GroupShape<N>::Q, G = 32 / Q;
+  __shared__ cpx<float> twq[N];
+  __shared__ cpx<float> slots[4 * G * group_ps<N>()];
+  load_twq<float, N>(twq);
+  __syncthreads();
+  const FftRun<float>& r = runs[blockIdx.y];
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, g = lane / Q;
+  cpx<float>* z = slots + (wib * G + g) * group_ps<N>();
+  const int pr = (blockIdx.x * 4 + wib) * G + g;
+  if (r.phi_fixed)
+    rows_r2c_pair<N, unsigned long long>((unsigned long long*)r.phi, r.in_scale, r.T1, pr, lane & (Q - 1), twq, z);
+  else
+    rows_r2c_pair<N, float>((float*)r.phi, 1.0, r.T1, pr, lane & (Q - 1), twq, z);
 }
 
 // Rows c2r of the three gradient components by group FFTs with whole nodes
@@ -2491,8 +2565,11 @@ static cudaError_t field_batch_e(const FftRun<T>* runs, int nruns, int stages, c
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
       nk += 1;
     } else {
-      launch_plain(kwb_rows_r2c<T, E>, dim3(rblocks, nruns), 256, 0, s, runs);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      if constexpr (group_rows<T, N>())
+        e = launch_plain(kwrb_rows_r2c<N>, dim3(N * N / 2 / (4 * (32 / GroupShape<N>::Q)), nruns), 128, 0, s, runs);
+      else
+        e = launch_plain(kwb_rows_r2c<T, E>, dim3(rblocks, nruns), 256, 0, s, runs);
+      if (e != cudaSuccess) return e;
       if ((e = kwb_cols_bc<T, E, -1>(runs, nruns, 1, bc, s)) != cudaSuccess) return e;
       nk += 2;
     }
