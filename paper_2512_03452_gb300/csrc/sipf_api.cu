@@ -1104,25 +1104,56 @@ int sipf_gather_dev(int precision, const void* x, const void* y, const void* z, 
   return SIPF_OK;
 }
 
+// The transforms' kernels take complex values as one 8- or 16-byte access; a
+// caller's spectrum at a lesser alignment goes through an aligned copy.
+}  // extern "C"
+
+namespace {
+template <typename Fn>
+int with_aligned_spec(void* spec, int precision, int32_t H, bool in, bool out, cudaStream_t s, Fn&& fn) {
+  const size_t esz = precision == 64 ? 16 : 8;
+  if ((reinterpret_cast<uintptr_t>(spec) & (esz - 1)) == 0) return fn(spec);
+  const size_t bytes = (size_t)H * H * (H / 2 + 1) * esz;
+  void* tmp = nullptr;
+  SIPF_CK(cudaMallocAsync(&tmp, bytes, s));
+  int r = SIPF_OK;
+  cudaError_t e = in ? cudaMemcpyAsync(tmp, spec, bytes, cudaMemcpyDeviceToDevice, s) : cudaSuccess;
+  if (e == cudaSuccess) r = fn(tmp);
+  if (e == cudaSuccess && !r && out) e = cudaMemcpyAsync(spec, tmp, bytes, cudaMemcpyDeviceToDevice, s);
+  const cudaError_t ef = cudaFreeAsync(tmp, s);
+  if (r) return r;
+  if (e == cudaSuccess) e = ef;
+  return e == cudaSuccess ? SIPF_OK : cuda_fail(e, "aligned copy of the spectrum");
+}
+
+template <typename T> int forward_ft(int32_t H, double L, const void* grid, void* spec, cudaStream_t s) {
+  const int nh = H / 2 + 1;
+  cpx<T>* o = (cpx<T>*)spec;
+  SIPF_CK(launch_rows_r2c<T>(grid, 0, 1.0, false, o, H, H * H, nullptr, s));
+  SIPF_CK(launch_cols<T>(o, H, H, nh, 1, 0, -1, 1.0, s));
+  SIPF_CK(launch_cols<T>(o, H, 1, H * nh, 1, 0, -1, 1.0 / (L * L * L), s));
+  return SIPF_OK;
+}
+template <typename T> int inverse_ft(int32_t H, void* spec, void* grid, cudaStream_t s) {
+  const int nh = H / 2 + 1;
+  cpx<T>* o = (cpx<T>*)spec;
+  SIPF_CK(launch_cols<T>(o, H, 1, H * nh, 1, 0, +1, 1.0, s));
+  SIPF_CK(launch_cols<T>(o, H, H, nh, 1, 0, +1, 1.0, s));
+  SIPF_CK(launch_rows_c2r<T>(o, 1, 0, (T*)grid, H, H * H, nullptr, s));
+  return SIPF_OK;
+}
+}  // namespace
+
+extern "C" {
+
 int sipf_forward_ft_dev(int precision, int32_t H, double L, const void* grid, void* spec, void* stream) {
   if (precision != 32 && precision != 64) return fail(SIPF_EINVAL, "precision");
   if (!is_pow2(H) || H < 8 || H > kNmax || !(L > 0) || !grid || !spec) return fail(SIPF_EINVAL, "forward_ft args");
   SIPF_CK(ensure_device_tables());
   cudaStream_t s = (cudaStream_t)stream;
-  const int nh = H / 2 + 1;
-  const double sc = 1.0 / (L * L * L);
-  if (precision == 64) {
-    cpx<double>* o = (cpx<double>*)spec;
-    SIPF_CK(launch_rows_r2c<double>(grid, 0, 1.0, false, o, H, H * H, nullptr, s));
-    SIPF_CK(launch_cols<double>(o, H, H, nh, 1, 0, -1, 1.0, s));
-    SIPF_CK(launch_cols<double>(o, H, 1, H * nh, 1, 0, -1, sc, s));
-  } else {
-    cpx<float>* o = (cpx<float>*)spec;
-    SIPF_CK(launch_rows_r2c<float>(grid, 0, 1.0, false, o, H, H * H, nullptr, s));
-    SIPF_CK(launch_cols<float>(o, H, H, nh, 1, 0, -1, 1.0, s));
-    SIPF_CK(launch_cols<float>(o, H, 1, H * nh, 1, 0, -1, sc, s));
-  }
-  return SIPF_OK;
+  return with_aligned_spec(spec, precision, H, false, true, s, [&](void* o) {
+    return precision == 64 ? forward_ft<double>(H, L, grid, o, s) : forward_ft<float>(H, L, grid, o, s);
+  });
 }
 
 int sipf_inverse_ft_dev(int precision, int32_t H, void* spec, void* grid, void* stream) {
@@ -1130,19 +1161,9 @@ int sipf_inverse_ft_dev(int precision, int32_t H, void* spec, void* grid, void* 
   if (!is_pow2(H) || H < 8 || H > kNmax || !grid || !spec) return fail(SIPF_EINVAL, "inverse_ft args");
   SIPF_CK(ensure_device_tables());
   cudaStream_t s = (cudaStream_t)stream;
-  const int nh = H / 2 + 1;
-  if (precision == 64) {
-    cpx<double>* o = (cpx<double>*)spec;
-    SIPF_CK(launch_cols<double>(o, H, 1, H * nh, 1, 0, +1, 1.0, s));
-    SIPF_CK(launch_cols<double>(o, H, H, nh, 1, 0, +1, 1.0, s));
-    SIPF_CK(launch_rows_c2r<double>(o, 1, 0, (double*)grid, H, H * H, nullptr, s));
-  } else {
-    cpx<float>* o = (cpx<float>*)spec;
-    SIPF_CK(launch_cols<float>(o, H, 1, H * nh, 1, 0, +1, 1.0, s));
-    SIPF_CK(launch_cols<float>(o, H, H, nh, 1, 0, +1, 1.0, s));
-    SIPF_CK(launch_rows_c2r<float>(o, 1, 0, (float*)grid, H, H * H, nullptr, s));
-  }
-  return SIPF_OK;
+  return with_aligned_spec(spec, precision, H, true, true, s, [&](void* o) {
+    return precision == 64 ? inverse_ft<double>(H, o, grid, s) : inverse_ft<float>(H, o, grid, s);
+  });
 }
 
 }  // extern "C"
@@ -1195,18 +1216,7 @@ extern "C" int sipf_inverse_ft_noalloc_dev(int precision, int32_t H, const void*
   if (r) return r;
   cudaStream_t s = (cudaStream_t)stream;
   SIPF_CK(cudaMemcpyAsync(work, spec, bytes, cudaMemcpyDeviceToDevice, s));
-  if (precision == 64) {
-    cpx<double>* o = (cpx<double>*)work;
-    SIPF_CK(launch_cols<double>(o, H, 1, H * (int)nh, 1, 0, +1, 1.0, s));
-    SIPF_CK(launch_cols<double>(o, H, H, (int)nh, 1, 0, +1, 1.0, s));
-    SIPF_CK(launch_rows_c2r<double>(o, 1, 0, (double*)grid, H, H * H, nullptr, s));
-  } else {
-    cpx<float>* o = (cpx<float>*)work;
-    SIPF_CK(launch_cols<float>(o, H, 1, H * (int)nh, 1, 0, +1, 1.0, s));
-    SIPF_CK(launch_cols<float>(o, H, H, (int)nh, 1, 0, +1, 1.0, s));
-    SIPF_CK(launch_rows_c2r<float>(o, 1, 0, (float*)grid, H, H * H, nullptr, s));
-  }
-  return SIPF_OK;
+  return precision == 64 ? inverse_ft<double>(H, work, grid, s) : inverse_ft<float>(H, work, grid, s);
 }
 
 // ===========================================================================

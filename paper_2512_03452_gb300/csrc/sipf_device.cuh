@@ -9,7 +9,9 @@
 
 namespace sipf {
 
-template <typename T> struct cpx { T x, y; };
+// Aligned to its size, so that a value is one 8- or 16-byte access (without the
+// alignment every load and store of a complex value is two).
+template <typename T> struct alignas(2 * sizeof(T)) cpx { T x, y; };
 
 // Programmatic dependent launch (see launch_k): in a grid of at most
 // kPdlBlocks blocks, waits until the kernel before this one has completed and
