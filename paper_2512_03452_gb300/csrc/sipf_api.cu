@@ -411,7 +411,7 @@ template <typename T> int step_impl(sipf_ctx* c, int64_t nsteps) {
     SIPF_CK(mark(&ev[5]));
     SIPF_CK(launch_chunk_list(cl_args(c, c->cursor[dst], c->lcap[c->lc], c->lbase[c->lc], c->cursor[src]), c->work,
                               c->timing ? c->ovf : nullptr, c->stream));
-    c->launches += (fr ? fk : 5) + 3;
+    c->launches += (fr ? fk : 5) + 1 + chunk_list_launches(c->NT);
     c->cur = dst;
     c->n += 1;
     if (++c->since_layout >= c->resort()) {
@@ -422,7 +422,7 @@ template <typename T> int step_impl(sipf_ctx* c, int64_t nsteps) {
       SIPF_CK(launch_binned_rebin<T>(bin_args<T>(c, c->cur, c->lc, d2, L), c->stream));
       SIPF_CK(launch_chunk_list(cl_args(c, c->cursor[d2], c->lcap[L], c->lbase[L], c->cursor[c->cur]), c->work, nullptr,
                                 c->stream));
-      c->launches += 4;
+      c->launches += 2 + chunk_list_launches(c->NT);
       c->cur = d2;
       c->lc = L;
       c->since_layout = 0;
@@ -641,7 +641,7 @@ template <typename T> int upload_soa_impl(sipf_ctx* c, const void* const src[3])
   }
   SIPF_CK(launch_chunk_list(cl_args(c, c->cursor[b], c->lcap[c->lc], c->lbase[c->lc], c->cursor[1 - b]), c->work,
                             nullptr, c->stream));
-  c->launches += 2;
+  c->launches += chunk_list_launches(c->NT);
   SIPF_CK(mark_positions(c));
   c->dep_pending = true;
   return SIPF_OK;

@@ -289,10 +289,11 @@ template <typename T> cudaError_t launch_move(const BinArgs<T>& a, cudaStream_t 
 // From fill cursors: clamped counts, chunk prefix sums and chunk descriptors
 // (slots from `base`); clears other_cursor and the work counter.  ovf_total
 // (nullable) accumulates the number of particles in the overflow bin.
-// Chunk list of one buffer: two launches (count, emit); clears work[0] and
+// Chunk list of one buffer: one launch, or two (count, emit) above 1023 tiles; clears work[0] and
 // work[1] (a context's deposit / re-bin and move counters) and adds the
 // overflow-bin count to *ovf_total when those are non-NULL.
 int chunk_list_blocks(int NT);
+inline int chunk_list_launches(int NT) { return chunk_list_blocks(NT) == 1 ? 1 : 2; }
 cudaError_t launch_chunk_list(const ChunkListArgs& a, unsigned long long* work, unsigned long long* ovf_total,
                               cudaStream_t s);
 cudaError_t launch_layout(const int* want, int* cap, long long* base, int NT, int ntx, int ovf_cap, cudaStream_t s);
