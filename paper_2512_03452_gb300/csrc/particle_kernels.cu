@@ -1255,43 +1255,36 @@ k_run_prefix(const ChunkListArgs* __restrict__ t, int nruns, long long* __restri
 // Capacities from the wanted counts (tile histogram) and their prefix sum.
 // Spare room: half the tile's own count, 64, and a quarter of what its six
 // face neighbours hold (particles diffuse in across steep density edges).
-// The overflow bin keeps capacity ovf_cap.  One block.
+// The overflow bin keeps capacity ovf_cap.  One block, 1024 consecutive bins at
+// a time (a contiguous range of bins for each thread read every neighbour
+// count with a stride: 183 -> 58 us for the 32768 bins of H = 256).
 __device__ __forceinline__ void layout_body(const int* __restrict__ want, int* __restrict__ cap,
                                             long long* __restrict__ base, int NT, int ntx, int ovf_cap) {
-  __shared__ long long s_part[1024];
-  const int per = (NT + blockDim.x - 1) / blockDim.x;
-  const int b0 = threadIdx.x * per;
-  long long local = 0;
-  for (int b = b0; b < min(b0 + per, NT); ++b) {
-    const int w = want[b];
-    const int tz = b % ntx, ty = (b / ntx) % ntx, tx = b / (ntx * ntx);
-    long long nsum = 0;
-    for (int d = -1; d <= 1; d += 2) {
-      nsum += want[((((tx + d + ntx) % ntx) * ntx) + ty) * ntx + tz];
-      nsum += want[((tx * ntx) + (ty + d + ntx) % ntx) * ntx + tz];
-      nsum += want[((tx * ntx) + ty) * ntx + (tz + d + ntx) % ntx];
+  long long first = 0;   // first slot of this group of bins
+  for (int b0 = 0; b0 < NT; b0 += blockDim.x) {
+    const int b = b0 + threadIdx.x;
+    long long c = 0;
+    if (b < NT) {
+      const int w = want[b];
+      const int tz = b % ntx, ty = (b / ntx) % ntx, tx = b / (ntx * ntx);
+      long long nsum = 0;
+      for (int d = -1; d <= 1; d += 2) {
+        nsum += want[((((tx + d + ntx) % ntx) * ntx) + ty) * ntx + tz];
+        nsum += want[((tx * ntx) + (ty + d + ntx) % ntx) * ntx + tz];
+        nsum += want[((tx * ntx) + ty) * ntx + (tz + d + ntx) % ntx];
+      }
+      long long cl = (long long)w + w / 2 + 64 + nsum / 4;
+      cl = cl < 0x7ffffff0LL ? cl : 0x7ffffff0LL;
+      c = (cl + 3) & ~3LL;   // 4-slot multiples keep every bin 16-byte aligned
+      cap[b] = (int)c;
     }
-    long long cl = (long long)w + w / 2 + 64 + nsum / 4;
-    cl = cl < 0x7ffffff0LL ? cl : 0x7ffffff0LL;
-    const int c = (int)((cl + 3) & ~3LL);   // 4-slot multiples keep every bin 16-byte aligned
-    cap[b] = c;
-    local += c;
+    long long total;
+    const long long ex = block_exclusive_scan_ll(c, total);
+    if (b < NT) base[b] = first + ex;
+    first += total;
   }
-  s_part[threadIdx.x] = local;
-  __syncthreads();
-  for (int off = 1; off < (int)blockDim.x; off <<= 1) {
-    const long long v = threadIdx.x >= (unsigned)off ? s_part[threadIdx.x - off] : 0;
-    __syncthreads();
-    s_part[threadIdx.x] += v;
-    __syncthreads();
-  }
-  long long run = s_part[threadIdx.x] - local;
-  for (int b = b0; b < min(b0 + per, NT); ++b) {
-    base[b] = run;
-    run += cap[b];
-  }
-  if (threadIdx.x == blockDim.x - 1) {
-    base[NT] = s_part[threadIdx.x];
+  if (threadIdx.x == 0) {
+    base[NT] = first;
     cap[NT] = (ovf_cap + 3) & ~3;
   }
 }
