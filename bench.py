@@ -37,15 +37,15 @@ P_FULL, H_FULL = 10_000_000, 128
 # algorithmic bytes of the particle kernel per particle-step (FP32): read X (12 B) + write X (12 B)
 BYTES_PER_PARTICLE = 24
 # DRAM traffic (read + write bytes) of the particle phase, move + re-bin
-# (299.6 MB) and deposit (133.6 MB) launches of one step, from ncu captures of
+# (296.4 MB) and deposit (133.4 MB) launches of one step, from ncu captures of
 # the torus workload, keyed by the SHA-256 of the kernel sources they were
 # taken on (a changed kernel reports null until it is captured again).
-MOVE_TRAFFIC = {"4dcf580b08ec301d09cbd40561b51f6355c651130cf8c66b76a9069438413064": 433.24e6}
+MOVE_TRAFFIC = {"ed31ca7102d5f72a4ffc3dc8845c3e64d574a29b3ac6455fcf4ba6195c8a3260": 429.84e6}
 FALLBACK_HBM_GBS = 6800.0
-# Warp-instructions of one move + re-bin launch (136.76 M) and one deposit
-# launch (114.26 M) at P = 1e7, H = 128, FP32, from the same ncu captures,
+# Warp-instructions of one move + re-bin launch (137.21 M) and one deposit
+# launch (96.04 M) at P = 1e7, H = 128, FP32, from the same ncu captures,
 # keyed like the traffic: the particle kernels against the SMs' issue rate.
-PARTICLE_WARP_INSTR = {"4dcf580b08ec301d09cbd40561b51f6355c651130cf8c66b76a9069438413064": 251.03e6}
+PARTICLE_WARP_INSTR = {"ed31ca7102d5f72a4ffc3dc8845c3e64d574a29b3ac6455fcf4ba6195c8a3260": 233.26e6}
 # FP64 form: FP64-pipe thread instructions (DFMA + DADD + DMUL) of one FP64 step
 # at P = 1e7, H = 128 (move 2.580e9, deposit 0.823e9, forward plane 0.112e9,
 # x pass 0.279e9, inverse plane 0.334e9), from an ncu capture of the bench's
@@ -479,7 +479,7 @@ def run_ours(args, world, rank, local):
                        "mu": w.mu, "eps": w.eps, "k": w.k, "tau": w.dt, "precision": "fp32",
                        "l2": "inputs larger than L2 (per step 2 x 16 B x 1e7 particle traffic + 76 MB of grids)",
                        "parallelism": f"replicas x{world}"},
-            "roofline": {"bound": "hbm", "kernel": "particle phase: k_move (move + re-bin) and k_binned (deposit)",
+            "roofline": {"bound": "hbm", "kernel": "particle phase: k_move (move + re-bin) and k_binned_deposit (deposit)",
                          "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                          "traffic": traffic, "peak_source": peak_kind, "bytes_per_particle": BYTES_PER_PARTICLE,
                          "kernel_ms": part_ms, "overflow_per_step": tim.overflow / max(tim.steps, 1),

@@ -2648,7 +2648,7 @@ template <typename T> FieldTune field_tune_default(int H) {
   t.rows_per_sm = 8;
   t.plane_mode = 0;
   t.plane_nw = kDefaultPlaneWarps;
-  t.spec_nw = kDefaultSpectralWarps;
+  t.spec_nw = 0;   // by the number of pencils
   switch (H) {
     case 32: t.sbc = default_sbc<T, 1>(); break;
     case 64: t.sbc = default_sbc<T, 2>(); break;
