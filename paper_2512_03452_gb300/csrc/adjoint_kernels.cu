@@ -119,11 +119,11 @@ __device__ __forceinline__ void stencil_grad_visit(int order, T px, T py, T pz, 
 // w (H/L) sum_gamma grad_lambda F_gamma(lambda(X)) phibar[q_gamma]: the
 // transpose of X -> I rho-hat(X) applied to the grid cotangent phibar.
 template <typename T>
-__device__ __forceinline__ A3<T> deposit_adjoint(const T* __restrict__ phibar, int order, T px, T py, T pz, T w_inv_h,
+__device__ __forceinline__ A3<T> deposit_adjoint(const T* phibar, int order, T px, T py, T pz, T w_inv_h,
                                                  const Geo<T>& g) {
   A3<T> s{T(0), T(0), T(0)};
   stencil_grad_visit<T>(order, px, py, pz, g, [&](int idx, T, T fx, T fy, T fz) {
-    const T f = __ldg(phibar + idx);
+    const T f = phibar[idx];
     s.x += fx * f;
     s.y += fy * f;
     s.z += fz * f;
@@ -139,16 +139,16 @@ __device__ __forceinline__ A3<T> deposit_adjoint(const T* __restrict__ phibar, i
 template <typename T> struct Quad { T v[4]; };
 template <typename T> __device__ __forceinline__ Quad<T> load_quad(const T* p);
 template <> __device__ __forceinline__ Quad<float> load_quad<float>(const float* p) {
-  const float4 v = __ldg(reinterpret_cast<const float4*>(p));
+  const float4 v = *reinterpret_cast<const float4*>(p);
   return {{v.x, v.y, v.z, v.w}};
 }
 template <> __device__ __forceinline__ Quad<double> load_quad<double>(const double* p) {
-  const double2 a = __ldg(reinterpret_cast<const double2*>(p)), b = __ldg(reinterpret_cast<const double2*>(p) + 1);
+  const double2 a = *reinterpret_cast<const double2*>(p), b = reinterpret_cast<const double2*>(p)[1];
   return {{a.x, a.y, b.x, b.y}};
 }
 
 template <typename T>
-__device__ __forceinline__ A3<T> deposit_adjoint4_quads(const T* __restrict__ quads, T px, T py, T pz, T w_inv_h,
+__device__ __forceinline__ A3<T> deposit_adjoint4_quads(const T* quads, T px, T py, T pz, T w_inv_h,
                                                         const Geo<T>& g) {
   int cx, cy, cz;
   T lx, ly, lz;
@@ -212,7 +212,7 @@ __device__ __forceinline__ A3<T> deposit_adjoint4_quads(const T* __restrict__ qu
 
 // phibar (H^3) -> its z-quads (4 H^3): quad n = phibar at z - 1, z, z + 1, z + 2 (periodic).
 template <typename T>
-__global__ void __launch_bounds__(256) k_adj_quads(const T* __restrict__ phibar, T* __restrict__ quads, int H,
+__global__ void __launch_bounds__(256) k_adj_quads(const T* phibar, T* __restrict__ quads, int H,
                                                    int64_t H3) {
   pdl_wait();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < H3; i += (int64_t)gridDim.x * blockDim.x) {
@@ -239,18 +239,18 @@ template <> __device__ __forceinline__ void red_node3<double>(double* node, doub
   atomicAdd(node + 2, c);
 }
 
-// One (x, y, z, -) node of the gradient grids, read through the read-only path.
+// One (x, y, z, -) node of the gradient grids.
 template <typename T> struct Node4;
 template <> struct Node4<float> {
   static __device__ __forceinline__ A3<float> load(const float* p) {
-    const float4 v = __ldg(reinterpret_cast<const float4*>(p));
+    const float4 v = *reinterpret_cast<const float4*>(p);
     return {v.x, v.y, v.z};
   }
 };
 template <> struct Node4<double> {
   static __device__ __forceinline__ A3<double> load(const double* p) {
-    const double2 v = __ldg(reinterpret_cast<const double2*>(p));
-    return {v.x, v.y, __ldg(p + 2)};
+    const double2 v = *reinterpret_cast<const double2*>(p);
+    return {v.x, v.y, p[2]};
   }
 };
 
@@ -392,8 +392,8 @@ __global__ void __launch_bounds__(256) k_adj_planes(T* __restrict__ gbar4, T* __
 // order) applied to phibar^N.
 template <typename T>
 __global__ void __launch_bounds__(256)
-k_adj_terminal(const T* __restrict__ x, const T* __restrict__ y, const T* __restrict__ z, int64_t P,
-               const T* __restrict__ phibar, int p2g, T w_inv_h, Geo<T> g, T* __restrict__ xb4) {
+k_adj_terminal(const T* x, const T* y, const T* z, int64_t P,
+               const T* phibar, int p2g, T w_inv_h, Geo<T> g, T* __restrict__ xb4) {
   pdl_wait();
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += (int64_t)gridDim.x * blockDim.x) {
     const A3<T> dp = deposit_adjoint<T>(phibar, p2g, x[p], y[p], z[p], w_inv_h, g);
@@ -407,7 +407,7 @@ k_adj_terminal(const T* __restrict__ x, const T* __restrict__ y, const T* __rest
 //   that gives the transpose of F_H).
 template <typename T>
 __global__ void __launch_bounds__(256)
-k_adj_spectral(const cpx<T>* __restrict__ ghat, cpx<T>* __restrict__ abar, cpx<T>* __restrict__ spec, int H,
+k_adj_spectral(const cpx<T>* ghat, cpx<T>* __restrict__ abar, cpx<T>* __restrict__ spec, int H,
                SpecConst<T> sk) {
   pdl_wait();
   const int nh = H / 2 + 1;

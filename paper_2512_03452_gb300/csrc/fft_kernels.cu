@@ -206,7 +206,7 @@ k_cols(cpx<T>* __restrict__ data, int lgH, int B, int lgBC, size_t comp_stride, 
 // ---------------------------------------------------------------------------
 template <typename T, int MODE>
 __global__ void __launch_bounds__(kThreads)
-k_spectral_x(const cpx<T>* __restrict__ T1, cpx<T>* __restrict__ alpha, cpx<T>* __restrict__ T2,
+k_spectral_x(const cpx<T>* T1, cpx<T>* __restrict__ alpha, cpx<T>* __restrict__ T2,
              int lgH, int lgBC, SpecConst<T> sk, double* alpha0_shadow) {
   pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -304,7 +304,7 @@ k_spectral_x(const cpx<T>* __restrict__ T1, cpx<T>* __restrict__ alpha, cpx<T>* 
 // ---------------------------------------------------------------------------
 template <typename T, int NCOMP>
 __global__ void __launch_bounds__(kThreads)
-k_rows_c2r(const cpx<T>* __restrict__ in, size_t comp_stride, T* __restrict__ out, int lgH, int rows,
+k_rows_c2r(const cpx<T>* in, size_t comp_stride, T* __restrict__ out, int lgH, int rows,
            int RP, double* max_acc) {
   pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -921,7 +921,7 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // own arrays, 8-byte aligned): all of them in flight at once as asynchronous
 // copies; the caller's wait is included, a block barrier is not.
 template <typename T, int N, int BC, bool ASYNC>
-__device__ __forceinline__ void load_tile(const cpx<T>* __restrict__ src, int B, int nb, cpx<T>* buf, int LD, int col) {
+__device__ __forceinline__ void load_tile(const cpx<T>* src, int B, int nb, cpx<T>* buf, int LD, int col) {
   for (int t = threadIdx.x; t < N * BC; t += blockDim.x) {
     const int j = t / BC, c = t - j * BC;
     if constexpr (ASYNC && sizeof(T) == 4) {
@@ -978,7 +978,7 @@ template <int E> constexpr bool two_spectra() { return E == 8; }
 // transforms a pencil, and a third less to write here and to read there (x pass
 // 170 -> 123 us, inverse y pass 125 -> 112).
 template <typename T, int E, int MODE, int BC, bool TWO = false>
-__device__ __forceinline__ void spectral_body(const cpx<T>* __restrict__ T1, cpx<T>* __restrict__ alpha,
+__device__ __forceinline__ void spectral_body(const cpx<T>* T1, cpx<T>* __restrict__ alpha,
                                               cpx<T>* __restrict__ T2, const SpecConst<T>& sk,
                                               double* alpha0_shadow,
                                               int b0, const cpx<T>* tw, const cpx<T>* twq, cpx<T>* buf) {
@@ -1090,7 +1090,7 @@ template <int N> constexpr size_t xreg_smem_bytes(int nw) {
 }
 
 template <int N, int MODE>
-__device__ __forceinline__ void spectral_reg_task(const cpx<float>* __restrict__ T1, cpx<float>* __restrict__ alpha,
+__device__ __forceinline__ void spectral_reg_task(const cpx<float>* T1, cpx<float>* __restrict__ alpha,
                                                   cpx<float>* __restrict__ T2, const SpecConst<float>& sk,
                                                   double* alpha0_shadow, int m0, const cpx<float>* twq,
                                                   cpx<float>* wslot) {
@@ -1185,7 +1185,7 @@ __device__ __forceinline__ void spectral_reg_task(const cpx<float>* __restrict__
 
 template <int N, int MODE>
 __global__ void __launch_bounds__(256)
-kwr_spectral_x(const cpx<float>* __restrict__ T1, cpx<float>* __restrict__ alpha, cpx<float>* __restrict__ T2,
+kwr_spectral_x(const cpx<float>* T1, cpx<float>* __restrict__ alpha, cpx<float>* __restrict__ T2,
                SpecConst<float> sk, double* alpha0_shadow) {
   pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1216,7 +1216,7 @@ __global__ void __launch_bounds__(512) kwrb_spectral_x(const FftRun<float>* __re
 
 template <typename T, int E, int MODE, int BC>
 __global__ void __launch_bounds__(256)
-kw_spectral_x(const cpx<T>* __restrict__ T1, cpx<T>* __restrict__ alpha, cpx<T>* __restrict__ T2, SpecConst<T> sk,
+kw_spectral_x(const cpx<T>* T1, cpx<T>* __restrict__ alpha, cpx<T>* __restrict__ T2, SpecConst<T> sk,
               double* alpha0_shadow) {
   pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1231,7 +1231,7 @@ kw_spectral_x(const cpx<T>* __restrict__ T1, cpx<T>* __restrict__ alpha, cpx<T>*
 // full pencil Z = A + i B from the Hermitian halves, inverse-transforms it,
 // and writes (gx, gy, gz, 0) nodes (NCOMP == 3) or a plain grid (NCOMP == 1).
 template <typename T, int E, int NCOMP>
-__device__ __forceinline__ void rows_c2r_body(const cpx<T>* __restrict__ in, size_t comp_stride, T* __restrict__ out,
+__device__ __forceinline__ void rows_c2r_body(const cpx<T>* in, size_t comp_stride, T* __restrict__ out,
                                               int rows, double* max_acc, int bx, int gx, const cpx<T>* tw,
                                               cpx<T>* zb_all, T* ob_all) {
   constexpr int N = 32 * E, NH = N / 2 + 1;
@@ -1336,7 +1336,7 @@ __device__ __forceinline__ void rows_c2r_body(const cpx<T>* __restrict__ in, siz
 
 template <typename T, int E, int NCOMP>
 __global__ void __launch_bounds__(256)
-kw_rows_c2r(const cpx<T>* __restrict__ in, size_t comp_stride, T* __restrict__ out, int rows, double* max_acc) {
+kw_rows_c2r(const cpx<T>* in, size_t comp_stride, T* __restrict__ out, int rows, double* max_acc) {
   pdl_wait();
   constexpr int N = 32 * E;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1714,7 +1714,7 @@ __device__ __forceinline__ void plane_fwd_body(Tin* __restrict__ in, double in_s
 }
 
 template <typename T, int E>
-__device__ __forceinline__ void plane_inv_body(const cpx<T>* __restrict__ in, T* __restrict__ out, int x, int d,
+__device__ __forceinline__ void plane_inv_body(const cpx<T>* in, T* __restrict__ out, int x, int d,
                                                const cpx<T>* tw, cpx<T>* P, cpx<T>* zball) {
   constexpr int N = 32 * E, NH = N / 2 + 1;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -1835,7 +1835,7 @@ template <typename T> __device__ __forceinline__ void store_node4(T* p, T a, T b
 }
 
 template <typename T, int E>
-__device__ __forceinline__ void plane_inv3_body(const cpx<T>* __restrict__ in, size_t S, T* __restrict__ out, int x,
+__device__ __forceinline__ void plane_inv3_body(const cpx<T>* in, size_t S, T* __restrict__ out, int x,
                                                 const cpx<T>* tw, cpx<T>* P, cpx<T>* zball, T* oball) {
   constexpr int N = 32 * E, NH = N / 2 + 1;
   constexpr int PL = N * NH + E;             // one padded plane
@@ -2060,7 +2060,7 @@ __device__ __forceinline__ void cplane_fwd_body(Tin* __restrict__ in, double in_
 }
 
 template <typename T, int E, int CS>
-__device__ __forceinline__ void cplane_inv_body(const cpx<T>* __restrict__ in, T* __restrict__ out, int x, int d,
+__device__ __forceinline__ void cplane_inv_body(const cpx<T>* in, T* __restrict__ out, int x, int d,
                                                 T two_pi_L, const cpx<T>* tw, cpx<T>* Q, cpx<T>* zball) {
   // H = 256: G_y and G_z from Phi alpha, as in kwb_cols_inv3
   const bool from_y = two_spectra<E>() && d == 1, from_z = two_spectra<E>() && d == 2;

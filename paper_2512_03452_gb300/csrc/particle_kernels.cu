@@ -104,21 +104,21 @@ template <typename T> struct V3 { T x, y, z; };
 template <typename T> struct Vec4;
 template <> struct Vec4<float> {
   static __device__ __forceinline__ V3<float> load(const float* p) {
-    const float4 v = __ldg(reinterpret_cast<const float4*>(p));
+    const float4 v = *reinterpret_cast<const float4*>(p);
     return {v.x, v.y, v.z};
   }
 };
 template <> struct Vec4<double> {
   static __device__ __forceinline__ V3<double> load(const double* p) {
-    const double2 a = __ldg(reinterpret_cast<const double2*>(p));
-    const double b = __ldg(p + 2);
+    const double2 a = *reinterpret_cast<const double2*>(p);
+    const double b = p[2];
     return {a.x, a.y, b};
   }
 };
 
 // Gather of the three gradient components (interleaved 4-wide nodes).
 template <typename T>
-__device__ __forceinline__ V3<T> gather_grad(const T* __restrict__ grad4, int order, T px, T py, T pz,
+__device__ __forceinline__ V3<T> gather_grad(const T* grad4, int order, T px, T py, T pz,
                                              const Geo<T>& g) {
   int cx, cy, cz;
   T lx, ly, lz;
@@ -675,8 +675,8 @@ k_binned_rebin(const __grid_constant__ BinArgs<T> a) {
 // all runs from one list.
 template <typename T, bool FIXED>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2)
-k_deposit_batch(const BinArgs<T>* __restrict__ table, const BatchItem* __restrict__ list,
-                const long long* __restrict__ total, unsigned long long* work) {
+k_deposit_batch(const BinArgs<T>* __restrict__ table, const BatchItem* list,
+                const long long* total, unsigned long long* work) {
   using A = typename WinType<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   A* win = reinterpret_cast<A*>(smem_raw);
@@ -981,8 +981,8 @@ k_move(BinArgs<T> a) {
 // run r's arguments at table[r]; the step index from device memory.
 template <typename T, bool MOVE, int G2P>
 __global__ void __launch_bounds__(kMoveThreads, move_min_blocks<T>())
-k_move_batch(const BinArgs<T>* __restrict__ table, const BatchItem* __restrict__ list,
-             const long long* __restrict__ total, unsigned long long* work, const uint32_t* step) {
+k_move_batch(const BinArgs<T>* __restrict__ table, const BatchItem* list,
+             const long long* total, unsigned long long* work, const uint32_t* step) {
   pdl_wait();
   __shared__ MoveSmem<T> sm;
   const uint32_t n = *step + 1;
@@ -1205,7 +1205,7 @@ __global__ void __launch_bounds__(kCLBlock) k_chunk_count_batch(const ChunkListA
 }
 
 __global__ void __launch_bounds__(kCLBlock)
-k_chunk_emit_batch(const ChunkListArgs* __restrict__ t, const long long* __restrict__ prefix, BatchItem* list) {
+k_chunk_emit_batch(const ChunkListArgs* __restrict__ t, const long long* prefix, BatchItem* list) {
   pdl_wait();
   const ChunkListArgs a = t[blockIdx.y];
   const int nblk = chunk_list_blocks_dev(a.NT);
@@ -1258,7 +1258,7 @@ k_run_prefix(const ChunkListArgs* __restrict__ t, int nruns, long long* __restri
 // The overflow bin keeps capacity ovf_cap.  One block, 1024 consecutive bins at
 // a time (a contiguous range of bins for each thread read every neighbour
 // count with a stride: 183 -> 58 us for the 32768 bins of H = 256).
-__device__ __forceinline__ void layout_body(const int* __restrict__ want, int* __restrict__ cap,
+__device__ __forceinline__ void layout_body(const int* want, int* __restrict__ cap,
                                             long long* __restrict__ base, int NT, int ntx, int ovf_cap) {
   long long first = 0;   // first slot of this group of bins
   for (int b0 = 0; b0 < NT; b0 += blockDim.x) {
@@ -1290,7 +1290,7 @@ __device__ __forceinline__ void layout_body(const int* __restrict__ want, int* _
 }
 
 __global__ void __launch_bounds__(1024)
-k_layout(const int* __restrict__ want, int* __restrict__ cap, long long* __restrict__ base, int NT, int ntx,
+k_layout(const int* want, int* __restrict__ cap, long long* __restrict__ base, int NT, int ntx,
          int ovf_cap) {
   pdl_wait();
   layout_body(want, cap, base, NT, ntx, ovf_cap);
@@ -1308,7 +1308,7 @@ __global__ void __launch_bounds__(1024) k_layout_batch(const LayoutArgs* __restr
 // the global histogram once; otherwise warps aggregate equal tiles.
 template <typename T>
 __global__ void __launch_bounds__(256)
-k_tile_hist(const T* __restrict__ x, const T* __restrict__ y, const T* __restrict__ z, int64_t P, Geo<T> g,
+k_tile_hist(const T* x, const T* y, const T* z, int64_t P, Geo<T> g,
             int shift, int ntx, int NT, int* __restrict__ hist, int use_smem) {
   pdl_wait();
   extern __shared__ int s_cnt[];
@@ -1357,10 +1357,10 @@ k_tile_hist(const T* __restrict__ x, const T* __restrict__ y, const T* __restric
 // nothing else depends on the order inside a bin.
 template <typename T>
 __global__ void __launch_bounds__(256)
-k_rebin_plain(const T* __restrict__ x, const T* __restrict__ y, const T* __restrict__ z,
-              const uint32_t* __restrict__ id, int64_t P, Geo<T> g, int shift, int ntx, int NT,
+k_rebin_plain(const T* x, const T* y, const T* z,
+              const uint32_t* id, int64_t P, Geo<T> g, int shift, int ntx, int NT,
               T* __restrict__ dx, T* __restrict__ dy, T* __restrict__ dz, uint32_t* __restrict__ did,
-              const long long* __restrict__ dst_base, const int* __restrict__ dst_cap, int* __restrict__ dst_cursor,
+              const long long* dst_base, const int* dst_cap, int* __restrict__ dst_cursor,
               int* err, int64_t id0, int wrap) {
   pdl_wait();
   extern __shared__ int s_cnt[];
@@ -1419,8 +1419,8 @@ __global__ void __launch_bounds__(256) k_slot_map(BinArgs<T> a, uint32_t* __rest
 
 template <typename T>
 __global__ void __launch_bounds__(256)
-k_gather_slots(const uint32_t* __restrict__ slot_of, const T* __restrict__ bx, const T* __restrict__ by,
-               const T* __restrict__ bz, int64_t P, T* __restrict__ ox, T* __restrict__ oy, T* __restrict__ oz) {
+k_gather_slots(const uint32_t* slot_of, const T* bx, const T* by,
+               const T* bz, int64_t P, T* __restrict__ ox, T* __restrict__ oy, T* __restrict__ oz) {
   pdl_wait();
   // four ids per thread and iteration, their gathers issued together
   constexpr int U = 4;
@@ -1578,8 +1578,8 @@ k_partition_pieces(BinArgs<T> a, PieceBounds pb, int* __restrict__ cursor, T* __
 // while its partial sectors fill.
 template <typename T>
 __global__ void __launch_bounds__(256)
-k_scatter_piece(const T* __restrict__ rx, const T* __restrict__ ry, const T* __restrict__ rz,
-                const uint32_t* __restrict__ rid, int64_t a0, int64_t n, int64_t P, T* __restrict__ ox,
+k_scatter_piece(const T* rx, const T* ry, const T* rz,
+                const uint32_t* rid, int64_t a0, int64_t n, int64_t P, T* __restrict__ ox,
                 T* __restrict__ oy, T* __restrict__ oz) {
   pdl_wait();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -1595,7 +1595,7 @@ k_scatter_piece(const T* __restrict__ rx, const T* __restrict__ ry, const T* __r
 
 template <typename T>
 __global__ void __launch_bounds__(256)
-k_aos4_to_soa(const T* __restrict__ aos, int64_t P, T* __restrict__ ox, T* __restrict__ oy, T* __restrict__ oz) {
+k_aos4_to_soa(const T* aos, int64_t P, T* __restrict__ ox, T* __restrict__ oy, T* __restrict__ oz) {
   pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += stride) {
@@ -1618,7 +1618,7 @@ __global__ void __launch_bounds__(256) k_iota(uint32_t* id, int64_t P) {
 // ---------------------------------------------------------------------------
 template <typename T>
 __global__ void __launch_bounds__(256)
-k_deposit(const T* __restrict__ x, const T* __restrict__ y, const T* __restrict__ z, int64_t P, Geo<T> g, T w,
+k_deposit(const T* x, const T* y, const T* z, int64_t P, Geo<T> g, T w,
           T* __restrict__ phi, int order) {
   pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -1681,7 +1681,7 @@ __device__ __forceinline__ void deposit_columns(float* phi, int order, const int
 }
 
 __global__ void __launch_bounds__(256)
-k_deposit_vec(const float* __restrict__ x, const float* __restrict__ y, const float* __restrict__ z, int64_t P,
+k_deposit_vec(const float* x, const float* y, const float* z, int64_t P,
               Geo<float> g, float w, float* __restrict__ phi, int order) {
   pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -1706,8 +1706,8 @@ k_deposit_vec(const float* __restrict__ x, const float* __restrict__ y, const fl
 
 template <typename T>
 __global__ void __launch_bounds__(256)
-k_gather(const T* __restrict__ x, const T* __restrict__ y, const T* __restrict__ z, int64_t P, Geo<T> g,
-         const T* __restrict__ f, int ncomp, int order, T* __restrict__ out) {
+k_gather(const T* x, const T* y, const T* z, int64_t P, Geo<T> g,
+         const T* f, int ncomp, int order, T* __restrict__ out) {
   pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const size_t N = (size_t)g.H * g.H * g.H;
@@ -1732,8 +1732,8 @@ k_gather(const T* __restrict__ x, const T* __restrict__ y, const T* __restrict__
 // lookups, one a lane for particles in random order.  Same order of the sums as
 // k_gather: 60 -> 48 us for 1e6 unsorted particles, three grids of 128^3.
 __global__ void __launch_bounds__(256)
-k_gather2_vec(const float* __restrict__ x, const float* __restrict__ y, const float* __restrict__ z, int64_t P,
-              Geo<float> g, const float* __restrict__ f, int ncomp, float* __restrict__ out) {
+k_gather2_vec(const float* x, const float* y, const float* z, int64_t P,
+              Geo<float> g, const float* f, int ncomp, float* __restrict__ out) {
   pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const size_t N = (size_t)g.H * g.H * g.H;
@@ -1754,8 +1754,8 @@ k_gather2_vec(const float* __restrict__ x, const float* __restrict__ y, const fl
       float n[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        q[k] = __ldg(reinterpret_cast<const float4*>(fc + col[k] + (z0 & ~3)));
-        n[k] = o == 3 ? __ldg(fc + col[k] + z1) : 0.f;
+        q[k] = *reinterpret_cast<const float4*>(fc + col[k] + (z0 & ~3));
+        n[k] = o == 3 ? fc[col[k] + z1] : 0.f;
       }
       float acc = 0.f;
 #pragma unroll
@@ -1791,7 +1791,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 // acc2[0] += sum |X|^2, acc2[1] += sum sqrt(x^2 + y^2)  (FP64)
 template <typename T>
 __global__ void __launch_bounds__(256)
-k_moments(const T* __restrict__ x, const T* __restrict__ y, const T* __restrict__ z, int64_t P, double* acc2) {
+k_moments(const T* x, const T* y, const T* z, int64_t P, double* acc2) {
   pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   double s2 = 0.0, sr = 0.0;
@@ -1810,7 +1810,7 @@ k_moments(const T* __restrict__ x, const T* __restrict__ y, const T* __restrict_
 
 template <typename T>
 __global__ void __launch_bounds__(256)
-k_aos_to_soa(const double* __restrict__ aos, int64_t P, Geo<T> g, T* x, T* y, T* z) {
+k_aos_to_soa(const double* aos, int64_t P, Geo<T> g, T* x, T* y, T* z) {
   pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += stride) {
@@ -1834,7 +1834,7 @@ __global__ void __launch_bounds__(256) k_wrap_soa(int64_t P, Geo<T> g, T* x, T* 
 // acc2[0] += sum_q mult |alpha_q|^2 over ||q|| >= 4, acc2[1] += the full sum
 // (mult = 2 for 0 < kz < H/2 accounts for the Hermitian partner).
 template <typename T>
-__global__ void __launch_bounds__(256) k_alpha_energy(const cpx<T>* __restrict__ alpha, int H, double* acc2) {
+__global__ void __launch_bounds__(256) k_alpha_energy(const cpx<T>* alpha, int H, double* acc2) {
   pdl_wait();
   const int nh = H / 2 + 1;
   const int64_t n = (int64_t)H * H * nh;

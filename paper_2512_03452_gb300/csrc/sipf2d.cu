@@ -76,7 +76,7 @@ __device__ __forceinline__ void stencil2d(int order, int cx, int cy, T lx, T ly,
 
 template <typename T>
 __global__ void __launch_bounds__(kT2)
-k2_deposit(const T* __restrict__ x, const T* __restrict__ y, int64_t P, Geo<T> g, T w, int order,
+k2_deposit(const T* x, const T* y, int64_t P, Geo<T> g, T w, int order,
            T* __restrict__ phi) {
   pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -107,7 +107,7 @@ template <typename T> int win2_rows(int H) {
 
 template <typename T>
 __global__ void __launch_bounds__(kT2Win, 1)
-k2_deposit_win(const T* __restrict__ x, const T* __restrict__ y, int64_t P, Geo<T> g, T w, int order, int rows,
+k2_deposit_win(const T* x, const T* y, int64_t P, Geo<T> g, T w, int order, int rows,
                T* __restrict__ phi) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* win = reinterpret_cast<T*>(smem_raw);
@@ -148,7 +148,7 @@ struct Spec2D {
 // One thread per mode of the H x (H/2+1) half spectrum.
 template <typename T>
 __global__ void __launch_bounds__(kT2)
-k2_spectral(const cpx<T>* __restrict__ T1, cpx<T>* __restrict__ alpha, cpx<T>* __restrict__ T2, int H,
+k2_spectral(const cpx<T>* T1, cpx<T>* __restrict__ alpha, cpx<T>* __restrict__ T2, int H,
             Spec2D<T> sp) {
   pdl_wait();
   const int NH = H / 2 + 1;
@@ -186,7 +186,7 @@ k2_spectral(const cpx<T>* __restrict__ T1, cpx<T>* __restrict__ alpha, cpx<T>* _
 
 template <typename T>
 __global__ void __launch_bounds__(kT2)
-k2_move(T* __restrict__ x, T* __restrict__ y, int64_t P, Geo<T> g, const T* __restrict__ grad4, int g2p, int split,
+k2_move(T* __restrict__ x, T* __restrict__ y, int64_t P, Geo<T> g, const T* grad4, int g2p, int split,
         T s_noise, T chitau, uint64_t seed, uint32_t n, int* err) {
   pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -228,7 +228,7 @@ __device__ __forceinline__ double warp_sum2(double v) {
 // acc[0] += sum |X|^2, acc[1] += sum of the grid (mass)
 template <typename T>
 __global__ void __launch_bounds__(kT2)
-k2_sums(const T* __restrict__ x, const T* __restrict__ y, int64_t P, const T* __restrict__ phi, int64_t N,
+k2_sums(const T* x, const T* y, int64_t P, const T* phi, int64_t N,
         double* acc) {
   pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -247,7 +247,7 @@ k2_sums(const T* __restrict__ x, const T* __restrict__ y, int64_t P, const T* __
 // acc[2] += energy of modes with ||q|| >= 4, acc[3] += total (full spectrum:
 // the columns ky = 0 and ky = H/2 once, the others twice)
 template <typename T>
-__global__ void __launch_bounds__(kT2) k2_energy(const cpx<T>* __restrict__ alpha, int H, double* acc) {
+__global__ void __launch_bounds__(kT2) k2_energy(const cpx<T>* alpha, int H, double* acc) {
   pdl_wait();
   const int NH = H / 2 + 1, S = H * NH;
   double hi = 0.0, tot = 0.0;
@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(kT2) k2_energy(const cpx<T>* __restrict__ alph
 
 template <typename T>
 __global__ void __launch_bounds__(kT2)
-k2_load_aos(const double* __restrict__ X, int64_t P, Geo<T> g, T* __restrict__ x, T* __restrict__ y) {
+k2_load_aos(const double* X, int64_t P, Geo<T> g, T* __restrict__ x, T* __restrict__ y) {
   pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += stride) {
@@ -280,7 +280,7 @@ k2_load_aos(const double* __restrict__ X, int64_t P, Geo<T> g, T* __restrict__ x
 
 template <typename T>
 __global__ void __launch_bounds__(kT2)
-k2_store_aos(const T* __restrict__ x, const T* __restrict__ y, int64_t P, double* __restrict__ X) {
+k2_store_aos(const T* x, const T* y, int64_t P, double* __restrict__ X) {
   pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += stride) {

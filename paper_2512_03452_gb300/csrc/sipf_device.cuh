@@ -18,6 +18,12 @@ template <typename T> struct alignas(2 * sizeof(T)) cpx { T x, y; };
 // its writes are visible.  (Larger grids are launched the ordinary way.)
 // Every block of such a kernel executes it first of all, so a kernel's
 // completion implies that of all kernels before it.
+// Such a kernel's lifetime overlaps its predecessor's last writes, while the
+// read-only data path (__ldg, and const __restrict__ kernel arguments, which the
+// compiler may load that way and ahead of the wait) is only defined for memory
+// that no one writes during the kernel.  So these kernels read what an earlier
+// kernel may have written through plain pointers; only argument tables and
+// constants, written before any of the kernels start, are read-only.
 constexpr unsigned kPdlBlocks = 152 * 8;
 __device__ __forceinline__ void pdl_wait() {
   if (gridDim.x * gridDim.y * gridDim.z <= kPdlBlocks) asm volatile("griddepcontrol.wait;" ::: "memory");
