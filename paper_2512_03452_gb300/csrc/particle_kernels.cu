@@ -102,17 +102,18 @@ __device__ __forceinline__ void win_add(long long* p, long long v) {
 
 template <typename T> struct V3 { T x, y, z; };
 template <typename T> struct Vec4;
+// (With plain loads the batched move waits for each node in turn: 249 -> 311 us a
+// step of 32 runs of 3e5 particles, H = 32.)
 template <> struct Vec4<float> {
   static __device__ __forceinline__ V3<float> load(const float* p) {
-    const float4 v = *reinterpret_cast<const float4*>(p);
+    const float4 v = ld_data(reinterpret_cast<const float4*>(p));
     return {v.x, v.y, v.z};
   }
 };
 template <> struct Vec4<double> {
   static __device__ __forceinline__ V3<double> load(const double* p) {
-    const double2 a = *reinterpret_cast<const double2*>(p);
-    const double b = p[2];
-    return {a.x, a.y, b};
+    const double2 a = ld_data(reinterpret_cast<const double2*>(p));
+    return {a.x, a.y, ld_data(p + 2)};
   }
 };
 

@@ -29,6 +29,32 @@ __device__ __forceinline__ void pdl_wait() {
   if (gridDim.x * gridDim.y * gridDim.z <= kPdlBlocks) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// Loads of an earlier kernel's data for gathers: ordinary global loads, but
+// stated without side effects, so that the compiler may issue them together and
+// past the kernel's own stores as it does with read-only loads.  The address
+// must depend on a value read after pdl_wait (a gather's position does), and
+// the kernel must not write the memory.
+__device__ __forceinline__ float ld_data(const float* p) {
+  float v;
+  asm("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double ld_data(const double* p) {
+  double v;
+  asm("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float4 ld_data(const float4* p) {
+  float4 v;
+  asm("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double2 ld_data(const double2* p) {
+  double2 v;
+  asm("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+  return v;
+}
+
 __device__ __forceinline__ int ilog2_dev(int v) { return 31 - __clz(v); }   // v a power of two
 __device__ __forceinline__ float t_floor(float v) { return floorf(v); }
 __device__ __forceinline__ double t_floor(double v) { return ::floor(v); }
