@@ -146,8 +146,8 @@ __device__ __forceinline__ int tile_of(int cx, int cy, int cz, int shift, int nt
 // drift can carry particles many cells in one step, so the deposit reads the
 // bins of the new positions, where every particle lies in the tile of its bin
 // and the window only needs the stencil halo.
-// WHOLE: the window is the whole (small) grid with periodic slots (H <= 16);
-// otherwise the window is the tile plus the halo of Gamma_4 (-1, +2).
+// The window is the tile plus the halo of Gamma_4 (-1, +2), or the whole (small)
+// grid with periodic slots (H <= 16, k_deposit_whole).
 // ---------------------------------------------------------------------------
 constexpr int kTileShift = 3;                 // tiles of 8^3 cells
 constexpr int kTileE = 1 << kTileShift;
@@ -344,26 +344,22 @@ __device__ __forceinline__ void tile_origin(int bin, int ntx, int& ox, int& oy, 
   oz = tz * kTileE - kMargin - 1;
 }
 
-// Deposit of one work item of a single bin by the block.  WHOLE: the window is
-// the whole grid (use_win: the launch has one).
-template <typename T, bool FIXED, bool WHOLE, typename Fetch>
+// Deposit of one work item of a single bin by the block.
+template <typename T, bool FIXED, typename Fetch>
 __device__ __forceinline__ void deposit_chunk(const BinArgs<T>& a, const ChunkDesc& cur,
-                                              typename WinType<T>::type* win, bool use_win, Fetch& fetch) {
+                                              typename WinType<T>::type* win, Fetch& fetch) {
   using A = typename WinType<T>::type;
-  const int H = a.g.H, mask = a.g.mask;
-  const int wslots = WHOLE ? H * H * H : kWinSlots;
+  const int mask = a.g.mask;
   const int lane = threadIdx.x & 31;
-  // lanes of a warp that land in the same cell add into different copies
-  A* const my_win = win + (lane & (kReplicas - 1)) * wslots;
   const int bin = cur.bin, len = cur.len;
   const long long start = cur.start;
-  const bool has_win = use_win && (WHOLE || (bin < a.NT && len >= kWinMinLen));
+  const bool has_win = bin < a.NT && len >= kWinMinLen;
   int ox = 0, oy = 0, oz = 0;   // node coordinates of window slot (0,0,0)
-  if (!WHOLE && bin < a.NT) tile_origin(bin, a.ntx, ox, oy, oz);
+  if (bin < a.NT) tile_origin(bin, a.ntx, ox, oy, oz);
   // window scale 2^K: no copy's node sum can reach 2^30 (int32 windows; see
   // win_copy_load) or 2^62 (int64 windows: the whole chunk's sum)
   const int K = FIXED ? a.fix_k
-                      : (sizeof(A) == 4 ? 30 - ceil_log2(win_copy_load(WHOLE ? 8 : 7, len, blockDim.x) + 1)
+                      : (sizeof(A) == 4 ? 30 - ceil_log2(win_copy_load(7, len, blockDim.x) + 1)
                                         : WinType<T>::bits - ceil_log2(len + 1));
   const T wwin = pow2<T>(K);
   // next particle's data is loaded one iteration ahead (streaming loads: the
@@ -396,17 +392,6 @@ __device__ __forceinline__ void deposit_chunk(const BinArgs<T>& a, const ChunkDe
       cell_lambda(y, a.g, cy, ly);
       cell_lambda(z, a.g, cz, lz);
       bool fits = i < len;
-      if (WHOLE) {
-        if (fits) {
-          int ix[4], iy[4], iz[4];
-          axis_layers_global(cx, mask, H * H, ix);
-          axis_layers_global(cy, mask, H, iy);
-          axis_layers_global(cz, mask, 1, iz);
-          stencil_visit<T>(a.p2g, ix, iy, iz, lx, ly, lz, wwin,
-                           [&](int idx, T f) { win_add(my_win + idx, WinType<T>::round(f)); });
-        }
-        continue;
-      }
       int slot = 0;
       if (fits && !tile_slot(cx, cy, cz, ox, oy, oz, mask, slot)) {
         fits = false;
@@ -432,7 +417,70 @@ __device__ __forceinline__ void deposit_chunk(const BinArgs<T>& a, const ChunkDe
       if (missed & 1u) deposit_global<T, FIXED>(a, start + i);
   if (has_win) {
     __syncthreads();
-    window_flush<T, FIXED, WHOLE>(a, win, wslots, ox, oy, oz, K);
+    window_flush<T, FIXED, false>(a, win, kWinSlots, ox, oy, oz, K);
+  }
+}
+
+// Deposit of a whole small grid (H <= 16, where a single tile holds every
+// particle): a block adds `len` consecutive particles into kReplicas copies of
+// the grid in shared memory, then those to the grid.  The ranges are the
+// deposit's own, not the move's work items: items of 64 particles (see
+// particle_chunk) are too few for a window, and added straight to the grid
+// their 32 reductions a particle met on 4096 nodes and rounded at every one:
+// P = 2e5, H = 16, single precision 334 us, and 3 to 10 times the windows'
+// error (FP64 P = 1e4: 1.3e-15 of the grid against 1.4e-16).
+template <typename T, bool FIXED>
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1)
+k_deposit_whole(const __grid_constant__ BinArgs<T> a, int len) {
+  using A = typename WinType<T>::type;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  A* win = reinterpret_cast<A*>(smem_raw);
+  const int H = a.g.H, mask = a.g.mask, nodes = H * H * H;
+  for (int i = threadIdx.x; i < kReplicas * nodes; i += blockDim.x) win[i] = A(0);
+  pdl_wait();
+  // lanes of a warp that land in the same cell add into different copies
+  A* const my_win = win + (threadIdx.x & (kReplicas - 1)) * nodes;
+  // the tile's particles, then the overflow bin's
+  const int c0 = a.src_count[0], total = c0 + a.src_count[1];
+  const long long base0 = a.src_base[0], base1 = a.src_base[1] - c0;
+  auto slot = [&](int i) { return i < c0 ? base0 + i : base1 + i; };
+  __syncthreads();
+  for (long long r = (long long)blockIdx.x * len; r < total; r += (long long)gridDim.x * len) {
+    const int r0 = (int)r, n = min(len, total - r0);
+    // window scale as in deposit_chunk; eight lanes of a warp share a copy
+    const int K = FIXED ? a.fix_k
+                        : (sizeof(A) == 4 ? 30 - ceil_log2(win_copy_load(8, n, blockDim.x) + 1)
+                                          : WinType<T>::bits - ceil_log2(n + 1));
+    const T wwin = pow2<T>(K);
+    T px = T(0), py = T(0), pz = T(0);   // the next particle, loaded one iteration ahead
+    if ((int)threadIdx.x < n) {
+      const long long s = slot(r0 + threadIdx.x);
+      px = __ldcs(a.sx + s);
+      py = __ldcs(a.sy + s);
+      pz = __ldcs(a.sz + s);
+    }
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      const T x = px, y = py, z = pz;
+      if (i + (int)blockDim.x < n) {
+        const long long s = slot(r0 + i + blockDim.x);
+        px = __ldcs(a.sx + s);
+        py = __ldcs(a.sy + s);
+        pz = __ldcs(a.sz + s);
+      }
+      int cx, cy, cz, ix[4], iy[4], iz[4];
+      T lx, ly, lz;
+      cell_lambda(x, a.g, cx, lx);
+      cell_lambda(y, a.g, cy, ly);
+      cell_lambda(z, a.g, cz, lz);
+      axis_layers_global(cx, mask, H * H, ix);
+      axis_layers_global(cy, mask, H, iy);
+      axis_layers_global(cz, mask, 1, iz);
+      stencil_visit<T>(a.p2g, ix, iy, iz, lx, ly, lz, wwin,
+                       [&](int idx, T f) { win_add(my_win + idx, WinType<T>::round(f)); });
+    }
+    __syncthreads();
+    window_flush<T, FIXED, true>(a, win, nodes, 0, 0, 0, K);
+    __syncthreads();
   }
 }
 
@@ -443,7 +491,7 @@ __device__ __forceinline__ void deposit_chunk(const BinArgs<T>& a, const ChunkDe
 // and dependent loads, and an item was as many of them.)  A bin adds at most once per particle to a
 // node, so K = 31 - ceil(log2(c + 1)) keeps c 2^K below 2^31: 24 for up to 127
 // particles, 23 for up to 255.
-template <typename T, bool FIXED, bool WHOLE>
+template <typename T, bool FIXED>
 __device__ __forceinline__ void deposit_merged(const BinArgs<T>& a, const ChunkDesc& cur,
                                                typename WinType<T>::type* win) {
   using A = typename WinType<T>::type;
@@ -455,9 +503,9 @@ __device__ __forceinline__ void deposit_merged(const BinArgs<T>& a, const ChunkD
     const int c = b < a.NT ? a.src_count[b] : 0;
     if (!bin_is_small(b, c, a.NT, a.small)) continue;
     const long long s0 = a.src_base[b];
-    const bool has_win = !WHOLE && c >= kWarpWinMin;
-    int ox = 0, oy = 0, oz = 0;
-    if (!WHOLE) tile_origin(b, a.ntx, ox, oy, oz);
+    const bool has_win = c >= kWarpWinMin;
+    int ox, oy, oz;
+    tile_origin(b, a.ntx, ox, oy, oz);
     const int K = FIXED ? a.fix_k : (sizeof(A) == 4 ? 31 : WinType<T>::bits) - ceil_log2(c + 1);
     const T wwin = pow2<T>(K);
     uint32_t missed = has_win ? 0u : 0xFFFFFFFFu;   // a bit per iteration (at most kSmallMax / 32)
@@ -629,24 +677,21 @@ __device__ __forceinline__ void for_items(const Item* list, long long n, unsigne
   }
 }
 
-template <typename T, bool FIXED, bool WHOLE>
+template <typename T, bool FIXED>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2)
-k_binned_deposit(const __grid_constant__ BinArgs<T> a, int use_win) {
+k_binned_deposit(const __grid_constant__ BinArgs<T> a) {
   using A = typename WinType<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   A* win = reinterpret_cast<A*>(smem_raw);
   __shared__ ChunkDesc s_item[2];
-  if (use_win) {
-    const int n = WHOLE ? kReplicas * a.g.H * a.g.H * a.g.H : kTileReps * kWinSlots;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) win[i] = A(0);
-  }
+  for (int i = threadIdx.x; i < kTileReps * kWinSlots; i += blockDim.x) win[i] = A(0);
   pdl_wait();
   for_items(a.chunks, a.chunk_start[a.NT + 1], a.work, s_item, [&](const ChunkDesc& cur, auto& fetch) {
     if (cur.bin >= 0) {
-      deposit_chunk<T, FIXED, WHOLE>(a, cur, win, use_win != 0, fetch);
+      deposit_chunk<T, FIXED>(a, cur, win, fetch);
     } else {
       fetch.load();
-      deposit_merged<T, FIXED, WHOLE>(a, cur, win);
+      deposit_merged<T, FIXED>(a, cur, win);
     }
     return true;
   });
@@ -687,10 +732,10 @@ k_deposit_batch(const BinArgs<T>* __restrict__ table, const BatchItem* list,
   for_items(list, *total, work, s_item, [&](const BatchItem& cur, auto& fetch) {
     const BinArgs<T>& a = table[cur.run];
     if (cur.d.bin >= 0) {
-      deposit_chunk<T, FIXED, false>(a, cur.d, win, true, fetch);
+      deposit_chunk<T, FIXED>(a, cur.d, win, fetch);
     } else {
       fetch.load();
-      deposit_merged<T, FIXED, false>(a, cur.d, win);
+      deposit_merged<T, FIXED>(a, cur.d, win);
     }
     return true;
   });
@@ -1886,24 +1931,37 @@ int particle_small(int chunk) {
   return s > kSmallMax ? kSmallMax : s < 32 ? 32 : s;
 }
 
-template <typename T, bool FIXED, bool WHOLE>
-static cudaError_t launch_deposit_t(const BinArgs<T>& a, cudaStream_t s) {
-  // whole-grid window: only for items with enough particles to pay for its flush
-  const int nodes = a.g.H * a.g.H * a.g.H;
-  const int use_win = !WHOLE || a.chunk >= nodes / 8;
-  const size_t slots = WHOLE ? (size_t)kReplicas * nodes : (size_t)kTileReps * kWinSlots;
-  const size_t smem = use_win ? slots * sizeof(typename WinType<T>::type) : 0;
-  auto kern = k_binned_deposit<T, FIXED, WHOLE>;
+// Particles of a block of k_deposit_whole: some 40 windows up to 4096 particles
+// each.  The windows' sums are added in floating point, and more windows of
+// fewer particles round more (FP64, P = 1e5, H = 16: 2.7e-16 of the grid with
+// windows of 1024, 2.1e-16 with 4096).  At least 512 in single precision, so that
+// the flush stays small next to them; 64 in double, whose weights want as many
+// SMs as there are.
+static int deposit_whole_len(int64_t P, bool fp64) {
+  int len = fp64 ? 64 : 512;
+  while (len < 4096 && P / len >= 40) len <<= 1;
+  return len;
+}
+
+template <typename T, bool FIXED> static cudaError_t launch_deposit_t(const BinArgs<T>& a, cudaStream_t s) {
+  using A = typename WinType<T>::type;
   int blocks = 0;
-  const cudaError_t e = resident_blocks((const void*)kern, 256, smem, &blocks);
+  if (a.g.H <= 16) {
+    const size_t smem = (size_t)kReplicas * a.g.H * a.g.H * a.g.H * sizeof(A);
+    const cudaError_t e = resident_blocks((const void*)k_deposit_whole<T, FIXED>, 256, smem, &blocks);
+    if (e != cudaSuccess) return e;
+    const int len = deposit_whole_len(a.P, sizeof(T) == 8);
+    const int64_t ranges = (a.P + len - 1) / len;
+    return launch_k(k_deposit_whole<T, FIXED>, ranges < blocks ? (int)ranges : blocks, 256, smem, s, a, len);
+  }
+  const size_t smem = (size_t)kTileReps * kWinSlots * sizeof(A);
+  const cudaError_t e = resident_blocks((const void*)k_binned_deposit<T, FIXED>, 256, smem, &blocks);
   if (e != cudaSuccess) return e;
-  launch_k(kern, min(blocks, a.max_items), 256, smem, s, a, use_win);
-  return cudaGetLastError();
+  return launch_k(k_binned_deposit<T, FIXED>, min(blocks, a.max_items), 256, smem, s, a);
 }
 
 template <typename T> cudaError_t launch_binned_deposit(const BinArgs<T>& a, cudaStream_t s) {
-  if (a.g.H <= 16) return a.fixed ? launch_deposit_t<T, true, true>(a, s) : launch_deposit_t<T, false, true>(a, s);
-  return a.fixed ? launch_deposit_t<T, true, false>(a, s) : launch_deposit_t<T, false, false>(a, s);
+  return a.fixed ? launch_deposit_t<T, true>(a, s) : launch_deposit_t<T, false>(a, s);
 }
 
 template <typename T> cudaError_t launch_binned_rebin(const BinArgs<T>& a, cudaStream_t s) {

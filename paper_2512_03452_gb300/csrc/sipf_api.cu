@@ -262,8 +262,8 @@ template <typename T> BinArgs<T> bin_args(sipf_ctx* c, int src_buf, int src_lay,
   a.ntx = c->ntx;
   a.tile_shift = c->shift;
   a.max_items = (int)std::min<int64_t>(c->max_chunks(), INT32_MAX);
-  a.chunk = c->chunk;
   a.small = c->small;
+  a.P = c->p.P;
   a.phi = c->phi;
   a.grad4 = (const T*)c->grad;
   a.g = make_geo<T>(c->p.L, c->p.H);

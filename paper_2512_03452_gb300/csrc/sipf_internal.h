@@ -228,7 +228,8 @@ struct BinArgs {
   unsigned long long* work;      // chunk counter of the persistent grid (zeroed before the launch)
   int NT, ntx, tile_shift;       // tiles, tiles per axis, log2 tile edge
   int max_items;                 // bound of the number of work items
-  int chunk, small;              // the chunk list's item length and merge threshold (see ChunkListArgs)
+  int small;                     // the chunk list's merge threshold (see ChunkListArgs)
+  int64_t P;                     // particles of the run
   // physics
   void* phi;                     // deposit target (T, or int64 fixed point)
   const T* grad4;                // H^3 nodes x 4 (gx, gy, gz, 0)
