@@ -177,7 +177,7 @@ constexpr int kWinMinLen = 64;
 // kMerge warps.  (Windows of 4 and 16 bins: 241 and 267 us per step of a batch
 // of 24 runs against 237; torus of 1e7 453 and 445 against 446.)
 constexpr int kMerge = 8;
-constexpr int kSmallMax = 256;
+constexpr int kSmallMax = 240;   // (see merged_k)
 // In a merged item's deposit, a warp takes a bin of at least this many
 // particles into a window of its own (below it: global reductions).
 constexpr int kWarpWinMin = 24;
@@ -484,13 +484,24 @@ k_deposit_whole(const __grid_constant__ BinArgs<T> a, int len) {
   }
 }
 
+// Unit 2^-K of the one-copy window of a bin of c < kSmallMax particles.  Each
+// adds at most once to a node, a weight in (-1/15, 1] ((lambda - lambda^3) / 6 <=
+// 0.0642 beyond the cell), so with c 2^K < 240 2^24 a 32-bit node sum lies in
+// (-16 2^24, 240 2^24) and its bits tell it apart (window_sum).  K = 24 for 120
+// to 239 particles, as in the block's windows, and one more for each halving.
+// (Taken as two's complement, c 2^K < 2^31: K = 23 from 128 particles on, up to
+// 3% of the whole FP32 deposit's error at H = 32.)
+__device__ __forceinline__ int merged_k(int c) { return 24 + 31 - __clz((kSmallMax - 1) / c); }
+__device__ __forceinline__ long long window_sum(int v) {
+  return (unsigned)v < 0xF0000000u ? (long long)(unsigned)v : (long long)v;
+}
+__device__ __forceinline__ long long window_sum(long long v) { return v; }
+
 // Deposit of a merged item: each warp takes small bins of its own, with a
 // window of one copy in its eighth of the block's window, so the bins of an
 // item run beside one another with no block barrier.  (Taken one after another
 // by the whole block, a bin of some 80 particles cost about 10 us of barriers
-// and dependent loads, and an item was as many of them.)  A bin adds at most once per particle to a
-// node, so K = 31 - ceil(log2(c + 1)) keeps c 2^K below 2^31: 24 for up to 127
-// particles, 23 for up to 255.
+// and dependent loads, and an item was as many of them.)
 template <typename T, bool FIXED>
 __device__ __forceinline__ void deposit_merged(const BinArgs<T>& a, const ChunkDesc& cur,
                                                typename WinType<T>::type* win) {
@@ -506,7 +517,7 @@ __device__ __forceinline__ void deposit_merged(const BinArgs<T>& a, const ChunkD
     const bool has_win = c >= kWarpWinMin;
     int ox, oy, oz;
     tile_origin(b, a.ntx, ox, oy, oz);
-    const int K = FIXED ? a.fix_k : (sizeof(A) == 4 ? 31 : WinType<T>::bits) - ceil_log2(c + 1);
+    const int K = FIXED ? a.fix_k : sizeof(A) == 4 ? merged_k(c) : WinType<T>::bits - ceil_log2(c + 1);
     const T wwin = pow2<T>(K);
     uint32_t missed = has_win ? 0u : 0xFFFFFFFFu;   // a bit per iteration (at most kSmallMax / 32)
     if (has_win) {
@@ -558,7 +569,7 @@ __device__ __forceinline__ void deposit_merged(const BinArgs<T>& a, const ChunkD
               wr[i] = 0;
               any = true;
             }
-            v[i] = sum_to_real<float>(c4) * unit;
+            v[i] = sum_to_real<float>(window_sum(c4)) * unit;
           }
           if (any) {
             const int sa = row / kWin, sb = row - sa * kWin;
@@ -573,7 +584,8 @@ __device__ __forceinline__ void deposit_merged(const BinArgs<T>& a, const ChunkD
           if (v != 0) {
             ww[s] = A(0);
             const int sc = s % kWin, sb = (s / kWin) % kWin, sa = s / (kWin * kWin);
-            add_node<T, FIXED>(a, (((ox + sa) & mask) * H + ((oy + sb) & mask)) * H + ((oz + sc) & mask), v, unit);
+            add_node<T, FIXED>(a, (((ox + sa) & mask) * H + ((oy + sb) & mask)) * H + ((oz + sc) & mask), window_sum(v),
+                               unit);
           }
         }
       }
