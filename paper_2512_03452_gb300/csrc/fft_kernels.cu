@@ -1199,9 +1199,10 @@ kwr_spectral_x(const cpx<float>* T1, cpx<float>* __restrict__ alpha, cpx<float>*
                                twq + N + wib * XRegShape<N>::WARP);
 }
 
-template <int N>
+// (Kernels with a DEP parameter: the form with the wait, see launch_sized.)
+template <int N, bool DEP>
 __global__ void __launch_bounds__(512) kwrb_spectral_x(const FftRun<float>* __restrict__ runs) {
-  pdl_wait();
+  if constexpr (DEP) pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<float>* twq = reinterpret_cast<cpx<float>*>(smem_raw);
   load_twq<float, N>(twq);
@@ -1777,9 +1778,9 @@ __device__ __forceinline__ void plane_inv_body(const cpx<T>* in, T* __restrict__
   }
 }
 
-template <typename T, int E>
+template <typename T, int E, bool DEP>
 __global__ void __launch_bounds__(group_rows<T, 32 * E>() ? 512 : 1024) kwp_fwd(const FftRun<T>* __restrict__ runs) {
-  pdl_wait();
+  if constexpr (DEP) pdl_wait();
   constexpr int N = 32 * E, NH = N / 2 + 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
@@ -1797,9 +1798,9 @@ __global__ void __launch_bounds__(group_rows<T, 32 * E>() ? 512 : 1024) kwp_fwd(
     plane_fwd_body<T, E, T>(static_cast<T*>(r.phi) + (size_t)x * N * N, 1.0, out, tw, P, zb);
 }
 
-template <typename T, int E>
+template <typename T, int E, bool DEP>
 __global__ void __launch_bounds__(group_rows<T, 32 * E>() ? 512 : 1024) kwp_inv(const FftRun<T>* __restrict__ runs) {
-  pdl_wait();
+  if constexpr (DEP) pdl_wait();
   constexpr int N = 32 * E, NH = N / 2 + 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
@@ -2154,9 +2155,9 @@ __device__ __forceinline__ void cplane_inv_body(const cpx<T>* in, T* __restrict_
   cluster.sync();
 }
 
-template <typename T, int E, int CS>
+template <typename T, int E, int CS, bool DEP>
 __global__ void __launch_bounds__(1024) kwc_fwd(const FftRun<T>* __restrict__ runs) {
-  pdl_wait();
+  if constexpr (DEP) pdl_wait();
   constexpr int N = 32 * E, NH = N / 2 + 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
@@ -2174,9 +2175,9 @@ __global__ void __launch_bounds__(1024) kwc_fwd(const FftRun<T>* __restrict__ ru
     cplane_fwd_body<T, E, CS, T>(static_cast<T*>(r.phi) + (size_t)x * N * N, 1.0, out, tw, Q, zb);
 }
 
-template <typename T, int E, int CS>
+template <typename T, int E, int CS, bool DEP>
 __global__ void __launch_bounds__(1024) kwc_inv(const FftRun<T>* __restrict__ runs) {
-  pdl_wait();
+  if constexpr (DEP) pdl_wait();
   constexpr int N = 32 * E, NH = N / 2 + 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
@@ -2191,10 +2192,14 @@ __global__ void __launch_bounds__(1024) kwc_inv(const FftRun<T>* __restrict__ ru
   cplane_inv_body<T, E, CS>(r.T2 + comp * S + (size_t)x * N * NH, r.grad, x, d, r.sk.two_pi_L, tw, Q, zb);
 }
 
-// Launch with a cluster of CS CTAs along x.
+// Launch with a cluster of CS CTAs along x (of the form for its size, see launch_sized).
 template <typename K, typename... Args>
-static cudaError_t launch_cluster(K kernel, dim3 grid, int threads, size_t smem, int cs, cudaStream_t s,
+static cudaError_t launch_cluster(K with_wait, K without, dim3 grid, int threads, size_t smem, int cs, cudaStream_t s,
                                   Args... args) {
+  const bool dep = grid.x * grid.y * grid.z <= kPdlBlocks;
+  K kernel = dep ? with_wait : without;
+  const cudaError_t e = set_smem(kernel, smem);
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(threads);
@@ -2208,7 +2213,7 @@ static cudaError_t launch_cluster(K kernel, dim3 grid, int threads, size_t smem,
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // see launch_k
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = grid.x * grid.y * grid.z <= kPdlBlocks ? 2 : 1;
+  cfg.numAttrs = dep ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
@@ -2491,9 +2496,10 @@ static cudaError_t kwb_spectral_launch(const FftRun<T>* runs, int nruns, int nw,
     if (nw == 0) nw = spread_warps(XRegShape<N>::TASKS * nruns, kDefaultSpectralWarps);
     const size_t smr = xreg_smem_bytes<N>(nw);
     if (smr > kMaxSmem) return cudaErrorInvalidValue;
-    if ((e = set_smem(kwrb_spectral_x<N>, smr)) != cudaSuccess) return e;
-    launch_k(kwrb_spectral_x<N>, dim3((XRegShape<N>::TASKS + nw - 1) / nw, nruns), 32 * nw, smr, s, runs);
-    return cudaGetLastError();
+    if ((e = set_smem(kwrb_spectral_x<N, true>, smr)) != cudaSuccess) return e;
+    if ((e = set_smem(kwrb_spectral_x<N, false>, smr)) != cudaSuccess) return e;
+    return launch_sized(kwrb_spectral_x<N, true>, kwrb_spectral_x<N, false>,
+                        dim3((XRegShape<N>::TASKS + nw - 1) / nw, nruns), 32 * nw, smr, s, runs);
   } else {
     if (nw == 0) nw = kDefaultSpectralWarps;
     const size_t sms = spectral_smem<T, E, SBC>();
@@ -2555,14 +2561,14 @@ static cudaError_t field_batch_e(const FftRun<T>* runs, int nruns, int stages, c
                                     : tune.inv3 == 0 && nruns * N >= 4 * 152 && 2 * i3sm <= kMaxSmem);
   if (stages & kFieldForward) {
     if (clusters) {
-      if ((e = set_smem(kwc_fwd<T, E, CS>, csm)) != cudaSuccess) return e;
-      if ((e = launch_cluster(kwc_fwd<T, E, CS>, dim3(N * CS, nruns), 32 * cnw, csm, CS, s, runs)) != cudaSuccess)
-        return e;
+      e = launch_cluster(kwc_fwd<T, E, CS, true>, kwc_fwd<T, E, CS, false>, dim3(N * CS, nruns), 32 * cnw, csm, CS, s, runs);
+      if (e != cudaSuccess) return e;
       nk += 1;
     } else if (planes) {
-      if ((e = set_smem(kwp_fwd<T, E>, fsm)) != cudaSuccess) return e;
-      launch_k(kwp_fwd<T, E>, dim3(N, nruns), 32 * fnw, fsm, s, runs);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      if ((e = set_smem(kwp_fwd<T, E, true>, fsm)) != cudaSuccess) return e;
+      if ((e = set_smem(kwp_fwd<T, E, false>, fsm)) != cudaSuccess) return e;
+      e = launch_sized(kwp_fwd<T, E, true>, kwp_fwd<T, E, false>, dim3(N, nruns), 32 * fnw, fsm, s, runs);
+      if (e != cudaSuccess) return e;
       nk += 1;
     } else {
       if constexpr (group_rows<T, N>())
@@ -2584,9 +2590,8 @@ static cudaError_t field_batch_e(const FftRun<T>* runs, int nruns, int stages, c
     nk += 1;
   }
   if ((stages & kFieldInverse) && clusters) {
-    if ((e = set_smem(kwc_inv<T, E, CS>, csm)) != cudaSuccess) return e;
-    if ((e = launch_cluster(kwc_inv<T, E, CS>, dim3(N * CS, 3, nruns), 32 * cnw, csm, CS, s, runs)) != cudaSuccess)
-      return e;
+    e = launch_cluster(kwc_inv<T, E, CS, true>, kwc_inv<T, E, CS, false>, dim3(N * CS, 3, nruns), 32 * cnw, csm, CS, s, runs);
+    if (e != cudaSuccess) return e;
     nk += 1;
   } else if ((stages & kFieldInverse) && inv3) {
     if constexpr (E <= 2) {
@@ -2596,9 +2601,10 @@ static cudaError_t field_batch_e(const FftRun<T>* runs, int nruns, int stages, c
       nk += 1;
     }
   } else if ((stages & kFieldInverse) && planes) {
-    if ((e = set_smem(kwp_inv<T, E>, ism)) != cudaSuccess) return e;
-    launch_k(kwp_inv<T, E>, dim3(N, 3, nruns), 32 * inw, ism, s, runs);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = set_smem(kwp_inv<T, E, true>, ism)) != cudaSuccess) return e;
+    if ((e = set_smem(kwp_inv<T, E, false>, ism)) != cudaSuccess) return e;
+    e = launch_sized(kwp_inv<T, E, true>, kwp_inv<T, E, false>, dim3(N, 3, nruns), 32 * inw, ism, s, runs);
+    if (e != cudaSuccess) return e;
     nk += 1;
   } else if (stages & kFieldInverse) {
     if constexpr (two_spectra<E>()) {

@@ -64,9 +64,12 @@ template <typename T> inline SpecConst<T> spec_const(const SpecParams& sp) {
 // the kernels, so that the next kernel's blocks come in as soon as there is
 // room, measured slower (643 us; FP64 P = 1e6 2.52 -> 2.77 ms): the early blocks
 // pile up on the SMs that drain first.
-// launch_plain: kernels only used for grids of many waves.  They do not contain
-// the wait: the instruction alone, executed or not, made such kernels slower
-// (y pass at H = 256, 6912 blocks: 125 -> 201 us; x pass 170 -> 198).
+// launch_plain: kernels without the wait.  The instruction alone, executed or
+// not, makes grids of many waves slower (y pass at H = 256, 6912 blocks: 125 ->
+// 201 us; x pass 170 -> 198; inverse plane kernel of 8 runs at H = 128, 3072
+// blocks: 272 -> 366).
+// launch_sized: a kernel in both forms, with and without the wait, for grids
+// that may be small or large.
 template <typename... KA, typename... A>
 inline cudaError_t launch_plain(void (*kernel)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                                 A&&... args) {
@@ -90,6 +93,13 @@ inline cudaError_t launch_k(void (*kernel)(KA...), dim3 grid, dim3 block, size_t
   cfg.attrs = attr;
   cfg.numAttrs = grid.x * grid.y * grid.z <= kPdlBlocks ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+
+template <typename... KA, typename... A>
+inline cudaError_t launch_sized(void (*with_wait)(KA...), void (*without)(KA...), dim3 grid, dim3 block, size_t smem,
+                                cudaStream_t s, A&&... args) {
+  return grid.x * grid.y * grid.z <= kPdlBlocks ? launch_k(with_wait, grid, block, smem, s, std::forward<A>(args)...)
+                                                : launch_plain(without, grid, block, smem, s, std::forward<A>(args)...);
 }
 
 enum SpecMode { kModeStep = 0, kModeDensity = 1, kModeField = 2, kModeGradOnly = 3 };
