@@ -383,9 +383,6 @@ k_rows_c2r(const cpx<T>* in, size_t comp_stride, T* __restrict__ out, int lgH, i
   }
 }
 
-template <typename K>
-static cudaError_t set_smem(K kernel, size_t bytes);
-
 // ===========================================================================
 // Warp FFTs for H = 32 E, E in {2, 4, 8}.  A warp holds one pencil of
 // length N = 32 E: lane l keeps elements j = l + 32 m (m < E) in registers.
@@ -2198,7 +2195,7 @@ static cudaError_t launch_cluster(K with_wait, K without, dim3 grid, int threads
                                   Args... args) {
   const bool dep = grid.x * grid.y * grid.z <= kPdlBlocks;
   K kernel = dep ? with_wait : without;
-  const cudaError_t e = set_smem(kernel, smem);
+  const cudaError_t e = allow_smem((const void*)kernel, smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
@@ -2238,7 +2235,7 @@ static cudaError_t warp_cols(cpx<T>* data, int A, int B, int ncomp, size_t comp_
   constexpr int BC = 16;
   const size_t smem = (tw_len<T, E>() + (size_t)32 * E * (BC + 1) + E) * sizeof(cpx<T>);
   auto k = kw_cols<T, E, DIR, BC>;
-  cudaError_t e = set_smem(k, smem);
+  cudaError_t e = allow_smem((const void*)k, smem);
   if (e != cudaSuccess) return e;
   dim3 grid((B + BC - 1) / BC, A, ncomp);
   launch_k(k, grid, 256, smem, s, data, B, comp_stride, (T)scale);
@@ -2253,7 +2250,7 @@ static cudaError_t warp_spectral(const cpx<T>* T1, cpx<T>* alpha, cpx<T>* T2, Sp
     const int nw = spread_warps(XRegShape<N>::TASKS, kDefaultSpectralWarps);
     const size_t smem = xreg_smem_bytes<N>(nw);
     auto k = kwr_spectral_x<N, MODE>;
-    cudaError_t e = set_smem(k, smem);
+    cudaError_t e = allow_smem((const void*)k, smem);
     if (e != cudaSuccess) return e;
     launch_k(k, (XRegShape<N>::TASKS + nw - 1) / nw, 32 * nw, smem, s, T1, alpha, T2, spec_const<T>(sp), shadow);
     return cudaGetLastError();
@@ -2262,7 +2259,7 @@ static cudaError_t warp_spectral(const cpx<T>* T1, cpx<T>* alpha, cpx<T>* T2, Sp
   const int B = N * (N / 2 + 1);
   const size_t smem = (kTwLen + twq_len<T, N>() + (size_t)N * (3 * BC + 1) + E) * sizeof(cpx<T>);
   auto k = kw_spectral_x<T, E, MODE, BC>;
-  cudaError_t e = set_smem(k, smem);
+  cudaError_t e = allow_smem((const void*)k, smem);
   if (e != cudaSuccess) return e;
   launch_k(k, (B + BC - 1) / BC, 256, smem, s, T1, alpha, T2, spec_const<T>(sp), shadow);
   return cudaGetLastError();
@@ -2275,7 +2272,7 @@ static cudaError_t warp_rows_c2r(const cpx<T>* in, size_t comp_stride, T* out, i
   constexpr int NOUT = NCOMP == 3 ? 4 : 1;
   const size_t smem = row_c2r_smem<T, E, NOUT>();
   auto k = kw_rows_c2r<T, E, NCOMP>;
-  cudaError_t e = set_smem(k, smem);
+  cudaError_t e = allow_smem((const void*)k, smem);
   if (e != cudaSuccess) return e;
   launch_k(k, warp_blocks(rows), 256, smem, s, in, comp_stride, out, rows, max_acc);
   return cudaGetLastError();
@@ -2284,12 +2281,6 @@ static cudaError_t warp_rows_c2r(const cpx<T>* in, size_t comp_stride, T* out, i
 // ---------------------------------------------------------------------------
 // Launchers.
 // ---------------------------------------------------------------------------
-template <typename K>
-static cudaError_t set_smem(K kernel, size_t bytes) {
-  if (bytes > 48 * 1024) return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  return cudaSuccess;
-}
-
 // Shapes of the H < 32 kernels: blocks as small as it takes to give every SM
 // one (a 16^3 grid has 256 rows and 144 x pencils; with 8 row pairs or 16
 // pencils a block its FP64 transforms ran on 9 to 16 SMs: a step of P = 1e4
@@ -2322,11 +2313,11 @@ cudaError_t launch_rows_r2c(const void* in, int in_kind, double in_scale, bool z
   cudaError_t e;
   if (in_kind == 0) {
     auto k = k_rows_r2c<T, T>;
-    if ((e = set_smem(k, smem)) != cudaSuccess) return e;
+    if ((e = allow_smem((const void*)k, smem)) != cudaSuccess) return e;
     launch_k(k, blocks, RP > 2 ? kThreads : kSmallThreads, smem, s, (T*)in, in_scale, zero_input ? 1 : 0, out, lgH, rows, RP, mass_acc);
   } else {
     auto k = k_rows_r2c<T, unsigned long long>;
-    if ((e = set_smem(k, smem)) != cudaSuccess) return e;
+    if ((e = allow_smem((const void*)k, smem)) != cudaSuccess) return e;
     launch_k(k, blocks, RP > 2 ? kThreads : kSmallThreads, smem, s, (unsigned long long*)in, in_scale, zero_input ? 1 : 0, out, lgH, rows,
                                      RP, mass_acc);
   }
@@ -2362,11 +2353,11 @@ cudaError_t launch_cols(cpx<T>* data, int H, int A, int B, int ncomp, size_t com
   cudaError_t e;
   if (dir < 0) {
     auto k = k_cols<T, -1>;
-    if ((e = set_smem(k, smem)) != cudaSuccess) return e;
+    if ((e = allow_smem((const void*)k, smem)) != cudaSuccess) return e;
     launch_k(k, grid, nt, smem, s, data, lgH, B, lgBC, comp_stride, (T)scale);
   } else {
     auto k = k_cols<T, +1>;
-    if ((e = set_smem(k, smem)) != cudaSuccess) return e;
+    if ((e = allow_smem((const void*)k, smem)) != cudaSuccess) return e;
     launch_k(k, grid, nt, smem, s, data, lgH, B, lgBC, comp_stride, (T)scale);
   }
   return cudaGetLastError();
@@ -2383,7 +2374,7 @@ static cudaError_t spectral_mode(const cpx<T>* T1, cpx<T>* alpha, cpx<T>* T2, in
   const int lgBC = ilog2(BC), nt = BC > 2 ? kThreads : kSmallThreads;
   const size_t smem = (kNmax / 2 + (size_t)H * 4 * BC) * sizeof(cpx<T>);
   auto k = k_spectral_x<T, MODE>;
-  cudaError_t e = set_smem(k, smem);
+  cudaError_t e = allow_smem((const void*)k, smem);
   if (e != cudaSuccess) return e;
   launch_k(k, (B + BC - 1) / BC, nt, smem, s, T1, alpha, T2, lgH, lgBC, spec_const<T>(sp), shadow);
   return cudaGetLastError();
@@ -2436,17 +2427,15 @@ cudaError_t launch_rows_c2r(const cpx<T>* in, int ncomp, size_t comp_stride, T* 
   cudaError_t e;
   if (ncomp == 3) {
     auto k = k_rows_c2r<T, 3>;
-    if ((e = set_smem(k, smem)) != cudaSuccess) return e;
+    if ((e = allow_smem((const void*)k, smem)) != cudaSuccess) return e;
     launch_k(k, blocks, RP > 2 ? kThreads : kSmallThreads, smem, s, in, comp_stride, out, lgH, rows, RP, nullptr);
   } else {
     auto k = k_rows_c2r<T, 1>;
-    if ((e = set_smem(k, smem)) != cudaSuccess) return e;
+    if ((e = allow_smem((const void*)k, smem)) != cudaSuccess) return e;
     launch_k(k, blocks, RP > 2 ? kThreads : kSmallThreads, smem, s, in, comp_stride, out, lgH, rows, RP, max_acc);
   }
   return cudaGetLastError();
 }
-
-constexpr size_t kMaxSmem = 227 * 1024;
 
 template <typename T, int E, int BC>
 static size_t cols_smem() {
@@ -2464,7 +2453,7 @@ static cudaError_t kwb_cols_launch(const FftRun<T>* runs, int nruns, int ncomp, 
   const size_t smc = cols_smem<T, E, BC>();
   if (smc > kMaxSmem) return cudaErrorInvalidValue;
   cudaError_t e;
-  if ((e = set_smem(kwb_cols<T, E, DIR, BC>, smc)) != cudaSuccess) return e;
+  if ((e = allow_smem((const void*)kwb_cols<T, E, DIR, BC>, smc)) != cudaSuccess) return e;
   launch_plain(kwb_cols<T, E, DIR, BC>, dim3((NHH + BC - 1) / BC, N, nruns * ncomp), 256, smc, s, runs, ncomp);
   return cudaGetLastError();
 }
@@ -2483,7 +2472,7 @@ static cudaError_t kwb_cols_inv3_launch(const FftRun<T>* runs, int nruns, cudaSt
   constexpr int N = 32 * E, NHH = N / 2 + 1;
   const size_t smc = cols_smem<T, E, BC>();
   if (smc > kMaxSmem) return cudaErrorInvalidValue;
-  const cudaError_t e = set_smem(kwb_cols_inv3<T, E, BC>, smc);
+  const cudaError_t e = allow_smem((const void*)kwb_cols_inv3<T, E, BC>, smc);
   if (e != cudaSuccess) return e;
   return launch_plain(kwb_cols_inv3<T, E, BC>, dim3((NHH + BC - 1) / BC, N, nruns), 256, smc, s, runs);
 }
@@ -2496,15 +2485,15 @@ static cudaError_t kwb_spectral_launch(const FftRun<T>* runs, int nruns, int nw,
     if (nw == 0) nw = spread_warps(XRegShape<N>::TASKS * nruns, kDefaultSpectralWarps);
     const size_t smr = xreg_smem_bytes<N>(nw);
     if (smr > kMaxSmem) return cudaErrorInvalidValue;
-    if ((e = set_smem(kwrb_spectral_x<N, true>, smr)) != cudaSuccess) return e;
-    if ((e = set_smem(kwrb_spectral_x<N, false>, smr)) != cudaSuccess) return e;
+    if ((e = allow_smem((const void*)kwrb_spectral_x<N, true>, smr)) != cudaSuccess) return e;
+    if ((e = allow_smem((const void*)kwrb_spectral_x<N, false>, smr)) != cudaSuccess) return e;
     return launch_sized(kwrb_spectral_x<N, true>, kwrb_spectral_x<N, false>,
                         dim3((XRegShape<N>::TASKS + nw - 1) / nw, nruns), 32 * nw, smr, s, runs);
   } else {
     if (nw == 0) nw = kDefaultSpectralWarps;
     const size_t sms = spectral_smem<T, E, SBC>();
     if (sms > kMaxSmem) return cudaErrorInvalidValue;
-    if ((e = set_smem(kwb_spectral_x<T, E, SBC>, sms)) != cudaSuccess) return e;
+    if ((e = allow_smem((const void*)kwb_spectral_x<T, E, SBC>, sms)) != cudaSuccess) return e;
     launch_plain(kwb_spectral_x<T, E, SBC>, dim3((N * NHH + SBC - 1) / SBC, nruns), 32 * nw, sms, s, runs);
     return cudaGetLastError();
   }
@@ -2565,8 +2554,8 @@ static cudaError_t field_batch_e(const FftRun<T>* runs, int nruns, int stages, c
       if (e != cudaSuccess) return e;
       nk += 1;
     } else if (planes) {
-      if ((e = set_smem(kwp_fwd<T, E, true>, fsm)) != cudaSuccess) return e;
-      if ((e = set_smem(kwp_fwd<T, E, false>, fsm)) != cudaSuccess) return e;
+      if ((e = allow_smem((const void*)kwp_fwd<T, E, true>, fsm)) != cudaSuccess) return e;
+      if ((e = allow_smem((const void*)kwp_fwd<T, E, false>, fsm)) != cudaSuccess) return e;
       e = launch_sized(kwp_fwd<T, E, true>, kwp_fwd<T, E, false>, dim3(N, nruns), 32 * fnw, fsm, s, runs);
       if (e != cudaSuccess) return e;
       nk += 1;
@@ -2595,14 +2584,14 @@ static cudaError_t field_batch_e(const FftRun<T>* runs, int nruns, int stages, c
     nk += 1;
   } else if ((stages & kFieldInverse) && inv3) {
     if constexpr (E <= 2) {
-      if ((e = set_smem(kwp_inv3<T, E>, i3sm)) != cudaSuccess) return e;
+      if ((e = allow_smem((const void*)kwp_inv3<T, E>, i3sm)) != cudaSuccess) return e;
       launch_plain(kwp_inv3<T, E>, dim3(N, nruns), 32 * i3nw, i3sm, s, runs);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
       nk += 1;
     }
   } else if ((stages & kFieldInverse) && planes) {
-    if ((e = set_smem(kwp_inv<T, E, true>, ism)) != cudaSuccess) return e;
-    if ((e = set_smem(kwp_inv<T, E, false>, ism)) != cudaSuccess) return e;
+    if ((e = allow_smem((const void*)kwp_inv<T, E, true>, ism)) != cudaSuccess) return e;
+    if ((e = allow_smem((const void*)kwp_inv<T, E, false>, ism)) != cudaSuccess) return e;
     e = launch_sized(kwp_inv<T, E, true>, kwp_inv<T, E, false>, dim3(N, 3, nruns), 32 * inw, ism, s, runs);
     if (e != cudaSuccess) return e;
     nk += 1;
@@ -2621,7 +2610,7 @@ static cudaError_t field_batch_e(const FftRun<T>* runs, int nruns, int stages, c
       e = launch_plain(kwrb_rows_c2r3<N>, dim3(N * N / 2 / (4 * (32 / GroupShape<N>::Q)), nruns), 128, 0, s, runs);
     } else {
       const size_t smr = row_c2r_smem<T, E, 4>();
-      if ((e = set_smem(kwb_rows_c2r<T, E>, smr)) != cudaSuccess) return e;
+      if ((e = allow_smem((const void*)kwb_rows_c2r<T, E>, smr)) != cudaSuccess) return e;
       e = launch_plain(kwb_rows_c2r<T, E>, dim3(rblocks, nruns), 256, smr, s, runs);
     }
     if (e != cudaSuccess) return e;

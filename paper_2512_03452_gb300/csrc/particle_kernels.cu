@@ -1061,9 +1061,7 @@ k_move_batch(const BinArgs<T>* __restrict__ table, const BatchItem* list,
 static cudaError_t resident_blocks(const void* kern, int threads, size_t smem, int* blocks, int blocks_per_sm = 0) {
   int dev = 0, sms = 0, per_sm = 0;
   cudaError_t e;
-  if (smem > 48 * 1024 &&
-      (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-    return e;
+  if ((e = allow_smem(kern, smem, 1024)) != cudaSuccess) return e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem)) != cudaSuccess) return e;

@@ -365,7 +365,7 @@ template <typename T> int deposit2(sipf2d_ctx* c) {
   if (c->p.P >= 8 * kT2Win) {
     const int rows = win2_rows<T>(c->p.H);
     const size_t smem = (size_t)rows * c->p.H * sizeof(T);
-    SIPF2_CK(cudaFuncSetAttribute(k2_deposit_win<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    SIPF2_CK(allow_smem((const void*)k2_deposit_win<T>, smem));
     SIPF2_CK(launch_k(k2_deposit_win<T>, grid_for2(c->p.P, kT2Win, 152), kT2Win, smem, c->stream, (const T*)c->x,
                       (const T*)c->y, c->p.P, geo2<T>(c), w, c->p.p2g_order, rows, (T*)c->phi));
     return SIPF_OK;

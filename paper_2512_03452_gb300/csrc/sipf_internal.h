@@ -102,6 +102,18 @@ inline cudaError_t launch_sized(void (*with_wait)(KA...), void (*without)(KA...)
                                                 : launch_plain(without, grid, block, smem, s, std::forward<A>(args)...);
 }
 
+// Dynamic shared memory above 48 KB has to be allowed per kernel first, and the
+// allowance belongs to the kernel, not to the launch: it is always set to the
+// same maximum, whatever this launch needs, so that a host thread with a smaller
+// window or plane never lowers it between another thread's setting and launch.
+// (own: bytes of static shared memory the kernel has besides, rounded up.)
+constexpr size_t kMaxSmem = 227 * 1024;
+inline cudaError_t allow_smem(const void* kernel, size_t bytes, size_t own = 0) {
+  return bytes > 48 * 1024
+             ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kMaxSmem - own))
+             : cudaSuccess;
+}
+
 enum SpecMode { kModeStep = 0, kModeDensity = 1, kModeField = 2, kModeGradOnly = 3 };
 
 // One run of a batch, as seen by the batched FFT kernels.
