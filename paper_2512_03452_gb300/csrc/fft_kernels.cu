@@ -112,9 +112,9 @@ static inline int ilog2(int v) { int l = 0; while ((1 << l) < v) ++l; return l; 
 // Rows r2c: rows 2c and 2c+1 of the block form z = a + i b; after the FFT,
 // A_k = (Z_k + conj Z_{n-k})/2 and B_k = -i (Z_k - conj Z_{n-k})/2.
 // ---------------------------------------------------------------------------
-template <typename T, typename Tin>
+template <typename T, typename Tin, typename C = cpx<T>>
 __global__ void __launch_bounds__(kThreads)
-k_rows_r2c(Tin* __restrict__ in, double in_scale, int zero_input, cpx<T>* __restrict__ out,
+k_rows_r2c(Tin* __restrict__ in, double in_scale, int zero_input, C* __restrict__ out,
            int lgH, int rows, int RP, double* mass_acc) {
   pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -164,16 +164,16 @@ k_rows_r2c(Tin* __restrict__ in, double in_scale, int zero_input, cpx<T>* __rest
 // ---------------------------------------------------------------------------
 // c2c along the middle axis of [A][H][B]: block = (column chunk, a, component).
 // ---------------------------------------------------------------------------
-template <typename T, int DIR>
+template <typename T, int DIR, typename C = cpx<T>>
 __global__ void __launch_bounds__(kThreads)
-k_cols(cpx<T>* __restrict__ data, int lgH, int B, int lgBC, size_t comp_stride, T scale) {
+k_cols(C* __restrict__ data, int lgH, int B, int lgBC, size_t comp_stride, T scale) {
   pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
   cpx<T>* buf = tw + kNmax / 2;
   const int H = 1 << lgH, BC = 1 << lgBC;
   load_twiddles(tw);
-  cpx<T>* base = data + blockIdx.z * comp_stride + (size_t)blockIdx.y * H * B;
+  C* base = data + blockIdx.z * comp_stride + (size_t)blockIdx.y * H * B;
   const int b0 = blockIdx.x * BC;
   const int nb = min(BC, B - b0);
   for (int t = threadIdx.x; t < H * BC; t += blockDim.x) {
@@ -302,9 +302,9 @@ k_spectral_x(const cpx<T>* T1, cpx<T>* __restrict__ alpha, cpx<T>* __restrict__ 
 // gives a + i b.  The imaginary parts of the k = 0 and k = n/2 entries are
 // dropped (they carry no real signal).
 // ---------------------------------------------------------------------------
-template <typename T, int NCOMP>
+template <typename T, int NCOMP, typename C = cpx<T>>
 __global__ void __launch_bounds__(kThreads)
-k_rows_c2r(const cpx<T>* in, size_t comp_stride, T* __restrict__ out, int lgH, int rows,
+k_rows_c2r(const C* in, size_t comp_stride, T* __restrict__ out, int lgH, int rows,
            int RP, double* max_acc) {
   pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -318,7 +318,7 @@ k_rows_c2r(const cpx<T>* in, size_t comp_stride, T* __restrict__ out, int lgH, i
   const int row0 = blockIdx.x * 2 * RP;
   const int nrow = min(2 * RP, rows - row0);
   for (int d = 0; d < NCOMP; ++d) {
-    const cpx<T>* src = in + d * comp_stride;
+    const C* src = in + d * comp_stride;
     for (int t = threadIdx.x; t < RP * H; t += blockDim.x) {
       const int c = t >> lgH, k = t & (H - 1);
       cpx<T> z{T(0), T(0)};
@@ -330,8 +330,10 @@ k_rows_c2r(const cpx<T>* in, size_t comp_stride, T* __restrict__ out, int lgH, i
           Bv = src[rb + k];
           if (k == 0 || k == H / 2) { A.y = T(0); Bv.y = T(0); }
         } else {
-          A = cconj(src[ra + (H - k)]);
-          Bv = cconj(src[rb + (H - k)]);
+          A = src[ra + (H - k)];
+          Bv = src[rb + (H - k)];
+          A.y = -A.y;
+          Bv.y = -Bv.y;
         }
         z = cpx<T>{A.x - Bv.y, A.y + Bv.x};
       }
@@ -812,9 +814,9 @@ template <typename T, int E, bool ROWS> __device__ __forceinline__ void load_tw_
 // (the *_batch kernels, one run per block row).
 
 // Rows r2c: each warp takes row pairs (two real rows as one complex pencil).
-template <typename T, int E, typename Tin>
+template <typename T, int E, typename Tin, typename C>
 __device__ __forceinline__ void rows_r2c_body(Tin* __restrict__ in, double in_scale, int zero_input,
-                                              cpx<T>* __restrict__ out, int rows, double* mass_acc, int bx, int gx,
+                                              C* __restrict__ out, int rows, double* mass_acc, int bx, int gx,
                                               const cpx<T>* tw, cpx<T>* zball) {
   constexpr int N = 32 * E, NH = N / 2 + 1;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -843,7 +845,7 @@ __device__ __forceinline__ void rows_r2c_body(Tin* __restrict__ in, double in_sc
         },
         [&](int, int g) { return zb + g * PS; },
         [&](int pr, int k, cpx<T> A, cpx<T> B) {
-          cpx<T>* oa = out + (size_t)(2 * (p0 + pr)) * NH;
+          C* oa = out + (size_t)(2 * (p0 + pr)) * NH;
           oa[k] = A;
           oa[NH + k] = B;
         });
@@ -879,7 +881,7 @@ __device__ __forceinline__ void rows_r2c_body(Tin* __restrict__ in, double in_sc
 #pragma unroll
     for (int k1 = 0; k1 < E; ++k1) zb[zpad(out_index(k1, E, lane))] = v[k1];
     __syncwarp();
-    cpx<T>* oa = out + (size_t)(2 * pr) * NH;
+    C* oa = out + (size_t)(2 * pr) * NH;
     for (int k = lane; k < NH; k += 32) {
       const cpx<T> zk = zb[zpad(k)];
       const cpx<T> zm = cconj(zb[zpad((N - k) & (N - 1))]);
@@ -896,9 +898,9 @@ __device__ __forceinline__ void rows_r2c_body(Tin* __restrict__ in, double in_sc
   }
 }
 
-template <typename T, int E, typename Tin>
+template <typename T, int E, typename Tin, typename C = cpx<T>>
 __global__ void __launch_bounds__(256)
-kw_rows_r2c(Tin* __restrict__ in, double in_scale, int zero_input, cpx<T>* __restrict__ out, int rows,
+kw_rows_r2c(Tin* __restrict__ in, double in_scale, int zero_input, C* __restrict__ out, int rows,
             double* mass_acc) {
   pdl_wait();
   __shared__ cpx<T> tw[tw_len<T, E>()];
@@ -917,22 +919,22 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // to shared column `col + c` (c < nb).  ASYNC (single precision, the library's
 // own arrays, 8-byte aligned): all of them in flight at once as asynchronous
 // copies; the caller's wait is included, a block barrier is not.
-template <typename T, int N, int BC, bool ASYNC>
-__device__ __forceinline__ void load_tile(const cpx<T>* src, int B, int nb, cpx<T>* buf, int LD, int col) {
+template <typename T, int N, int BC, bool ASYNC, typename C>
+__device__ __forceinline__ void load_tile(const C* src, int B, int nb, cpx<T>* buf, int LD, int col) {
   for (int t = threadIdx.x; t < N * BC; t += blockDim.x) {
     const int j = t / BC, c = t - j * BC;
     if constexpr (ASYNC && sizeof(T) == 4) {
       if (c < nb) cp_async8(buf + tpad(j, LD, col + c), src + (size_t)j * B + c);
     } else {
-      buf[tpad(j, LD, col + c)] = c < nb ? src[(size_t)j * B + c] : cpx<T>{T(0), T(0)};
+      buf[tpad(j, LD, col + c)] = c < nb ? cpx<T>(src[(size_t)j * B + c]) : cpx<T>{T(0), T(0)};
     }
   }
 }
 
 // c2c along the middle axis of [A][H][B]: a block stages an H x BC tile
 // (coalesced row segments), warps transform its columns from shared memory.
-template <typename T, int E, int DIR, int BC, bool ASYNC = false>
-__device__ __forceinline__ void cols_body(cpx<T>* __restrict__ base, int B, T scale, int b0, const cpx<T>* tw,
+template <typename T, int E, int DIR, int BC, bool ASYNC = false, typename C>
+__device__ __forceinline__ void cols_body(C* __restrict__ base, int B, T scale, int b0, const cpx<T>* tw,
                                           cpx<T>* buf) {
   constexpr int N = 32 * E, LD = BC + 1;
   const int nb = min(BC, B - b0);
@@ -951,14 +953,14 @@ __device__ __forceinline__ void cols_body(cpx<T>* __restrict__ base, int B, T sc
   }
 }
 
-template <typename T, int E, int DIR, int BC>
+template <typename T, int E, int DIR, int BC, typename C = cpx<T>>
 __global__ void __launch_bounds__(256)
-kw_cols(cpx<T>* __restrict__ data, int B, size_t comp_stride, T scale) {
+kw_cols(C* __restrict__ data, int B, size_t comp_stride, T scale) {
   pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* tw = reinterpret_cast<cpx<T>*>(smem_raw);
   load_tw_group<T, E, false>(tw);
-  cpx<T>* base = data + blockIdx.z * comp_stride + (size_t)blockIdx.y * (32 * E) * B;
+  C* base = data + blockIdx.z * comp_stride + (size_t)blockIdx.y * (32 * E) * B;
   cols_body<T, E, DIR, BC>(base, B, scale, blockIdx.x * BC, tw, tw + tw_len<T, E>());
 }
 
@@ -1228,8 +1230,8 @@ kw_spectral_x(const cpx<T>* T1, cpx<T>* __restrict__ alpha, cpx<T>* __restrict__
 // Rows c2r: each warp takes a row pair of every component, rebuilds the
 // full pencil Z = A + i B from the Hermitian halves, inverse-transforms it,
 // and writes (gx, gy, gz, 0) nodes (NCOMP == 3) or a plain grid (NCOMP == 1).
-template <typename T, int E, int NCOMP>
-__device__ __forceinline__ void rows_c2r_body(const cpx<T>* in, size_t comp_stride, T* __restrict__ out,
+template <typename T, int E, int NCOMP, typename C>
+__device__ __forceinline__ void rows_c2r_body(const C* in, size_t comp_stride, T* __restrict__ out,
                                               int rows, double* max_acc, int bx, int gx, const cpx<T>* tw,
                                               cpx<T>* zb_all, T* ob_all) {
   constexpr int N = 32 * E, NH = N / 2 + 1;
@@ -1249,11 +1251,11 @@ __device__ __forceinline__ void rows_c2r_body(const cpx<T>* in, size_t comp_stri
     for (int c0 = 0; c0 < cnt; c0 += chunk) {
       const int cc = min(chunk, cnt - c0), q0 = p0 + c0;
       for (int d = 0; d < NCOMP; ++d) {
-        const cpx<T>* src = in + d * comp_stride;
+        const C* src = in + d * comp_stride;
         group_c2r_pairs<T, N>(
             cc, 0, tw + kTwLen,
             [&](int pr, int k, cpx<T>& A, cpx<T>& B) {
-              const cpx<T>* ra = src + (size_t)(2 * (q0 + pr)) * NH;
+              const C* ra = src + (size_t)(2 * (q0 + pr)) * NH;
               A = ra[k];
               B = ra[NH + k];
             },
@@ -1276,8 +1278,8 @@ __device__ __forceinline__ void rows_c2r_body(const cpx<T>* in, size_t comp_stri
   const int nwarps = gx * 8;
   for (int pr = bx * 8 + wib; pr < rows / 2; pr += nwarps) {
     for (int d = 0; d < NCOMP; ++d) {
-      const cpx<T>* ra = in + d * comp_stride + (size_t)(2 * pr) * NH;
-      const cpx<T>* rb = ra + NH;
+      const C* ra = in + d * comp_stride + (size_t)(2 * pr) * NH;
+      const C* rb = ra + NH;
       for (int k = lane; k < NH; k += 32) {
         cpx<T> A = ra[k], Bv = rb[k];
         if (k == 0 || k == N / 2) {
@@ -1332,9 +1334,9 @@ __device__ __forceinline__ void rows_c2r_body(const cpx<T>* in, size_t comp_stri
   }
 }
 
-template <typename T, int E, int NCOMP>
+template <typename T, int E, int NCOMP, typename C = cpx<T>>
 __global__ void __launch_bounds__(256)
-kw_rows_c2r(const cpx<T>* in, size_t comp_stride, T* __restrict__ out, int rows, double* max_acc) {
+kw_rows_c2r(const C* in, size_t comp_stride, T* __restrict__ out, int rows, double* max_acc) {
   pdl_wait();
   constexpr int N = 32 * E;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -2219,22 +2221,23 @@ static int warp_blocks(int rows) {
   return b > 152 * 8 ? 152 * 8 : (b < 1 ? 1 : b);
 }
 
-template <typename T, int E>
-static cudaError_t warp_rows_r2c(const void* in, int in_kind, double in_scale, bool zero_input, cpx<T>* out, int rows,
+template <typename T, int E, typename C>
+static cudaError_t warp_rows_r2c(const void* in, int in_kind, double in_scale, bool zero_input, C* out, int rows,
                                  double* mass_acc, cudaStream_t s) {
+  const int zero = zero_input ? 1 : 0;
   if (in_kind == 0)
-    launch_k(kw_rows_r2c<T, E, T>, warp_blocks(rows), 256, 0, s, (T*)in, in_scale, zero_input ? 1 : 0, out, rows, mass_acc);
-  else
-    launch_k(kw_rows_r2c<T, E, unsigned long long>, warp_blocks(rows), 256, 0, s, (unsigned long long*)in, in_scale,
-                                                                           zero_input ? 1 : 0, out, rows, mass_acc);
-  return cudaGetLastError();
+    return launch_k(kw_rows_r2c<T, E, T, C>, warp_blocks(rows), 256, 0, s, (T*)in, in_scale, zero, out, rows, mass_acc);
+  if constexpr (std::is_same<C, cpx<T>>::value)
+    return launch_k(kw_rows_r2c<T, E, unsigned long long>, warp_blocks(rows), 256, 0, s, (unsigned long long*)in,
+                    in_scale, zero, out, rows, mass_acc);
+  return cudaErrorInvalidValue;
 }
 
-template <typename T, int E, int DIR>
-static cudaError_t warp_cols(cpx<T>* data, int A, int B, int ncomp, size_t comp_stride, double scale, cudaStream_t s) {
+template <typename T, int E, int DIR, typename C>
+static cudaError_t warp_cols(C* data, int A, int B, int ncomp, size_t comp_stride, double scale, cudaStream_t s) {
   constexpr int BC = 16;
   const size_t smem = (tw_len<T, E>() + (size_t)32 * E * (BC + 1) + E) * sizeof(cpx<T>);
-  auto k = kw_cols<T, E, DIR, BC>;
+  auto k = kw_cols<T, E, DIR, BC, C>;
   cudaError_t e = allow_smem((const void*)k, smem);
   if (e != cudaSuccess) return e;
   dim3 grid((B + BC - 1) / BC, A, ncomp);
@@ -2266,12 +2269,12 @@ static cudaError_t warp_spectral(const cpx<T>* T1, cpx<T>* alpha, cpx<T>* T2, Sp
   }
 }
 
-template <typename T, int E, int NCOMP>
-static cudaError_t warp_rows_c2r(const cpx<T>* in, size_t comp_stride, T* out, int rows, double* max_acc,
+template <typename T, int E, int NCOMP, typename C>
+static cudaError_t warp_rows_c2r(const C* in, size_t comp_stride, T* out, int rows, double* max_acc,
                                  cudaStream_t s) {
   constexpr int NOUT = NCOMP == 3 ? 4 : 1;
   const size_t smem = row_c2r_smem<T, E, NOUT>();
-  auto k = kw_rows_c2r<T, E, NCOMP>;
+  auto k = kw_rows_c2r<T, E, NCOMP, C>;
   cudaError_t e = allow_smem((const void*)k, smem);
   if (e != cudaSuccess) return e;
   launch_k(k, warp_blocks(rows), 256, smem, s, in, comp_stride, out, rows, max_acc);
@@ -2299,8 +2302,8 @@ static int rows_per_pair_block(int H, int rows, size_t elem, bool with_out4) {
   return rp;
 }
 
-template <typename T>
-cudaError_t launch_rows_r2c(const void* in, int in_kind, double in_scale, bool zero_input, cpx<T>* out,
+template <typename T, typename C>
+cudaError_t launch_rows_r2c(const void* in, int in_kind, double in_scale, bool zero_input, C* out,
                             int H, int rows, double* mass_acc, cudaStream_t s) {
   if (H == 32) return warp_rows_r2c<T, 1>(in, in_kind, in_scale, zero_input, out, rows, mass_acc, s);
   if (H == 64) return warp_rows_r2c<T, 2>(in, in_kind, in_scale, zero_input, out, rows, mass_acc, s);
@@ -2311,17 +2314,18 @@ cudaError_t launch_rows_r2c(const void* in, int in_kind, double in_scale, bool z
   const size_t smem = (kNmax / 2 + (size_t)RP * (H + 1)) * sizeof(cpx<T>);
   const int blocks = (rows + 2 * RP - 1) / (2 * RP);
   cudaError_t e;
+  const int nt = RP > 2 ? kThreads : kSmallThreads, zero = zero_input ? 1 : 0;
   if (in_kind == 0) {
-    auto k = k_rows_r2c<T, T>;
+    auto k = k_rows_r2c<T, T, C>;
     if ((e = allow_smem((const void*)k, smem)) != cudaSuccess) return e;
-    launch_k(k, blocks, RP > 2 ? kThreads : kSmallThreads, smem, s, (T*)in, in_scale, zero_input ? 1 : 0, out, lgH, rows, RP, mass_acc);
-  } else {
+    return launch_k(k, blocks, nt, smem, s, (T*)in, in_scale, zero, out, lgH, rows, RP, mass_acc);
+  }
+  if constexpr (std::is_same<C, cpx<T>>::value) {
     auto k = k_rows_r2c<T, unsigned long long>;
     if ((e = allow_smem((const void*)k, smem)) != cudaSuccess) return e;
-    launch_k(k, blocks, RP > 2 ? kThreads : kSmallThreads, smem, s, (unsigned long long*)in, in_scale, zero_input ? 1 : 0, out, lgH, rows,
-                                     RP, mass_acc);
+    return launch_k(k, blocks, nt, smem, s, (unsigned long long*)in, in_scale, zero, out, lgH, rows, RP, mass_acc);
   }
-  return cudaGetLastError();
+  return cudaErrorInvalidValue;
 }
 
 template <typename T>
@@ -2332,8 +2336,8 @@ static int col_chunk(int H, int slots) {
   return bc;
 }
 
-template <typename T>
-cudaError_t launch_cols(cpx<T>* data, int H, int A, int B, int ncomp, size_t comp_stride, int dir, double scale,
+template <typename T, typename C>
+cudaError_t launch_cols(C* data, int H, int A, int B, int ncomp, size_t comp_stride, int dir, double scale,
                         cudaStream_t s) {
   if (H == 32) return dir < 0 ? warp_cols<T, 1, -1>(data, A, B, ncomp, comp_stride, scale, s)
                               : warp_cols<T, 1, +1>(data, A, B, ncomp, comp_stride, scale, s);
@@ -2352,11 +2356,11 @@ cudaError_t launch_cols(cpx<T>* data, int H, int A, int B, int ncomp, size_t com
   dim3 grid((B + BC - 1) / BC, A, ncomp);
   cudaError_t e;
   if (dir < 0) {
-    auto k = k_cols<T, -1>;
+    auto k = k_cols<T, -1, C>;
     if ((e = allow_smem((const void*)k, smem)) != cudaSuccess) return e;
     launch_k(k, grid, nt, smem, s, data, lgH, B, lgBC, comp_stride, (T)scale);
   } else {
-    auto k = k_cols<T, +1>;
+    auto k = k_cols<T, +1, C>;
     if ((e = allow_smem((const void*)k, smem)) != cudaSuccess) return e;
     launch_k(k, grid, nt, smem, s, data, lgH, B, lgBC, comp_stride, (T)scale);
   }
@@ -2408,33 +2412,30 @@ cudaError_t launch_spectral_x(const cpx<T>* T1, cpx<T>* alpha, cpx<T>* T2, int H
   return cudaErrorInvalidValue;
 }
 
-template <typename T>
-cudaError_t launch_rows_c2r(const cpx<T>* in, int ncomp, size_t comp_stride, T* out, int H, int rows,
-                            double* max_acc, cudaStream_t s) {
-  if (H == 32) return ncomp == 3 ? warp_rows_c2r<T, 1, 3>(in, comp_stride, out, rows, nullptr, s)
-                                 : warp_rows_c2r<T, 1, 1>(in, comp_stride, out, rows, max_acc, s);
-  if (H == 64) return ncomp == 3 ? warp_rows_c2r<T, 2, 3>(in, comp_stride, out, rows, nullptr, s)
-                                 : warp_rows_c2r<T, 2, 1>(in, comp_stride, out, rows, max_acc, s);
-  if (H == 128) return ncomp == 3 ? warp_rows_c2r<T, 4, 3>(in, comp_stride, out, rows, nullptr, s)
-                                  : warp_rows_c2r<T, 4, 1>(in, comp_stride, out, rows, max_acc, s);
-  if (H == 256) return ncomp == 3 ? warp_rows_c2r<T, 8, 3>(in, comp_stride, out, rows, nullptr, s)
-                                  : warp_rows_c2r<T, 8, 1>(in, comp_stride, out, rows, max_acc, s);
+template <typename T, int NCOMP, typename C>
+static cudaError_t rows_c2r_comps(const C* in, size_t comp_stride, T* out, int H, int rows, double* max_acc,
+                                  cudaStream_t s) {
+  if (H == 32) return warp_rows_c2r<T, 1, NCOMP>(in, comp_stride, out, rows, max_acc, s);
+  if (H == 64) return warp_rows_c2r<T, 2, NCOMP>(in, comp_stride, out, rows, max_acc, s);
+  if (H == 128) return warp_rows_c2r<T, 4, NCOMP>(in, comp_stride, out, rows, max_acc, s);
+  if (H == 256) return warp_rows_c2r<T, 8, NCOMP>(in, comp_stride, out, rows, max_acc, s);
   const int lgH = ilog2(H);
   const int RP = rows_per_pair_block(H, rows, sizeof(T), true);
-  const int NOUT = ncomp == 3 ? 4 : 1;
+  const int NOUT = NCOMP == 3 ? 4 : 1;
   const size_t smem = (kNmax / 2 + (size_t)RP * (H + 1)) * sizeof(cpx<T>) + (size_t)2 * RP * H * NOUT * sizeof(T);
   const int blocks = (rows + 2 * RP - 1) / (2 * RP);
-  cudaError_t e;
-  if (ncomp == 3) {
-    auto k = k_rows_c2r<T, 3>;
-    if ((e = allow_smem((const void*)k, smem)) != cudaSuccess) return e;
-    launch_k(k, blocks, RP > 2 ? kThreads : kSmallThreads, smem, s, in, comp_stride, out, lgH, rows, RP, nullptr);
-  } else {
-    auto k = k_rows_c2r<T, 1>;
-    if ((e = allow_smem((const void*)k, smem)) != cudaSuccess) return e;
-    launch_k(k, blocks, RP > 2 ? kThreads : kSmallThreads, smem, s, in, comp_stride, out, lgH, rows, RP, max_acc);
-  }
-  return cudaGetLastError();
+  auto k = k_rows_c2r<T, NCOMP, C>;
+  const cudaError_t e = allow_smem((const void*)k, smem);
+  if (e != cudaSuccess) return e;
+  return launch_k(k, blocks, RP > 2 ? kThreads : kSmallThreads, smem, s, in, comp_stride, out, lgH, rows, RP, max_acc);
+}
+
+template <typename T, typename C>
+cudaError_t launch_rows_c2r(const C* in, int ncomp, size_t comp_stride, T* out, int H, int rows, double* max_acc,
+                            cudaStream_t s) {
+  if (ncomp != 3) return rows_c2r_comps<T, 1>(in, comp_stride, out, H, rows, max_acc, s);
+  if constexpr (std::is_same<C, cpx<T>>::value) return rows_c2r_comps<T, 3>(in, comp_stride, out, H, rows, nullptr, s);
+  return cudaErrorInvalidValue;
 }
 
 template <typename T, int E, int BC>
@@ -2676,18 +2677,21 @@ cudaError_t launch_field_batch(const FftRun<T>* runs, int nruns, int H, int stag
   return cudaErrorInvalidValue;
 }
 
+#define SIPF_INST_C(T, C)                                                                                     \
+  template cudaError_t launch_rows_r2c<T, C>(const void*, int, double, bool, C*, int, int, double*, cudaStream_t); \
+  template cudaError_t launch_cols<T, C>(C*, int, int, int, int, size_t, int, double, cudaStream_t);           \
+  template cudaError_t launch_rows_c2r<T, C>(const C*, int, size_t, T*, int, int, double*, cudaStream_t);
 #define SIPF_INST(T)                                                                                          \
-  template cudaError_t launch_rows_r2c<T>(const void*, int, double, bool, cpx<T>*, int, int, double*,        \
-                                          cudaStream_t);                                                    \
-  template cudaError_t launch_cols<T>(cpx<T>*, int, int, int, int, size_t, int, double, cudaStream_t);       \
+  SIPF_INST_C(T, cpx<T>)                                                                                      \
+  SIPF_INST_C(T, cpx_parts<T>)                                                                                \
   template cudaError_t launch_spectral_x<T>(const cpx<T>*, cpx<T>*, cpx<T>*, int, SpecParams, int, double*,  \
                                             cudaStream_t);                                                  \
-  template cudaError_t launch_rows_c2r<T>(const cpx<T>*, int, size_t, T*, int, int, double*, cudaStream_t);     \
   template cudaError_t launch_field_batch<T>(const FftRun<T>*, int, int, int, cudaStream_t, const FieldTune&, int*); \
   template bool field_tune_valid<T>(int, const FieldTune&);                                                   \
   template FieldTune field_tune_default<T>(int);
 SIPF_INST(float)
 SIPF_INST(double)
 #undef SIPF_INST
+#undef SIPF_INST_C
 
 }  // namespace sipf

@@ -1104,43 +1104,36 @@ int sipf_gather_dev(int precision, const void* x, const void* y, const void* z, 
   return SIPF_OK;
 }
 
-// The transforms' kernels take complex values as one 8- or 16-byte access; a
-// caller's spectrum at a lesser alignment goes through an aligned copy.
 }  // extern "C"
 
 namespace {
-template <typename Fn>
-int with_aligned_spec(void* spec, int precision, int32_t H, bool in, bool out, cudaStream_t s, Fn&& fn) {
-  const size_t esz = precision == 64 ? 16 : 8;
-  if ((reinterpret_cast<uintptr_t>(spec) & (esz - 1)) == 0) return fn(spec);
-  const size_t bytes = (size_t)H * H * (H / 2 + 1) * esz;
-  void* tmp = nullptr;
-  SIPF_CK(cudaMallocAsync(&tmp, bytes, s));
-  int r = SIPF_OK;
-  cudaError_t e = in ? cudaMemcpyAsync(tmp, spec, bytes, cudaMemcpyDeviceToDevice, s) : cudaSuccess;
-  if (e == cudaSuccess) r = fn(tmp);
-  if (e == cudaSuccess && !r && out) e = cudaMemcpyAsync(spec, tmp, bytes, cudaMemcpyDeviceToDevice, s);
-  const cudaError_t ef = cudaFreeAsync(tmp, s);
-  if (r) return r;
-  if (e == cudaSuccess) e = ef;
-  return e == cudaSuccess ? SIPF_OK : cuda_fail(e, "aligned copy of the spectrum");
-}
-
-template <typename T> int forward_ft(int32_t H, double L, const void* grid, void* spec, cudaStream_t s) {
+// C: cpx<T>, or cpx_parts<T> for a caller's spectrum at a lesser alignment.
+template <typename T, typename C> int forward_ft(int32_t H, double L, const void* grid, void* spec, cudaStream_t s) {
   const int nh = H / 2 + 1;
-  cpx<T>* o = (cpx<T>*)spec;
+  C* o = (C*)spec;
   SIPF_CK(launch_rows_r2c<T>(grid, 0, 1.0, false, o, H, H * H, nullptr, s));
   SIPF_CK(launch_cols<T>(o, H, H, nh, 1, 0, -1, 1.0, s));
   SIPF_CK(launch_cols<T>(o, H, 1, H * nh, 1, 0, -1, 1.0 / (L * L * L), s));
   return SIPF_OK;
 }
-template <typename T> int inverse_ft(int32_t H, void* spec, void* grid, cudaStream_t s) {
+template <typename T, typename C> int inverse_ft(int32_t H, void* spec, void* grid, cudaStream_t s) {
   const int nh = H / 2 + 1;
-  cpx<T>* o = (cpx<T>*)spec;
+  C* o = (C*)spec;
   SIPF_CK(launch_cols<T>(o, H, 1, H * nh, 1, 0, +1, 1.0, s));
   SIPF_CK(launch_cols<T>(o, H, H, nh, 1, 0, +1, 1.0, s));
   SIPF_CK(launch_rows_c2r<T>(o, 1, 0, (T*)grid, H, H * H, nullptr, s));
   return SIPF_OK;
+}
+template <typename T> bool whole_complex(const void* spec) {
+  return (reinterpret_cast<uintptr_t>(spec) & (sizeof(cpx<T>) - 1)) == 0;
+}
+template <typename T> int forward_ft_any(int32_t H, double L, const void* grid, void* spec, cudaStream_t s) {
+  return whole_complex<T>(spec) ? forward_ft<T, cpx<T>>(H, L, grid, spec, s)
+                                : forward_ft<T, cpx_parts<T>>(H, L, grid, spec, s);
+}
+template <typename T> int inverse_ft_any(int32_t H, void* spec, void* grid, cudaStream_t s) {
+  return whole_complex<T>(spec) ? inverse_ft<T, cpx<T>>(H, spec, grid, s)
+                                : inverse_ft<T, cpx_parts<T>>(H, spec, grid, s);
 }
 }  // namespace
 
@@ -1151,9 +1144,7 @@ int sipf_forward_ft_dev(int precision, int32_t H, double L, const void* grid, vo
   if (!is_pow2(H) || H < 8 || H > kNmax || !(L > 0) || !grid || !spec) return fail(SIPF_EINVAL, "forward_ft args");
   SIPF_CK(ensure_device_tables());
   cudaStream_t s = (cudaStream_t)stream;
-  return with_aligned_spec(spec, precision, H, false, true, s, [&](void* o) {
-    return precision == 64 ? forward_ft<double>(H, L, grid, o, s) : forward_ft<float>(H, L, grid, o, s);
-  });
+  return precision == 64 ? forward_ft_any<double>(H, L, grid, spec, s) : forward_ft_any<float>(H, L, grid, spec, s);
 }
 
 int sipf_inverse_ft_dev(int precision, int32_t H, void* spec, void* grid, void* stream) {
@@ -1161,9 +1152,7 @@ int sipf_inverse_ft_dev(int precision, int32_t H, void* spec, void* grid, void* 
   if (!is_pow2(H) || H < 8 || H > kNmax || !grid || !spec) return fail(SIPF_EINVAL, "inverse_ft args");
   SIPF_CK(ensure_device_tables());
   cudaStream_t s = (cudaStream_t)stream;
-  return with_aligned_spec(spec, precision, H, true, true, s, [&](void* o) {
-    return precision == 64 ? inverse_ft<double>(H, o, grid, s) : inverse_ft<float>(H, o, grid, s);
-  });
+  return precision == 64 ? inverse_ft_any<double>(H, spec, grid, s) : inverse_ft_any<float>(H, spec, grid, s);
 }
 
 }  // extern "C"
@@ -1216,7 +1205,8 @@ extern "C" int sipf_inverse_ft_noalloc_dev(int precision, int32_t H, const void*
   if (r) return r;
   cudaStream_t s = (cudaStream_t)stream;
   SIPF_CK(cudaMemcpyAsync(work, spec, bytes, cudaMemcpyDeviceToDevice, s));
-  return precision == 64 ? inverse_ft<double>(H, work, grid, s) : inverse_ft<float>(H, work, grid, s);
+  return precision == 64 ? inverse_ft<double, cpx<double>>(H, work, grid, s)
+                         : inverse_ft<float, cpx<float>>(H, work, grid, s);
 }
 
 // ===========================================================================

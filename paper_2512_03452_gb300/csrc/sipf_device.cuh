@@ -12,6 +12,17 @@ namespace sipf {
 // Aligned to its size, so that a value is one 8- or 16-byte access (without the
 // alignment every load and store of a complex value is two).
 template <typename T> struct alignas(2 * sizeof(T)) cpx { T x, y; };
+// A complex value in a caller's array that is only aligned to its real type:
+// two accesses of one part each.  The transforms' kernels take either.
+template <typename T> struct cpx_parts {
+  T x, y;
+  __device__ __forceinline__ operator cpx<T>() const { return cpx<T>{x, y}; }
+  __device__ __forceinline__ cpx_parts& operator=(const cpx<T>& v) {
+    x = v.x;
+    y = v.y;
+    return *this;
+  }
+};
 
 // Programmatic dependent launch (see launch_k): in a grid of at most
 // kPdlBlocks blocks, waits until the kernel before this one has completed and

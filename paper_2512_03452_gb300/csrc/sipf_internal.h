@@ -137,13 +137,13 @@ cudaError_t ensure_device_tables();
 // rows r2c: `rows` real rows of length H (in) -> half-spectrum rows (out).
 // in_kind: 0 = T, 1 = int64 fixed point scaled by in_scale.  zero_input
 // clears the input after reading.  mass_acc (nullable) receives the FP64 sum.
-template <typename T>
+template <typename T, typename C>
 cudaError_t launch_rows_r2c(const void* in, int in_kind, double in_scale, bool zero_input,
-                            cpx<T>* out, int H, int rows, double* mass_acc, cudaStream_t s);
+                            C* out, int H, int rows, double* mass_acc, cudaStream_t s);
 // c2c along the middle axis of [A][H][B] complex arrays, ncomp arrays spaced
 // comp_stride apart.  dir = -1 forward, +1 inverse.
-template <typename T>
-cudaError_t launch_cols(cpx<T>* data, int H, int A, int B, int ncomp, size_t comp_stride, int dir,
+template <typename T, typename C>
+cudaError_t launch_cols(C* data, int H, int A, int B, int ncomp, size_t comp_stride, int dir,
                         double scale, cudaStream_t s);
 // x-axis pass fused with the spectral work (see SpecMode).
 template <typename T>
@@ -152,8 +152,8 @@ cudaError_t launch_spectral_x(const cpx<T>* T1, cpx<T>* alpha, cpx<T>* T2, int H
 // rows c2r of ncomp (1 or 3) half-spectrum arrays spaced comp_stride apart;
 // ncomp == 3 writes interleaved 4-wide nodes (gx, gy, gz, 0), ncomp == 1 a
 // plain real grid.  max_acc (nullable, ncomp == 1): FP64 max of the output.
-template <typename T>
-cudaError_t launch_rows_c2r(const cpx<T>* in, int ncomp, size_t comp_stride, T* out, int H,
+template <typename T, typename C>
+cudaError_t launch_rows_c2r(const C* in, int ncomp, size_t comp_stride, T* out, int H,
                             int rows, double* max_acc, cudaStream_t s);
 
 // The whole field solve of a step (F_H of phi, update of alpha, gradient
