@@ -1760,11 +1760,14 @@ k_deposit_vec(const float* x, const float* y, const float* z, int64_t P,
   }
 }
 
+// The stateless gathers do not overlap the caller's kernels (no pdl_wait), so
+// their inputs may take the read-only path, which leaves the compiler free to
+// order the loads: with the wait and plain loads 34 -> 38 us for 1e6 particles,
+// three grids of 32^3.
 template <typename T>
 __global__ void __launch_bounds__(256)
-k_gather(const T* x, const T* y, const T* z, int64_t P, Geo<T> g,
-         const T* f, int ncomp, int order, T* __restrict__ out) {
-  pdl_wait();
+k_gather(const T* __restrict__ x, const T* __restrict__ y, const T* __restrict__ z, int64_t P, Geo<T> g,
+         const T* __restrict__ f, int ncomp, int order, T* __restrict__ out) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const size_t N = (size_t)g.H * g.H * g.H;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += stride) {
@@ -1782,15 +1785,17 @@ k_gather(const T* x, const T* y, const T* z, int64_t P, Geo<T> g,
   }
 }
 
-// Gamma_2 gather in single precision from 16-byte aligned grids: the two z nodes
-// of an (x, y) column by one 16-byte load of their quad (and a second load where
-// they straddle two), instead of a load each: the kernel is bound by the L1's
-// lookups, one a lane for particles in random order.  Same order of the sums as
-// k_gather: 60 -> 48 us for 1e6 unsorted particles, three grids of 128^3.
+// Gamma_2 gather in single precision from 8-byte aligned grids: the two z nodes of
+// an (x, y) column by one 8-byte load where the first is even, else by a load
+// each.  The kernel is bound by the L1's lookups, one a lane for particles in
+// random order.  Same order of the sums as k_gather.  us for three grids, k_gather
+// -> here, particles unsorted / sorted by tiles of 8^3 cells: P = 1e6, H = 128 61 -> 51 /
+// 38 -> 36; H = 64 51 -> 42 / 36 -> 34; H = 32 34 -> 30 / 32 -> 34; P = 4e6, H = 32
+// 140 -> 99 / 127 -> 117.  (One 16-byte load of the column's quad: 50 / 44 at P = 1e6,
+// H = 128, and 34 / 42 at H = 32: sorted particles' lanes share words, not quads.)
 __global__ void __launch_bounds__(256)
-k_gather2_vec(const float* x, const float* y, const float* z, int64_t P,
-              Geo<float> g, const float* f, int ncomp, float* __restrict__ out) {
-  pdl_wait();
+k_gather2_pairs(const float* __restrict__ x, const float* __restrict__ y, const float* __restrict__ z, int64_t P,
+              Geo<float> g, const float* __restrict__ f, int ncomp, float* __restrict__ out) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const size_t N = (size_t)g.H * g.H * g.H;
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += stride) {
@@ -1800,27 +1805,30 @@ k_gather2_vec(const float* x, const float* y, const float* z, int64_t P,
     cell_lambda(y[p], g, cy, ly);
     cell_lambda(z[p], g, cz, lz);
     const float wx[2] = {1.f - lx, lx}, wy[2] = {1.f - ly, ly}, wz[2] = {1.f - lz, lz};
-    const int z0 = cz & g.mask, z1 = (cz + 1) & g.mask, o = z0 & 3;
+    const int z0 = cz & g.mask, z1 = (cz + 1) & g.mask;
     int col[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) col[k] = (((cx + (k >> 1)) & g.mask) * g.H + ((cy + (k & 1)) & g.mask)) * g.H;
     for (int c = 0; c < ncomp; ++c) {
       const float* fc = f + c * N;
-      float4 q[4];
-      float n[4];
+      float v0[4], v1[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        q[k] = *reinterpret_cast<const float4*>(fc + col[k] + (z0 & ~3));
-        n[k] = o == 3 ? fc[col[k] + z1] : 0.f;
+        if (z0 & 1) {
+          v0[k] = fc[col[k] + z0];
+          v1[k] = fc[col[k] + z1];
+        } else {
+          const float2 q = *reinterpret_cast<const float2*>(fc + col[k] + z0);
+          v0[k] = q.x;
+          v1[k] = q.y;
+        }
       }
       float acc = 0.f;
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        const float v0 = o == 0 ? q[k].x : o == 1 ? q[k].y : o == 2 ? q[k].z : q[k].w;
-        const float v1 = o == 0 ? q[k].y : o == 1 ? q[k].z : o == 2 ? q[k].w : n[k];
         const float wab = wx[k >> 1] * wy[k & 1];
-        acc += wab * wz[0] * v0;
-        acc += wab * wz[1] * v1;
+        acc += wab * wz[0] * v0[k];
+        acc += wab * wz[1] * v1[k];
       }
       out[(size_t)c * P + p] = acc;
     }
@@ -2154,10 +2162,10 @@ template <typename T>
 cudaError_t launch_gather(const T* x, const T* y, const T* z, int64_t P, Geo<T> g, const T* f, int ncomp, int order,
                           T* out, cudaStream_t s) {
   if constexpr (sizeof(T) == 4) {
-    if (order == 2 && (reinterpret_cast<uintptr_t>(f) & 15) == 0)
-      return launch_k(k_gather2_vec, grid_for(P, 256), 256, 0, s, x, y, z, P, g, f, ncomp, out);
+    if (order == 2 && (reinterpret_cast<uintptr_t>(f) & 7) == 0)
+      return launch_plain(k_gather2_pairs, grid_for(P, 256), 256, 0, s, x, y, z, P, g, f, ncomp, out);
   }
-  return launch_k(k_gather<T>, grid_for(P, 256), 256, 0, s, x, y, z, P, g, f, ncomp, order, out);
+  return launch_plain(k_gather<T>, grid_for(P, 256), 256, 0, s, x, y, z, P, g, f, ncomp, order, out);
 }
 
 template <typename T>
