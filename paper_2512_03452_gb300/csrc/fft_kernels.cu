@@ -2195,7 +2195,7 @@ __global__ void __launch_bounds__(1024) kwc_inv(const FftRun<T>* __restrict__ ru
 template <typename K, typename... Args>
 static cudaError_t launch_cluster(K with_wait, K without, dim3 grid, int threads, size_t smem, int cs, cudaStream_t s,
                                   Args... args) {
-  const bool dep = grid.x * grid.y * grid.z <= kPdlBlocks;
+  const bool dep = grid.x * grid.y * grid.z <= one_wave(threads, smem);
   K kernel = dep ? with_wait : without;
   const cudaError_t e = allow_smem((const void*)kernel, smem);
   if (e != cudaSuccess) return e;
@@ -2488,7 +2488,7 @@ static cudaError_t kwb_spectral_launch(const FftRun<T>* runs, int nruns, int nw,
     if (smr > kMaxSmem) return cudaErrorInvalidValue;
     if ((e = allow_smem((const void*)kwrb_spectral_x<N, true>, smr)) != cudaSuccess) return e;
     if ((e = allow_smem((const void*)kwrb_spectral_x<N, false>, smr)) != cudaSuccess) return e;
-    return launch_sized(kwrb_spectral_x<N, true>, kwrb_spectral_x<N, false>,
+    return launch_sized(kwrb_spectral_x<N, true>, kwrb_spectral_x<N, false>, kPdlBlocks,
                         dim3((XRegShape<N>::TASKS + nw - 1) / nw, nruns), 32 * nw, smr, s, runs);
   } else {
     if (nw == 0) nw = kDefaultSpectralWarps;
@@ -2557,7 +2557,8 @@ static cudaError_t field_batch_e(const FftRun<T>* runs, int nruns, int stages, c
     } else if (planes) {
       if ((e = allow_smem((const void*)kwp_fwd<T, E, true>, fsm)) != cudaSuccess) return e;
       if ((e = allow_smem((const void*)kwp_fwd<T, E, false>, fsm)) != cudaSuccess) return e;
-      e = launch_sized(kwp_fwd<T, E, true>, kwp_fwd<T, E, false>, dim3(N, nruns), 32 * fnw, fsm, s, runs);
+      e = launch_sized(kwp_fwd<T, E, true>, kwp_fwd<T, E, false>, one_wave(32 * fnw, fsm), dim3(N, nruns), 32 * fnw, fsm,
+                       s, runs);
       if (e != cudaSuccess) return e;
       nk += 1;
     } else {
@@ -2593,7 +2594,8 @@ static cudaError_t field_batch_e(const FftRun<T>* runs, int nruns, int stages, c
   } else if ((stages & kFieldInverse) && planes) {
     if ((e = allow_smem((const void*)kwp_inv<T, E, true>, ism)) != cudaSuccess) return e;
     if ((e = allow_smem((const void*)kwp_inv<T, E, false>, ism)) != cudaSuccess) return e;
-    e = launch_sized(kwp_inv<T, E, true>, kwp_inv<T, E, false>, dim3(N, 3, nruns), 32 * inw, ism, s, runs);
+    e = launch_sized(kwp_inv<T, E, true>, kwp_inv<T, E, false>, one_wave(32 * inw, ism), dim3(N, 3, nruns), 32 * inw, ism,
+                     s, runs);
     if (e != cudaSuccess) return e;
     nk += 1;
   } else if (stages & kFieldInverse) {

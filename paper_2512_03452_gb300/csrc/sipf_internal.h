@@ -69,7 +69,9 @@ template <typename T> inline SpecConst<T> spec_const(const SpecParams& sp) {
 // 201 us; x pass 170 -> 198; inverse plane kernel of 8 runs at H = 128, 3072
 // blocks: 272 -> 366).
 // launch_sized: a kernel in both forms, with and without the wait, for grids
-// that may be small or large.
+// that may be small or large: the wait where at most `most` blocks are launched,
+// for a kernel of few blocks per SM its first wave (inverse plane kernel of two
+// runs at H = 128, 768 blocks of which 456 are resident: 72 us without, 85 with).
 template <typename... KA, typename... A>
 inline cudaError_t launch_plain(void (*kernel)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                                 A&&... args) {
@@ -95,11 +97,16 @@ inline cudaError_t launch_k(void (*kernel)(KA...), dim3 grid, dim3 block, size_t
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 
+inline unsigned one_wave(unsigned threads, size_t smem) {
+  const unsigned by_threads = 2048 / threads, by_smem = (unsigned)(228 * 1024 / (smem + 1024));
+  const unsigned blocks = 152 * (by_threads < by_smem ? by_threads : by_smem);
+  return blocks < kPdlBlocks ? blocks : kPdlBlocks;
+}
 template <typename... KA, typename... A>
-inline cudaError_t launch_sized(void (*with_wait)(KA...), void (*without)(KA...), dim3 grid, dim3 block, size_t smem,
-                                cudaStream_t s, A&&... args) {
-  return grid.x * grid.y * grid.z <= kPdlBlocks ? launch_k(with_wait, grid, block, smem, s, std::forward<A>(args)...)
-                                                : launch_plain(without, grid, block, smem, s, std::forward<A>(args)...);
+inline cudaError_t launch_sized(void (*with_wait)(KA...), void (*without)(KA...), unsigned most, dim3 grid, dim3 block,
+                                size_t smem, cudaStream_t s, A&&... args) {
+  return grid.x * grid.y * grid.z <= most ? launch_k(with_wait, grid, block, smem, s, std::forward<A>(args)...)
+                                          : launch_plain(without, grid, block, smem, s, std::forward<A>(args)...);
 }
 
 // Dynamic shared memory above 48 KB has to be allowed per kernel first, and the
