@@ -2656,6 +2656,8 @@ template <typename T> FieldTune field_tune_default(int H) {
   return t;
 }
 
+template <typename T> bool field_rows_tunable(int H) { return !(H == 256 && group_rows<T, 256>()); }
+
 template <typename T> bool field_tune_valid(int H, const FieldTune& t) {
   switch (H) {
     case 32: return field_tune_valid_e<T, 1>(t);
@@ -2690,6 +2692,7 @@ cudaError_t launch_field_batch(const FftRun<T>* runs, int nruns, int H, int stag
                                             cudaStream_t);                                                  \
   template cudaError_t launch_field_batch<T>(const FftRun<T>*, int, int, int, cudaStream_t, const FieldTune&, int*); \
   template bool field_tune_valid<T>(int, const FieldTune&);                                                   \
+  template bool field_rows_tunable<T>(int);                                                                   \
   template FieldTune field_tune_default<T>(int);
 SIPF_INST(float)
 SIPF_INST(double)

@@ -1445,6 +1445,7 @@ template <typename T> int batch_autotune_impl(sipf_batch* b, int trial, sipf_bat
     // pencil-pass shapes (which only matter if pencils won)
     static const std::vector<int> cand[7] = {{0, 1, 2}, {8, 16, 32}, {1, 2}, {4, 8, 16}, {8, 16}, {8, 16, 32}, {4, 8, 16}};
     for (int dim = 0; dim < 7; ++dim) {
+      if (dim == 6 && !field_rows_tunable<T>(b->group_H[g])) continue;   // three times the same launch
       for (int v : cand[dim]) {
         FieldTune t = best_t;
         int* f[7] = {&t.plane_mode, &t.plane_nw, &t.inv3, &t.sbc, &t.spec_nw, &t.bc, &t.rows_per_sm};

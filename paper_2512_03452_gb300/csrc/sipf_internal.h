@@ -180,7 +180,7 @@ struct FieldTune {
   int plane_mode = 0;   // 0: plane kernels for the inner axes where they fit (H <= 128), 1: pencil passes,
                         // 2: cluster plane kernels (H >= 64; each x-plane over 2 or 4 blocks)
   int plane_nw = 0;     // warps per block of the plane kernels (8, 16, 32)
-  int spec_nw = 0;      // warps per block of the fused x pass (8, 16)
+  int spec_nw = 0;      // warps per block of the fused x pass (8, 16; 0: by the number of pencils)
   int inv3 = 0;         // inverse plane kernel: 0 by grid size, 1 one block per x-plane for all three
                         // gradient components (H <= 64), 2 one block per (component, x-plane)
 };
@@ -189,6 +189,8 @@ cudaError_t launch_field_batch(const FftRun<T>* runs, int nruns, int H, int stag
                                const FieldTune& tune = FieldTune{}, int* launched = nullptr);   // += kernels launched
 template <typename T> bool field_tune_valid(int H, const FieldTune& t);
 template <typename T> FieldTune field_tune_default(int H);   // the shapes used when a field is 0
+// Whether rows_per_sm has an effect (not in single precision at H = 256: one row pair per group of lanes).
+template <typename T> bool field_rows_tunable(int H);
 
 // FP64 FMA throughput probe: blocks x 256 threads x 8 chains x iters FMAs.
 cudaError_t launch_fp64_fma(int blocks, int iters, double* sink, cudaStream_t s);
