@@ -1465,8 +1465,8 @@ __global__ void __launch_bounds__(256) kwb_rows_c2r(const FftRun<T>* __restrict_
 // soon as registers are free (the persistent pass over row pairs left the
 // memory idle between a warp's pairs: 76 -> 71 us at H = 256).
 template <int N, typename Tin>
-__device__ __forceinline__ void rows_r2c_pair(Tin* __restrict__ in, double in_scale, cpx<float>* __restrict__ out, int pr,
-                                              int q, const cpx<float>* twq, cpx<float>* z) {
+__device__ __forceinline__ void rows_r2c_pair(Tin* __restrict__ in, double in_scale, cpx<float>* __restrict__ out,
+                                              int pr, int q, const cpx<float>* twq, cpx<float>* z) {
   using T = float;
   constexpr int F = GroupShape<N>::F, Q = GroupShape<N>::Q, R = F / Q, NH = N / 2 + 1;
   constexpr int KI = (NH + Q - 1) / Q;
@@ -2551,14 +2551,15 @@ static cudaError_t field_batch_e(const FftRun<T>* runs, int nruns, int stages, c
                                     : tune.inv3 == 0 && nruns * N >= 4 * 152 && 2 * i3sm <= kMaxSmem);
   if (stages & kFieldForward) {
     if (clusters) {
-      e = launch_cluster(kwc_fwd<T, E, CS, true>, kwc_fwd<T, E, CS, false>, dim3(N * CS, nruns), 32 * cnw, csm, CS, s, runs);
+      e = launch_cluster(kwc_fwd<T, E, CS, true>, kwc_fwd<T, E, CS, false>, dim3(N * CS, nruns), 32 * cnw, csm, CS, s,
+                         runs);
       if (e != cudaSuccess) return e;
       nk += 1;
     } else if (planes) {
       if ((e = allow_smem((const void*)kwp_fwd<T, E, true>, fsm)) != cudaSuccess) return e;
       if ((e = allow_smem((const void*)kwp_fwd<T, E, false>, fsm)) != cudaSuccess) return e;
-      e = launch_sized(kwp_fwd<T, E, true>, kwp_fwd<T, E, false>, one_wave(32 * fnw, fsm), dim3(N, nruns), 32 * fnw, fsm,
-                       s, runs);
+      e = launch_sized(kwp_fwd<T, E, true>, kwp_fwd<T, E, false>, one_wave(32 * fnw, fsm), dim3(N, nruns), 32 * fnw,
+                       fsm, s, runs);
       if (e != cudaSuccess) return e;
       nk += 1;
     } else {
@@ -2581,7 +2582,8 @@ static cudaError_t field_batch_e(const FftRun<T>* runs, int nruns, int stages, c
     nk += 1;
   }
   if ((stages & kFieldInverse) && clusters) {
-    e = launch_cluster(kwc_inv<T, E, CS, true>, kwc_inv<T, E, CS, false>, dim3(N * CS, 3, nruns), 32 * cnw, csm, CS, s, runs);
+    e = launch_cluster(kwc_inv<T, E, CS, true>, kwc_inv<T, E, CS, false>, dim3(N * CS, 3, nruns), 32 * cnw, csm, CS, s,
+                       runs);
     if (e != cudaSuccess) return e;
     nk += 1;
   } else if ((stages & kFieldInverse) && inv3) {
@@ -2594,8 +2596,8 @@ static cudaError_t field_batch_e(const FftRun<T>* runs, int nruns, int stages, c
   } else if ((stages & kFieldInverse) && planes) {
     if ((e = allow_smem((const void*)kwp_inv<T, E, true>, ism)) != cudaSuccess) return e;
     if ((e = allow_smem((const void*)kwp_inv<T, E, false>, ism)) != cudaSuccess) return e;
-    e = launch_sized(kwp_inv<T, E, true>, kwp_inv<T, E, false>, one_wave(32 * inw, ism), dim3(N, 3, nruns), 32 * inw, ism,
-                     s, runs);
+    e = launch_sized(kwp_inv<T, E, true>, kwp_inv<T, E, false>, one_wave(32 * inw, ism), dim3(N, 3, nruns), 32 * inw,
+                     ism, s, runs);
     if (e != cudaSuccess) return e;
     nk += 1;
   } else if (stages & kFieldInverse) {

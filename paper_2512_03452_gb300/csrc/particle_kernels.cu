@@ -19,6 +19,7 @@
 //             to the grid with coalesced reductions; the bins of a merged
 //             item a warp each, in windows of one copy.  Particles outside the
 //             window (the overflow bin) deposit with global reductions.
+//             Grids up to 16^3 are a single tile: k_deposit_whole.
 // Batched forms take the work items of many runs from one counter.  Also
 // here: the re-binning of particle-order arrays, the read-backs to particle
 // order (through a slot map, or by pieces of ids) and the bin-order copy of
@@ -649,7 +650,7 @@ __device__ __forceinline__ void rebin_run(const BinArgs<T>& a, long long start, 
 
 // Work items are taken from a global counter by persistent blocks.  Thread 0
 // takes the next item's index when the current item starts and loads its
-// description when fn calls mid(), by when the counter's answer has come
+// description when fn calls load(), by when the counter's answer has come
 // back, so that neither latency lies between two items (batch of 24 runs, which
 // also searched the runs for each item: move 62.5 -> 60.5 us a step, deposit 61.1
 // -> 60.2).
@@ -720,7 +721,7 @@ k_binned_rebin(const __grid_constant__ BinArgs<T> a) {
       rebin_run(a, cur.start, cur.len, threadIdx.x, blockDim.x);
       return true;
     }
-      for (int k = threadIdx.x >> 5; k < kMerge; k += (int)(blockDim.x >> 5)) {   // a warp per small bin
+    for (int k = threadIdx.x >> 5; k < kMerge; k += (int)(blockDim.x >> 5)) {   // a warp per small bin
       const int b = (int)cur.start * kMerge + k;
       const int c = b < a.NT ? a.src_count[b] : 0;
       if (bin_is_small(b, c, a.NT, a.small)) rebin_run(a, a.src_base[b], c, threadIdx.x & 31, 32);
@@ -1242,8 +1243,8 @@ k_chunk_emit(ChunkListArgs a, unsigned long long* work, unsigned long long* ovf_
   chunk_emit_body(a, blockIdx.x, gridDim.x, work, ovf_total);
 }
 
-// Both passes by one block, where it holds all bins (H <= 64): one launch less in every step of a small run
-// (4.4 -> 3.0 us of kernels).
+// Both passes by one block, where it holds all bins (H <= 64): one launch less in
+// every step of a small run (4.4 -> 3.0 us of kernels).
 __global__ void __launch_bounds__(kCLBlock)
 k_chunk_list_one(ChunkListArgs a, unsigned long long* work, unsigned long long* ovf_total) {
   pdl_wait();
@@ -1932,11 +1933,12 @@ int binned_tile_shift(int H) { return H <= 16 ? 30 : kTileShift; }
 // items each, so that few particles still spread over the chip and the last
 // wave of many is short, but long enough that a tile window's flush stays
 // small next to its particles.  Measured per step (us) by item length:
-//   FP32, P = 1e7, H = 128: 512 612, 2048 455, 4096 453; P = 1e6, H = 64: 512 103,
-//   1024 95, 4096 110; P = 2e5, H = 64: 128 78, 512 63, 2048 63; P = 16384,
-//   H = 32: 64 to 256 46, 1024 54, 4096 65;
-//   FP64 (the FP64 pipe wants every SM busy), P = 1e6, H = 64: 256 1170, 1024
-//   1159, 4096 1273; P = 1e4, H = 16 (whole-grid tile): 32 98, 64 86, 256 124, 4096 866.
+//   FP32, P = 1e7, H = 128: 512 617, 2048 463, 4096 468; P = 1e6, H = 64: 512 88,
+//   1024 80, 4096 106; P = 2e5, H = 64: 128 60, 512 49, 2048 56; P = 16384,
+//   H = 32: 64 to 256 28 to 29, 1024 37, 4096 38;
+//   FP64 (the FP64 pipe wants every SM busy), P = 1e6, H = 64: 256 1006, 1024
+//   1041, 4096 1845; P = 1e4, H = 16 (one tile, whose deposit has ranges of its
+//   own): 32 69, 64 60, 256 67, 4096 314.
 int particle_chunk(int64_t P, int H, bool fp64) {
   const int least = H <= 16 ? kChunkMin : fp64 ? 128 : P < (1 << 16) ? 256 : 512;
   int c = kChunkMax;
@@ -2068,10 +2070,8 @@ bool launch_rebin_plain(const T* x, const T* y, const T* z, const uint32_t* id, 
                         const int* dst_cap, int* dst_cursor, int* err, cudaStream_t s, cudaError_t* e, int64_t id0,
                         bool wrap) {
   if (NT > kMaxSmemTiles) return false;
-  launch_k(k_rebin_plain<T>, plain_blocks(P), 256, NT * sizeof(int), s, x, y, z, id, P, g, shift, ntx, NT, dx, dy, dz, did,
-                                                                 dst_base, dst_cap, dst_cursor, err, id0,
-                                                                 wrap ? 1 : 0);
-  *e = cudaGetLastError();
+  *e = launch_k(k_rebin_plain<T>, plain_blocks(P), 256, NT * sizeof(int), s, x, y, z, id, P, g, shift, ntx, NT, dx, dy,
+                dz, did, dst_base, dst_cap, dst_cursor, err, id0, wrap ? 1 : 0);
   return true;
 }
 
@@ -2109,8 +2109,8 @@ cudaError_t launch_read_back_mapped(const BinArgs<T>& a, int64_t max_chunks, uin
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int64_t b = (P + 255) / 256;
-  launch_k(k_gather_slots<T>, (unsigned)(b > 152 * 16 ? 152 * 16 : b), 256, 0, s, slot_of, a.sx, a.sy, a.sz, P, x, y, z);
-  return cudaGetLastError();
+  return launch_k(k_gather_slots<T>, (unsigned)(b > 152 * 16 ? 152 * 16 : b), 256, 0, s, slot_of, a.sx, a.sy, a.sz, P, x,
+                  y, z);
 }
 
 template <typename T>

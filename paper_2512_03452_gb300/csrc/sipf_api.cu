@@ -1340,8 +1340,8 @@ template <typename T> int batch_issue_step(sipf_batch* b) {
     SIPF_CK(mark(2 * g + 1));
   }
   SIPF_CK(mark(2 * G));
-  SIPF_CK(launch_move_batch<T>((const BinArgs<T>*)b->move_tab[b->cur][b->lc], b->list, b->prefix + R, b->work + 1, b->step, true,
-                               s, b->move_bps, b->g2p));
+  SIPF_CK(launch_move_batch<T>((const BinArgs<T>*)b->move_tab[b->cur][b->lc], b->list, b->prefix + R, b->work + 1,
+                               b->step, true, s, b->move_bps, b->g2p));
   SIPF_CK(launch_chunk_list_batch(b->cl_tab[1 - b->cur][b->lc], R, b->max_NT, b->prefix, b->work, b->step, 1, b->list,
                                   s));
   SIPF_CK(mark(2 * G + 1));
@@ -1350,8 +1350,8 @@ template <typename T> int batch_issue_step(sipf_batch* b) {
   b->cur = 1 - b->cur;
   if (++b->since >= kBatchResort) {
     SIPF_CK(launch_layout_batch(b->ly_tab[b->cur][1 - b->lc], R, s));
-    SIPF_CK(launch_move_batch<T>((const BinArgs<T>*)b->rebin_tab[b->cur][b->lc], b->list, b->prefix + R, b->work, b->step, false,
-                                 s, b->move_bps));
+    SIPF_CK(launch_move_batch<T>((const BinArgs<T>*)b->rebin_tab[b->cur][b->lc], b->list, b->prefix + R, b->work,
+                                 b->step, false, s, b->move_bps));
     SIPF_CK(launch_chunk_list_batch(b->cl_tab[1 - b->cur][1 - b->lc], R, b->max_NT, b->prefix, b->work, b->step, 0,
                                     b->list, s));
     b->launches += 5;
@@ -1360,8 +1360,8 @@ template <typename T> int batch_issue_step(sipf_batch* b) {
     b->since = 0;
   }
   SIPF_CK(mark(2 * G + 2));
-  SIPF_CK(launch_deposit_batch<T>((const BinArgs<T>*)b->dep_tab[b->cur][b->lc], b->list, b->prefix + R, b->work, b->fixed, s,
-                                  b->dep_bps));
+  SIPF_CK(launch_deposit_batch<T>((const BinArgs<T>*)b->dep_tab[b->cur][b->lc], b->list, b->prefix + R, b->work,
+                                  b->fixed, s, b->dep_bps));
   SIPF_CK(mark(2 * G + 3));
   b->launches += 1;
   b->n += 1;
