@@ -171,13 +171,16 @@ constexpr int kChunkMax = 4096, kChunkMin = 64;
 // their 32 reductions per particle.
 constexpr int kWinMinLen = 64;
 // Sparse bins are taken together: the bins with fewer than `small` particles
-// (the overflow bin excepted) of each window of kMerge consecutive bins form
+// (the overflow bin excepted) of each window of `merge` consecutive bins form
 // one work item, marked by bin = -1 with the window index in `start` and the
 // bins' total in `len`.  A sparse region then costs the move one round per
-// window instead of one per bin, and the deposit a warp per bin: a block has
-// kMerge warps.  (Windows of 4 and 16 bins: 241 and 267 us per step of a batch
-// of 24 runs against 237; torus of 1e7 453 and 445 against 446.)
-constexpr int kMerge = 8;
+// window instead of one per bin, and the deposit a warp per bin.  `merge` (a power
+// of two) is 8, the block's warps, and 16 for the runs of a batch with few
+// particles a tile (see particle_merge).
+// MERGE, a template parameter of the move and the deposit: kMerge, or 0 for the
+// window in the run's arguments (as an argument everywhere it costs a run of 1e6
+// particles at H = 32 1.7%: 69.8 -> 71.0 us a step).
+constexpr int kMerge = 8, kMergeMax = 16;
 constexpr int kSmallMax = 240;   // (see merged_k)
 // In a merged item's deposit, a warp takes a bin of at least this many
 // particles into a window of its own (below it: global reductions).
@@ -194,8 +197,8 @@ __device__ __forceinline__ void item_slots(const BinArgs<T>& a, const ChunkDesc&
     for (int i = threadIdx.x; i < d.len; i += blockDim.x) fn(d.start + i);
     return;
   }
-  for (int k = 0; k < kMerge; ++k) {
-    const int b = (int)d.start * kMerge + k;
+  for (int k = 0; k < a.merge; ++k) {
+    const int b = (int)d.start * a.merge + k;
     if (b > a.NT) break;
     const int c = a.src_count[b];
     if (!bin_is_small(b, c, a.NT, a.small)) continue;
@@ -503,15 +506,16 @@ __device__ __forceinline__ long long window_sum(long long v) { return v; }
 // item run beside one another with no block barrier.  (Taken one after another
 // by the whole block, a bin of some 80 particles cost about 10 us of barriers
 // and dependent loads, and an item was as many of them.)
-template <typename T, bool FIXED>
+template <typename T, bool FIXED, int MERGE>
 __device__ __forceinline__ void deposit_merged(const BinArgs<T>& a, const ChunkDesc& cur,
                                                typename WinType<T>::type* win) {
   using A = typename WinType<T>::type;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = (int)(blockDim.x >> 5);
   const int H = a.g.H, mask = a.g.mask;
   A* const ww = win + warp * kWinSlots;
-  for (int k = warp; k < kMerge; k += nwarps) {
-    const int b = (int)cur.start * kMerge + k;
+  const int merge = MERGE ? MERGE : a.merge;
+  for (int k = warp; k < merge; k += nwarps) {
+    const int b = (int)cur.start * merge + k;
     const int c = b < a.NT ? a.src_count[b] : 0;
     if (!bin_is_small(b, c, a.NT, a.small)) continue;
     const long long s0 = a.src_base[b];
@@ -690,7 +694,7 @@ __device__ __forceinline__ void for_items(const Item* list, long long n, unsigne
   }
 }
 
-template <typename T, bool FIXED>
+template <typename T, bool FIXED, int MERGE>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2)
 k_binned_deposit(const __grid_constant__ BinArgs<T> a) {
   using A = typename WinType<T>::type;
@@ -704,7 +708,7 @@ k_binned_deposit(const __grid_constant__ BinArgs<T> a) {
       deposit_chunk<T, FIXED>(a, cur, win, fetch);
     } else {
       fetch.load();
-      deposit_merged<T, FIXED>(a, cur, win);
+      deposit_merged<T, FIXED, MERGE>(a, cur, win);
     }
     return true;
   });
@@ -721,8 +725,8 @@ k_binned_rebin(const __grid_constant__ BinArgs<T> a) {
       rebin_run(a, cur.start, cur.len, threadIdx.x, blockDim.x);
       return true;
     }
-    for (int k = threadIdx.x >> 5; k < kMerge; k += (int)(blockDim.x >> 5)) {   // a warp per small bin
-      const int b = (int)cur.start * kMerge + k;
+    for (int k = threadIdx.x >> 5; k < a.merge; k += (int)(blockDim.x >> 5)) {   // a warp per small bin
+      const int b = (int)cur.start * a.merge + k;
       const int c = b < a.NT ? a.src_count[b] : 0;
       if (bin_is_small(b, c, a.NT, a.small)) rebin_run(a, a.src_base[b], c, threadIdx.x & 31, 32);
     }
@@ -748,7 +752,7 @@ k_deposit_batch(const BinArgs<T>* __restrict__ table, const BatchItem* list,
       deposit_chunk<T, FIXED>(a, cur.d, win, fetch);
     } else {
       fetch.load();
-      deposit_merged<T, FIXED>(a, cur.d, win);
+      deposit_merged<T, FIXED, 0>(a, cur.d, win);
     }
     return true;
   });
@@ -783,8 +787,8 @@ struct MoveSmem {
   int meta[R];        // neighbour slot (0..124) | rank << 7, or -1 - tile for far moves
   int cnt[kNbr], base[kNbr], tile[kNbr], cap[kNbr];
   long long gbase[kNbr];   // first slot of each destination bin
-  long long seg_base[kMerge];   // merged items: first slot and particles of each small bin
-  int seg_cnt[kMerge];
+  long long seg_base[kMergeMax];   // merged items: first slot and particles of each small bin
+  int seg_cnt[kMergeMax];
   __align__(8) uint64_t bar;
   int abort;
 };
@@ -864,15 +868,17 @@ template <typename T> __device__ __forceinline__ void move_write_out(const BinAr
 // source tiles, are read straight from their bins in rounds, moved, staged
 // and written out, each reserving its own destination slot (sparse bins, so
 // the destination cursors see little contention).
-template <typename T, bool MOVE, int G2P, typename Fetch>
+template <typename T, bool MOVE, int G2P, int MERGE, typename Fetch>
 __device__ __forceinline__ void move_merged(const BinArgs<T>& a, const ChunkDesc& cur, uint32_t n, MoveSmem<T>& sm,
                                             Fetch& fetch) {
   constexpr int R = MoveRound<T>::n;
-  if (threadIdx.x < kMerge) {
-    const int b = (int)cur.start * kMerge + threadIdx.x;
+  constexpr int most = MERGE ? MERGE : kMergeMax;
+  const int merge = MERGE ? MERGE : a.merge;
+  if (threadIdx.x < most) {
+    const int b = (int)cur.start * merge + threadIdx.x;
     int c = 0;
     long long base = 0;
-    if (b <= a.NT) {
+    if ((int)threadIdx.x < merge && b <= a.NT) {
       c = a.src_count[b];
       base = a.src_base[b];
       if (!bin_is_small(b, c, a.NT, a.small)) c = 0;
@@ -888,7 +894,7 @@ __device__ __forceinline__ void move_merged(const BinArgs<T>& a, const ChunkDesc
     for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
       // the bin holding item particle r0 + i
       int k = 0, o = r0 + i;
-      while (k < kMerge - 1 && o >= sm.seg_cnt[k]) o -= sm.seg_cnt[k++];
+      while (k < most - 1 && o >= sm.seg_cnt[k]) o -= sm.seg_cnt[k++];
       const long long slot = sm.seg_base[k] + o;
       T x = a.sx[slot], y = a.sy[slot], z = a.sz[slot];
       const uint32_t id = a.sid[slot];
@@ -922,11 +928,11 @@ __device__ __forceinline__ void prefetch_round(const BinArgs<T>& a, long long s0
 // fetch: the block's next work item, loaded while this one's first round is
 // staged; its first round is prefetched (args_of: its run's arguments) during
 // this item's last round.
-template <typename T, bool MOVE, int G2P, typename Fetch, typename ArgsOf>
+template <typename T, bool MOVE, int G2P, int MERGE, typename Fetch, typename ArgsOf>
 __device__ __forceinline__ void move_chunk(const BinArgs<T>& a, const ChunkDesc& cur, uint32_t n, MoveSmem<T>& sm,
                                            uint32_t& phase, Fetch& fetch, ArgsOf&& args_of) {
   if (cur.bin < 0) {
-    move_merged<T, MOVE, G2P>(a, cur, n, sm, fetch);
+    move_merged<T, MOVE, G2P, MERGE>(a, cur, n, sm, fetch);
     return;
   }
   constexpr int R = MoveRound<T>::n;
@@ -1017,7 +1023,7 @@ __device__ __forceinline__ void move_chunk(const BinArgs<T>& a, const ChunkDesc&
   }
 }
 
-template <typename T, int G2P>
+template <typename T, int G2P, int MERGE>
 __global__ void __launch_bounds__(kMoveThreads, move_min_blocks<T>())
 k_move(BinArgs<T> a) {
   pdl_wait();
@@ -1029,8 +1035,8 @@ k_move(BinArgs<T> a) {
   uint32_t phase = 0;
   for_items(a.chunks, a.chunk_start[a.NT + 1], a.work, reinterpret_cast<ChunkDesc*>(sm.item),
             [&](const ChunkDesc& cur, auto& fetch) {
-              move_chunk<T, true, G2P>(a, cur, a.n, sm, phase, fetch,
-                                       [&](const ChunkDesc&) -> const BinArgs<T>& { return a; });
+              move_chunk<T, true, G2P, MERGE>(a, cur, a.n, sm, phase, fetch,
+                                              [&](const ChunkDesc&) -> const BinArgs<T>& { return a; });
               return sm.abort == 0;
             });
 }
@@ -1051,8 +1057,8 @@ k_move_batch(const BinArgs<T>* __restrict__ table, const BatchItem* list,
   }
   uint32_t phase = 0;
   for_items(list, *total, work, sm.item, [&](const BatchItem& cur, auto& fetch) {
-    move_chunk<T, MOVE, G2P>(table[cur.run], cur.d, n, sm, phase, fetch,
-                             [&](const BatchItem& i) -> const BinArgs<T>& { return table[i.run]; });
+    move_chunk<T, MOVE, G2P, 0>(table[cur.run], cur.d, n, sm, phase, fetch,
+                                [&](const BatchItem& i) -> const BinArgs<T>& { return table[i.run]; });
     return sm.abort == 0;
   });
 }
@@ -1075,7 +1081,8 @@ static cudaError_t resident_blocks(const void* kern, int threads, size_t smem, i
 // lengthen the launch.)
 template <typename T> cudaError_t launch_move(const BinArgs<T>& a, cudaStream_t s) {
   int blocks = 0;
-  auto k = a.g2p == 4 ? k_move<T, 4> : k_move<T, 2>;
+  auto k = a.merge == kMerge ? (a.g2p == 4 ? k_move<T, 4, kMerge> : k_move<T, 2, kMerge>)
+                             : (a.g2p == 4 ? k_move<T, 4, 0> : k_move<T, 2, 0>);
   const cudaError_t e = resident_blocks((const void*)k, kMoveThreads, 0, &blocks);
   if (e != cudaSuccess) return e;
   launch_k(k, min(blocks, a.max_items), kMoveThreads, 0, s, a);
@@ -1157,11 +1164,11 @@ __device__ __forceinline__ void chunk_count_body(const ChunkListArgs& a, int blk
     ch = small ? 0 : (c + a.chunk - 1) / a.chunk;
     a.other_cursor[b] = 0;
   }
-  // the first bin of a window (kMerge lanes of a warp) also holds the
+  // the first bin of a window (`merge` lanes of a warp) also holds the
   // window's merged item, if it has small bins
   const unsigned sm = __ballot_sync(0xFFFFFFFFu, small);
-  const int lane = threadIdx.x & 31;
-  if ((lane & (kMerge - 1)) == 0 && ((sm >> lane) & ((1u << kMerge) - 1u)) != 0u) ch += 1;
+  const int lane = threadIdx.x & 31, merge = a.merge;
+  if ((lane & (merge - 1)) == 0 && ((sm >> lane) & ((1u << merge) - 1u)) != 0u) ch += 1;
   long long total;
   const long long ex = block_exclusive_scan_ll(ch, total);
   if (b < nb) a.chunk_start[b] = ex;
@@ -1199,15 +1206,17 @@ __device__ __forceinline__ void chunk_emit_body(const ChunkListArgs& a, int blk,
       if (s_ls[i + step] <= q) i += step;
     const int bin = blk * kCLBlock + i;
     int j = (int)(q - s_ls[i]);
-    if ((bin & (kMerge - 1)) == 0) {
+    const int merge = a.merge;
+    if ((bin & (merge - 1)) == 0) {
       int tot = 0;
-      for (int k = 0; k < kMerge && bin + k < nb; ++k) {
-        const int cc = a.count[bin + k];
+#pragma unroll
+      for (int k = 0; k < kMergeMax; ++k) {   // (all counts loaded at once)
+        const int cc = k < merge && bin + k < nb ? a.count[bin + k] : 0;
         if (bin_is_small(bin + k, cc, a.NT, a.small)) tot += cc;
       }
       if (tot > 0) {
         if (j == 0) {   // the window's merged item comes first
-          const ChunkDesc d{(long long)(bin / kMerge), -1, tot};
+          const ChunkDesc d{(long long)(bin >> (__ffs(merge) - 1)), -1, tot};
           a.chunks[off + q] = d;
           if (list) list[off + q] = BatchItem{d, run, 0};
           continue;
@@ -1515,15 +1524,15 @@ k_compact(BinArgs<T> a, unsigned long long* cursor, T* __restrict__ ox, T* __res
   pdl_wait();
   // a merged item's bins looked up together, then its particles copied in one
   // pass (bin after bin, each lookup waited for, 14.3 -> 6.2 us for 2e5 particles)
-  __shared__ long long s_out, s_base[kMerge];
-  __shared__ int s_cnt[kMerge];
+  __shared__ long long s_out, s_base[kMergeMax];
+  __shared__ int s_cnt[kMergeMax];
   const long long c = blockIdx.x;
   if (c >= a.chunk_start[a.NT + 1]) return;
   const ChunkDesc d = a.chunks[c];
-  if (threadIdx.x < kMerge) {
-    const int b = (int)d.start * kMerge + threadIdx.x;
+  if (threadIdx.x < kMergeMax) {
+    const int b = (int)d.start * a.merge + threadIdx.x;
     int n = 0;
-    if (d.bin < 0 && b < a.NT) {
+    if (d.bin < 0 && (int)threadIdx.x < a.merge && b < a.NT) {
       n = a.src_count[b];
       if (!bin_is_small(b, n, a.NT, a.small)) n = 0;
     }
@@ -1537,7 +1546,7 @@ k_compact(BinArgs<T> a, unsigned long long* cursor, T* __restrict__ ox, T* __res
     long long s = d.start + i;
     if (d.bin < 0) {
       int k = 0, j = i;
-      while (k < kMerge - 1 && j >= s_cnt[k]) j -= s_cnt[k++];
+      while (k < kMergeMax - 1 && j >= s_cnt[k]) j -= s_cnt[k++];
       s = s_base[k] + j;
     }
     ox[o + i] = a.sx[s];
@@ -1945,11 +1954,20 @@ int particle_chunk(int64_t P, int H, bool fp64) {
   while (c > least && P / c < 152 * 6) c >>= 1;
   return c;
 }
-// A merged item (up to kMerge bins) is then at most twice an item of one bin.
+// A merged item of eight bins is then at most twice an item of one bin.
 int particle_small(int chunk) {
   const int s = chunk / 4;
   return s > kSmallMax ? kSmallMax : s < 32 ? 32 : s;
 }
+
+// Bins of a merge window: 8; 16 for a run of a batch with fewer than 16 particles
+// a tile, whose items are short and many (us per step with 8 and with 16: 32 runs
+// of 1e4 at H = 128, 2.4 a tile, 2266 and 2150, of 6e4, 15 a tile, 2629 and 2536;
+// at H = 64 32 runs of 1000, 2 a tile, 282 and 272, of 1e4, 20 a tile, 351 and
+// 357, of 6e4 425 and 454).  A run by itself has too few items to be short of
+// blocks (P = 1e4, H = 64: 40 and 49); windows of 4: 241 us per step of 24 runs of
+// 1e4 to 1e5 against 237 with 8 and 267 with 16.
+int particle_merge(int64_t P, int NT, bool in_batch) { return in_batch && P < 16 * (int64_t)NT ? kMergeMax : kMerge; }
 
 // Particles of a block of k_deposit_whole: some 40 windows up to 4096 particles
 // each.  The windows' sums are added in floating point, and more windows of
@@ -1975,9 +1993,10 @@ template <typename T, bool FIXED> static cudaError_t launch_deposit_t(const BinA
     return launch_k(k_deposit_whole<T, FIXED>, ranges < blocks ? (int)ranges : blocks, 256, smem, s, a, len);
   }
   const size_t smem = (size_t)kTileReps * kWinSlots * sizeof(A);
-  const cudaError_t e = resident_blocks((const void*)k_binned_deposit<T, FIXED>, 256, smem, &blocks);
+  auto k = a.merge == kMerge ? k_binned_deposit<T, FIXED, kMerge> : k_binned_deposit<T, FIXED, 0>;
+  const cudaError_t e = resident_blocks((const void*)k, 256, smem, &blocks);
   if (e != cudaSuccess) return e;
-  return launch_k(k_binned_deposit<T, FIXED>, min(blocks, a.max_items), 256, smem, s, a);
+  return launch_k(k, min(blocks, a.max_items), 256, smem, s, a);
 }
 
 template <typename T> cudaError_t launch_binned_deposit(const BinArgs<T>& a, cudaStream_t s) {

@@ -190,7 +190,7 @@ struct sipf_ctx {
   bool fixed() const { return p.deposit_mode == SIPF_DEPOSIT_DETERMINISTIC; }
   int64_t max_chunks() const { return p.P / chunk + NT + 2; }
   int resort() const { return p.resort_every > 0 ? p.resort_every : 16; }
-  int chunk = 4096, small = 256;   // work-item length and merge threshold (particle_chunk, particle_small)
+  int chunk = 0, small = 0, merge = 0;   // work-item length, merge threshold and window (particle_chunk, _small, _merge)
 };
 
 enum { kDscMass = 0, kDscAlpha0 = 1, kDscM2 = 2, kDscRing = 3, kDscHF = 4, kDscTot = 5, kDscMax = 6, kDscCount = 8 };
@@ -263,6 +263,7 @@ template <typename T> BinArgs<T> bin_args(sipf_ctx* c, int src_buf, int src_lay,
   a.tile_shift = c->shift;
   a.max_items = (int)std::min<int64_t>(c->max_chunks(), INT32_MAX);
   a.small = c->small;
+  a.merge = c->merge;
   a.P = c->p.P;
   a.phi = c->phi;
   a.grad4 = (const T*)c->grad;
@@ -285,7 +286,7 @@ template <typename T> BinArgs<T> bin_args(sipf_ctx* c, int src_buf, int src_lay,
 // arrays; `other` are the cursors to clear for the next pass.
 ChunkListArgs cl_args(sipf_ctx* c, const int* cursor, const int* cap, const long long* base, int* other) {
   return ChunkListArgs{cursor, cap, base, c->count, c->chunk_start, c->chunks, other, c->NT, c->part,
-                       c->chunk, c->small};
+                       c->chunk, c->small, c->merge};
 }
 
 // The current bins are final (positions of step n, before their deposit):
@@ -832,6 +833,7 @@ int sipf_init(const sipf_params* p, const double* X0, void* stream, sipf_ctx** o
   c->NT = c->ntx * c->ntx * c->ntx;
   c->chunk = particle_chunk(p->P, p->H, p->precision == 64);
   c->small = particle_small(c->chunk);
+  c->merge = particle_merge(p->P, c->NT, false);
   const size_t nb = (size_t)c->NT + 1;
   // bins hold at most 1.5 P + 64 NT + 6 P / 4 (capacities with spare room), the overflow bin P
   c->cap_total = (int64_t)(4 * P + 68 * (size_t)c->NT + 1024);
@@ -1584,6 +1586,7 @@ int sipf_batch_init(int32_t nruns, const sipf_params* params, const double* cons
     // (their counts are unchanged)
     c->chunk = std::max(c->chunk, particle_chunk(total, c->p.H, c->p.precision == 64));
     c->small = particle_small(c->chunk);
+    c->merge = particle_merge(c->p.P, c->NT, true);
     cudaError_t e = launch_chunk_list(cl_args(c, c->cursor[c->cur], c->lcap[c->lc], c->lbase[c->lc],
                                               c->cursor[1 - c->cur]),
                                       c->work, nullptr, c->stream);

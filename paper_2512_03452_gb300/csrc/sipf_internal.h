@@ -259,7 +259,7 @@ struct BinArgs {
   unsigned long long* work;      // chunk counter of the persistent grid (zeroed before the launch)
   int NT, ntx, tile_shift;       // tiles, tiles per axis, log2 tile edge
   int max_items;                 // bound of the number of work items
-  int small;                     // the chunk list's merge threshold (see ChunkListArgs)
+  int small, merge;              // the chunk list's merge threshold and window (see ChunkListArgs)
   int64_t P;                     // particles of the run
   // physics
   void* phi;                     // deposit target (T, or int64 fixed point)
@@ -285,7 +285,8 @@ struct ChunkListArgs {
   int* other_cursor;        // cursors of the other buffer (cleared)
   int NT;
   long long* part;          // chunk totals of the blocks of kCLBlock bins (chunk_list_blocks(NT))
-  int chunk, small;         // most particles of an item of one bin; bins below `small` are merged
+  int chunk, small, merge;  // most particles of an item of one bin; bins below `small` are merged, by windows of
+                            // `merge` bins
 };
 struct LayoutArgs {
   const int* want;
@@ -312,6 +313,8 @@ cudaError_t launch_layout_batch(const LayoutArgs* t, int nruns, cudaStream_t s);
 // Work-item length for P particles on an H^3 grid, and the bin size below which bins are merged.
 int particle_chunk(int64_t P, int H, bool fp64);
 int particle_small(int chunk);
+// Bins of a merge window (NT: tiles of the grid).
+int particle_merge(int64_t P, int NT, bool in_batch);
 int binned_tile_shift(int H);
 // Deposit of the source bins; re-bin of the source bins into the destination bins.
 template <typename T> cudaError_t launch_binned_deposit(const BinArgs<T>& a, cudaStream_t s);
