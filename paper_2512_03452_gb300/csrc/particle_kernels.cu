@@ -177,9 +177,9 @@ constexpr int kWinMinLen = 64;
 // window instead of one per bin, and the deposit a warp per bin.  `merge` (a power
 // of two) is 8, the block's warps, and 16 for the runs of a batch with few
 // particles a tile (see particle_merge).
-// MERGE, a template parameter of the move and the deposit: kMerge, or 0 for the
-// window in the run's arguments (as an argument everywhere it costs a run of 1e6
-// particles at H = 32 1.7%: 69.8 -> 71.0 us a step).
+// MERGE, a template parameter of the move, the deposit and the chunk lists: kMerge,
+// or 0 for the window in the run's arguments (as an argument everywhere it costs a
+// run of 1e6 particles at H = 32 1.7%: 69.8 -> 71.0 us a step).
 constexpr int kMerge = 8, kMergeMax = 16;
 constexpr int kSmallMax = 240;   // (see merged_k)
 // In a merged item's deposit, a warp takes a bin of at least this many
@@ -355,7 +355,11 @@ __device__ __forceinline__ void deposit_chunk(const BinArgs<T>& a, const ChunkDe
   using A = typename WinType<T>::type;
   const int mask = a.g.mask;
   const int lane = threadIdx.x & 31;
-  const int bin = cur.bin, len = cur.len;
+  const int bin = cur.bin, len = cur.dep;
+  if (len == 0) {   // (its particles are another item's)
+    fetch.load();
+    return;
+  }
   const long long start = cur.start;
   const bool has_win = bin < a.NT && len >= kWinMinLen;
   int ox = 0, oy = 0, oz = 0;   // node coordinates of window slot (0,0,0)
@@ -1152,7 +1156,7 @@ __device__ __forceinline__ long long block_exclusive_scan_ll(long long v, long l
   return ex;
 }
 
-__device__ __forceinline__ void chunk_count_body(const ChunkListArgs& a, int blk) {
+template <int MERGE> __device__ __forceinline__ void chunk_count_body(const ChunkListArgs& a, int blk) {
   const int nb = a.NT + 1;
   const int b = blk * kCLBlock + threadIdx.x;
   long long ch = 0;
@@ -1167,7 +1171,7 @@ __device__ __forceinline__ void chunk_count_body(const ChunkListArgs& a, int blk
   // the first bin of a window (`merge` lanes of a warp) also holds the
   // window's merged item, if it has small bins
   const unsigned sm = __ballot_sync(0xFFFFFFFFu, small);
-  const int lane = threadIdx.x & 31, merge = a.merge;
+  const int lane = threadIdx.x & 31, merge = MERGE ? MERGE : a.merge;
   if ((lane & (merge - 1)) == 0 && ((sm >> lane) & ((1u << merge) - 1u)) != 0u) ch += 1;
   long long total;
   const long long ex = block_exclusive_scan_ll(ch, total);
@@ -1175,7 +1179,21 @@ __device__ __forceinline__ void chunk_count_body(const ChunkListArgs& a, int blk
   if (threadIdx.x == 0) a.part[blk] = total;
 }
 
+// Particles of a bin of c that the deposit takes into one window: an item, or as
+// many as leave at most twelve windows to a bin, up to kChunkMax.  The windows'
+// sums are added to the grid in floating point, so a node that holds much of a
+// dense bin rounds once a window; many short items are what the move wants, not
+// the deposit (1.25e5 particles in a few cells, FP32: 1.8e-7 of the grid with
+// windows of 1024, 1.0e-7 with 4096; the peak of the collapsed blob of 1e6, H = 64:
+// 1.5e-7 and 0.8e-7).  It costs the collapsed blob 78 -> 90 us a step, 1e6 particles
+// spread over the box nothing.  (The long ones first, each on an SM of its own: 88.)
+__device__ __forceinline__ int deposit_len(int chunk, int c) {
+  while (chunk < kChunkMax && c > 12 * chunk) chunk <<= 1;
+  return chunk;
+}
+
 // (list: a batch's items, where this run's go from its entry on)
+template <int MERGE>
 __device__ __forceinline__ void chunk_emit_body(const ChunkListArgs& a, int blk, int nblk, unsigned long long* work,
                                                 unsigned long long* ovf_total, BatchItem* list = nullptr, int run = 0) {
   __shared__ long long s_off;
@@ -1206,17 +1224,17 @@ __device__ __forceinline__ void chunk_emit_body(const ChunkListArgs& a, int blk,
       if (s_ls[i + step] <= q) i += step;
     const int bin = blk * kCLBlock + i;
     int j = (int)(q - s_ls[i]);
-    const int merge = a.merge;
+    const int merge = MERGE ? MERGE : a.merge;
     if ((bin & (merge - 1)) == 0) {
       int tot = 0;
 #pragma unroll
-      for (int k = 0; k < kMergeMax; ++k) {   // (all counts loaded at once)
+      for (int k = 0; k < (MERGE ? MERGE : kMergeMax); ++k) {   // (all counts loaded at once)
         const int cc = k < merge && bin + k < nb ? a.count[bin + k] : 0;
         if (bin_is_small(bin + k, cc, a.NT, a.small)) tot += cc;
       }
       if (tot > 0) {
         if (j == 0) {   // the window's merged item comes first
-          const ChunkDesc d{(long long)(bin >> (__ffs(merge) - 1)), -1, tot};
+          const ChunkDesc d{(long long)(bin >> (__ffs(merge) - 1)), -1, tot, tot, 0};
           a.chunks[off + q] = d;
           if (list) list[off + q] = BatchItem{d, run, 0};
           continue;
@@ -1225,7 +1243,8 @@ __device__ __forceinline__ void chunk_emit_body(const ChunkListArgs& a, int blk,
       }
     }
     const int c = a.count[bin];
-    const ChunkDesc d{a.base[bin] + (long long)j * a.chunk, bin, min(a.chunk, c - j * a.chunk)};
+    const int p0 = j * a.chunk, dl = bin < a.NT ? deposit_len(a.chunk, c) : a.chunk;
+    const ChunkDesc d{a.base[bin] + p0, bin, min(a.chunk, c - p0), (p0 & (dl - 1)) == 0 ? min(dl, c - p0) : 0, 0};
     a.chunks[off + q] = d;
     if (list) list[off + q] = BatchItem{d, run, 0};
   }
@@ -1241,25 +1260,27 @@ __device__ __forceinline__ void chunk_emit_body(const ChunkListArgs& a, int blk,
 
 __device__ __forceinline__ int chunk_list_blocks_dev(int NT) { return (NT + 1 + kCLBlock - 1) / kCLBlock; }
 
-__global__ void __launch_bounds__(kCLBlock) k_chunk_count(ChunkListArgs a) {
+template <int MERGE> __global__ void __launch_bounds__(kCLBlock) k_chunk_count(ChunkListArgs a) {
   pdl_wait();
-  chunk_count_body(a, blockIdx.x);
+  chunk_count_body<MERGE>(a, blockIdx.x);
 }
 
+template <int MERGE>
 __global__ void __launch_bounds__(kCLBlock)
 k_chunk_emit(ChunkListArgs a, unsigned long long* work, unsigned long long* ovf_total) {
   pdl_wait();
-  chunk_emit_body(a, blockIdx.x, gridDim.x, work, ovf_total);
+  chunk_emit_body<MERGE>(a, blockIdx.x, gridDim.x, work, ovf_total);
 }
 
 // Both passes by one block, where it holds all bins (H <= 64): one launch less in
 // every step of a small run (4.4 -> 3.0 us of kernels).
+template <int MERGE>
 __global__ void __launch_bounds__(kCLBlock)
 k_chunk_list_one(ChunkListArgs a, unsigned long long* work, unsigned long long* ovf_total) {
   pdl_wait();
-  chunk_count_body(a, 0);
+  chunk_count_body<MERGE>(a, 0);
   __syncthreads();
-  chunk_emit_body(a, 0, 1, work, ovf_total);
+  chunk_emit_body<MERGE>(a, 0, 1, work, ovf_total);
 }
 
 // Batched: grid (blocks of the largest run, runs).
@@ -1267,7 +1288,7 @@ __global__ void __launch_bounds__(kCLBlock) k_chunk_count_batch(const ChunkListA
   pdl_wait();
   const ChunkListArgs a = t[blockIdx.y];
   if ((int)blockIdx.x >= chunk_list_blocks_dev(a.NT)) return;
-  chunk_count_body(a, blockIdx.x);
+  chunk_count_body<0>(a, blockIdx.x);
 }
 
 __global__ void __launch_bounds__(kCLBlock)
@@ -1276,7 +1297,7 @@ k_chunk_emit_batch(const ChunkListArgs* __restrict__ t, const long long* prefix,
   const ChunkListArgs a = t[blockIdx.y];
   const int nblk = chunk_list_blocks_dev(a.NT);
   if ((int)blockIdx.x >= nblk) return;
-  chunk_emit_body(a, blockIdx.x, nblk, nullptr, nullptr, list + prefix[blockIdx.y], blockIdx.y);
+  chunk_emit_body<0>(a, blockIdx.x, nblk, nullptr, nullptr, list + prefix[blockIdx.y], blockIdx.y);
 }
 
 // Work items of a run from its blocks' totals (k_chunk_count_batch).
@@ -2016,12 +2037,12 @@ int chunk_list_blocks(int NT) { return (NT + 1 + kCLBlock - 1) / kCLBlock; }
 cudaError_t launch_chunk_list(const ChunkListArgs& a, unsigned long long* work, unsigned long long* ovf_total,
                               cudaStream_t s) {
   const int nblk = chunk_list_blocks(a.NT);
-  if (nblk == 1) return launch_k(k_chunk_list_one, 1, kCLBlock, 0, s, a, work, ovf_total);
-  launch_k(k_chunk_count, nblk, kCLBlock, 0, s, a);
-  cudaError_t e = cudaGetLastError();
+  const bool own = a.merge == kMerge;
+  if (nblk == 1)
+    return launch_k(own ? k_chunk_list_one<kMerge> : k_chunk_list_one<0>, 1, kCLBlock, 0, s, a, work, ovf_total);
+  const cudaError_t e = launch_k(own ? k_chunk_count<kMerge> : k_chunk_count<0>, nblk, kCLBlock, 0, s, a);
   if (e != cudaSuccess) return e;
-  launch_k(k_chunk_emit, nblk, kCLBlock, 0, s, a, work, ovf_total);
-  return cudaGetLastError();
+  return launch_k(own ? k_chunk_emit<kMerge> : k_chunk_emit<0>, nblk, kCLBlock, 0, s, a, work, ovf_total);
 }
 
 template <typename T>
