@@ -360,7 +360,7 @@ __device__ __forceinline__ void deposit_chunk(const BinArgs<T>& a, const ChunkDe
     fetch.load();
     return;
   }
-  const long long start = cur.start;
+  const long long start = cur.start - cur.back;
   const bool has_win = bin < a.NT && len >= kWinMinLen;
   int ox = 0, oy = 0, oz = 0;   // node coordinates of window slot (0,0,0)
   if (bin < a.NT) tile_origin(bin, a.ntx, ox, oy, oz);
@@ -1186,7 +1186,7 @@ template <int MERGE> __device__ __forceinline__ void chunk_count_body(const Chun
 // the deposit (1.25e5 particles in a few cells, FP32: 1.8e-7 of the grid with
 // windows of 1024, 1.0e-7 with 4096; the peak of the collapsed blob of 1e6, H = 64:
 // 1.5e-7 and 0.8e-7).  It costs the collapsed blob 78 -> 90 us a step, 1e6 particles
-// spread over the box nothing.  (The long ones first, each on an SM of its own: 88.)
+// spread over the box nothing.
 __device__ __forceinline__ int deposit_len(int chunk, int c) {
   while (chunk < kChunkMax && c > 12 * chunk) chunk <<= 1;
   return chunk;
@@ -1243,8 +1243,15 @@ __device__ __forceinline__ void chunk_emit_body(const ChunkListArgs& a, int blk,
       }
     }
     const int c = a.count[bin];
+    // groups of dl / chunk items are deposited with one of them, the first of the
+    // first group, the second of the second, ...: always the first would fall on
+    // every second or fourth block, and so on a part of the SMs
     const int p0 = j * a.chunk, dl = bin < a.NT ? deposit_len(a.chunk, c) : a.chunk;
-    const ChunkDesc d{a.base[bin] + p0, bin, min(a.chunk, c - p0), (p0 & (dl - 1)) == 0 ? min(dl, c - p0) : 0, 0};
+    const int lgG = __ffs(dl) - __ffs(a.chunk), group = j >> lgG, first = group << lgG;
+    const int items = min(1 << lgG, (c + a.chunk - 1) / a.chunk - first);
+    const bool carries = j - first == min(group & ((1 << lgG) - 1), items - 1);
+    const ChunkDesc d{a.base[bin] + p0, bin, min(a.chunk, c - p0), carries ? min(dl, c - first * a.chunk) : 0,
+                      carries ? p0 - first * a.chunk : 0};
     a.chunks[off + q] = d;
     if (list) list[off + q] = BatchItem{d, run, 0};
   }

@@ -234,7 +234,7 @@ cudaError_t launch_adj_spectral(const cpx<T>* ghat, cpx<T>* abar, cpx<T>* spec, 
 struct ChunkDesc {
   long long start;
   int bin, len;
-  int dep, pad;   // particles from `start` on that the deposit takes with this item (0: with an item before it)
+  int dep, back;   // the deposit's share: `dep` particles from slot start - back on (0: another item's)
 };
 
 // One work item of a batch: run `run`'s item d.
