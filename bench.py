@@ -37,20 +37,20 @@ P_FULL, H_FULL = 10_000_000, 128
 # algorithmic bytes of the particle kernel per particle-step (FP32): read X (12 B) + write X (12 B)
 BYTES_PER_PARTICLE = 24
 # DRAM traffic (read + write bytes) of the particle phase, move + re-bin
-# (299.6 MB) and deposit (133.5 MB) launches of one step, from ncu captures of
+# (299.4 MB) and deposit (133.7 MB) launches of one step, from ncu captures of
 # the torus workload, keyed by the SHA-256 of the kernel sources they were
 # taken on (a changed kernel reports null until it is captured again).
-MOVE_TRAFFIC = {"f67b6b67bc29ee7f3cf81d685029ab365b6ab17290bf90c694f61e0c4b779a4d": 433.13e6}
+MOVE_TRAFFIC = {"d3225297c04164e4785196ac72a2ad089f8301a0c15c3763a8e9f5dba6d23f0b": 433.02e6}
 FALLBACK_HBM_GBS = 6800.0
-# Warp-instructions of one move + re-bin launch (137.17 M) and one deposit
-# launch (96.61 M) at P = 1e7, H = 128, FP32, from the same ncu captures,
+# Warp-instructions of one move + re-bin launch (137.61 M) and one deposit
+# launch (96.77 M) at P = 1e7, H = 128, FP32, from the same ncu captures,
 # keyed like the traffic: the particle kernels against the SMs' issue rate.
-PARTICLE_WARP_INSTR = {"f67b6b67bc29ee7f3cf81d685029ab365b6ab17290bf90c694f61e0c4b779a4d": 233.78e6}
+PARTICLE_WARP_INSTR = {"d3225297c04164e4785196ac72a2ad089f8301a0c15c3763a8e9f5dba6d23f0b": 234.38e6}
 # FP64 form: FP64-pipe thread instructions (DFMA + DADD + DMUL) of one FP64 step
 # at P = 1e7, H = 128 (move 2.010e9, deposit 0.808e9, forward plane 0.112e9,
 # x pass 0.270e9, inverse plane 0.334e9), from an ncu capture of the bench's
 # FP64 leg, keyed by the SHA-256 of the kernel sources it was taken on.
-FP64_PIPE_INSTR = {"cbf35c0a25cad6a8db2738722c4f3355b26d9154c776daad46c76b5ad895c0fa": 3.53359e9}
+FP64_PIPE_INSTR = {"754f56710156764c03334ec91ad342566e5fcc756e69a4ec3d3275f87b16e20e": 3.53359e9}
 
 
 def _env_int(name, default):
